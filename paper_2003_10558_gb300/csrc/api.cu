@@ -188,7 +188,7 @@ vsr_status scene_setup(vsr_scene sc, const float* tris_dev, int64_t T, const flo
     }
     sc->T = T;
     for (int q = 0; q < 12; ++q) sc->cam[q] = cam[q];
-    // the record layout is field-major with stride T: keep it dense
+    // the records are laid out for exactly T triangles
     vsr_status s = launch_setup(tris_dev, (int)T, cam, sc->rec, st);
     sc->gen = g_gen.fetch_add(1);
     return s == VSR_OK ? scene_used(sc, st) : s;

@@ -333,8 +333,8 @@ __global__ void __launch_bounds__(128, CB == 1 ? 12 : (CB == 2 ? 10 : 1)) bin_ke
     float sx = 0.0f, sy = 0.0f, sz = 1.0f, cb = 1.0f, sb = 0.0f;
     int r0 = 0, c0i = 0, ncol = 0, segs = 1, rowpairs = 0, npairs = 0;
     if (lane < TPW && t < T) {
-        const float4 q0 = v.rec[RF_CAP * TT + t];
-        const float4 q1 = v.rec[RF_CAP2 * TT + t];
+        const float4 q0 = v.rec[rec_at(TT, t, RF_CAP)];
+        const float4 q1 = v.rec[rec_at(TT, t, RF_CAP2)];
         if (q1.w != 0.0f) {
             sx = q0.x;
             sy = q0.y;
@@ -649,8 +649,8 @@ __device__ __forceinline__ int tri_col(float lon, int nlon, float cell)
 __device__ __forceinline__ bool tri_cap(const float4* __restrict__ rec, size_t TT, int t, float hmax, int pstep,
                                         float4& q0, float& cb, float& sb)
 {
-    q0 = rec[RF_CAP * TT + t];
-    const float4 q1 = rec[RF_CAP2 * TT + t];
+    q0 = rec[rec_at(TT, t, RF_CAP)];
+    const float4 q1 = rec[rec_at(TT, t, RF_CAP2)];
     if (q1.w == 0.0f) return false;
     if (pstep) {
         const float2 c = pstep_cap(q0.w, q1.x, hmax);

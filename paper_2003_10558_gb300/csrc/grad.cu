@@ -347,8 +347,8 @@ __global__ void __launch_bounds__(TILE_PIX) frag_backward_kernel(BackView v)
         if (dm != 0.0f && x.z > 0.0f && x.z < 1.0f) {
             // the minimising distance (any one of equal minima is a valid
             // subgradient); the forward's g_min from its own m^f
-            const float4 n1 = v.rec[RF_N1 * TT + t], n2 = v.rec[RF_N2 * TT + t], n3 = v.rec[RF_N3 * TT + t];
-            const float4 cp = v.rec[RF_CAP * TT + t], cp2 = v.rec[RF_CAP2 * TT + t];
+            const float4 n1 = v.rec[rec_at(TT, t, RF_N1)], n2 = v.rec[rec_at(TT, t, RF_N2)], n3 = v.rec[rec_at(TT, t, RF_N3)];
+            const float4 cp = v.rec[rec_at(TT, t, RF_CAP)], cp2 = v.rec[rec_at(TT, t, RF_CAP2)];
             const float g1 = dot3f(g.x, g.y, g.z, n1), g2 = dot3f(g.x, g.y, g.z, n2), g3 = dot3f(g.x, g.y, g.z, n3);
             const float mx = g.x - cp.x, my = g.y - cp.y, mz = g.z - cp.z;
             const float g4 = (cp2.y - fmaf(mx, mx, fmaf(my, my, mz * mz))) * cp2.z;
@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(TILE_PIX) frag_backward_kernel(BackView v)
             }
         }
         if (dsh != 0.0f) {
-            const float4 pl = v.rec[RF_PL * TT + t];
+            const float4 pl = v.rec[rec_at(TT, t, RF_PL)];
             const float u = dot3f(g.x, g.y, g.z, pl);
             const float col = v.colors ? v.colors[t] : 1.0f;
             const float du = u > 0.0f ? dsh * col : (u < 0.0f ? -dsh * col : 0.0f);
@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(TILE_PIX) frag_backward_kernel(BackView v)
     if (dD != 0.0f && v.id) {
         const uint32_t t = v.id[o];
         if (t < (uint32_t)v.T) {
-            const float4 pl = v.rec[RF_PL * TT + t];
+            const float4 pl = v.rec[rec_at(TT, t, RF_PL)];
             const float u = dot3f(g.x, g.y, g.z, pl);
             const float r = pl.w / u;
             const float dGN = -dD * r / u;
@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(128) setup_backward_kernel(const float* __rest
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= T) return;
     const size_t TT = (size_t)T;
-    const float4 cp2 = rec[RF_CAP2 * TT + t];
+    const float4 cp2 = rec[rec_at(TT, t, RF_CAP2)];
     float* out = dtris ? dtris + (size_t)t * 9 : nullptr;
     const float4 gpl = grad[GF_PL * TT + t];
     if (dcolors) dcolors[t] = cp2.w != 0.0f ? gpl.w : 0.0f;
@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(128) setup_backward_kernel(const float* __rest
         dV[q] = f3(0.0f, 0.0f, 0.0f);
     }
     // edge normals
-    const float4 n1s = rec[RF_N1 * TT + t];
+    const float4 n1s = rec[rec_at(TT, t, RF_N1)];
     const F3 x0 = cross(V[0], V[1]);
     const float sigma = dot(xyz(n1s), x0) < 0.0f ? -1.0f : 1.0f;
 #pragma unroll

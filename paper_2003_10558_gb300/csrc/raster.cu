@@ -567,7 +567,7 @@ __global__ void __launch_bounds__(RT) raster_dense_kernel(RasterView view, int* 
         __syncthreads();
         if ((int)threadIdx.x < n) {
             const uint32_t t = (uint32_t)(base + threadIdx.x);
-            if (view.rec[RF_CAP2 * TT + t].w == 0.0f)  // culled at set-up
+            if (view.rec[rec_at(TT, t, RF_CAP2)].w == 0.0f)  // culled at set-up
                 st.s6[threadIdx.x] = make_float4(0.0f, 0.0f, 0.0f, __uint_as_float(STAGE_EMPTY));
             else
                 stage_triangle(view.rec, TT, t, ax, ay, az, st, threadIdx.x);

@@ -172,23 +172,29 @@ __global__ void __launch_bounds__(128, VSR_SETUP_PAIR_CTAS) setup_pair_kernel(co
         const bool bad = c ? bad1 : bad0;
         auto pick = [c](float2 v) { return c ? v.y : v.x; };
         if (bad) {
+            const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
-            for (int f = 0; f < REC_F; ++f) rec[f * TT + t] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            for (int f = 0; f < REC_F; f += 2) st_f8(rec + rec_at(TT, t, f), z, z);
             continue;
         }
         const unsigned ties = first_positive_c(pick(n1.x.hi), pick(n1.y.hi), pick(n1.z.hi)) |
                               (first_positive_c(pick(n2.x.hi), pick(n2.y.hi), pick(n2.z.hi)) << 1) |
                               (first_positive_c(pick(n3.x.hi), pick(n3.y.hi), pick(n3.z.hi)) << 2);
-        rec[RF_CAP * TT + t] = make_float4(pick(Sh.x.hi), pick(Sh.y.hi), pick(Sh.z.hi), pick(slen.hi));
-        rec[RF_CAP2 * TT + t] = make_float4(pick(sr.hi), pick(K), pick(inv2sr), 1.0f);
-        rec[RF_N1 * TT + t] = make_float4(pick(n1.x.hi), pick(n1.y.hi), pick(n1.z.hi), __uint_as_float(ties));
-        rec[RF_N2 * TT + t] = make_float4(pick(n2.x.hi), pick(n2.y.hi), pick(n2.z.hi), 0.0f);
-        rec[RF_N3 * TT + t] = make_float4(pick(n3.x.hi), pick(n3.y.hi), pick(n3.z.hi), 0.0f);
-        rec[RF_PL * TT + t] = make_float4(pick(Nh.x.hi), pick(Nh.y.hi), pick(Nh.z.hi), pick(dN.hi));
-        rec[RF_N1L * TT + t] = make_float4(pick(n1.x.lo), pick(n1.y.lo), pick(n1.z.lo), pick(Sh.x.lo));
-        rec[RF_N2L * TT + t] = make_float4(pick(n2.x.lo), pick(n2.y.lo), pick(n2.z.lo), pick(Sh.y.lo));
-        rec[RF_N3L * TT + t] = make_float4(pick(n3.x.lo), pick(n3.y.lo), pick(n3.z.lo), pick(Sh.z.lo));
-        rec[RF_PLL * TT + t] = make_float4(pick(Nh.x.lo), pick(Nh.y.lo), pick(Nh.z.lo), 0.0f);
+        st_f8(rec + rec_at(TT, t, RF_CAP),
+              make_float4(pick(Sh.x.hi), pick(Sh.y.hi), pick(Sh.z.hi), pick(slen.hi)),
+              make_float4(pick(sr.hi), pick(K), pick(inv2sr), 1.0f));
+        st_f8(rec + rec_at(TT, t, RF_N1),
+              make_float4(pick(n1.x.hi), pick(n1.y.hi), pick(n1.z.hi), __uint_as_float(ties)),
+              make_float4(pick(n2.x.hi), pick(n2.y.hi), pick(n2.z.hi), 0.0f));
+        st_f8(rec + rec_at(TT, t, RF_N3),
+              make_float4(pick(n3.x.hi), pick(n3.y.hi), pick(n3.z.hi), 0.0f),
+              make_float4(pick(Nh.x.hi), pick(Nh.y.hi), pick(Nh.z.hi), pick(dN.hi)));
+        st_f8(rec + rec_at(TT, t, RF_N1L),
+              make_float4(pick(n1.x.lo), pick(n1.y.lo), pick(n1.z.lo), pick(Sh.x.lo)),
+              make_float4(pick(n2.x.lo), pick(n2.y.lo), pick(n2.z.lo), pick(Sh.y.lo)));
+        st_f8(rec + rec_at(TT, t, RF_N3L),
+              make_float4(pick(n3.x.lo), pick(n3.y.lo), pick(n3.z.lo), pick(Sh.z.lo)),
+              make_float4(pick(Nh.x.lo), pick(Nh.y.lo), pick(Nh.z.lo), 0.0f));
     }
 }
 

@@ -30,12 +30,12 @@ constexpr uint32_t STAGE_EMPTY = 0xffffffffu;  // s6.w of a slot that holds no t
 __device__ __forceinline__ void stage_triangle(const float4* __restrict__ rec, size_t TT, uint32_t t, float ax,
                                                float ay, float az, Stage& st, int j)
 {
-    const float4 cp = rec[RF_CAP * TT + t];
-    const float4 cp2 = rec[RF_CAP2 * TT + t];
-    const float4 n1 = rec[RF_N1 * TT + t], n2 = rec[RF_N2 * TT + t], n3 = rec[RF_N3 * TT + t];
-    const float4 pl = rec[RF_PL * TT + t];
-    const float4 l1 = rec[RF_N1L * TT + t], l2 = rec[RF_N2L * TT + t], l3 = rec[RF_N3L * TT + t];
-    const float4 ll = rec[RF_PLL * TT + t];
+    const F8 n12 = ld_f8(rec + rec_at(TT, t, RF_N1)), n3p = ld_f8(rec + rec_at(TT, t, RF_N3));
+    const F8 l12 = ld_f8(rec + rec_at(TT, t, RF_N1L)), l3p = ld_f8(rec + rec_at(TT, t, RF_N3L));
+    const F8 cap = ld_f8(rec + rec_at(TT, t, RF_CAP));
+    const float4 &n1 = n12.a, &n2 = n12.b, &n3 = n3p.a, &pl = n3p.b;
+    const float4 &l1 = l12.a, &l2 = l12.b, &l3 = l3p.a, &ll = l3p.b;
+    const float4 &cp = cap.a, &cp2 = cap.b;
     const float c1 = dot_f_df(ax, ay, az, {{n1.x, l1.x}, {n1.y, l1.y}, {n1.z, l1.z}});
     const float c2 = dot_f_df(ax, ay, az, {{n2.x, l2.x}, {n2.y, l2.y}, {n2.z, l2.z}});
     const float c3 = dot_f_df(ax, ay, az, {{n3.x, l3.x}, {n3.y, l3.y}, {n3.z, l3.z}});

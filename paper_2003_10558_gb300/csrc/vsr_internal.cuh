@@ -13,22 +13,51 @@ constexpr int TILE = 16;
 constexpr int TILE_PIX = TILE * TILE;
 
 // ---------------------------------------------------------------------------
-// Per-triangle set-up record: REC_F float4 fields stored field-major
-// (field f of triangle t at rec[f * T + t]) so that the binner reads its two
-// cap fields coalesced.
+// Per-triangle set-up record: REC_F float4 fields in two arrays, the bodies
+// (8 fields, one 128-byte line per triangle) first, then the caps (2 fields,
+// one 32-byte sector per triangle).  The raster gathers the records of the
+// triangles of a bin, in no order of memory: a record is five whole sectors
+// (with every field in an array of its own it was ten half-used ones).  The
+// binner reads the caps alone, coalesced.
 enum {
-    RF_CAP = 0,   // (S-hat.hi xyz, cos rho)            miter cap centre and radius
-    RF_CAP2 = 1,  // (sin rho, 2(1 - cos rho), 1/(2 sin rho), valid ? 1 : 0)
-    RF_N1 = 2,    // (n_AB.hi xyz, tie flags)          edge normals, FP32 high parts
-    RF_N2 = 3,    // (n_BC.hi xyz, 0)
-    RF_N3 = 4,    // (n_CA.hi xyz, 0)
-    RF_PL = 5,    // (N-hat.hi xyz, (A'.N)/|N|)         plane for the ray-plane depth
-    RF_N1L = 6,   // (n_AB.lo xyz, S-hat.lo.x)          low parts
-    RF_N2L = 7,   // (n_BC.lo xyz, S-hat.lo.y)
-    RF_N3L = 8,   // (n_CA.lo xyz, S-hat.lo.z)
-    RF_PLL = 9,   // (N-hat.lo xyz, 0)
+    RF_N1 = 0,   // body: (n_AB.hi xyz, tie flags)      edge normals, FP32 high parts
+    RF_N2 = 1,   // (n_BC.hi xyz, 0)
+    RF_N3 = 2,   // (n_CA.hi xyz, 0)
+    RF_PL = 3,   // (N-hat.hi xyz, (A'.N)/|N|)         plane for the ray-plane depth
+    RF_N1L = 4,  // (n_AB.lo xyz, S-hat.lo.x)          low parts
+    RF_N2L = 5,  // (n_BC.lo xyz, S-hat.lo.y)
+    RF_N3L = 6,  // (n_CA.lo xyz, S-hat.lo.z)
+    RF_PLL = 7,  // (N-hat.lo xyz, 0)
+    REC_BODY = 8,
+    RF_CAP = 8,  // cap: (S-hat.hi xyz, cos rho)        miter cap centre and radius
+    RF_CAP2 = 9, // (sin rho, 2(1 - cos rho), 1/(2 sin rho), valid ? 1 : 0)
     REC_F = 10
 };
+// field f of triangle t in the records of TT triangles
+__host__ __device__ __forceinline__ size_t rec_at(size_t TT, size_t t, int f)
+{
+    return f < REC_BODY ? REC_BODY * t + f : REC_BODY * TT + (REC_F - REC_BODY) * t + (f - REC_BODY);
+}
+
+// Two consecutive fields (32 bytes, 32-byte aligned: an even field) in one
+// 256-bit access of sm_100+.
+struct __align__(16) F8 {
+    float4 a, b;
+};
+__device__ __forceinline__ F8 ld_f8(const float4* p)
+{
+    F8 v;
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(v.a.x), "=f"(v.a.y), "=f"(v.a.z), "=f"(v.a.w), "=f"(v.b.x), "=f"(v.b.y), "=f"(v.b.z), "=f"(v.b.w)
+        : "l"(p));
+    return v;
+}
+__device__ __forceinline__ void st_f8(float4* p, const float4& a, const float4& b)
+{
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(a.x), "f"(a.y), "f"(a.z),
+                 "f"(a.w), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w)
+                 : "memory");
+}
 
 // tie flags in RF_N1.w (as integer bits): bit i set <=> the first nonzero
 // component of edge normal i is positive (simulation-of-simplicity rule for
