@@ -147,3 +147,17 @@ __device__ __forceinline__ df3_2 df3_2_sel(bool cx, bool cy, df3_2 a, df3_2 b)
 {
     return {df2_sel(cx, cy, a.x, b.x), df2_sel(cx, cy, a.y, b.y), df2_sel(cx, cy, a.z, b.z)};
 }
+
+// dot_f_df of the FP32 vector a with two double-word vectors at once (b's
+// components x and y), bit for bit the scalar function's results.
+__device__ __forceinline__ float2 dot_f_df2(float ax, float ay, float az, df3_2 b)
+{
+    const df2 p = two_prod2(f2(ax), b.x.hi);
+    const df2 q = two_prod2(f2(ay), b.y.hi);
+    const df2 r = two_prod2(f2(az), b.z.hi);
+    const df2 s = two_sum2(p.hi, q.hi);
+    const df2 t = two_sum2(s.hi, r.hi);
+    const float2 err = add2(add2(add2(p.lo, q.lo), add2(r.lo, s.lo)), t.lo);
+    const float2 lo = fma2(f2(ax), b.x.lo, fma2(f2(ay), b.y.lo, mul2(f2(az), b.z.lo)));
+    return add2(t.hi, add2(err, lo));
+}

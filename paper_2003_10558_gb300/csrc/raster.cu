@@ -85,60 +85,85 @@ __device__ __forceinline__ bool cone_may_hit(const float4& a, const float4& b, c
                                   fmaf(c0.x, n3.x, fmaf(c0.y, n3.y, c0.z * n3.z)) > lim));
 }
 
-// View cone of a group of WIDTH lanes (xor-shuffle width; 32: the warp's
-// block) from the lanes' valid pixels: axis = normalised sum, cos alpha = min G.axis less a margin, h =
-// the widest ramp half-width; a group without a valid pixel gets valid = 0,
-// a degenerate sum the whole sphere.
-template <int WIDTH>
-__device__ __forceinline__ void group_cone(const float* gx, const float* gy, const float* gz, const float* h,
+// View cone of the warp's 8x8 block from its valid pixels: axis = normalised
+// sum, cos alpha = min G.axis less a margin, h = the widest ramp half-width;
+// a block without a valid pixel gets valid = 0, a degenerate sum the whole
+// sphere.  The cone only culls, so the sums may be taken in any order: the
+// axis by shuffles, the two extrema by the integer reductions of sm_80+
+// (non-negative floats order as their bits; the minimum of G.axis <= 1 + a
+// few ulp as the maximum of 2 - G.axis, whose rounding of 1.2e-7 the margin
+// covers).
+__device__ __forceinline__ void block_cone(const float* gx, const float* gy, const float* gz, const float* h,
                                            const bool* pv, float4& c0, float4& c1)
 {
-    float sx = 0.0f, sy = 0.0f, sz = 0.0f, cn = 0.0f, hw = 0.0f;
+    const unsigned FULL = 0xffffffffu;
+    const int cn = __popc(__ballot_sync(FULL, pv[0])) + __popc(__ballot_sync(FULL, pv[1]));
+    float sx = 0.0f, sy = 0.0f, sz = 0.0f, hw = 0.0f;
 #pragma unroll
     for (int p = 0; p < PPT; ++p)
         if (pv[p]) {
             sx += gx[p];
             sy += gy[p];
             sz += gz[p];
-            cn += 1.0f;
             hw = fmaxf(hw, h[p]);
         }
 #pragma unroll
-    for (int o = 1; o < WIDTH; o <<= 1) {
-        sx += __shfl_xor_sync(0xffffffffu, sx, o);
-        sy += __shfl_xor_sync(0xffffffffu, sy, o);
-        sz += __shfl_xor_sync(0xffffffffu, sz, o);
-        cn += __shfl_xor_sync(0xffffffffu, cn, o);
-        hw = fmaxf(hw, __shfl_xor_sync(0xffffffffu, hw, o));
+    for (int o = 1; o < 32; o <<= 1) {
+        sx += __shfl_xor_sync(FULL, sx, o);
+        sy += __shfl_xor_sync(FULL, sy, o);
+        sz += __shfl_xor_sync(FULL, sz, o);
     }
-    const float len = sqrtf(sx * sx + sy * sy + sz * sz);
-    const bool deg = !(len > 1e-6f * fmaxf(cn, 1.0f));
-    const float ax = deg ? 0.0f : sx / len, ay = deg ? 0.0f : sy / len, az = deg ? 1.0f : sz / len;
-    float cm = 2.0f;
+    hw = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(hw)));
+    const float len2 = fmaf(sx, sx, fmaf(sy, sy, sz * sz));
+    const bool deg = !(len2 > 1e-12f * (float)(cn * cn));
+    const float inv = rsqrtf(len2);
+    const float ax = deg ? 0.0f : sx * inv, ay = deg ? 0.0f : sy * inv, az = deg ? 1.0f : sz * inv;
+    float away = 0.0f;
 #pragma unroll
     for (int p = 0; p < PPT; ++p)
-        if (pv[p]) cm = fminf(cm, gx[p] * ax + gy[p] * ay + gz[p] * az);
-#pragma unroll
-    for (int o = 1; o < WIDTH; o <<= 1) cm = fminf(cm, __shfl_xor_sync(0xffffffffu, cm, o));
+        if (pv[p]) away = fmaxf(away, 2.0f - fmaf(gx[p], ax, fmaf(gy[p], ay, gz[p] * az)));
+    const float cm = 2.0f - __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(away)));
     float cs = fmaxf(-1.0f, fminf(1.0f, cm - 2e-6f));
     if (deg) cs = -1.0f;
     c0 = make_float4(ax, ay, az, cs);
-    c1 = make_float4(sqrtf(fmaxf(0.0f, 1.0f - cs * cs)), hw, cn > 0.0f ? 1.0f : 0.0f, 0.0f);
+    c1 = make_float4(sqrtf(fmaxf(0.0f, 1.0f - cs * cs)), hw, cn > 0 ? 1.0f : 0.0f, 0.0f);
 }
 
 // One lane's two pixels as the evaluation sees them.
 struct PixPair {
-    float2 dgx, dgy, dgz;  // G - a (tile axis) of both pixels
+    float2 dgx, dgy, dgz;  // G - a (tile axis) of both pixels; 0 at an invalid pixel
     float2 eg;             // |G|^2 - 1
     float delta[PPT];      // global delta (0: invalid pixel)
     float lim[PPT];        // fragment iff min distance > lim (-1/(2 delta); +inf if invalid)
-    uint32_t acc[PPT];     // coverage, 2^-22 fixed point
-    unsigned long long key[PPT];  // (bits(r) << 32) | t of the nearest centre-inside fragment
+    uint32_t acc[PPT];     // coverage, 2^-22 fixed point (not meaningful at an invalid pixel)
+    unsigned long long key[PPT];  // ((bits(r) - 1) << 32) | t of the nearest centre-inside fragment, or KEY_NONE
     int32_t cnt_in[PPT];   // centre-inside fragments (statistics)
 };
+// A depth 0 < r < inf has bits(r) - 1 < DEPTH_LIM (unsigned; NaN, zeros and
+// negative numbers do not), so a key below KEY_NONE is a valid depth's.
+constexpr uint32_t DEPTH_LIM = 0x7f7fffffu;
+constexpr unsigned long long KEY_NONE = (unsigned long long)DEPTH_LIM << 32;
+
+// 1/x to the precision of the hardware's reciprocal; x neither denormal nor
+// above 2^126: the quotient a * rcp_fast(x) is then __fdividef(a, x) bit for
+// bit, without the instructions that scale its operands.
+__device__ __forceinline__ float rcp_fast(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
 
 // Evaluate staged slot j at the lane's two pixels and merge the fragments into the pixels' coverage and keys.
 // Called by all 32 lanes of a warp together (warp votes).
+//
+// Issue-bound, the compares and selects (ALU pipe, half rate) above all.  So:
+// the coverage of a lane without a fragment is added too (its ramp value
+// rounds to 0 in the 2^-22 fixed point: gm <= -1/(2 delta) rounded leaves at
+// most 2^-25 after the 1/2); the depth test is folded into the key, whose
+// high word is bits(r) - 1; and everything rare -- a distance exactly on an
+// edge plane (tie rule), a plane distance too small for the plain reciprocal
+// -- is one warp-uniform decision to run the general copy.
 template <bool STATS>
 __device__ __forceinline__ void eval_slot(const Stage& st, int j, PixPair& q, uint32_t& cnt_alg)
 {
@@ -152,7 +177,7 @@ __device__ __forceinline__ void eval_slot(const Stage& st, int j, PixPair& q, ui
     const float2 g2p = plane_distance2(q.dgx, q.dgy, q.dgz, st.s3[j]);
     const float2 g3p = plane_distance2(q.dgx, q.dgy, q.dgz, st.s4[j]);
     const float g4[PPT] = {g4p.x, g4p.y};
-    float g3m[PPT] = {fminf(fminf(g1p.x, g2p.x), g3p.x), fminf(fminf(g1p.y, g2p.y), g3p.y)};
+    const float g3m[PPT] = {fminf(fminf(g1p.x, g2p.x), g3p.x), fminf(fminf(g1p.y, g2p.y), g3p.y)};
     float gm[PPT];
     bool frag[PPT], anyf = false;
 #pragma unroll
@@ -164,55 +189,72 @@ __device__ __forceinline__ void eval_slot(const Stage& st, int j, PixPair& q, ui
     }
     if (!__any_sync(0xffffffffu, anyf)) return;
     const float2 Dp = plane_distance2(q.dgx, q.dgy, q.dgz, st.s5[j]);
-    const float D2[PPT] = {Dp.x, Dp.y};
-    const float dgx[PPT] = {q.dgx.x, q.dgx.y}, dgy[PPT] = {q.dgy.x, q.dgy.y}, dgz[PPT] = {q.dgz.x, q.dgz.y};
-    const unsigned long long tbits = (unsigned long long)__float_as_uint(e.w);
-    // The exact-zero tie rule needs its branch only where some pixel of
-    // the warp has a fragment on an edge plane (rare): decide once for
-    // the warp, and run a copy of the loop without the branch otherwise.
-    auto post = [&](auto tie_t) {
-        constexpr bool TIE = decltype(tie_t)::value;
-        float rr[PPT];
+    const float D[PPT] = {Dp.x, Dp.y};
+    auto post = [&](auto rare_t) {
+        constexpr bool RARE = decltype(rare_t)::value;
+        uint32_t rq[PPT];
         bool inn[PPT];
 #pragma unroll
         for (int p = 0; p < PPT; ++p) {
-            // predicated: every lane computes, non-fragments add nothing
-            const float r = __fdividef(b.w, D2[p]);
-            // 0 < r < inf (NaN excluded) as one unsigned compare of the bits
-            const bool f = frag[p] && __float_as_uint(r) - 1u < 0x7f7fffffu;
+            const float r = RARE ? __fdividef(b.w, D[p]) : __fmul_rn(b.w, rcp_fast(D[p]));
+            rq[p] = __float_as_uint(r) - 1u;
             const float m = __saturatef(fmaf(gm[p], q.delta[p], 0.5f));
-            q.acc[p] += f ? cov_fixed(m) : 0u;
+            if (rq[p] < DEPTH_LIM) q.acc[p] += cov_fixed(m);
             // centre-inside: all three edge distances >= 0; an exact zero
             // takes the tie rule on the three distances, recomputed from
             // the staged planes (the scalar form gives the packed values
             // bit for bit), so they need not stay live in registers here
-            bool in = f && g3m[p] > 0.0f;
-            if (TIE && f && g3m[p] == 0.0f)
-                in = centre_inside(plane_distance(dgx[p], dgy[p], dgz[p], st.s2[j]),
-                                   plane_distance(dgx[p], dgy[p], dgz[p], st.s3[j]),
-                                   plane_distance(dgx[p], dgy[p], dgz[p], st.s4[j]), g3m[p],
-                                   __float_as_uint(st.s0[j].w));
-            rr[p] = r;
-            inn[p] = in;
-            if (STATS) q.cnt_in[p] += in;
+            inn[p] = frag[p] && g3m[p] > 0.0f;
+            if (RARE && frag[p] && g3m[p] == 0.0f) {
+                const float dx = p ? q.dgx.y : q.dgx.x, dy = p ? q.dgy.y : q.dgy.x, dz = p ? q.dgz.y : q.dgz.x;
+                inn[p] = centre_inside(plane_distance(dx, dy, dz, st.s2[j]), plane_distance(dx, dy, dz, st.s3[j]),
+                                       plane_distance(dx, dy, dz, st.s4[j]), g3m[p], __float_as_uint(st.s0[j].w));
+            }
+            if (STATS) q.cnt_in[p] += inn[p] && rq[p] < DEPTH_LIM;
         }
         // the visibility keys only where some lane of the warp has a
         // centre-inside fragment
         if (__any_sync(0xffffffffu, inn[0] || inn[1])) {
 #pragma unroll
             for (int p = 0; p < PPT; ++p) {
-                const unsigned long long k = ((unsigned long long)__float_as_uint(rr[p]) << 32) | tbits;
+                const unsigned long long k = ((unsigned long long)rq[p] << 32) | __float_as_uint(e.w);
                 q.key[p] = inn[p] && k < q.key[p] ? k : q.key[p];
             }
         }
     };
-    bool z = false;
-#pragma unroll
-    for (int p = 0; p < PPT; ++p) z |= frag[p] && g3m[p] == 0.0f;
-    if (__any_sync(0xffffffffu, z))
+    const float tiny = fminf(fminf(fabsf(g3m[0]), fabsf(g3m[1])), fminf(fabsf(D[0]), fabsf(D[1])));
+    if (__any_sync(0xffffffffu, tiny < 1.17549435e-38f))
         post(std::true_type{});
     else
         post(std::false_type{});
+}
+
+// The pixel pair's loop state from its directions (xyz, delta) and the tile
+// axis; invalid pixels (delta 0) evaluate at the axis and never pass.
+__device__ __forceinline__ void pix_pair(PixPair& q, const float4& g0, const float4& g1, float ax, float ay, float az)
+{
+    const bool v0 = g0.w > 0.0f, v1 = g1.w > 0.0f;
+    q.dgx = make_float2(v0 ? g0.x - ax : 0.0f, v1 ? g1.x - ax : 0.0f);
+    q.dgy = make_float2(v0 ? g0.y - ay : 0.0f, v1 ? g1.y - ay : 0.0f);
+    q.dgz = make_float2(v0 ? g0.z - az : 0.0f, v1 ? g1.z - az : 0.0f);
+    const float2 eg = norm2_minus_one2(make_float2(g0.x, g1.x), make_float2(g0.y, g1.y), make_float2(g0.z, g1.z));
+    q.eg = make_float2(v0 ? eg.x : 0.0f, v1 ? eg.y : 0.0f);
+    q.delta[0] = g0.w;
+    q.delta[1] = g1.w;
+    q.lim[0] = v0 ? -(0.5f / g0.w) : INFINITY;
+    q.lim[1] = v1 ? -(0.5f / g1.w) : INFINITY;
+#pragma unroll
+    for (int p = 0; p < PPT; ++p) {
+        q.acc[p] = 0u;
+        q.key[p] = KEY_NONE;
+        q.cnt_in[p] = 0;
+    }
+}
+
+// Coverage of a finished pixel: saturated, 0 at an invalid pixel.
+__device__ __forceinline__ uint32_t final_acc(const PixPair& q, int p)
+{
+    return q.lim[p] < INFINITY ? min(q.acc[p], COV_ONE) : 0u;
 }
 
 // ROWS: the outputs go through shared memory and leave in whole tile rows
@@ -245,35 +287,25 @@ __device__ __forceinline__ void raster_tile(const RasterView& view, int tile, St
     const Cone tc = tiles[tile];
     const float ax = tc.c0.x, ay = tc.c0.y, az = tc.c0.z;
 
-    float gx[PPT], gy[PPT], gz[PPT], h[PPT];
-    bool pv[PPT], inimg[PPT];
+    bool inimg[PPT];
     PixPair q;
-#pragma unroll
-    for (int p = 0; p < PPT; ++p) {
-        const int py = py0 + 4 * p;
-        inimg[p] = px < W && py < H;
-        float4 g = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (inimg[p]) g = map[(size_t)py * W + px];
-        pv[p] = g.w > 0.0f;
-        gx[p] = g.x;
-        gy[p] = g.y;
-        gz[p] = g.z;
-        h[p] = pv[p] ? 0.5f / g.w : 0.0f;
-        q.delta[p] = g.w;
-        q.lim[p] = pv[p] ? -h[p] : INFINITY;
-        q.acc[p] = 0u;
-        q.key[p] = ~0ull;
-        q.cnt_in[p] = 0;
-    }
-    q.dgx = make_float2(gx[0] - ax, gx[1] - ax);
-    q.dgy = make_float2(gy[0] - ay, gy[1] - ay);
-    q.dgz = make_float2(gz[0] - az, gz[1] - az);
-    q.eg = make_float2(pv[0] ? norm2_minus_one(gx[0], gy[0], gz[0]) : 0.0f,
-                       pv[1] ? norm2_minus_one(gx[1], gy[1], gz[1]) : 0.0f);
-
     // the warp's own view cone (its 8x8 pixels)
     float4 wc0, wc1;
-    group_cone<32>(gx, gy, gz, h, pv, wc0, wc1);
+    {
+        float4 g[PPT];
+#pragma unroll
+        for (int p = 0; p < PPT; ++p) {
+            const int py = py0 + 4 * p;
+            inimg[p] = px < W && py < H;
+            g[p] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (inimg[p]) g[p] = map[(size_t)py * W + px];
+        }
+        pix_pair(q, g[0], g[1], ax, ay, az);
+        const float gx[PPT] = {g[0].x, g[1].x}, gy[PPT] = {g[0].y, g[1].y}, gz[PPT] = {g[0].z, g[1].z};
+        const bool pv[PPT] = {g[0].w > 0.0f, g[1].w > 0.0f};
+        const float h[PPT] = {pv[0] ? -q.lim[0] : 0.0f, pv[1] ? -q.lim[1] : 0.0f};
+        block_cone(gx, gy, gz, h, pv, wc0, wc1);
+    }
     const bool warp_active = wc1.z > 0.0f;
 
     uint32_t b0 = 0, b1 = 0;
@@ -322,8 +354,9 @@ __device__ __forceinline__ void raster_tile(const RasterView& view, int tile, St
                 keep = cone_may_hit(st.s0[jj], st.s1[jj], st.s2[jj], st.s3[jj], st.s4[jj], wc0, wc1, count_alg);
             unsigned mask = __ballot_sync(0xffffffffu, keep);
             while (mask) {
-                const int j = gbase + __ffs(mask) - 1;
-                mask &= mask - 1;
+                const int k = 31 - __clz(mask);  // any order: from the top, one instruction less than from the bottom
+                mask ^= 1u << k;
+                const int j = gbase + k;
                 if (STATS) ++cnt_exec;
                 eval_slot<STATS>(st, j, q, cnt_alg);
             }
@@ -331,7 +364,7 @@ __device__ __forceinline__ void raster_tile(const RasterView& view, int tile, St
     }
 
 #pragma unroll
-    for (int p = 0; p < PPT; ++p) q.acc[p] = min(q.acc[p], COV_ONE);
+    for (int p = 0; p < PPT; ++p) q.acc[p] = final_acc(q, p);
 
     if (split_slot >= 0) {
         // merge into the tile's slot; the last item to arrive writes it out
@@ -341,7 +374,7 @@ __device__ __forceinline__ void raster_tile(const RasterView& view, int tile, St
 #pragma unroll
         for (int p = 0; p < PPT; ++p) {
             if (q.acc[p]) atomicAdd(&sacc[lp0 + TILE * 4 * p], (unsigned long long)q.acc[p]);
-            if (q.key[p] != ~0ull) atomicMin(&skey[lp0 + TILE * 4 * p], q.key[p]);
+            if (q.key[p] != KEY_NONE) atomicMin(&skey[lp0 + TILE * 4 * p], q.key[p]);
         }
         __threadfence();
         __syncthreads();
@@ -353,7 +386,7 @@ __device__ __forceinline__ void raster_tile(const RasterView& view, int tile, St
 #pragma unroll
         for (int p = 0; p < PPT; ++p) {
             q.acc[p] = (uint32_t)min(atomicExch(&sacc[lp0 + TILE * 4 * p], 0ull), (unsigned long long)COV_ONE);
-            q.key[p] = atomicExch(&skey[lp0 + TILE * 4 * p], ~0ull);
+            q.key[p] = min(atomicExch(&skey[lp0 + TILE * 4 * p], ~0ull), KEY_NONE);
         }
         if (threadIdx.x == 0) split.done[split_slot] = 0u;
     }
@@ -363,9 +396,9 @@ __device__ __forceinline__ void raster_tile(const RasterView& view, int tile, St
         for (int p = 0; p < PPT; ++p) {
             if (!inimg[p]) continue;
             const size_t o = (size_t)(py0 + 4 * p) * W + px;
-            const bool hit = q.key[p] != ~0ull;
+            const bool hit = q.key[p] != KEY_NONE;
             if (out_id) out_id[o] = hit ? (uint32_t)(q.key[p] & 0xffffffffull) : 0xffffffffu;
-            if (out_depth) out_depth[o] = hit ? __uint_as_float((uint32_t)(q.key[p] >> 32)) : INFINITY;
+            if (out_depth) out_depth[o] = hit ? __uint_as_float((uint32_t)(q.key[p] >> 32) + 1u) : INFINITY;
             if (out_cov) out_cov[o] = (float)q.acc[p] * (1.0f / (float)COV_ONE);
             if (STATS && n_inside) n_inside[o] = q.cnt_in[p];
         }
@@ -377,9 +410,9 @@ __device__ __forceinline__ void raster_tile(const RasterView& view, int tile, St
 #pragma unroll
         for (int p = 0; p < PPT; ++p) {
             const int lp = lx + TILE * (ly0 + 4 * p);
-            const bool hit = q.key[p] != ~0ull;
+            const bool hit = q.key[p] != KEY_NONE;
             s_out[0][lp] = hit ? (uint32_t)(q.key[p] & 0xffffffffull) : 0xffffffffu;
-            s_out[1][lp] = hit ? (uint32_t)(q.key[p] >> 32) : __float_as_uint(INFINITY);
+            s_out[1][lp] = hit ? (uint32_t)(q.key[p] >> 32) + 1u : __float_as_uint(INFINITY);
             s_out[2][lp] = __float_as_uint((float)q.acc[p] * (1.0f / (float)COV_ONE));
             if (STATS && n_inside && inimg[p]) n_inside[(size_t)(py0 + 4 * p) * W + px] = q.cnt_in[p];
         }
@@ -534,29 +567,18 @@ __global__ void __launch_bounds__(RT) raster_dense_kernel(RasterView view, int* 
     const Cone tc = view.tiles[tile];
     const float ax = tc.c0.x, ay = tc.c0.y, az = tc.c0.z;
     PixPair q;
-    float gx[PPT], gy[PPT], gz[PPT];
-    bool pv[PPT], inimg[PPT];
+    bool inimg[PPT];
+    {
+        float4 g[PPT];
 #pragma unroll
-    for (int p = 0; p < PPT; ++p) {
-        const int py = py0 + 4 * p;
-        inimg[p] = px < W && py < H;
-        float4 g = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (inimg[p]) g = view.map[(size_t)py * W + px];
-        pv[p] = g.w > 0.0f;
-        gx[p] = g.x;
-        gy[p] = g.y;
-        gz[p] = g.z;
-        q.delta[p] = g.w;
-        q.lim[p] = pv[p] ? -0.5f / g.w : INFINITY;
-        q.acc[p] = 0u;
-        q.key[p] = ~0ull;
-        q.cnt_in[p] = 0;
+        for (int p = 0; p < PPT; ++p) {
+            const int py = py0 + 4 * p;
+            inimg[p] = px < W && py < H;
+            g[p] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (inimg[p]) g[p] = view.map[(size_t)py * W + px];
+        }
+        pix_pair(q, g[0], g[1], ax, ay, az);
     }
-    q.dgx = make_float2(gx[0] - ax, gx[1] - ax);
-    q.dgy = make_float2(gy[0] - ay, gy[1] - ay);
-    q.dgz = make_float2(gz[0] - az, gz[1] - az);
-    q.eg = make_float2(pv[0] ? norm2_minus_one(gx[0], gy[0], gz[0]) : 0.0f,
-                       pv[1] ? norm2_minus_one(gx[1], gy[1], gz[1]) : 0.0f);
     const bool active = tc.c1.z > 0.0f;
     const size_t TT = (size_t)T;
     uint32_t unused = 0;
@@ -585,10 +607,10 @@ __global__ void __launch_bounds__(RT) raster_dense_kernel(RasterView view, int* 
     for (int p = 0; p < PPT; ++p) {
         if (!inimg[p]) continue;
         const size_t o = (size_t)(py0 + 4 * p) * W + px;
-        const uint32_t acc = min(q.acc[p], COV_ONE);
-        const bool hit = q.key[p] != ~0ull;
+        const uint32_t acc = final_acc(q, p);
+        const bool hit = q.key[p] != KEY_NONE;
         if (view.out_id) view.out_id[o] = hit ? (uint32_t)(q.key[p] & 0xffffffffull) : 0xffffffffu;
-        if (view.out_depth) view.out_depth[o] = hit ? __uint_as_float((uint32_t)(q.key[p] >> 32)) : INFINITY;
+        if (view.out_depth) view.out_depth[o] = hit ? __uint_as_float((uint32_t)(q.key[p] >> 32) + 1u) : INFINITY;
         if (view.out_cov) view.out_cov[o] = (float)acc * (1.0f / (float)COV_ONE);
     }
 }

@@ -10,6 +10,7 @@
 #pragma once
 
 #include "df.cuh"
+#include "df2.cuh"
 #include "vsr_internal.cuh"
 
 constexpr int STAGE_CHUNK = 128;  // triangles staged per pass
@@ -36,10 +37,15 @@ __device__ __forceinline__ void stage_triangle(const float4* __restrict__ rec, s
     const float4 &n1 = n12.a, &n2 = n12.b, &n3 = n3p.a, &pl = n3p.b;
     const float4 &l1 = l12.a, &l2 = l12.b, &l3 = l3p.a, &ll = l3p.b;
     const float4 &cp = cap.a, &cp2 = cap.b;
-    const float c1 = dot_f_df(ax, ay, az, {{n1.x, l1.x}, {n1.y, l1.y}, {n1.z, l1.z}});
-    const float c2 = dot_f_df(ax, ay, az, {{n2.x, l2.x}, {n2.y, l2.y}, {n2.z, l2.z}});
-    const float c3 = dot_f_df(ax, ay, az, {{n3.x, l3.x}, {n3.y, l3.y}, {n3.z, l3.z}});
-    const float cN = dot_f_df(ax, ay, az, {{pl.x, ll.x}, {pl.y, ll.y}, {pl.z, ll.z}});
+    // the four centring terms two at a time in packed FP32x2
+    auto pair3 = [](const float4& u, const float4& ul, const float4& w, const float4& wl) {
+        return df3_2{{make_float2(u.x, w.x), make_float2(ul.x, wl.x)},
+                     {make_float2(u.y, w.y), make_float2(ul.y, wl.y)},
+                     {make_float2(u.z, w.z), make_float2(ul.z, wl.z)}};
+    };
+    const float2 c12 = dot_f_df2(ax, ay, az, pair3(n1, l1, n2, l2));
+    const float2 c3N = dot_f_df2(ax, ay, az, pair3(n3, l3, pl, ll));
+    const float c1 = c12.x, c2 = c12.y, c3 = c3N.x, cN = c3N.y;
     st.s0[j] = make_float4(cp.x, cp.y, cp.z, n1.w);
     st.s1[j] = make_float4(cp2.x, cp2.y, cp2.z, pl.w);
     st.s2[j] = make_float4(n1.x, n1.y, n1.z, c1);
@@ -47,10 +53,11 @@ __device__ __forceinline__ void stage_triangle(const float4* __restrict__ rec, s
     st.s4[j] = make_float4(n3.x, n3.y, n3.z, c3);
     st.s5[j] = make_float4(pl.x, pl.y, pl.z, cN);
     // S-hat - a from the pair S-hat (exact differences, then one rounding)
-    const df dsx = df_add(two_sum(cp.x, -ax), df_make(l1.w));
-    const df dsy = df_add(two_sum(cp.y, -ay), df_make(l2.w));
+    const df2 dsxy = df2_add(two_sum2(make_float2(cp.x, cp.y), make_float2(-ax, -ay)),
+                             df2_make(make_float2(l1.w, l2.w)));
     const df dsz = df_add(two_sum(cp.z, -az), df_make(l3.w));
-    st.s6[j] = make_float4(__fadd_rn(dsx.hi, dsx.lo), __fadd_rn(dsy.hi, dsy.lo), __fadd_rn(dsz.hi, dsz.lo),
+    const float2 dxy = add2(dsxy.hi, dsxy.lo);
+    st.s6[j] = make_float4(dxy.x, dxy.y, __fadd_rn(dsz.hi, dsz.lo),
                            __uint_as_float(t));
 }
 
@@ -64,6 +71,16 @@ __device__ __forceinline__ float norm2_minus_one(float x, float y, float z)
     const df s2 = two_sum(s1.hi, pz2.hi);
     const float tail = __fadd_rn(__fadd_rn(__fadd_rn(px2.lo, py2.lo), __fadd_rn(pz2.lo, s1.lo)), s2.lo);
     return __fadd_rn(__fadd_rn(s2.hi, -1.0f), tail);
+}
+
+// the same of two directions at once, bit for bit
+__device__ __forceinline__ float2 norm2_minus_one2(float2 x, float2 y, float2 z)
+{
+    const df2 px2 = two_prod2(x, x), py2 = two_prod2(y, y), pz2 = two_prod2(z, z);
+    const df2 s1 = two_sum2(px2.hi, py2.hi);
+    const df2 s2 = two_sum2(s1.hi, pz2.hi);
+    const float2 tail = add2(add2(add2(px2.lo, py2.lo), add2(pz2.lo, s1.lo)), s2.lo);
+    return add2(add2(s2.hi, f2(-1.0f)), tail);
 }
 
 // Miter distance in the chord form (4 sin^2(rho/2) - |G - S-hat|^2 +
