@@ -213,20 +213,15 @@ int64_t vsr_scene_size(vsr_scene s);
  * accumulated in 2^-22 fixed point and is bit-reproducible.
  * Binning (which triangles may cover which 16x16 tile: the enlarged cap of
  * each triangle against the tile's view cone, the region mask of Sec.
- * 1.1.3): with at most 64 triangles per tile, tile-major (the triangles
- * filed by cap cell, then each tile over the cells in its reach), else
- * triangle-major over the map's tile index (built on the first such
- * binning after each update of the map); both give the same outputs.
- * Scratch (tile bins, the triangle index of the tile-major binning: about
- * 57 MB plus 24 B per triangle) is held by the scene handle.  It is sized
- * with one synchronisation of `stream` the first time and whenever the
- * map's tile count or the scene's T changes; otherwise no call
- * synchronises: the bins
- * grow ahead of need from the pair count of an earlier frame, and a frame
- * that still outgrows them (e.g. after the camera moved) raises
- * VSR_ERR_BIN_OVERFLOW in the device status (vsr_last_device_status) with
- * that frame's outputs incomplete, the next call growing the bins.  A scene
- * must not be rasterized on two streams at the same time. */
+ * 1.1.3): the set-up files its triangles by cap on latitude-longitude grids
+ * of the view sphere, and each tile tests those within its reach.  The first
+ * frame of a shape (the map's tile count, the scene's T) goes through stored
+ * bins, as vsr_bin and vsr_raster_tiles, sized with one synchronisation of
+ * `stream`; later frames bin and rasterize in one launch that stores none,
+ * and do not synchronise.  The outputs are the same.
+ * Scratch (the grid, 28 B per triangle; the bins, sized by the first frame;
+ * accumulators of shared tiles) is held by the scene handle.  A scene must
+ * not be rasterized on two streams at the same time. */
 vsr_status vsr_raster(vsr_map m, vsr_scene s, uint32_t* id_dev, float* depth_dev, float* cov_dev, void* stream);
 
 /* vsr_raster_pstep: vsr_raster with the per-fragment pixel step of Sec.
@@ -243,8 +238,16 @@ vsr_status vsr_raster_pstep(vsr_map m, vsr_scene s, uint32_t* id_dev, float* dep
 /* The two halves of vsr_raster, for callers that reuse one binning:
  * vsr_bin builds the tile bins of (m, s) (as described for vsr_raster);
  * vsr_raster_tiles runs the tile coverage/depth kernel on the current bins
- * and returns VSR_ERR_INVALID_ARG if they were built for another map or an
- * older set-up of the scene. */
+ * (made first, if the last vsr_raster of (m, s) stored none) and returns
+ * VSR_ERR_INVALID_ARG if there is neither a binning nor a vsr_raster of this
+ * map and set-up.
+ * Bins are sized with one synchronisation of `stream` the first time and
+ * whenever the map's tile count or the scene's T changes; otherwise no call
+ * synchronises: the bins grow ahead of need from the pair count of an earlier
+ * binning, and a binning that still outgrows them (e.g. after the camera
+ * moved) raises VSR_ERR_BIN_OVERFLOW in the device status
+ * (vsr_last_device_status) with that frame's outputs incomplete, the next
+ * call growing the bins. */
 vsr_status vsr_bin(vsr_map m, vsr_scene s, void* stream);
 
 /* Diagnostics of one rasterization (all optional, NULL to skip). */
@@ -300,8 +303,8 @@ vsr_status vsr_raster_dense(vsr_map m, vsr_scene s, uint32_t* id_dev, float* dep
 vsr_status vsr_raster_noalloc(vsr_map m, vsr_scene s, uint32_t* id_dev, float* depth_dev, float* cov_dev,
                               int32_t* status_dev, void* stream);
 
-/* Number of (tile, triangle) pairs in the last binning of this scene
- * (synchronises `stream`). */
+/* Number of (tile, triangle) pairs in the last binning of this scene, stored
+ * or not (synchronises `stream`). */
 vsr_status vsr_scene_bin_pairs(vsr_scene s, void* stream, int64_t* pairs);
 
 /* ---- end to end from host memory ------------------------------------------
@@ -311,10 +314,9 @@ vsr_status vsr_scene_bin_pairs(vsr_scene s, void* stream, int64_t* pairs);
  * work scene `s` (a handle from vsr_scene_create, whose device buffers are
  * reused across calls) on `tris_host` ([T][3][3] FP32, host), rasterizes
  * into the map and returns id/depth/cov (W*H each, host; any may be NULL),
- * then synchronises `stream`.  Same outputs as vsr_raster, but always
- * complete: since the call waits for the frame, a frame that outgrew the
- * scene's bins (see vsr_raster) is rendered again with grown bins before it
- * returns, and a bin overflow that persists is returned by the call
+ * then synchronises `stream`.  Same outputs as vsr_raster.  A bin overflow
+ * of a frame through stored bins would be rendered again with grown bins
+ * before the call returns, and one that persists returned by the call
  * (VSR_ERR_BIN_OVERFLOW) instead of being raised in the per-device status.
  * Buffers in pinned host memory mapped into the device's address space
  * (cudaHostAlloc, cudaMallocHost, torch pin_memory) are read and written in
@@ -353,8 +355,8 @@ vsr_status vsr_render_host_wait(vsr_scene s);
 
 /* ---- batched multi-view rendering -------------------------------------------
  * A batch renders V views of one scene as one CUDA graph.  Each view is the
- * chain of vsr_setup (with the view's camera, Sec. 1.1, 1.1.2, 1.1.4), vsr_bin
- * and vsr_raster_tiles on a workspace of its own; the chains are spread over
+ * chain of vsr_setup (with the view's camera, Sec. 1.1, 1.1.2, 1.1.4) and
+ * vsr_raster on a workspace of its own; the chains are spread over
  * S parallel streams inside the graph, so every view keeps its working set
  * in L2 while independent views overlap on the GPU, and no launch pays host
  * overhead.  Outputs per view are those of vsr_raster.
@@ -365,26 +367,28 @@ vsr_status vsr_render_host_wait(vsr_scene s);
  * caller-owned device pointers, [H_v][W_v] each; the arrays themselves or
  * any entry may be NULL).  The first call for a configuration (the same
  * maps, map contents, scene buffer and T, output pointers) renders the
- * views eagerly, synchronises `stream` once to size every view's bins, then
+ * views eagerly (where pooled launches may be kept, with one synchronisation
+ * of `stream` to size every view's bins), then
  * captures graphs of two kinds for each S in {1, 2, 4, 8}: each view's chain
- * ending in its own raster launch, and chains that end after binning and
- * work-item assignment, the views rasterized in G in {1, 4, 16} pooled
+ * ending in its own raster launch, and chains that end after storing their
+ * bins and work items, the views rasterized in G in {1, 4, 16} pooled
  * launches -- persistent CTAs (resident CTAs per SM x SMs) that take the
  * (view, item) work of a group of views from a shared queue (an atomic
  * counter; no CTA waits for another), each group's launch on a stream of its
  * own as soon as its views are binned, beside the next groups' chains.
- * It times their replays, keeps the fastest, then tries 256 and 1024
- * triangles per work item of a long bin at that S and kind (the autotuner;
+ * It times their replays, keeps the fastest, then, if that is a pooled one,
+ * tries 256 and 1024 triangles per work item of a long bin (the autotuner;
  * vsr_batch_set_mode can restrict the kinds); later calls with the same configuration
  * copy only the cameras (into pinned staging of the batch) and replay the
  * graph on `stream`.  Each call waits for the previous frame of the batch to
- * finish; a replay leaves every view's (tile, triangle) pair total in pinned
- * memory, and a call that finds a view within 1/8 of its bin capacity
- * re-sizes the bins and captures again (as for a new configuration).  A
- * frame whose cameras outgrow the bins before that raises
+ * finish.  With pooled launches a replay leaves every view's (tile, triangle)
+ * pair total in pinned memory, and a call that finds a view within 1/8 of its
+ * bin capacity re-sizes the bins and captures again (as for a new
+ * configuration); a frame whose cameras outgrow the bins before that raises
  * VSR_ERR_BIN_OVERFLOW in the device status with its outputs incomplete; the
- * next call grows the bins.  Device memory per view: T x 228 B of set-up
- * records and bin caches plus its bins.  A batch must not render on two
+ * next call grows the bins.  Device memory per view: T x 188 B of set-up
+ * records and triangle grid, 4 MB of accumulators, and for pooled launches
+ * its bins.  A batch must not render on two
  * streams at once. */
 typedef struct vsr_batch_s* vsr_batch;
 vsr_status vsr_batch_create(vsr_batch* out);

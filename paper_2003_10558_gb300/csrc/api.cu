@@ -1,7 +1,7 @@
 // api.cu -- host side of the C ABI declared in include/vsr.h: handles,
 // device memory, argument checks and the launch sequence of one frame
-//   map (once per lens) -> set-up (once per scene/camera) -> bin count ->
-//   scan -> bin fill -> tile raster.
+//   map (once per lens) -> set-up and triangle grid (once per scene/camera)
+//   -> raster (each tile walks the grid, or bins stored before).
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
@@ -176,6 +176,27 @@ vsr_status ensure_tile_index(vsr_map m, cudaStream_t st)
     return s;
 }
 
+// Set-up of T triangles with the camera in host (cam) or device (cam_dev)
+// memory: records, and the triangle grid where it is used.
+vsr_status setup_records(const float* tris_dev, int64_t T, const float* cam, const float* cam_dev, float4* rec,
+                         TriGrid& grid, cudaStream_t st)
+{
+    const TriGrid* g = grid_used(T) ? &grid : nullptr;
+    vsr_status s;
+    if (g) {
+        if ((s = grid_alloc(&grid, T)) != VSR_OK) return s;
+        // until the filing is queued, a failure leaves counters behind
+        const bool was_dirty = grid.dirty;
+        grid.dirty = true;
+        if (was_dirty)
+            VSR_CUDA_TRY(cudaMemsetAsync(grid.counts, 0, sizeof(uint32_t) * ((size_t)GRID_WORDS + GRID_HDR), st));
+    }
+    s = cam_dev ? launch_setup_view(tris_dev, (int)T, cam_dev, rec, g, st)
+                : launch_setup(tris_dev, (int)T, cam, rec, g, st);
+    if (s == VSR_OK && g && (s = launch_grid_file(rec, (int)T, grid, st)) == VSR_OK) grid.dirty = false;
+    return s;
+}
+
 vsr_status scene_setup(vsr_scene sc, const float* tris_dev, int64_t T, const float cam[12], cudaStream_t st)
 {
     if (T > sc->T_alloc) {
@@ -189,45 +210,48 @@ vsr_status scene_setup(vsr_scene sc, const float* tris_dev, int64_t T, const flo
     sc->T = T;
     for (int q = 0; q < 12; ++q) sc->cam[q] = cam[q];
     // the records are laid out for exactly T triangles
-    vsr_status s = launch_setup(tris_dev, (int)T, cam, sc->rec, st);
+    vsr_status s = setup_records(tris_dev, T, cam, nullptr, sc->rec, sc->grid, st);
     sc->gen = g_gen.fetch_add(1);
     return s == VSR_OK ? scene_used(sc, st) : s;
 }
 
-// bin ids and the triangle-major count pass's pair list, both of `want`
-// entries (frees the old ones, which waits for the launches still using
-// them)
+// bin ids, `want` entries (frees the old ones, which waits for the launches
+// still using them)
 vsr_status bins_realloc(vsr_scene sc, uint32_t want)
 {
     cudaFree(sc->ids);
-    cudaFree(sc->pairs);
     sc->ids = nullptr;
-    sc->pairs = nullptr;
     sc->cap = 0;
-    vsr_status s;
-    if ((s = dalloc(&sc->ids, (size_t)want)) != VSR_OK) return s;
-    if ((s = dalloc(&sc->pairs, (size_t)want)) != VSR_OK) {
-        cudaFree(sc->ids);
-        sc->ids = nullptr;
-        return s;
-    }
-    sc->cap = want;
-    return VSR_OK;
+    vsr_status s = dalloc(&sc->ids, (size_t)want);
+    if (s == VSR_OK) sc->cap = want;
+    return s;
 }
 
-vsr_status ensure_ws(vsr_scene sc, int ntiles)
+vsr_status ensure_ws(vsr_scene sc, int ntiles, cudaStream_t st)
 {
+    vsr_status s;
+    if (!sc->bin_ctr) {
+        if ((s = dalloc(&sc->bin_ctr, 2)) != VSR_OK) return s;
+        VSR_CUDA_TRY(cudaMemsetAsync(sc->bin_ctr, 0, 2 * sizeof(uint32_t), st));
+    }
     if (ntiles <= sc->ws_tiles) return VSR_OK;
     cudaFree(sc->ends);
     cudaFree(sc->offsets);
-    sc->ends = sc->offsets = nullptr;
+    cudaFree(sc->tile_pairs);
+    sc->ends = sc->offsets = sc->tile_pairs = nullptr;
     sc->ws_tiles = 0;
-    vsr_status s;
-    if ((s = dalloc(&sc->ends, (size_t)ntiles + 1)) != VSR_OK) return s;  // (+1: the triangle-major pair cursor)
+    if ((s = dalloc(&sc->ends, (size_t)ntiles)) != VSR_OK) return s;
     if ((s = dalloc(&sc->offsets, (size_t)ntiles + 1)) != VSR_OK) return s;
+    if ((s = dalloc(&sc->tile_pairs, (size_t)ntiles)) != VSR_OK) return s;
     sc->ws_tiles = ntiles;
     sc->sized_shape = 0;
     return VSR_OK;
+}
+
+// the bins' sizes depend on the map, the scene and the step's cap width
+uint64_t bin_shape_of(vsr_map m, vsr_scene sc, int pstep)
+{
+    return ((uint64_t)(m->tx * m->ty) << 32) ^ (uint64_t)sc->T ^ ((uint64_t)(pstep != 0) << 63);
 }
 
 }  // namespace
@@ -492,9 +516,11 @@ void vsr_scene_free(vsr_scene sc)
     cudaFree(sc->rec);
     cudaFree(sc->ends);
     cudaFree(sc->offsets);
+    cudaFree(sc->tile_pairs);
+    cudaFree(sc->bin_ctr);
     cudaFree(sc->ids);
-    cudaFree(sc->pairs);
-    tri_index_free(&sc->tri);
+    grid_free(&sc->grid);
+    walk_work_free(&sc->walk);
     raster_work_free(&sc->work);
     cudaFree(sc->tris_dev);
     cudaFree(sc->out_dev);
@@ -531,7 +557,7 @@ vsr_status vsr_raster_pstep(vsr_map m, vsr_scene sc, uint32_t* id_dev, float* de
     vsr_status s = bin_scene(m, sc, 1, st);
     if (s != VSR_OK) return s;
     const RasterView v{m->map,  m->p.W, m->p.H, m->tiles, m->tx,     sc->rec,   (int)sc->T, sc->offsets,
-                       sc->ids, sc->cap, id_dev, depth_dev, cov_dev, scene_ends(sc)};
+                       sc->ids, sc->cap, id_dev, depth_dev, cov_dev, sc->ends};
     s = launch_raster_pstep(v, m->deriv, scene_status(sc), st);
     return s == VSR_OK ? scene_used(sc, st) : s;
 }
@@ -541,27 +567,17 @@ vsr_status vsr_raster_pstep(vsr_map m, vsr_scene sc, uint32_t* id_dev, float* de
 static vsr_status bin_scene(vsr_map m, vsr_scene sc, int pstep, cudaStream_t st)
 {
     const int ntiles = m->tx * m->ty;
-    vsr_status s = ensure_ws(sc, ntiles);
+    vsr_status s = ensure_ws(sc, ntiles, st);
     if (s != VSR_OK) return s;
     const int T = (int)sc->T;
     sc->last_ntiles = ntiles;
-    // The binner: tile-major while the triangles are few per tile (each
-    // tile's warp then walks a short window), else the triangle-major search
-    // over the map's tile index (its work spread over the triangles).
-    sc->tile_major = (int64_t)T <= TILE_MAJOR_TRIS_PER_TILE * (int64_t)ntiles;
-    if (sc->tile_major) {
-        if ((s = tri_index_alloc(&sc->tri, T, ntiles)) != VSR_OK) return s;
-    } else if ((s = ensure_tile_index(m, st)) != VSR_OK) {
-        return s;
-    }
     // Bin capacity.  Sized synchronously the first time and whenever the
     // number of tiles or triangles changes (the first time only, for a scene
     // with async_sizing); otherwise the pair total of the previous binning
     // (copied to pinned memory, read only once its event has completed, never
     // waited for) grows the capacity ahead of need, and the binning kernels
     // report any overflow in the status word.
-    // the bins' sizes depend on the map, the scene and the step's cap width
-    const uint64_t shape = ((uint64_t)ntiles << 32) ^ (uint64_t)sc->T ^ ((uint64_t)(pstep != 0) << 63);
+    const uint64_t shape = bin_shape_of(m, sc, pstep);
     const bool resize = sc->cap == 0 || (!sc->async_sizing && sc->sized_shape != shape);
     if (!resize && sc->total_pending && cudaEventQuery(sc->total_event) == cudaSuccess) {
         sc->total_pending = false;
@@ -576,31 +592,19 @@ static vsr_status bin_scene(vsr_map m, vsr_scene sc, int pstep, cudaStream_t st)
     // unless an earlier total has not been read yet -- and always when this
     // binning sizes the bins, which reads this total
     const bool record = resize || !sc->total_pending;
-    uint32_t* total_host = record ? sc->h_total_dev : nullptr;
-    // triangle-major: per-tile counters and the pair cursor in the end array
-    uint32_t* counts = sc->ends;
-    uint32_t* cursor = counts + ntiles;
-    uint2* pairs = sc->pairs;
-    const uint32_t pair_cap = sc->cap;
-    if (sc->tile_major) {
-        // one pass (a sizing pass reports no overflow: its bins are grown and
-        // binned again)
-        if ((s = launch_bin_tiles(sc->rec, T, m->idx, m->tiles, ntiles, sc->tri, sc->offsets, sc->ends, sc->ids,
-                                  sc->cap, resize ? nullptr : scene_status(sc), total_host, st, pstep)) != VSR_OK)
-            return s;
-    } else {
-        VSR_CUDA_TRY(cudaMemsetAsync(counts, 0, sizeof(uint32_t) * ((size_t)ntiles + 1), st));
-        if ((s = launch_bin_count(sc->rec, T, m->idx, counts, cursor, pairs, pair_cap, st, pstep)) != VSR_OK)
-            return s;
-        if ((s = launch_scan(counts, nullptr, ntiles, nullptr, sc->offsets, st, total_host)) != VSR_OK) return s;
-    }
+    const WalkIndex wi = walk_index(sc->grid, sc->T, pstep);
+    auto walk = [&](int* status, uint32_t* total_host) {
+        return launch_bin_walk(sc->rec, T, wi, m->idx.geom, m->tiles, ntiles, sc->bin_ctr, sc->offsets, sc->ends,
+                               sc->ids, sc->cap, status, total_host, st);
+    };
+    // (a sizing pass reports no overflow: its bins are grown and binned again)
+    if ((s = walk(resize ? nullptr : scene_status(sc), record ? sc->h_total_dev : nullptr)) != VSR_OK) return s;
     if (record) {
         VSR_CUDA_TRY(cudaEventRecord(sc->total_event, st));
         sc->total_pending = true;
         sc->total_map = m->gen;
         sc->total_scene = sc->gen;
     }
-    bool grown = false;
     if (resize) {
         VSR_CUDA_TRY(cudaEventSynchronize(sc->total_event));
         sc->total_pending = false;
@@ -609,21 +613,13 @@ static vsr_status bin_scene(vsr_map m, vsr_scene sc, int pstep, cudaStream_t st)
             uint64_t want = (uint64_t)total + total / 4 + 4096;
             if (want > 0xffffffffull) want = 0xffffffffull;
             if ((s = bins_realloc(sc, (uint32_t)want)) != VSR_OK) return s;
-            pairs = nullptr;  // this frame's pair list went with the old buffer: search again
-            grown = true;
+            if ((s = walk(scene_status(sc), nullptr)) != VSR_OK) return s;
         }
         sc->sized_shape = shape;
     }
-    if (sc->tile_major) {
-        if (grown && (s = launch_bin_tiles(sc->rec, T, m->idx, m->tiles, ntiles, sc->tri, sc->offsets, sc->ends,
-                                           sc->ids, sc->cap, scene_status(sc), nullptr, st, pstep)) != VSR_OK)
-            return s;
-    } else if ((s = launch_bin_fill(sc->rec, T, m->idx, sc->offsets, counts, cursor, pairs, pair_cap, sc->ids,
-                                    sc->cap, scene_status(sc), st, pstep)) != VSR_OK) {
-        return s;
-    }
     sc->binned_map = m->gen;
     sc->binned_scene = sc->gen;
+    sc->walked_last = false;
     return scene_used(sc, st);
 }
 
@@ -632,7 +628,12 @@ static vsr_status raster_tiles(vsr_map m, vsr_scene sc, uint32_t* id_dev, float*
                                const vsr_raster_stats* stats, void* stream, bool host_out)
 {
     if (!m || !sc) return VSR_ERR_INVALID_ARG;
-    if (sc->binned_map != m->gen || sc->binned_scene != sc->gen) return VSR_ERR_INVALID_ARG;
+    if (sc->binned_map != m->gen || sc->binned_scene != sc->gen) {
+        // the last frame of this pair stored no bins: make them now
+        if (sc->walked_map != m->gen || sc->walked_scene != sc->gen) return VSR_ERR_INVALID_ARG;
+        const vsr_status s = bin_scene(m, sc, 0, (cudaStream_t)stream);
+        if (s != VSR_OK) return s;
+    }
     const uint32_t ntiles = (uint32_t)(m->tx * m->ty);
     if (!stats || (!stats->n_alg_dev && !stats->n_exec_dev && !stats->n_inside_dev)) {
         // timed path: work items, large bins split over several CTAs
@@ -644,7 +645,7 @@ static vsr_status raster_tiles(vsr_map m, vsr_scene sc, uint32_t* id_dev, float*
             sc->work_tiles = ntiles;
         }
         const RasterView v{m->map,  m->p.W, m->p.H, m->tiles, m->tx,     sc->rec,   (int)sc->T, sc->offsets,
-                           sc->ids, sc->cap, id_dev, depth_dev, cov_dev, scene_ends(sc)};
+                           sc->ids, sc->cap, id_dev, depth_dev, cov_dev, sc->ends};
         const vsr_status s = launch_raster_items(v, sc->offsets, ntiles, sc->cap, sc->work, SPLIT_MAX_DEFAULT,
                                                  scene_status(sc), (cudaStream_t)stream, host_out);
         return s == VSR_OK ? scene_used(sc, (cudaStream_t)stream) : s;
@@ -654,8 +655,37 @@ static vsr_status raster_tiles(vsr_map m, vsr_scene sc, uint32_t* id_dev, float*
         launch_raster(m->map, m->p.W, m->p.H, m->tiles, sc->rec, (int)sc->T, sc->offsets, sc->ids, sc->cap, id_dev,
                       depth_dev, cov_dev, stats ? (unsigned long long*)stats->n_alg_dev : nullptr,
                       stats ? (unsigned long long*)stats->n_exec_dev : nullptr, stats ? stats->n_inside_dev : nullptr,
-                      scene_status(sc), (cudaStream_t)stream, scene_ends(sc));
+                      scene_status(sc), (cudaStream_t)stream, sc->ends);
     return s == VSR_OK ? scene_used(sc, (cudaStream_t)stream) : s;
+}
+
+// One frame of (m, s) without statistics.  The walking raster needs no bins
+// (1920x1080, 220k triangles: see the figures at raster_walk_kernel), but the
+// first frame of a shape goes through stored ones, as does every frame of a
+// scene that renders again on a bin overflow (async_sizing): the bins are
+// then allocated and sized, with the one synchronisation of a new shape, and
+// a vsr_raster_tiles that follows later needs neither, also under capture.
+static vsr_status raster_frame(vsr_map m, vsr_scene sc, uint32_t* id_dev, float* depth_dev, float* cov_dev,
+                               cudaStream_t st, bool host_out)
+{
+    if (!m || !sc) return VSR_ERR_INVALID_ARG;
+    vsr_status s;
+    if (sc->async_sizing || sc->cap == 0 || sc->sized_shape != bin_shape_of(m, sc, 0)) {
+        if ((s = bin_scene(m, sc, 0, st)) != VSR_OK) return s;
+        return raster_tiles(m, sc, id_dev, depth_dev, cov_dev, nullptr, st, host_out);
+    }
+    const int ntiles = m->tx * m->ty;
+    if ((s = ensure_ws(sc, ntiles, st)) != VSR_OK || (s = walk_work_alloc(&sc->walk, st)) != VSR_OK) return s;
+    const RasterView v{m->map, m->p.W, m->p.H, m->tiles, m->tx,   sc->rec,   (int)sc->T,
+                       nullptr, nullptr, 0u,   id_dev,   depth_dev, cov_dev};
+    if ((s = launch_raster_walk(v, walk_index(sc->grid, sc->T), m->idx.geom, sc->walk, sc->tile_pairs,
+                                scene_status(sc), st, host_out)) != VSR_OK)
+        return s;
+    sc->last_ntiles = ntiles;
+    sc->walked_map = m->gen;
+    sc->walked_scene = sc->gen;
+    sc->walked_last = true;
+    return scene_used(sc, st);
 }
 
 extern "C" {
@@ -679,6 +709,8 @@ vsr_status vsr_raster_dense(vsr_map m, vsr_scene sc, uint32_t* id_dev, float* de
 vsr_status vsr_raster_ex(vsr_map m, vsr_scene sc, uint32_t* id_dev, float* depth_dev, float* cov_dev,
                          const vsr_raster_stats* stats, void* stream)
 {
+    if (!stats || (!stats->n_alg_dev && !stats->n_exec_dev && !stats->n_inside_dev))
+        return raster_frame(m, sc, id_dev, depth_dev, cov_dev, (cudaStream_t)stream, false);
     vsr_status s = vsr_bin(m, sc, stream);
     if (s != VSR_OK) return s;
     return vsr_raster_tiles(m, sc, id_dev, depth_dev, cov_dev, stats, stream);
@@ -695,17 +727,16 @@ vsr_status vsr_scene_bin_pairs(vsr_scene sc, void* stream, int64_t* pairs)
     cudaStream_t st = (cudaStream_t)stream;
     VSR_CUDA_TRY(cudaStreamSynchronize(st));
     const size_t n = (size_t)sc->last_ntiles;
-    if (!sc->tile_major) {  // bins in tile order: the scan's total
+    if (!sc->walked_last) {
         uint32_t v = 0;
         VSR_CUDA_TRY(cudaMemcpy(&v, sc->offsets + n, sizeof(uint32_t), cudaMemcpyDeviceToHost));
         *pairs = v;
         return VSR_OK;
     }
-    std::vector<uint32_t> b0(n), b1(n);
-    VSR_CUDA_TRY(cudaMemcpy(b0.data(), sc->offsets, sizeof(uint32_t) * n, cudaMemcpyDeviceToHost));
-    VSR_CUDA_TRY(cudaMemcpy(b1.data(), sc->ends, sizeof(uint32_t) * n, cudaMemcpyDeviceToHost));
+    std::vector<uint32_t> c(n);
+    VSR_CUDA_TRY(cudaMemcpy(c.data(), sc->tile_pairs, sizeof(uint32_t) * n, cudaMemcpyDeviceToHost));
     int64_t v = 0;
-    for (size_t u = 0; u < n; ++u) v += (int64_t)(b1[u] - b0[u]);
+    for (size_t u = 0; u < n; ++u) v += c[u];
     *pairs = v;
     return VSR_OK;
 }
@@ -811,8 +842,7 @@ vsr_status host_frame_back(vsr_map m, vsr_scene sc, const HostFrame& f, uint32_t
 {
     int* const saved_status = sc->status;
     sc->status = sc->host_status;
-    vsr_status s = vsr_bin(m, sc, st);
-    if (s == VSR_OK) s = raster_tiles(m, sc, f.id_d, f.depth_d, f.cov_d, nullptr, st, f.in_place);
+    vsr_status s = raster_frame(m, sc, f.id_d, f.depth_d, f.cov_d, st, f.in_place);
     sc->status = saved_status;
     if (s == VSR_OK && f.stage_id && cudaMemcpyAsync(id_host, f.id_d, 4 * f.npix, cudaMemcpyDeviceToHost, st))
         s = VSR_ERR_CUDA;
@@ -960,13 +990,11 @@ extern "C" vsr_status vsr_raster_noalloc(vsr_map m, vsr_scene sc, uint32_t* id_d
     // the array keeps the previous call's contents: clear what starts at zero
     VSR_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int), st));
     VSR_CUDA_TRY(cudaMemsetAsync(counts, 0, sizeof(uint32_t) * (size_t)ntiles, st));
-    // the triangle-major search over the map's tile index (no pair list: the
-    // fill searches again)
+    // the triangle-major search over the map's tile index
     if ((s = ensure_tile_index(m, st)) != VSR_OK) return s;
-    if ((s = launch_bin_count(sc->rec, T, m->idx, counts, nullptr, nullptr, 0, st)) != VSR_OK) return s;
-    if ((s = launch_scan(counts, nullptr, ntiles, nullptr, offsets, st)) != VSR_OK) return s;
-    if ((s = launch_bin_fill(sc->rec, T, m->idx, offsets, counts, nullptr, nullptr, 0, ids, NA_PAIRS_MAX, status,
-                             st)) != VSR_OK)
+    if ((s = launch_bin_count(sc->rec, T, m->idx, counts, st)) != VSR_OK) return s;
+    if ((s = launch_scan(counts, ntiles, offsets, st)) != VSR_OK) return s;
+    if ((s = launch_bin_fill(sc->rec, T, m->idx, offsets, counts, ids, NA_PAIRS_MAX, status, st)) != VSR_OK)
         return s;
     if ((s = launch_raster(m->map, m->p.W, m->p.H, m->tiles, sc->rec, T, offsets, ids, NA_PAIRS_MAX, id_dev,
                            depth_dev, cov_dev, nullptr, nullptr, nullptr, status, st)) != VSR_OK)
@@ -979,28 +1007,29 @@ extern "C" vsr_status vsr_raster_noalloc(vsr_map m, vsr_scene sc, uint32_t* id_d
 //
 // V views of one scene as one CUDA graph: each view is a chain of the
 // single-view launches (set-up with the view's camera read from device
-// memory, bin count, scan, bin fill, raster work items) on its own
-// workspace, and the chains are spread over S parallel streams inside the
-// graph, so each view keeps its working set in L2 while independent views
-// overlap on the GPU and no launch pays host overhead.  The first call for a
-// configuration runs the views eagerly (sizing every view's bins with one
+// memory, triangle grid, raster) on its own workspace, and the chains are
+// spread over S parallel streams inside the graph, so each view keeps its
+// working set in L2 while independent views overlap on the GPU and no launch
+// pays host overhead.  The first call for a configuration runs the views
+// eagerly (for pooled rasters, sizing every view's bins with one
 // synchronisation), then captures one graph per candidate (S in {1, 2, 4, 8}
-// streams; the views' own raster launches or 1, 4 or 16 pooled ones; then the
-// work-item size), times their replays and keeps the fastest (the
-// autotuner).  Later calls
-// with the same configuration copy the cameras into pinned staging and
-// replay.
+// streams; the views' own raster launches or 1, 4 or 16 pooled ones over
+// stored bins; then the latter's work-item size), times their replays and
+// keeps the fastest (the autotuner).  Later calls with the same configuration
+// copy the cameras into pinned staging and replay.
 namespace {
 
 constexpr int BATCH_STREAMS_MAX = 8;
 
 struct BatchView {
     float4* rec = nullptr;
-    uint32_t* counts = nullptr;
-    uint32_t* offsets = nullptr;
-    uint32_t* partials = nullptr;
+    TriGrid grid;
+    WalkWork walk;  // split slots of the view's own raster launch
+    // stored bins and work items of the pooled raster launches
+    uint32_t* ctr = nullptr;      // 2, zero between binnings
+    uint32_t* offsets = nullptr;  // tiles + 1
+    uint32_t* ends = nullptr;     // tiles
     uint32_t* ids = nullptr;
-    uint2* pairs = nullptr;  // the count pass's hits, cap entries
     uint32_t cap = 0;
     int tiles = 0;
     int64_t T = 0;
@@ -1010,11 +1039,12 @@ struct BatchView {
 void batch_view_free(BatchView& v)
 {
     cudaFree(v.rec);
-    cudaFree(v.counts);
+    grid_free(&v.grid);
+    walk_work_free(&v.walk);
+    cudaFree(v.ctr);
     cudaFree(v.offsets);
-    cudaFree(v.partials);
+    cudaFree(v.ends);
     cudaFree(v.ids);
-    cudaFree(v.pairs);
     raster_work_free(&v.work);
     v = BatchView{};
 }
@@ -1051,7 +1081,8 @@ struct vsr_batch_s {
 
 namespace {
 
-vsr_status batch_view_alloc(BatchView& v, int64_t T, int tiles)
+// pooled: also the stored bins' workspace
+vsr_status batch_view_alloc(BatchView& v, int64_t T, int tiles, bool pooled, cudaStream_t st)
 {
     vsr_status s;
     if (T > v.T) {
@@ -1061,57 +1092,57 @@ vsr_status batch_view_alloc(BatchView& v, int64_t T, int tiles)
         if ((s = dalloc(&v.rec, (size_t)REC_F * (size_t)T)) != VSR_OK) return s;
         v.T = T;
     }
+    if (grid_used(T) && (s = grid_alloc(&v.grid, T)) != VSR_OK) return s;
+    if (grid_used(T) && v.grid.dirty) {  // here, not inside a capture
+        VSR_CUDA_TRY(cudaMemsetAsync(v.grid.counts, 0, sizeof(uint32_t) * ((size_t)GRID_WORDS + GRID_HDR), st));
+        v.grid.dirty = false;
+    }
+    if ((s = walk_work_alloc(&v.walk, st)) != VSR_OK) return s;
+    if (!pooled) return VSR_OK;
+    if (!v.ctr) {
+        if ((s = dalloc(&v.ctr, 2)) != VSR_OK) return s;
+        VSR_CUDA_TRY(cudaMemsetAsync(v.ctr, 0, 2 * sizeof(uint32_t), st));
+    }
     if (tiles > v.tiles) {
-        cudaFree(v.counts);
         cudaFree(v.offsets);
-        cudaFree(v.partials);
+        cudaFree(v.ends);
         raster_work_free(&v.work);
-        v.counts = v.offsets = v.partials = nullptr;
+        v.offsets = v.ends = nullptr;
         v.tiles = 0;
-        if ((s = dalloc(&v.counts, (size_t)tiles + 1)) != VSR_OK) return s;  // counts | pair cursor
         if ((s = dalloc(&v.offsets, (size_t)tiles + 1)) != VSR_OK) return s;
-        if ((s = dalloc(&v.partials, 2 * (size_t)((tiles + 4095) / 4096) + 2)) != VSR_OK) return s;
+        if ((s = dalloc(&v.ends, (size_t)tiles)) != VSR_OK) return s;
         if ((s = raster_work_alloc(&v.work, (uint32_t)tiles)) != VSR_OK) return s;
         v.tiles = tiles;
     }
     return VSR_OK;
 }
 
-// set-up, count and scan of view v (before its bins are sized); with
-// use_pairs the count records its hits for the fill (not while the bins may
-// still be re-sized)
-vsr_status batch_view_front(vsr_batch b, int v, vsr_map m, const float* tris, int64_t T, bool use_pairs,
-                            cudaStream_t st)
+vsr_status batch_view_setup(vsr_batch b, int v, const float* tris, int64_t T, cudaStream_t st)
 {
     BatchView& bv = b->views[v];
-    const int tiles = m->tx * m->ty;
-    vsr_status s;
-    if ((s = launch_setup_views(tris, (int)T, b->cams_dev + 12 * v, 1, bv.rec, st)) != VSR_OK) return s;
-    VSR_CUDA_TRY(cudaMemsetAsync(bv.counts, 0, sizeof(uint32_t) * ((size_t)tiles + 1), st));
-    if ((s = launch_bin_count(bv.rec, (int)T, m->idx, bv.counts, bv.counts + tiles, use_pairs ? bv.pairs : nullptr,
-                              use_pairs ? bv.cap : 0u, st)) != VSR_OK)
-        return s;
-    return tiles <= 65536 ? launch_scan(bv.counts, nullptr, tiles, nullptr, bv.offsets, st)
-                          : launch_scan_large(bv.counts, nullptr, tiles, bv.partials, bv.offsets, st);
+    return setup_records(tris, T, nullptr, b->cams_dev + 12 * v, bv.rec, bv.grid, st);
 }
 
-// fill and raster of view v (pooled: fill and item assignment only; the
-// pooled launch rasterizes the view)
-vsr_status batch_view_back(vsr_batch b, int v, vsr_map m, int64_t T, bool use_pairs, uint32_t* id, float* depth,
-                           float* cov, cudaStream_t st, int split_max = SPLIT_MAX_DEFAULT, bool pooled = false)
+// the raster of view v on its own: binning and raster in one launch
+vsr_status batch_view_raster(vsr_batch b, int v, vsr_map m, int64_t T, uint32_t* id, float* depth, float* cov,
+                             cudaStream_t st)
+{
+    BatchView& bv = b->views[v];
+    const RasterView rv{m->map, m->p.W, m->p.H, m->tiles, m->tx, bv.rec, (int)T, nullptr, nullptr, 0u, id, depth, cov};
+    return launch_raster_walk(rv, walk_index(bv.grid, T), m->idx.geom, bv.walk, nullptr, status_word(), st);
+}
+
+// the stored bins of view v, for a pooled launch (or, without a status, to
+// size them); the total to its pinned word
+vsr_status batch_view_bin(vsr_batch b, int v, vsr_map m, int64_t T, int* status, cudaStream_t st)
 {
     BatchView& bv = b->views[v];
     const int tiles = m->tx * m->ty;
-    vsr_status s;
-    if ((s = launch_bin_fill(bv.rec, (int)T, m->idx, bv.offsets, bv.counts, bv.counts + tiles,
-                             use_pairs ? bv.pairs : nullptr, use_pairs ? bv.cap : 0u, bv.ids, bv.cap, status_word(),
-                             st)) != VSR_OK)
-        return s;
-    if (pooled) return launch_raster_assign(bv.offsets, (uint32_t)tiles, bv.cap, bv.work, split_max, st);
-    const RasterView rv{m->map, m->p.W, m->p.H, m->tiles, m->tx, bv.rec, (int)T, bv.offsets,
-                        bv.ids, bv.cap, id, depth, cov};
-    return launch_raster_items(rv, bv.offsets, (uint32_t)tiles, bv.cap, bv.work, split_max, status_word(),
-                               st);
+    vsr_status s = launch_bin_walk(bv.rec, (int)T, walk_index(bv.grid, T), m->idx.geom, m->tiles, tiles, bv.ctr,
+                                   bv.offsets, bv.ends, bv.ids, bv.cap, status, nullptr, st);
+    if (s != VSR_OK) return s;
+    VSR_CUDA_TRY(cudaMemcpyAsync(b->h_total + v, bv.offsets + tiles, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+    return VSR_OK;
 }
 
 constexpr int POOL_GROUPS_MAX = 16;
@@ -1155,7 +1186,7 @@ vsr_status batch_pool_upload(vsr_batch b, int nviews, const vsr_map* maps, int64
         const uint32_t tiles = (uint32_t)(m->tx * m->ty);
         pv[v].view = RasterView{m->map, m->p.W, m->p.H, m->tiles, m->tx, bv.rec, (int)T, bv.offsets,
                                 bv.ids, bv.cap, id ? id[v] : nullptr, depth ? depth[v] : nullptr,
-                                cov ? cov[v] : nullptr};
+                                cov ? cov[v] : nullptr, bv.ends};
         pv[v].n_tiles = tiles;
         pv[v].nsplit_of = bv.work.nsplit_of;
         pv[v].split_slot = bv.work.split_slot;
@@ -1251,13 +1282,14 @@ vsr_status vsr_batch_render(vsr_batch b, int nviews, const vsr_map* maps, const 
     const size_t cam_bytes = sizeof(float) * 12 * (size_t)nviews;
 
     if (b->exec && key == b->key) {
-        // replay: new cameras only.  The previous replay (complete once its
-        // event has) left each view's pair total in pinned memory: a view
-        // within 1/8 of its bin capacity rebuilds the configuration with
-        // larger bins before this frame instead of overflowing in a later one.
+        // replay: new cameras only.  With pooled rasters the previous replay
+        // (complete once its event has) left each view's pair total in pinned
+        // memory: a view within 1/8 of its bin capacity rebuilds the
+        // configuration with larger bins before this frame instead of
+        // overflowing in a later one.
         VSR_CUDA_TRY(cudaEventSynchronize(b->cams_done));
         bool grow = false;
-        for (int v = 0; v < nviews && !grow; ++v) {
+        for (int v = 0; v < nviews && !grow && b->pool_groups > 0; ++v) {
             const uint64_t last = b->h_total[v];
             grow = last + last / 8 > b->views[v].cap;
         }
@@ -1294,43 +1326,37 @@ vsr_status vsr_batch_render(vsr_batch b, int nviews, const vsr_map* maps, const 
         b->cams_alloc = nviews;
     }
     if ((int)b->views.size() < nviews) b->views.resize(nviews);
+    const bool try_chains = b->mode != VSR_BATCH_POOLED, try_pool = b->mode != VSR_BATCH_CHAINS;
     for (int v = 0; v < nviews; ++v)
-        if ((s = batch_view_alloc(b->views[v], T, maps[v]->tx * maps[v]->ty)) != VSR_OK) return s;
+        if ((s = batch_view_alloc(b->views[v], T, maps[v]->tx * maps[v]->ty, try_pool, st)) != VSR_OK) return s;
     memcpy(b->cams_host, cams, cam_bytes);
     VSR_CUDA_TRY(cudaMemcpyAsync(b->cams_dev, b->cams_host, cam_bytes, cudaMemcpyHostToDevice, st));
 
-    // the views' binning searches their maps' tile indexes (built once per
-    // generation of a map; the key holds the generations)
-    for (int v = 0; v < nviews; ++v)
-        if ((s = ensure_tile_index(maps[v], st)) != VSR_OK) return s;
-    // eager frame: fronts, one synchronisation to size every view's bins, backs
+    // eager frame; for pooled rasters the views' bins are sized from it, with
+    // one synchronisation
     for (int v = 0; v < nviews; ++v) {
-        if ((s = batch_view_front(b, v, maps[v], tris_dev, T, false, st)) != VSR_OK) return s;
-        const int tiles = maps[v]->tx * maps[v]->ty;
-        VSR_CUDA_TRY(cudaMemcpyAsync(b->h_total + v, b->views[v].offsets + tiles, sizeof(uint32_t),
-                                     cudaMemcpyDeviceToHost, st));
+        if ((s = batch_view_setup(b, v, tris_dev, T, st)) != VSR_OK) return s;
+        if (try_pool && (s = batch_view_bin(b, v, maps[v], T, nullptr, st)) != VSR_OK) return s;
+        if ((s = batch_view_raster(b, v, maps[v], T, out_ptr(id_dev, v), out_ptr(depth_dev, v), out_ptr(cov_dev, v),
+                                   st)) != VSR_OK)
+            return s;
     }
-    VSR_CUDA_TRY(cudaStreamSynchronize(st));
-    for (int v = 0; v < nviews; ++v) {
-        BatchView& bv = b->views[v];
-        const uint32_t total = b->h_total[v];
-        if (total + total / 8 > bv.cap || !bv.ids) {
-            cudaFree(bv.ids);
-            cudaFree(bv.pairs);
-            bv.ids = nullptr;
-            bv.pairs = nullptr;
-            bv.cap = 0;
-            uint64_t want = (uint64_t)total + total / 4 + 4096;
-            if (want > 0xffffffffull) want = 0xffffffffull;
-            if ((s = dalloc(&bv.ids, (size_t)want)) != VSR_OK) return s;
-            if ((s = dalloc(&bv.pairs, (size_t)want)) != VSR_OK) return s;
-            bv.cap = (uint32_t)want;
+    if (try_pool) {
+        VSR_CUDA_TRY(cudaStreamSynchronize(st));
+        for (int v = 0; v < nviews; ++v) {
+            BatchView& bv = b->views[v];
+            const uint32_t total = b->h_total[v];
+            if (total + total / 8 > bv.cap || !bv.ids) {
+                cudaFree(bv.ids);
+                bv.ids = nullptr;
+                bv.cap = 0;
+                uint64_t want = (uint64_t)total + total / 4 + 4096;
+                if (want > 0xffffffffull) want = 0xffffffffull;
+                if ((s = dalloc(&bv.ids, (size_t)want)) != VSR_OK) return s;
+                bv.cap = (uint32_t)want;
+            }
         }
     }
-    for (int v = 0; v < nviews; ++v)
-        if ((s = batch_view_back(b, v, maps[v], T, false, out_ptr(id_dev, v), out_ptr(depth_dev, v),
-                                 out_ptr(cov_dev, v), st)) != VSR_OK)
-            return s;
     VSR_CUDA_TRY(cudaEventRecord(b->cams_done, st));
 
     // autotune: capture one graph per candidate (parallel streams S, raster
@@ -1366,14 +1392,17 @@ vsr_status vsr_batch_render(vsr_batch b, int nviews, const vsr_map* maps, const 
         int group = 0;
         for (int v = 0; cst == VSR_OK && v < nviews; ++v) {
             cudaStream_t vs = b->streams[v % S];
-            cst = batch_view_front(b, v, maps[v], tris_dev, T, true, vs);
-            const int tiles = maps[v]->tx * maps[v]->ty;
-            if (cst == VSR_OK && cudaMemcpyAsync(b->h_total + v, b->views[v].offsets + tiles, sizeof(uint32_t),
-                                                 cudaMemcpyDeviceToHost, vs) != cudaSuccess)
-                cst = VSR_ERR_CUDA;
-            if (cst == VSR_OK)
-                cst = batch_view_back(b, v, maps[v], T, true, out_ptr(id_dev, v), out_ptr(depth_dev, v),
-                                      out_ptr(cov_dev, v), vs, split, pooled);
+            cst = batch_view_setup(b, v, tris_dev, T, vs);
+            if (cst == VSR_OK && !pooled)
+                cst = batch_view_raster(b, v, maps[v], T, out_ptr(id_dev, v), out_ptr(depth_dev, v),
+                                        out_ptr(cov_dev, v), vs);
+            if (cst == VSR_OK && pooled) {
+                const BatchView& bv = b->views[v];
+                cst = batch_view_bin(b, v, maps[v], T, status_word(), vs);
+                if (cst == VSR_OK)
+                    cst = launch_raster_assign(bv.offsets, (uint32_t)(maps[v]->tx * maps[v]->ty), bv.cap, bv.work,
+                                               split, vs, bv.ends);
+            }
             if (cst == VSR_OK && pooled && v + 1 == pool_first(group + 1, groups, nviews)) {
                 // the group's views are binned once every stream reaches this point
                 for (int i = 0; cst == VSR_OK && i < S; ++i)
@@ -1433,9 +1462,9 @@ vsr_status vsr_batch_render(vsr_batch b, int nviews, const vsr_map* maps, const 
         return VSR_OK;
     };
     // the per-view raster launches and the pooled one: each at every stream
-    // count and the default split, then the splits at the best of them
+    // count and the default split, then the splits (of the pooled launches'
+    // stored bins) at the best of them
     vsr_status ts = VSR_OK;
-    const bool try_chains = b->mode != VSR_BATCH_POOLED, try_pool = b->mode != VSR_BATCH_CHAINS;
     for (int S : {1, 2, 4, 8}) {
         if (ts == VSR_OK && try_chains) ts = candidate(S, SPLIT_MAX_DEFAULT, 0);
         for (int groups : {1, 4, 16})
@@ -1444,7 +1473,7 @@ vsr_status vsr_batch_render(vsr_batch b, int nviews, const vsr_map* maps, const 
     const int bestS = b->nstreams;
     const int best_groups = b->pool_groups;
     for (int split : {256, 1024})
-        if (ts == VSR_OK && b->exec) ts = candidate(bestS, split, best_groups);
+        if (ts == VSR_OK && b->exec && best_groups > 0) ts = candidate(bestS, split, best_groups);
     // the kept graph's pooled views must carry its split and grouping
     if (ts == VSR_OK && b->exec && b->pool_groups > 0)
         ts = batch_pool_upload(b, nviews, maps, T, id_dev, depth_dev, cov_dev, b->split_max, b->pool_groups);

@@ -1,25 +1,19 @@
-// bin.cu -- tile binning: which triangles may produce a fragment in which
-// 16x16 tile.
+// bin.cu -- the triangle-major binner of the fixed-array path
+// (vsr_raster_noalloc) and the tile index it searches; scans.
 //
 // A fragment of triangle t at pixel direction G needs G inside the miter
 // cap enlarged by the ramp half-width (the gbpxstep test of the miter plane,
-// Sec. 1.1.1 / 1.1.2): G.S-hat - cos rho > -h sin rho, h = 1/(2 delta).  A
+// Sec. 1.1.1 / 1.1.2): G.S-hat - cos rho > -h sin rho, h = 1/(2 delta).  The
 // binner keeps (tile, t) when that enlarged cap can reach the tile's view
-// cone (cap_hits_cone).  The paper's analogue is the low-resolution region
-// mask widened by fwidth/2 (getPolygonRegion).
+// cone.  The paper's analogue is the low-resolution region mask widened by
+// fwidth/2 (getPolygonRegion).
 //
-// Two binners with the same cap / cone test:
-//  * tile-major (every frame of a scene or batch view): the frame's
-//    triangles filed by the cell of their cap centre on a latitude-longitude
-//    grid, then one warp per tile over the cells within its reach, in one
-//    pass (tri_file_kernel, bin_tiles_kernel; see TriIndex);
-//  * triangle-major (the fixed-array path, vsr_raster_noalloc): every
-//    triangle visits the cells of the map's tile index within beta +
-//    alpha_small_max of its cap centre (a few dozen cone tests whatever the
-//    map's size; no tile is found twice); count (atomic per-tile counters)
-//    -> exclusive scan -> fill (atomic per-tile cursors).
-// The order of ids inside a bin is not fixed; the raster kernels' results
-// do not depend on it.
+// Every triangle visits the cells of the map's tile index within beta +
+// alpha_small_max of its cap centre (a few dozen cone tests whatever the map's
+// size; no tile is found twice): count (atomic per-tile counters) -> exclusive
+// scan -> fill (atomic per-tile cursors).  It needs no memory but the bins and
+// one word per tile.  The scenes' own rasters walk the triangle grid instead
+// (walk.cuh).
 #include <math.h>
 #include <stddef.h>
 
@@ -250,20 +244,11 @@ __global__ void __launch_bounds__(IDX_FUSED_THREADS) idx_fused_kernel(const Cone
 // dependent loads of the search run on all lanes at once instead of one
 // lane walking its whole window.
 //
-// count: counts[tile] += 1 per hit (no value returned, so nothing waits),
-// and the hit is recorded as (tile, triangle) in the pair list -- staged per
-// warp in shared memory and appended with one atomic per warp and round.
-// fill: a map over the pair list that takes slot counts[tile] - 1 by atomic
-// decrement (one pair per thread, so the atomics' latency overlaps) and
-// writes ids[offsets[tile] + slot] = triangle.  When the list would overflow
-// (the first binning of a new shape, whose capacity is not known yet, or a
-// caller without a list) the fill searches again instead, with the same
-// decrement.  The counts return to zero either way; the order of ids inside
-// a bin is not fixed and the raster kernels' results do not depend on it.
-// (Keeping each hit's slot -- the old value of its counter -- would spare
-// the fill its atomics, but makes the count pass wait for each counter's
-// return: measured 44.3 -> 58.7 us for the count against 17.2 -> 8.6 us for
-// the fill on the 1080p frame.)
+// count: counts[tile] += 1 per hit (no value returned, so nothing waits);
+// fill: the same search, each hit taking slot counts[tile] - 1 by atomic
+// decrement and writing ids[offsets[tile] + slot] = triangle.  The counts
+// return to zero; the order of ids inside a bin is not fixed and the raster
+// kernels' results do not depend on it.
 
 constexpr int BIN_BIG_CHUNK = 16;
 // cones per step of the search for grids beyond one resident wave
@@ -284,8 +269,6 @@ constexpr int BIN_BIG_CHUNK = 16;
 #ifndef VSR_BIN_CB_LARGE
 #define VSR_BIN_CB_LARGE 1
 #endif
-constexpr int BIN_STAGE = 256;  // hits staged per warp (appended when half full)
-
 // FILL: false = count + record, true = fill by searching again.
 // CB: cones each lane fetches per step.  The search is bound by load latency:
 // a grid larger than one resident wave hides it with warps (CB = 1: 40
@@ -302,7 +285,6 @@ __global__ void __launch_bounds__(128, CB == 1 ? 12 : (CB == 2 ? 10 : 1)) bin_ke
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int t = (int)(blockIdx.x * 4 + warp) * TPW + lane;
-    if (FILL && v.pairs && *v.cursor <= v.pair_cap) return;  // the pair list is complete: bin_pairs_kernel fills
     const size_t TT = (size_t)T;
     // The index header, with every count that becomes an index clamped to
     // the arrays it indexes (identity for an index built by launch_tile_index),
@@ -324,10 +306,6 @@ __global__ void __launch_bounds__(128, CB == 1 ? 12 : (CB == 2 ? 10 : 1)) bin_ke
     sincosf(fminf(vang, PI_F), &vsin, &vcos);
     const uint32_t nbig = min(v.hdr->n_big, v.ntiles);
     const int bigpairs = (int)((nbig + BIN_BIG_CHUNK - 1) / BIN_BIG_CHUNK);
-    __shared__ uint2 s_hit[4][BIN_STAGE];
-    __shared__ uint32_t s_nhit[4];
-    if (!FILL && lane == 0) s_nhit[warp] = 0u;
-    __syncwarp();
 
     // phase 1: this lane's triangle
     float sx = 0.0f, sy = 0.0f, sz = 1.0f, cb = 1.0f, sb = 0.0f;
@@ -341,14 +319,8 @@ __global__ void __launch_bounds__(128, CB == 1 ? 12 : (CB == 2 ? 10 : 1)) bin_ke
             sz = q0.z;
             // the cap enlarged once by the map's widest ramp (>= every tile's
             // own): cos / sin of its radius beta, so each tile test is a few FMAs
-            if (v.pstep) {
-                const float2 c = pstep_cap(q0.w, q1.x, hmax);
-                cb = c.x;
-                sb = c.y;
-            } else {
-                cb = fmaxf(-1.0f, fminf(1.0f, q0.w - hmax * q1.x));
-                sb = sqrtf(fmaxf(0.0f, 1.0f - cb * cb));
-            }
+            cb = fmaxf(-1.0f, fminf(1.0f, q0.w - hmax * q1.x));
+            sb = sqrtf(fmaxf(0.0f, 1.0f - cb * cb));
             // outside the field of view: no window, no pairs.  The cap of
             // radius beta reaches the view cone iff angle(S, +z) <= beta +
             // view angle, i.e. S.z >= cos(beta + view angle) while the sum
@@ -431,15 +403,6 @@ __global__ void __launch_bounds__(128, CB == 1 ? 12 : (CB == 2 ? 10 : 1)) bin_ke
         auto hit = [&](uint32_t tile, uint32_t tri) {
             if (!FILL) {
                 atomicAdd(&v.counts[tile], 1u);
-                if (v.pairs) {
-                    const uint32_t j = atomicAdd(&s_nhit[warp], 1u);
-                    if (j < BIN_STAGE) {
-                        s_hit[warp][j] = make_uint2(tile, tri);
-                    } else {  // a round with more hits than the stage holds: straight to the list
-                        const uint32_t g = atomicAdd(v.cursor, 1u);
-                        if (g < v.pair_cap) v.pairs[g] = make_uint2(tile, tri);
-                    }
-                }
             } else {
                 const uint32_t pos = v.offsets[tile] + atomicSub(&v.counts[tile], 1u) - 1u;
                 if (pos < cap && pos < v.offsets[tile + 1])
@@ -508,62 +471,17 @@ __global__ void __launch_bounds__(128, CB == 1 ? 12 : (CB == 2 ? 10 : 1)) bin_ke
                 if (tile < v.ntiles) hit(tile, ot);
             }
         }
-        if (!FILL && v.pairs) {
-            // append the staged hits to the pair list once the stage is half
-            // full (a round adds about one hit per lane), and at the end
-            __syncwarp();
-            const uint32_t n = min(s_nhit[warp], (uint32_t)BIN_STAGE);
-            if (n >= BIN_STAGE / 2 || base + 32 >= total) {
-                uint32_t g0 = 0;
-                if (lane == 0 && n) g0 = atomicAdd(v.cursor, n);
-                g0 = __shfl_sync(FULL, g0, 0);
-                for (uint32_t j = lane; j < n; j += 32)
-                    if (g0 + j < v.pair_cap) v.pairs[g0 + j] = s_hit[warp][j];
-                __syncwarp();
-                if (lane == 0) s_nhit[warp] = 0u;
-                __syncwarp();
-            }
-        }
     }
 }
 
-// The fill as a map over the pair list of the count pass (when it is
-// complete): slot = --counts[tile], ids[offsets[tile] + slot] = triangle.
-__global__ void __launch_bounds__(256) bin_pairs_kernel(const uint2* __restrict__ pairs,
-                                                         const uint32_t* __restrict__ cursor, uint32_t pair_cap,
-                                                         const uint32_t* __restrict__ offsets,
-                                                         uint32_t* __restrict__ counts, uint32_t* __restrict__ ids,
-                                                         uint32_t cap, int* status, int overflow_here)
-{
-    const uint32_t n = *cursor;
-    if (n > pair_cap) {
-        // incomplete: the search-based fill runs instead -- or, when the list
-        // holds as many pairs as the bins, the bins overflow too: report it
-        if (overflow_here && blockIdx.x == 0 && threadIdx.x == 0) raise_status(status, VSR_ERR_BIN_OVERFLOW);
-        return;
-    }
-    for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
-        const uint2 e = pairs[p];
-        const uint32_t pos = offsets[e.x] + atomicSub(&counts[e.x], 1u) - 1u;
-        if (pos < cap && pos < offsets[e.x + 1])
-            ids[pos] = e.y;
-        else
-            raise_status(status, VSR_ERR_BIN_OVERFLOW);
-    }
-}
-
-// Exclusive scan of n counts (+ extra, when not NULL) into offsets[0..n] by
-// one CTA of 1024 threads:
+// Exclusive scan of n counts into offsets[0..n] by one CTA of 1024 threads:
 // chunks of 4096 (four consecutive elements per thread), carried across
-// chunks.  n comes from n_dev when it is not NULL.
-__global__ void __launch_bounds__(1024) scan_kernel(const uint32_t* __restrict__ counts,
-                                                     const uint32_t* __restrict__ extra, int n_host,
-                                                     const int* __restrict__ n_dev, uint32_t* __restrict__ offsets,
-                                                     volatile uint32_t* total_host)
+// chunks.
+__global__ void __launch_bounds__(1024) scan_kernel(const uint32_t* __restrict__ counts, int n,
+                                                     uint32_t* __restrict__ offsets)
 {
     __shared__ uint32_t warp_sums[32];
     __shared__ uint32_t carry_s;
-    const int n = n_dev ? *n_dev : n_host;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) carry_s = 0;
     __syncthreads();
@@ -571,7 +489,7 @@ __global__ void __launch_bounds__(1024) scan_kernel(const uint32_t* __restrict__
         const int b = base + 4 * tid;
         uint32_t v[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) v[q] = b + q < n ? counts[b + q] + (extra ? extra[b + q] : 0u) : 0u;
+        for (int q = 0; q < 4; ++q) v[q] = b + q < n ? counts[b + q] : 0u;
         const uint32_t local = v[0] + v[1] + v[2] + v[3];
         uint32_t x = local;
         for (int o = 1; o < 32; o <<= 1) {
@@ -599,532 +517,15 @@ __global__ void __launch_bounds__(1024) scan_kernel(const uint32_t* __restrict__
         if (tid == 0) carry_s += warp_sums[31];
         __syncthreads();
     }
-    if (tid == 0) {
-        offsets[n] = carry_s;
-        if (total_host) {  // the total straight into the host's pinned word (read after an event)
-            *total_host = carry_s;
-            __threadfence_system();
-        }
-    }
-}
-
-// ---- tile-major binning -----------------------------------------------------
-//
-// Per frame: tri_file (every triangle into its cell) -> bin_tiles (every
-// tile's bin, in one pass).
-
-constexpr float TRI_CELL0 = PI_F / TRI_NLAT0;
-constexpr float TRI_CELL1 = PI_F / TRI_NLAT1;
-// entries of a tile binned by its own warp (its hits staged in shared
-// memory); a tile with more goes to the heavy list
-constexpr uint32_t BIN_STAGE_HITS = 1024;
-constexpr int BIN_HEAVY_WARPS = 16;  // warps per heavy tile
-// steps of the walk whose loads are issued together: 2 (measured on the
-// 1080p frame: bin stage 38.9 us against 40.7 us at 4; 12 resident CTAs
-// per SM instead of 8, which caps the registers: 40.8 - 48.6 us)
-#ifndef VSR_BIN_WALK_U
-#define VSR_BIN_WALK_U 2
-#endif
-constexpr int BIN_WALK_U = VSR_BIN_WALK_U;
-// resident CTAs per SM the tile pass is compiled for (its register cap)
-#ifndef VSR_BIN_TILES_CTAS
-#define VSR_BIN_TILES_CTAS 8
-#endif
-
-__device__ __forceinline__ int tri_row(float lat, int nlat, float cell)
-{
-    return min(nlat - 1, max(0, (int)floorf((lat + 0.5f * PI_F) / cell)));
-}
-
-__device__ __forceinline__ int tri_col(float lon, int nlon, float cell)
-{
-    int c = (int)floorf((lon + PI_F) / cell);
-    c %= nlon;
-    return c < 0 ? c + nlon : c;
-}
-
-// The enlarged cap of triangle t as the triangle-major search forms it: its
-// centre (q0.xyz) and (cos, sin) of its radius; false for a triangle
-// without a cap.
-__device__ __forceinline__ bool tri_cap(const float4* __restrict__ rec, size_t TT, int t, float hmax, int pstep,
-                                        float4& q0, float& cb, float& sb)
-{
-    q0 = rec[rec_at(TT, t, RF_CAP)];
-    const float4 q1 = rec[rec_at(TT, t, RF_CAP2)];
-    if (q1.w == 0.0f) return false;
-    if (pstep) {
-        const float2 c = pstep_cap(q0.w, q1.x, hmax);
-        cb = c.x;
-        sb = c.y;
-    } else {
-        cb = fmaxf(-1.0f, fminf(1.0f, q0.w - hmax * q1.x));
-        sb = sqrtf(fmaxf(0.0f, 1.0f - cb * cb));
-    }
-    return true;
-}
-
-// Every triangle into its cell (counters cleared before): the fine grid
-// when its cap fits and the cell has room, else the coarse grid under the
-// same conditions, else the list; each grid's largest cap radius into the
-// header.
-__global__ void __launch_bounds__(256) tri_file_kernel(const float4* __restrict__ rec, int T,
-                                                       const TileIndexHdr* __restrict__ ihdr, TriIndex ti, int pstep)
-{
-    uint32_t* __restrict__ cnt = ti.counts;
-    const int gt = blockIdx.x * 256 + threadIdx.x;
-    unsigned b0 = 0u, b1 = 0u;  // float bits of non-negative radii order as the floats
-    if (gt < T) {
-        const int t = gt;
-        float4 q0;
-        float cb, sb;
-        if (tri_cap(rec, (size_t)T, t, __uint_as_float((uint32_t)ihdr->h_gen), pstep, q0, cb, sb)) {
-            const float beta = acosf(cb);
-            const unsigned bb = __float_as_uint(fmaxf(beta, 1e-30f));  // nonzero: the grid holds a triangle
-            uint32_t e = 0xffffffffu;
-            if (beta <= 2.0f * TRI_CELL1) {
-                const float lat = asinf(fmaxf(-1.0f, fminf(1.0f, q0.y)));
-                const float lon = atan2f(q0.x, q0.z);
-                if (beta <= 2.0f * TRI_CELL0) {
-                    const int cell = tri_row(lat, TRI_NLAT0, TRI_CELL0) * TRI_NLON0 + tri_col(lon, TRI_NLON0, TRI_CELL0);
-                    const uint32_t k = atomicAdd(&cnt[cell], 1u);
-                    if (k < (uint32_t)TRI_K0) {
-                        e = (uint32_t)cell * TRI_K0 + k;
-                        b0 = bb;
-                    }
-                }
-                if (e == 0xffffffffu) {
-                    const int cell = tri_row(lat, TRI_NLAT1, TRI_CELL1) * TRI_NLON1 + tri_col(lon, TRI_NLON1, TRI_CELL1);
-                    const uint32_t k = atomicAdd(&cnt[TRI_CELLS0 + cell], 1u);
-                    if (k < (uint32_t)TRI_K1) {
-                        e = TRI_E1 + (uint32_t)cell * TRI_K1 + k;
-                        b1 = bb;
-                    }
-                }
-            }
-            if (e == 0xffffffffu) {
-                // (below the list's capacity unless an earlier binning left its counters behind)
-                const uint32_t k = atomicAdd(&cnt[TRI_LARGE], 1u);
-                if (k < (uint32_t)ti.T) e = TRI_E2 + k;
-            }
-            if (e != 0xffffffffu) {
-                ti.cap[e] = make_float4(q0.x, q0.y, q0.z, cb);
-                ti.cs[e] = make_float2(sb, __uint_as_float((uint32_t)t));
-            }
-        }
-    }
-    for (int o = 16; o; o >>= 1) {
-        b0 = max(b0, __shfl_xor_sync(0xffffffffu, b0, o));
-        b1 = max(b1, __shfl_xor_sync(0xffffffffu, b1, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-        if (b0) atomicMax(&cnt[TRI_HDR], b0);
-        if (b1) atomicMax(&cnt[TRI_HDR + 1], b1);
-    }
-}
-
-// A window of one grid: rows r0 .. r0 + nr - 1, columns c0 .. c0 + ncol - 1
-// (mod nlon).
-struct TriWin {
-    int r0, nr, c0, ncol;
-};
-
-// The cells holding every direction within gamma of (lat, lon).
-__device__ __forceinline__ TriWin tri_window(float lat, float lon, float gamma, int nlat, float cell)
-{
-    const int nlon = 2 * nlat;
-    TriWin w{0, nlat, 0, nlon};
-    if (!(gamma < PI_F)) return w;
-    const int r0 = tri_row(lat - gamma, nlat, cell), r1 = tri_row(lat + gamma, nlat, cell);
-    w.r0 = r0;
-    w.nr = r1 - r0 + 1;
-    if (fabsf(lat) + gamma < 0.5f * PI_F - 1e-3f) {
-        // longitude half-width of a cap that holds no pole
-        const float dl = asinf(fminf(1.0f, sinf(gamma) / cosf(lat))) + 1e-4f;
-        int c0 = (int)floorf((lon - dl + PI_F) / cell);
-        const int c1 = (int)floorf((lon + dl + PI_F) / cell);
-        w.ncol = max(1, min(nlon, c1 - c0 + 1));
-        c0 %= nlon;
-        if (c0 < 0) c0 += nlon;
-        w.c0 = c0;
-    }
-    return w;
-}
-
-__device__ __forceinline__ TriWin shfl_win(const TriWin& w, int src)
-{
-    return TriWin{__shfl_sync(0xffffffffu, w.r0, src), __shfl_sync(0xffffffffu, w.nr, src),
-                  __shfl_sync(0xffffffffu, w.c0, src), __shfl_sync(0xffffffffu, w.ncol, src)};
-}
-
-// The candidate triangles of one tile, as one warp sees them: the cells of
-// the tile's two windows and the list, one range of sorted entries each.
-struct TileWalk {
-    float ax, ay, az, ca, sa;  // the tile's cone
-    TriWin w0, w1;             // its windows on the fine and coarse grid
-    int R0, R1, R;             // ranges: fine cells, coarse cells, then the list (none for an empty tile)
-
-    // every lane of the warp, the same tile
-    __device__ __forceinline__ void init(const float4& g, const Cone& c, const uint32_t* __restrict__ hdr, int lane)
-    {
-        ax = c.c0.x;
-        ay = c.c0.y;
-        az = c.c0.z;
-        ca = c.c0.w;
-        sa = c.c1.x;
-        TriWin w{0, 0, 0, 1};
-        R = 0;
-        if (g.w >= 0.0f) {  // h < 0: an empty tile
-            // lane 0 forms the fine grid's window, lane 1 the coarse grid's
-            // (none for a grid that holds no triangle)
-            const unsigned bm = lane < 2 ? hdr[lane] : 0u;
-            if (bm)
-                w = tri_window(g.y, g.z, g.x + __uint_as_float(bm) + 2e-4f, lane ? TRI_NLAT1 : TRI_NLAT0,
-                               lane ? TRI_CELL1 : TRI_CELL0);
-        }
-        w0 = shfl_win(w, 0);
-        w1 = shfl_win(w, 1);
-        R0 = w0.nr * w0.ncol;
-        R1 = w1.nr * w1.ncol;
-        R = g.w >= 0.0f ? R0 + R1 + 1 : 0;
-    }
-
-    // range i < R: first entry and length
-    __device__ __forceinline__ void range(const uint32_t* __restrict__ cnt, uint32_t listcap, int i, uint32_t& a,
-                                          int& len) const
-    {
-        if (i < R0) {
-            const int row = w0.r0 + i / w0.ncol;
-            int col = w0.c0 + i % w0.ncol;
-            if (col >= TRI_NLON0) col -= TRI_NLON0;
-            const int cell = row * TRI_NLON0 + col;
-            a = (uint32_t)cell * TRI_K0;
-            len = (int)min(cnt[cell], (uint32_t)TRI_K0);
-        } else if (i < R0 + R1) {
-            const int j = i - R0;
-            const int row = w1.r0 + j / w1.ncol;
-            int col = w1.c0 + j % w1.ncol;
-            if (col >= TRI_NLON1) col -= TRI_NLON1;
-            const int cell = row * TRI_NLON1 + col;
-            a = TRI_E1 + (uint32_t)cell * TRI_K1;
-            len = (int)min(cnt[TRI_CELLS0 + cell], (uint32_t)TRI_K1);
-        } else {
-            a = TRI_E2;
-            len = (int)min(cnt[TRI_LARGE], listcap);
-        }
-    }
-
-    // entries of all ranges (every lane gets the sum)
-    __device__ __forceinline__ uint32_t entries(const uint32_t* __restrict__ cnt, uint32_t listcap, int lane) const
-    {
-        uint32_t e = 0;
-        for (int rb = 0; rb < R; rb += 32) {
-            uint32_t a = 0;
-            int len = 0;
-            if (rb + lane < R) range(cnt, listcap, rb + lane, a, len);
-            e += (uint32_t)len;
-        }
-        for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-        return e;
-    }
-
-    // The walk, shared by nwarps warps (this one is number wr): the ranges go
-    // one per lane, 32 at a time; their entries are numbered across the warp
-    // and every lane tests the next one each step, finding the range that
-    // holds it by a search over the lanes; the warps take the steps in turn,
-    // BIN_WALK_U steps' loads at a time.  sink(hit mask, hit, triangle, this
-    // warp's hits before the step) for every step with a hit, on all lanes;
-    // returns this warp's hits.
-    template <class Sink>
-    __device__ __forceinline__ uint32_t walk(const TriIndex& ti, int lane, int wr, int nwarps, Sink sink) const
-    {
-        const unsigned FULL = 0xffffffffu;
-        uint32_t hits = 0;
-        for (int rb = 0; rb < R; rb += 32) {
-            uint32_t a = 0;
-            int len = 0;
-            if (rb + lane < R) range(ti.counts, (uint32_t)ti.T, rb + lane, a, len);
-            int incl = len;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(FULL, incl, o);
-                if (lane >= o) incl += y;
-            }
-            const int total = __shfl_sync(FULL, incl, 31);
-            const int excl = incl - len;
-            for (int k0 = 32 * BIN_WALK_U * wr; k0 < total; k0 += 32 * BIN_WALK_U * nwarps) {
-                float4 q[BIN_WALK_U];
-                float2 r[BIN_WALK_U];
-                bool in[BIN_WALK_U];
-#pragma unroll
-                for (int u = 0; u < BIN_WALK_U; ++u) {
-                    const int idx = k0 + 32 * u + lane;
-                    int o = 0;  // the last lane whose range starts at or before entry idx
-                    for (int st = 16; st > 0; st >>= 1) {
-                        const int x = __shfl_sync(FULL, excl, o + st);
-                        if (x <= idx) o += st;
-                    }
-                    const uint32_t e = __shfl_sync(FULL, a, o) + (uint32_t)(idx - __shfl_sync(FULL, excl, o));
-                    in[u] = idx < total;
-                    if (in[u]) {
-                        q[u] = ti.cap[e];
-                        r[u] = ti.cs[e];
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < BIN_WALK_U; ++u) {
-                    bool hit = false;
-                    if (in[u]) {
-                        // the cap / cone test of the triangle-major search, operand for operand
-                        const float cg = fmaf(q[u].x, ax, fmaf(q[u].y, ay, q[u].z * az));
-                        hit = q[u].w + ca <= 2e-6f || cg >= fmaf(ca, q[u].w, -sa * r[u].x) - 2e-6f;
-                    }
-                    const unsigned m = __ballot_sync(FULL, hit);
-                    if (m) sink(m, hit, __float_as_uint(r[u].y), hits);
-                    hits += (uint32_t)__popc(m);
-                }
-            }
-        }
-        return hits;
-    }
-};
-
-// The tiles, one warp each (a resident grid: warp w of W takes tiles w,
-// w + W, ...).  A tile whose ranges hold at most
-// BIN_STAGE_HITS entries is binned here: its hits staged in shared memory,
-// its range of the bins taken with one atomic on the cursor.  A larger tile
-// goes to the heavy list for bin_heavy_kernel.  With no heavy tile the last
-// CTA to finish stores the total.
-__global__ void __launch_bounds__(128, VSR_BIN_TILES_CTAS) bin_tiles_kernel(const float4* __restrict__ geom,
-                                                                            const Cone* __restrict__ tiles,
-                                                                            int ntiles, TriIndex ti,
-                                                                            uint32_t* __restrict__ starts,
-                                                                            uint32_t* __restrict__ ends,
-                                                                            uint32_t* __restrict__ ids, uint32_t cap,
-                                                                            int* status, uint32_t* total_host)
-{
-    __shared__ uint32_t s_hit[4][BIN_STAGE_HITS];
-    const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t* hdr = ti.counts + TRI_HDR;
-    const uint32_t lt = (1u << lane) - 1u;
-    for (int tile = blockIdx.x * 4 + warp; tile < ntiles; tile += gridDim.x * 4) {
-        const float4 g = geom[tile];
-        TileWalk tw;
-        tw.init(g, g.w >= 0.0f ? tiles[tile] : Cone{}, hdr, lane);
-        const uint32_t E = tw.entries(ti.counts, (uint32_t)ti.T, lane);
-        if (E <= BIN_STAGE_HITS) {
-            uint32_t* __restrict__ stage = s_hit[warp];
-            const uint32_t n = tw.walk(ti, lane, 0, 1, [&](unsigned m, bool hit, uint32_t t, uint32_t before) {
-                if (hit) stage[before + (uint32_t)__popc(m & lt)] = t;
-            });
-            uint32_t start = 0;
-            if (lane == 0 && n) start = atomicAdd(&hdr[TRI_H_CURSOR], n);
-            start = __shfl_sync(FULL, start, 0);
-            __syncwarp();
-            if (lane == 0 && (uint64_t)start + n > cap) raise_status(status, VSR_ERR_BIN_OVERFLOW);
-            for (uint32_t j = lane; j < n; j += 32)
-                if (start + j < cap) ids[start + j] = stage[j];
-            __syncwarp();  // the stage is read before the next tile's hits
-            if (lane == 0) {
-                starts[tile] = start;
-                ends[tile] = start + n;
-            }
-        } else if (lane == 0) {
-            const uint32_t j = atomicAdd(&hdr[TRI_H_HEAVY], 1u);
-            if (j < (uint32_t)ntiles) ti.heavy[j] = (uint32_t)tile;
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        if (atomicAdd(&hdr[TRI_H_DONE], 1u) == gridDim.x - 1) {
-            __threadfence();
-            if (atomicAdd(&hdr[TRI_H_HEAVY], 0u) == 0u) {
-                const uint32_t total = atomicAdd(&hdr[TRI_H_CURSOR], 0u);
-                starts[ntiles] = total;
-                if (total_host) {  // straight into the host's pinned word (read after an event)
-                    *total_host = total;
-                    __threadfence_system();
-                }
-            }
-        }
-    }
-}
-
-// The heavy tiles, one CTA of BIN_HEAVY_WARPS warps each, the CTAs taking
-// the next tile of the list until none is left (a grid of resident CTAs;
-// nothing waits).  The warps take the walk's steps in turn: a first walk
-// counts the tile's hits, one atomic takes its range of the bins, a second
-// walk writes them, each step's hits taking their places from a
-// shared-memory counter.  The last CTA to finish stores the total (when the
-// tile pass left it to this one) and clears the counters and the header for
-// the next binning.
-__global__ void __launch_bounds__(32 * BIN_HEAVY_WARPS) bin_heavy_kernel(const float4* __restrict__ geom,
-                                                                        const Cone* __restrict__ tiles, int ntiles,
-                                                                        TriIndex ti, uint32_t* __restrict__ starts,
-                                                                        uint32_t* __restrict__ ends,
-                                                                        uint32_t* __restrict__ ids, uint32_t cap,
-                                                                        int* status, uint32_t* total_host)
-{
-    __shared__ uint32_t s_tile, s_n, s_start;
-    const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t* hdr = ti.counts + TRI_HDR;
-    const uint32_t lt = (1u << lane) - 1u;
-    const uint32_t nheavy = min(hdr[TRI_H_HEAVY], (uint32_t)ntiles);
-    if (!nheavy) {
-        // nothing reads the cell counters any more: each CTA clears a slice
-        uint4* c4 = reinterpret_cast<uint4*>(ti.counts);
-        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < TRI_HDR / 4; i += gridDim.x * blockDim.x)
-            c4[i] = make_uint4(0u, 0u, 0u, 0u);
-    }
-    for (; nheavy;) {
-        __syncthreads();  // the previous tile's counter is read
-        if (threadIdx.x == 0) {
-            const uint32_t j = atomicAdd(&hdr[TRI_H_NEXT], 1u);
-            s_tile = j < nheavy ? ti.heavy[j] : 0xffffffffu;
-            s_n = 0u;
-        }
-        __syncthreads();
-        const uint32_t tile = s_tile;
-        if (tile >= (uint32_t)ntiles) break;
-        const float4 g = geom[tile];
-        TileWalk tw;
-        tw.init(g, tiles[tile], hdr, lane);
-        const uint32_t mine = tw.walk(ti, lane, warp, BIN_HEAVY_WARPS, [](unsigned, bool, uint32_t, uint32_t) {});
-        if (lane == 0 && mine) atomicAdd(&s_n, mine);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const uint32_t n = s_n;
-            const uint32_t start = n ? atomicAdd(&hdr[TRI_H_CURSOR], n) : 0u;
-            if ((uint64_t)start + n > cap) raise_status(status, VSR_ERR_BIN_OVERFLOW);
-            starts[tile] = start;
-            ends[tile] = start + n;
-            s_start = start;
-            s_n = 0u;
-        }
-        __syncthreads();
-        const uint32_t start = s_start;
-        tw.walk(ti, lane, warp, BIN_HEAVY_WARPS, [&](unsigned m, bool hit, uint32_t t, uint32_t) {
-            uint32_t base = 0;
-            if (lane == 0) base = atomicAdd(&s_n, (uint32_t)__popc(m));
-            base = __shfl_sync(FULL, base, 0);
-            if (hit) {
-                const uint32_t pos = start + base + (uint32_t)__popc(m & lt);
-                if (pos < cap) ids[pos] = t;
-            }
-        });
-    }
-    // the last CTA to finish (every tile's range is taken by then: the tile
-    // pass ran before, and each CTA's own before this)
-    __shared__ bool s_last;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        s_last = atomicAdd(&hdr[TRI_H_DONE2], 1u) == gridDim.x - 1;
-        if (s_last && nheavy) {
-            __threadfence();
-            const uint32_t total = atomicAdd(&hdr[TRI_H_CURSOR], 0u);
-            starts[ntiles] = total;
-            if (total_host) {  // straight into the host's pinned word (read after an event)
-                *total_host = total;
-                __threadfence_system();
-            }
-        }
-    }
-    __syncthreads();
-    if (s_last) {
-        // nothing reads the counters any more: clear the rest of them (all,
-        // after heavy tiles) and the header
-        const int from = nheavy ? 0 : TRI_HDR / 4;
-        uint4* c4 = reinterpret_cast<uint4*>(ti.counts);
-        for (int i = from + threadIdx.x; i < TRI_WORDS / 4; i += blockDim.x) c4[i] = make_uint4(0u, 0u, 0u, 0u);
-        if (threadIdx.x < TRI_WORDS % 4) ti.counts[(TRI_WORDS / 4) * 4 + threadIdx.x] = 0u;
-    }
+    if (tid == 0) offsets[n] = carry_s;
 }
 
 }  // namespace
 
-vsr_status launch_scan(const uint32_t* counts, const uint32_t* extra, int n, const int* n_dev, uint32_t* offsets,
-                       cudaStream_t st, uint32_t* total_host)
+vsr_status launch_scan(const uint32_t* counts, int n, uint32_t* offsets, cudaStream_t st)
 {
-    scan_kernel<<<1, 1024, 0, st>>>(counts, extra, n, n_dev, offsets, total_host);
+    scan_kernel<<<1, 1024, 0, st>>>(counts, n, offsets);
     VSR_CUDA_TRY(cudaGetLastError());
-    return VSR_OK;
-}
-
-vsr_status tri_index_alloc(TriIndex* ti, int64_t T, int ntiles)
-{
-    if (!ti->counts) {
-        VSR_CUDA_TRY(cudaMalloc(&ti->counts, sizeof(uint32_t) * TRI_WORDS));
-        ti->dirty = true;  // cleared by the first binning
-    }
-    if (!ti->heavy || ntiles > ti->ntiles) {
-        cudaFree(ti->heavy);
-        ti->heavy = nullptr;
-        ti->ntiles = 0;
-        VSR_CUDA_TRY(cudaMalloc(&ti->heavy, sizeof(uint32_t) * (size_t)(ntiles > 0 ? ntiles : 1)));
-        ti->ntiles = ntiles;
-    }
-    if (!ti->cap || T > ti->T) {
-        cudaFree(ti->cap);
-        cudaFree(ti->cs);
-        ti->cap = nullptr;
-        ti->cs = nullptr;
-        ti->T = 0;
-        const size_t n = (size_t)TRI_E2 + (size_t)T;
-        VSR_CUDA_TRY(cudaMalloc(&ti->cap, sizeof(float4) * n));
-        VSR_CUDA_TRY(cudaMalloc(&ti->cs, sizeof(float2) * n));
-        ti->T = T;
-    }
-    return VSR_OK;
-}
-
-void tri_index_free(TriIndex* ti)
-{
-    cudaFree(ti->counts);
-    cudaFree(ti->heavy);
-    cudaFree(ti->cap);
-    cudaFree(ti->cs);
-    *ti = TriIndex{};
-}
-
-size_t tri_index_bytes(int64_t T, int ntiles)
-{
-    return sizeof(uint32_t) * ((size_t)TRI_WORDS + (size_t)ntiles) +
-           (sizeof(float4) + sizeof(float2)) * ((size_t)TRI_E2 + (size_t)T);
-}
-
-vsr_status launch_bin_tiles(const float4* rec, int T, const TileIndex& idx, const Cone* tiles, int ntiles,
-                            TriIndex& ti, uint32_t* starts, uint32_t* ends, uint32_t* ids, uint32_t cap, int* status,
-                            uint32_t* total_host, cudaStream_t st, int pstep)
-{
-    if (T < 0 || (int64_t)T > ti.T || !ti.counts || !ti.cap || ntiles <= 0 || ntiles > ti.ntiles)
-        return VSR_ERR_INVALID_ARG;
-    // until the clearing kernel is queued, a failure leaves the counters behind
-    const bool was_dirty = ti.dirty;
-    ti.dirty = true;
-    if (was_dirty) VSR_CUDA_TRY(cudaMemsetAsync(ti.counts, 0, sizeof(uint32_t) * TRI_WORDS, st));
-    if (T > 0) {
-        tri_file_kernel<<<(T + 255) / 256, 256, 0, st>>>(rec, T, idx.hdr, ti, pstep);
-        VSR_CUDA_TRY(cudaGetLastError());
-    }
-    const int sms = sm_count();
-    if (sms < 0) return VSR_ERR_CUDA;
-    // one resident wave (the tile pass's occupancy, looked up once)
-    static std::atomic<int> per_sm{0};
-    int k = per_sm.load();
-    if (k <= 0) {
-        VSR_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, bin_tiles_kernel, 128, 0));
-        if (k <= 0) k = 1;
-        per_sm.store(k);
-    }
-    const int grid = std::min((ntiles + 3) / 4, k * sms);
-    bin_tiles_kernel<<<grid, 128, 0, st>>>(idx.geom, tiles, ntiles, ti, starts, ends, ids, cap, status, total_host);
-    VSR_CUDA_TRY(cudaGetLastError());
-    bin_heavy_kernel<<<sms, 32 * BIN_HEAVY_WARPS, 0, st>>>(idx.geom, tiles, ntiles, ti, starts, ends, ids, cap, status,
-                                                           total_host);
-    VSR_CUDA_TRY(cudaGetLastError());
-    ti.dirty = false;
     return VSR_OK;
 }
 
@@ -1171,12 +572,10 @@ static int bin_shape(int T, int sms)
     return 1;
 }
 
-vsr_status launch_bin_count(const float4* rec, int T, TileIndex idx, uint32_t* counts, uint32_t* cursor,
-                            uint2* pairs, uint32_t pair_cap, cudaStream_t st, int pstep)
+vsr_status launch_bin_count(const float4* rec, int T, TileIndex idx, uint32_t* counts, cudaStream_t st)
 {
     if (T == 0) return VSR_OK;
-    const BinView v{idx.hdr,  idx.cell_start, idx.sorted, idx.big, rec,   counts,
-                    nullptr,  pairs,          pair_cap,   cursor,  pstep, idx.ntiles};
+    const BinView v{idx.hdr, idx.cell_start, idx.sorted, idx.big, rec, counts, nullptr, idx.ntiles};
     const int sms = sm_count();
     if (sms < 0) return VSR_ERR_CUDA;
     switch (bin_shape(T, sms)) {
@@ -1192,22 +591,10 @@ vsr_status launch_bin_count(const float4* rec, int T, TileIndex idx, uint32_t* c
 }
 
 vsr_status launch_bin_fill(const float4* rec, int T, TileIndex idx, const uint32_t* offsets, uint32_t* counts,
-                           const uint32_t* cursor, const uint2* pairs, uint32_t pair_cap, uint32_t* ids, uint32_t cap,
-                           int* status, cudaStream_t st, int pstep)
+                           uint32_t* ids, uint32_t cap, int* status, cudaStream_t st)
 {
     if (T == 0) return VSR_OK;
-    const BinView v{idx.hdr, idx.cell_start, idx.sorted, idx.big, rec, counts, offsets, const_cast<uint2*>(pairs),
-                    pair_cap, const_cast<uint32_t*>(cursor), pstep, idx.ntiles};
-    // a pair list as long as the bins is complete unless the bins overflow,
-    // so the search-based fill is needed only without one or with a shorter one
-    const bool search = !pairs || pair_cap < cap;
-    if (pairs) {
-        constexpr int BIN_PAIR_BLOCKS = 152 * 8;
-        bin_pairs_kernel<<<BIN_PAIR_BLOCKS, 256, 0, st>>>(pairs, cursor, pair_cap, offsets, counts, ids, cap,
-                                                          status, search ? 0 : 1);
-        VSR_CUDA_TRY(cudaGetLastError());
-    }
-    if (!search) return VSR_OK;
+    const BinView v{idx.hdr, idx.cell_start, idx.sorted, idx.big, rec, counts, offsets, idx.ntiles};
     const int sms = sm_count();
     if (sms < 0) return VSR_ERR_CUDA;
     switch (bin_shape(T, sms)) {
@@ -1226,8 +613,7 @@ vsr_status launch_bin_fill(const float4* rec, int T, TileIndex idx, const uint32
 // pass 1: per 4096-element block sums; pass 2: one CTA scans the block sums
 // (partials[nb] = total); pass 3: per block, local scan plus the block's base.
 
-__global__ void __launch_bounds__(1024) scan_block_sums(const uint32_t* __restrict__ counts,
-                                                         const uint32_t* __restrict__ extra, int n,
+__global__ void __launch_bounds__(1024) scan_block_sums(const uint32_t* __restrict__ counts, int n,
                                                          uint32_t* __restrict__ partials)
 {
     __shared__ uint32_t ws[32];
@@ -1235,7 +621,7 @@ __global__ void __launch_bounds__(1024) scan_block_sums(const uint32_t* __restri
     uint32_t v = 0;
 #pragma unroll
     for (int q = 0; q < 4; ++q)
-        if (b + q < n) v += counts[b + q] + (extra ? extra[b + q] : 0u);
+        if (b + q < n) v += counts[b + q];
     for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
     __syncthreads();
@@ -1246,8 +632,7 @@ __global__ void __launch_bounds__(1024) scan_block_sums(const uint32_t* __restri
     }
 }
 
-__global__ void __launch_bounds__(1024) scan_blocks_apply(const uint32_t* __restrict__ counts,
-                                                           const uint32_t* __restrict__ extra, int n,
+__global__ void __launch_bounds__(1024) scan_blocks_apply(const uint32_t* __restrict__ counts, int n,
                                                            const uint32_t* __restrict__ bases,
                                                            uint32_t* __restrict__ offsets)
 {
@@ -1256,7 +641,7 @@ __global__ void __launch_bounds__(1024) scan_blocks_apply(const uint32_t* __rest
     const int b = blockIdx.x * 4096 + 4 * tid;
     uint32_t v[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) v[q] = b + q < n ? counts[b + q] + (extra ? extra[b + q] : 0u) : 0u;
+    for (int q = 0; q < 4; ++q) v[q] = b + q < n ? counts[b + q] : 0u;
     const uint32_t local = v[0] + v[1] + v[2] + v[3];
     uint32_t x = local;
     for (int o = 1; o < 32; o <<= 1) {
@@ -1283,16 +668,15 @@ __global__ void __launch_bounds__(1024) scan_blocks_apply(const uint32_t* __rest
     if (blockIdx.x == gridDim.x - 1 && tid == 0) offsets[n] = bases[gridDim.x];
 }
 
-vsr_status launch_scan_large(const uint32_t* counts, const uint32_t* extra, int n, uint32_t* partials,
-                             uint32_t* offsets, cudaStream_t st)
+vsr_status launch_scan_large(const uint32_t* counts, int n, uint32_t* partials, uint32_t* offsets, cudaStream_t st)
 {
     const int nb = (n + 4095) / 4096;
-    if (nb <= 1) return launch_scan(counts, extra, n, nullptr, offsets, st);
-    scan_block_sums<<<nb, 1024, 0, st>>>(counts, extra, n, partials);
+    if (nb <= 1) return launch_scan(counts, n, offsets, st);
+    scan_block_sums<<<nb, 1024, 0, st>>>(counts, n, partials);
     // scan the nb block sums in place into partials[nb + 1 ...]: reuse the one-CTA scan
-    vsr_status s = launch_scan(partials, nullptr, nb, nullptr, partials + nb + 1, st);
+    vsr_status s = launch_scan(partials, nb, partials + nb + 1, st);
     if (s != VSR_OK) return s;
-    scan_blocks_apply<<<nb, 1024, 0, st>>>(counts, extra, n, partials + nb + 1, offsets);
+    scan_blocks_apply<<<nb, 1024, 0, st>>>(counts, n, partials + nb + 1, offsets);
     VSR_CUDA_TRY(cudaGetLastError());
     return VSR_OK;
 }

@@ -65,7 +65,7 @@ FragArgs frag_args(vsr_map m, vsr_scene sc, const float* colors, vsr_frags f)
     a.rec = sc->rec;
     a.T = (int)sc->T;
     a.offsets = sc->offsets;
-    a.ends = scene_ends(sc);
+    a.ends = sc->ends;
     a.ids = sc->ids;
     a.cap = sc->cap;
     a.colors = colors;
@@ -119,7 +119,7 @@ vsr_status vsr_raster_shaded(vsr_map m, vsr_scene sc, const float* colors_dev, v
     FragArgs a = frag_args(m, sc, colors_dev, f);
     if ((s = launch_frag_count(a, st)) != VSR_OK) return s;
     const int npix = W * H;
-    if ((s = launch_scan_large(f->counts, nullptr, npix, f->scan_part, f->foff, st)) != VSR_OK) return s;
+    if ((s = launch_scan_large(f->counts, npix, f->scan_part, f->foff, st)) != VSR_OK) return s;
     VSR_CUDA_TRY(cudaMemcpyAsync(f->h_total, f->foff + npix, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
     VSR_CUDA_TRY(cudaStreamSynchronize(st));
     const uint32_t total = *f->h_total;

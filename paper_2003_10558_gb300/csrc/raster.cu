@@ -38,6 +38,7 @@
 #include <type_traits>
 
 #include "stage.cuh"
+#include "walk.cuh"
 
 namespace {
 
@@ -257,61 +258,191 @@ __device__ __forceinline__ uint32_t final_acc(const PixPair& q, int p)
     return q.lim[p] < INFINITY ? min(q.acc[p], COV_ONE) : 0u;
 }
 
+// A thread's place in its tile: warp w covers the 8x8 block (w & 1, w >> 1),
+// a lane the pixels (lx, ly) and (lx, ly + 4).
+struct TilePos {
+    int tx, ty, lx, ly, px, py;
+    __device__ __forceinline__ TilePos(int tile, int tiles_x)
+    {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        tx = tile % tiles_x;
+        ty = tile / tiles_x;
+        lx = (warp & 1) * 8 + (lane & 7);
+        ly = (warp >> 1) * 8 + (lane >> 3);
+        px = tx * TILE + lx;
+        py = ty * TILE + ly;
+    }
+};
+
+// The lane's pixels from the map (zero outside the picture).
+__device__ __forceinline__ void load_pixels(const RasterView& view, const TilePos& tp, float4 (&g)[PPT])
+{
+#pragma unroll
+    for (int p = 0; p < PPT; ++p) {
+        const int y = tp.py + 4 * p;
+        g[p] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (tp.px < view.W && y < view.H) g[p] = view.map[(size_t)y * view.W + tp.px];
+    }
+}
+
+// The warps' view cones (their 8x8 pixels; block_cone), in shared memory: the
+// cull reads them once per 32 triangles, and held in registers they would
+// spill others out of the evaluation loop.
+struct WarpCones {
+    float4 c[RT / 32][2];
+};
+
+// The pixels' loop state, and the warp's own view cone; returns whether the
+// warp has a valid pixel.
+__device__ __forceinline__ bool start_pixels(const float4 (&g)[PPT], const float4& axis, PixPair& q, WarpCones& wc)
+{
+    pix_pair(q, g[0], g[1], axis.x, axis.y, axis.z);
+    const float gx[PPT] = {g[0].x, g[1].x}, gy[PPT] = {g[0].y, g[1].y}, gz[PPT] = {g[0].z, g[1].z};
+    const bool pv[PPT] = {g[0].w > 0.0f, g[1].w > 0.0f};
+    const float h[PPT] = {pv[0] ? -q.lim[0] : 0.0f, pv[1] ? -q.lim[1] : 0.0f};
+    float4 c0, c1;
+    block_cone(gx, gy, gz, h, pv, c0, c1);
+    if ((threadIdx.x & 31) == 0) {
+        wc.c[threadIdx.x >> 5][0] = c0;
+        wc.c[threadIdx.x >> 5][1] = c1;
+    }
+    __syncwarp();
+    return c1.z > 0.0f;
+}
+
+// Stage triangle t into slot j (an index beyond the records -- never left by a
+// completed binning or grid -- empties the slot and raises the status).
+__device__ __forceinline__ void stage_checked(const float4* __restrict__ rec, int T, uint32_t t, const float4& axis,
+                                              Stage& st, int j, int* status)
+{
+    if (t >= (uint32_t)T) {
+        raise_status(status, VSR_ERR_BIN_OVERFLOW);
+        st.s6[j] = make_float4(0.0f, 0.0f, 0.0f, __uint_as_float(STAGE_EMPTY));
+    } else {
+        stage_triangle(rec, (size_t)T, t, axis.x, axis.y, axis.z, st, j);
+    }
+}
+
+// The n staged triangles of a chunk at the warp's pixels: a lane-parallel cull
+// of 32 triangles at a time against the warp's cone, then the survivors one by
+// one.
+template <bool STATS>
+__device__ __forceinline__ void eval_chunk(const Stage& st, int n, const WarpCones& wc, bool count_alg, PixPair& q,
+                                           uint32_t& cnt_alg, uint32_t& cnt_exec)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int gbase = 0; gbase < n; gbase += 32) {
+        const float4 wc0 = wc.c[warp][0], wc1 = wc.c[warp][1];
+        bool keep = false;
+        const int jj = gbase + lane;
+        if (jj < n && __float_as_uint(st.s6[jj].w) != STAGE_EMPTY)
+            keep = cone_may_hit(st.s0[jj], st.s1[jj], st.s2[jj], st.s3[jj], st.s4[jj], wc0, wc1, count_alg);
+        unsigned mask = __ballot_sync(0xffffffffu, keep);
+        while (mask) {
+            const int k = 31 - __clz(mask);  // any order: from the top, one instruction less than from the bottom
+            mask ^= 1u << k;
+            if (STATS) ++cnt_exec;
+            eval_slot<STATS>(st, gbase + k, q, cnt_alg);
+        }
+    }
+}
+
+// Merge the lane's pixels into accumulator slot `slot` of a tile processed in
+// several parts; the part that brings the count of `done` units to `target`
+// gets the tile's result in q, clears the slot and returns true.  Called by
+// every thread of the CTA.
+__device__ __forceinline__ bool merge_slot(const SplitAcc& split, int slot, const TilePos& tp, PixPair& q,
+                                           uint32_t units, uint32_t target)
+{
+    __shared__ int s_last;
+    const int lp0 = tp.lx + TILE * tp.ly;
+    unsigned long long* __restrict__ sacc = split.acc + (size_t)slot * TILE_PIX;
+    unsigned long long* __restrict__ skey = split.key + (size_t)slot * TILE_PIX;
+#pragma unroll
+    for (int p = 0; p < PPT; ++p) {
+        if (q.acc[p]) atomicAdd(&sacc[lp0 + TILE * 4 * p], (unsigned long long)q.acc[p]);
+        if (q.key[p] != KEY_NONE) atomicMin(&skey[lp0 + TILE * 4 * p], q.key[p]);
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&split.done[slot], units) + units == target;
+    __syncthreads();
+    if (!s_last) return false;
+    __threadfence();
+#pragma unroll
+    for (int p = 0; p < PPT; ++p) {
+        q.acc[p] = (uint32_t)min(atomicExch(&sacc[lp0 + TILE * 4 * p], 0ull), (unsigned long long)COV_ONE);
+        q.key[p] = min(atomicExch(&skey[lp0 + TILE * 4 * p], ~0ull), KEY_NONE);
+    }
+    if (threadIdx.x == 0) split.done[slot] = 0u;
+    return true;
+}
+
 // ROWS: the outputs go through shared memory and leave in whole tile rows
 // (pinned host outputs written in place over the host link).
+template <bool STATS, bool ROWS>
+__device__ __forceinline__ void write_tile(const RasterView& view, const TilePos& tp, const PixPair& q,
+                                           int32_t* __restrict__ n_inside)
+{
+    const int W = view.W, H = view.H;
+    if constexpr (!ROWS) {
+#pragma unroll
+        for (int p = 0; p < PPT; ++p) {
+            if (tp.px >= W || tp.py + 4 * p >= H) continue;
+            const size_t o = (size_t)(tp.py + 4 * p) * W + tp.px;
+            const bool hit = q.key[p] != KEY_NONE;
+            if (view.out_id) view.out_id[o] = hit ? (uint32_t)(q.key[p] & 0xffffffffull) : 0xffffffffu;
+            if (view.out_depth) view.out_depth[o] = hit ? __uint_as_float((uint32_t)(q.key[p] >> 32) + 1u) : INFINITY;
+            if (view.out_cov) view.out_cov[o] = (float)q.acc[p] * (1.0f / (float)COV_ONE);
+            if (STATS && n_inside) n_inside[o] = q.cnt_in[p];
+        }
+    } else {
+        // Through shared memory, so that each warp store covers two whole tile
+        // rows (16 pixels, 64 B each) instead of four 8-pixel pieces: over the
+        // host link 32-byte pieces cost about a quarter of its bandwidth.
+        __shared__ uint32_t s_out[3][TILE_PIX];
+#pragma unroll
+        for (int p = 0; p < PPT; ++p) {
+            const int lp = tp.lx + TILE * (tp.ly + 4 * p);
+            const bool hit = q.key[p] != KEY_NONE;
+            s_out[0][lp] = hit ? (uint32_t)(q.key[p] & 0xffffffffull) : 0xffffffffu;
+            s_out[1][lp] = hit ? (uint32_t)(q.key[p] >> 32) + 1u : __float_as_uint(INFINITY);
+            s_out[2][lp] = __float_as_uint((float)q.acc[p] * (1.0f / (float)COV_ONE));
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = threadIdx.x; i < TILE_PIX; i += RT) {
+            const int ox = tp.tx * TILE + (i % TILE), oy = tp.ty * TILE + i / TILE;
+            if (ox >= W || oy >= H) continue;
+            const size_t o = (size_t)oy * W + ox;
+            if (view.out_id) view.out_id[o] = s_out[0][i];
+            if (view.out_depth) view.out_depth[o] = __uint_as_float(s_out[1][i]);
+            if (view.out_cov) view.out_cov[o] = __uint_as_float(s_out[2][i]);
+        }
+        __syncthreads();  // read before the CTA's next tile writes it
+    }
+}
+
 template <bool STATS, bool ROWS = false>
 __device__ __forceinline__ void raster_tile(const RasterView& view, int tile, Stage& st, bool count_alg,
                                             uint32_t& cnt_alg, uint32_t& cnt_exec, int32_t* __restrict__ n_inside,
                                             int* __restrict__ status, int range_lo = 0, int range_hi = -1,
                                             int split_slot = -1, int nsplit = 1, SplitAcc split = SplitAcc{})
 {
-    const float4* __restrict__ map = view.map;
-    const int W = view.W, H = view.H, tiles_x = view.tiles_x, T = view.T;
-    const Cone* __restrict__ tiles = view.tiles;
-    const float4* __restrict__ rec = view.rec;
-    const uint32_t* __restrict__ offsets = view.offsets;
     const uint32_t* __restrict__ ids = view.ids;
     const uint32_t cap = view.cap;
-    uint32_t* __restrict__ out_id = view.out_id;
-    float* __restrict__ out_depth = view.out_depth;
-    float* __restrict__ out_cov = view.out_cov;
-
-    const int tx = tile % tiles_x, ty = tile / tiles_x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // pixel (in tile) of this lane's first pixel; its second is four rows below
-    const int lx = (warp & 1) * 8 + (lane & 7);
-    const int ly0 = (warp >> 1) * 8 + (lane >> 3);
-    const int px = tx * TILE + lx;
-    const int py0 = ty * TILE + ly0;
-
-    const Cone tc = tiles[tile];
-    const float ax = tc.c0.x, ay = tc.c0.y, az = tc.c0.z;
-
-    bool inimg[PPT];
+    const TilePos tp(tile, view.tiles_x);
+    const Cone tc = view.tiles[tile];
     PixPair q;
-    // the warp's own view cone (its 8x8 pixels)
-    float4 wc0, wc1;
-    {
-        float4 g[PPT];
-#pragma unroll
-        for (int p = 0; p < PPT; ++p) {
-            const int py = py0 + 4 * p;
-            inimg[p] = px < W && py < H;
-            g[p] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (inimg[p]) g[p] = map[(size_t)py * W + px];
-        }
-        pix_pair(q, g[0], g[1], ax, ay, az);
-        const float gx[PPT] = {g[0].x, g[1].x}, gy[PPT] = {g[0].y, g[1].y}, gz[PPT] = {g[0].z, g[1].z};
-        const bool pv[PPT] = {g[0].w > 0.0f, g[1].w > 0.0f};
-        const float h[PPT] = {pv[0] ? -q.lim[0] : 0.0f, pv[1] ? -q.lim[1] : 0.0f};
-        block_cone(gx, gy, gz, h, pv, wc0, wc1);
-    }
-    const bool warp_active = wc1.z > 0.0f;
+    __shared__ WarpCones wc;
+    float4 g[PPT];
+    load_pixels(view, tp, g);
+    const bool warp_active = start_pixels(g, tc.c0, q, wc);
 
     uint32_t b0 = 0, b1 = 0;
     if (tc.c1.z > 0.0f) {
-        b0 = offsets[tile];
-        b1 = view.ends ? view.ends[tile] : offsets[tile + 1];
+        b0 = view.offsets[tile];
+        b1 = view.ends ? view.ends[tile] : view.offsets[tile + 1];
         if (b1 > cap) {
             if (threadIdx.x == 0) raise_status(status, VSR_ERR_BIN_OVERFLOW);
             b1 = cap;
@@ -323,8 +454,6 @@ __device__ __forceinline__ void raster_tile(const RasterView& view, int tile, St
             b1 = min(hi, b1);
         }
     }
-
-    const size_t TT = (size_t)T;
     static_assert(PPT == 2, "packed pairs hold the thread's two pixels");
 
     for (uint32_t base = b0; base < b1; base += CHUNK) {
@@ -333,100 +462,15 @@ __device__ __forceinline__ void raster_tile(const RasterView& view, int tile, St
 #pragma unroll
         for (int p = 0; p < PPT; ++p) q.acc[p] = min(q.acc[p], COV_ONE);
         __syncthreads();
-        if ((int)threadIdx.x < n) {
-            const uint32_t t = ids[base + threadIdx.x];
-            if (t >= (uint32_t)T) {
-                // never produced by a completed binning: a stale or overflowed
-                // bin must not index outside the records
-                raise_status(status, VSR_ERR_BIN_OVERFLOW);
-                st.s6[threadIdx.x] = make_float4(0.0f, 0.0f, 0.0f, __uint_as_float(STAGE_EMPTY));
-            } else {
-                stage_triangle(rec, TT, t, ax, ay, az, st, threadIdx.x);
-            }
-        }
+        if ((int)threadIdx.x < n) stage_checked(view.rec, view.T, ids[base + threadIdx.x], tc.c0, st, threadIdx.x, status);
         __syncthreads();
-        if (!warp_active) continue;
-        for (int gbase = 0; gbase < n; gbase += 32) {
-            // lane-parallel cull of 32 triangles against this warp's cone
-            bool keep = false;
-            const int jj = gbase + lane;
-            if (jj < n && __float_as_uint(st.s6[jj].w) != STAGE_EMPTY)
-                keep = cone_may_hit(st.s0[jj], st.s1[jj], st.s2[jj], st.s3[jj], st.s4[jj], wc0, wc1, count_alg);
-            unsigned mask = __ballot_sync(0xffffffffu, keep);
-            while (mask) {
-                const int k = 31 - __clz(mask);  // any order: from the top, one instruction less than from the bottom
-                mask ^= 1u << k;
-                const int j = gbase + k;
-                if (STATS) ++cnt_exec;
-                eval_slot<STATS>(st, j, q, cnt_alg);
-            }
-        }
+        if (warp_active) eval_chunk<STATS>(st, n, wc, count_alg, q, cnt_alg, cnt_exec);
     }
 
 #pragma unroll
     for (int p = 0; p < PPT; ++p) q.acc[p] = final_acc(q, p);
-
-    if (split_slot >= 0) {
-        // merge into the tile's slot; the last item to arrive writes it out
-        const int lp0 = lx + TILE * ly0;
-        unsigned long long* __restrict__ sacc = split.acc + (size_t)split_slot * TILE_PIX;
-        unsigned long long* __restrict__ skey = split.key + (size_t)split_slot * TILE_PIX;
-#pragma unroll
-        for (int p = 0; p < PPT; ++p) {
-            if (q.acc[p]) atomicAdd(&sacc[lp0 + TILE * 4 * p], (unsigned long long)q.acc[p]);
-            if (q.key[p] != KEY_NONE) atomicMin(&skey[lp0 + TILE * 4 * p], q.key[p]);
-        }
-        __threadfence();
-        __syncthreads();
-        __shared__ int s_last;
-        if (threadIdx.x == 0) s_last = atomicAdd(&split.done[split_slot], 1u) == (unsigned)(nsplit - 1);
-        __syncthreads();
-        if (!s_last) return;
-        __threadfence();
-#pragma unroll
-        for (int p = 0; p < PPT; ++p) {
-            q.acc[p] = (uint32_t)min(atomicExch(&sacc[lp0 + TILE * 4 * p], 0ull), (unsigned long long)COV_ONE);
-            q.key[p] = min(atomicExch(&skey[lp0 + TILE * 4 * p], ~0ull), KEY_NONE);
-        }
-        if (threadIdx.x == 0) split.done[split_slot] = 0u;
-    }
-
-    if constexpr (!ROWS) {
-#pragma unroll
-        for (int p = 0; p < PPT; ++p) {
-            if (!inimg[p]) continue;
-            const size_t o = (size_t)(py0 + 4 * p) * W + px;
-            const bool hit = q.key[p] != KEY_NONE;
-            if (out_id) out_id[o] = hit ? (uint32_t)(q.key[p] & 0xffffffffull) : 0xffffffffu;
-            if (out_depth) out_depth[o] = hit ? __uint_as_float((uint32_t)(q.key[p] >> 32) + 1u) : INFINITY;
-            if (out_cov) out_cov[o] = (float)q.acc[p] * (1.0f / (float)COV_ONE);
-            if (STATS && n_inside) n_inside[o] = q.cnt_in[p];
-        }
-    } else {
-        // Through shared memory, so that each warp store covers two whole tile
-        // rows (16 pixels, 64 B each) instead of four 8-pixel pieces: over the
-        // host link 32-byte pieces cost about a quarter of its bandwidth.
-        __shared__ uint32_t s_out[3][TILE_PIX];
-#pragma unroll
-        for (int p = 0; p < PPT; ++p) {
-            const int lp = lx + TILE * (ly0 + 4 * p);
-            const bool hit = q.key[p] != KEY_NONE;
-            s_out[0][lp] = hit ? (uint32_t)(q.key[p] & 0xffffffffull) : 0xffffffffu;
-            s_out[1][lp] = hit ? (uint32_t)(q.key[p] >> 32) + 1u : __float_as_uint(INFINITY);
-            s_out[2][lp] = __float_as_uint((float)q.acc[p] * (1.0f / (float)COV_ONE));
-            if (STATS && n_inside && inimg[p]) n_inside[(size_t)(py0 + 4 * p) * W + px] = q.cnt_in[p];
-        }
-        __syncthreads();
-#pragma unroll
-        for (int i = threadIdx.x; i < TILE_PIX; i += RT) {
-            const int ox = tx * TILE + (i % TILE), oy = ty * TILE + i / TILE;
-            if (ox >= W || oy >= H) continue;
-            const size_t o = (size_t)oy * W + ox;
-            if (out_id) out_id[o] = s_out[0][i];
-            if (out_depth) out_depth[o] = __uint_as_float(s_out[1][i]);
-            if (out_cov) out_cov[o] = __uint_as_float(s_out[2][i]);
-        }
-    }
+    if (split_slot >= 0 && !merge_slot(split, split_slot, tp, q, 1u, (uint32_t)nsplit)) return;
+    write_tile<STATS, ROWS>(view, tp, q, n_inside);
 }
 
 template <bool STATS>
@@ -548,6 +592,205 @@ __global__ void __launch_bounds__(RT, VSR_RASTER_CTAS_PER_SM) raster_pool_kernel
     }
 }
 
+// Binning and raster in one launch: every tile's CTA walks its candidates
+// (walk.cuh) WALK_BLOCK at a time, lists the hits in shared memory and
+// rasterizes them, so the bins are never stored and no pass over the tiles
+// runs before.  Against the tile pass, the heavy-tile pass, the work-item pass
+// and the raster over stored bins (four launches), the walk's latency is
+// hidden by the other CTAs' evaluation (see the measured figures at
+// vsr_raster).
+//
+// A tile with many candidates is processed by several CTAs that merge in an
+// accumulator slot (merge_slot): the tile's own CTA takes a free slot and
+// publishes the tile there, the CTAs past the tiles (helpers) look for such
+// tiles, and each block of candidates goes to whoever adds 1 to the slot's
+// claim word next, (tile << 32) | blocks claimed.  An owner without a slot
+// works alone, a helper that finds nothing ends, and the part that finishes
+// the last block writes the tile and frees the slot.  A claim names its tile,
+// so one made on a slot that has changed hands is still a claim of the slot's
+// present tile; a claim past the tile's last block is no block.  While a part
+// holds unmerged blocks its slot cannot be freed.  Nobody waits for another,
+// but that helpers which start together with the tiles (fewer tiles than
+// resident CTAs) look again for about 10 us before they give up.
+struct WalkSlots {
+    SplitAcc split;             // WALK_SLOTS accumulators
+    unsigned long long* claim;  // WALK_SLOTS: (tile << 32) | blocks claimed
+    uint32_t* nblk;             // WALK_SLOTS: blocks of the slot's tile; 0 free, ~0 being set up
+    uint32_t* hits;             // WALK_SLOTS: hits of the parts merged so far
+    uint32_t* hint;             // where the next owner looks first
+    uint32_t* active;           // published tiles
+};
+
+// What a CTA knows of its tile, in shared memory: uniform, and needed only
+// between the evaluations, whose loop has no registers to spare.
+struct WalkTile {
+    Cone cone;
+    uint32_t nblk, next;  // blocks of the tile, this CTA's next one
+    uint32_t units, hits;  // blocks done and hits found by this CTA
+    int tile, slot;        // slot: -1 unless the tile is shared
+    uint32_t n;            // hits of the current block
+};
+
+template <bool ROWS>
+__global__ void __launch_bounds__(RT, VSR_RASTER_CTAS_PER_SM) raster_walk_kernel(RasterView view, WalkIndex wi,
+                                                                                 const float4* __restrict__ geom,
+                                                                                 int ntiles, uint32_t block,
+                                                                                 uint32_t split_blocks, int looks,
+                                                                                 WalkSlots slots,
+                                                                                 uint32_t* __restrict__ tile_pairs,
+                                                                                 int* __restrict__ status)
+{
+    __shared__ Stage st;
+    __shared__ WalkShared ws;
+    __shared__ WarpCones wc;
+    __shared__ WalkTile wt;
+    __shared__ uint32_t s_ids[WALK_BLOCK];
+    static_assert(RT == WALK_THREADS, "the walk's CTA");
+    const unsigned FULL = 0xffffffffu;
+    const bool helper = blockIdx.x >= (uint32_t)ntiles;
+    for (;;) {
+        PixPair q;
+        bool warp_active;
+        {
+            int tile = (int)blockIdx.x, slot = -1;
+            uint32_t first = 0u;
+            if (helper) {
+                // a published tile with blocks left: the lowest such slot from
+                // a start of this CTA's own
+                __syncthreads();
+                if (threadIdx.x == 0) {
+                    while (!*(volatile uint32_t*)slots.active && looks > 0) {
+                        --looks;
+                        __nanosleep(250);
+                    }
+                    wt.slot = *(volatile uint32_t*)slots.active ? WALK_SLOTS : -1;
+                }
+                __syncthreads();
+                if (wt.slot < 0) return;
+                const int from = (int)((blockIdx.x * 37u) % WALK_SLOTS);
+                int mine = WALK_SLOTS;
+                for (int i = threadIdx.x; i < WALK_SLOTS && mine == WALK_SLOTS; i += RT) {
+                    const int c = (from + i) % WALK_SLOTS;
+                    const uint32_t nb = *(volatile uint32_t*)&slots.nblk[c];
+                    if (nb != 0u && nb != 0xffffffffu &&
+                        (uint32_t)*(volatile unsigned long long*)&slots.claim[c] < nb)
+                        mine = i;
+                }
+                if (mine < WALK_SLOTS) atomicMin(&wt.slot, mine);
+                __syncthreads();
+                slot = wt.slot;
+                if (slot == WALK_SLOTS) return;
+                slot = (from + slot) % WALK_SLOTS;
+                if (threadIdx.x == 0) {
+                    const unsigned long long c = atomicAdd(&slots.claim[slot], 1ull);
+                    wt.tile = (int)(c >> 32);
+                    wt.next = (uint32_t)c;
+                }
+                __syncthreads();
+                tile = wt.tile;
+                first = wt.next;
+                if (tile >= ntiles) return;
+            }
+            const float4 axis = view.tiles[tile].c0;
+            float4 g[PPT];
+            load_pixels(view, TilePos(tile, view.tiles_x), g);  // in flight while the first warp finds the ranges
+            if (threadIdx.x == RT - 1) wt.cone = view.tiles[tile];
+            if (threadIdx.x < 32) walk_ranges(wi, view.T, geom[tile], axis.y, ws);
+            if (threadIdx.x == 0) {
+                const uint32_t nblk = (ws.total + block - 1) / block;
+                if (!helper && nblk > split_blocks) {
+                    const uint32_t from = atomicAdd(slots.hint, 1u);
+                    for (uint32_t i = 0; i < 8u && slot < 0; ++i) {
+                        const uint32_t c = (from + i) % WALK_SLOTS;
+                        if (atomicCAS(&slots.nblk[c], 0u, 0xffffffffu) == 0u) {
+                            atomicExch(&slots.claim[c], (unsigned long long)(uint32_t)tile << 32 | 1ull);
+                            __threadfence();
+                            atomicExch(&slots.nblk[c], nblk);
+                            atomicAdd(slots.active, 1u);
+                            slot = (int)c;
+                        }
+                    }
+                }
+                wt.tile = tile;
+                wt.slot = slot;
+                wt.nblk = nblk;
+                wt.next = first;
+                wt.units = wt.hits = wt.n = 0u;
+            }
+            warp_active = start_pixels(g, axis, q, wc);
+            __syncthreads();
+            if (helper && first >= wt.nblk) continue;  // finished meanwhile
+        }
+        while (wt.next < wt.nblk) {
+            {
+                Walk w;
+                w.init(wi, wt.cone, ws);
+                const uint32_t e0 = wt.next * block, e1 = min(ws.total, e0 + block);
+                const int lane = threadIdx.x & 31;
+                for (uint32_t i0 = e0; i0 < e1; i0 += RT) {
+                    const uint32_t idx = i0 + threadIdx.x;
+                    uint32_t t;
+                    const bool hit = w.test(wi, view.rec, view.T, ws, idx, idx < e1, t);
+                    const unsigned m = __ballot_sync(FULL, hit);
+                    if (!m) continue;
+                    uint32_t base = 0;
+                    if (lane == 0) base = atomicAdd(&wt.n, (uint32_t)__popc(m));
+                    base = __shfl_sync(FULL, base, 0);
+                    if (hit) s_ids[base + (uint32_t)__popc(m & ((1u << lane) - 1u))] = t;
+                }
+            }
+            __syncthreads();
+            for (uint32_t base = 0; base < wt.n; base += CHUNK) {
+                const int nc = (int)min((uint32_t)CHUNK, wt.n - base);
+#pragma unroll
+                for (int p = 0; p < PPT; ++p) q.acc[p] = min(q.acc[p], COV_ONE);
+                if (base) __syncthreads();
+                if ((int)threadIdx.x < nc)
+                    stage_checked(view.rec, view.T, s_ids[base + threadIdx.x], wt.cone.c0, st, threadIdx.x, status);
+                __syncthreads();
+                uint32_t ca = 0, ce = 0;
+                if (warp_active) eval_chunk<false>(st, nc, wc, false, q, ca, ce);
+            }
+            // the only block of a tile that is not shared (almost every tile):
+            // no one waits for the others' evaluation
+            if (wt.nblk == 1u && wt.slot < 0) break;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                wt.hits += wt.n;
+                wt.n = 0u;
+                ++wt.units;
+                wt.next = wt.slot >= 0 ? (uint32_t)atomicAdd(&slots.claim[wt.slot], 1ull) : wt.next + 1u;
+            }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int p = 0; p < PPT; ++p) q.acc[p] = final_acc(q, p);
+        const int tile = wt.tile, slot = wt.slot;
+        const TilePos tp(tile, view.tiles_x);
+        uint32_t hits = wt.hits + wt.n;
+        bool last = true;
+        if (slot >= 0) {
+            if (threadIdx.x == 0 && hits) atomicAdd(&slots.hits[slot], hits);
+            last = merge_slot(slots.split, slot, tp, q, wt.units, wt.nblk);
+            if (last) {
+                __threadfence();
+                __syncthreads();
+                if (threadIdx.x == 0) {
+                    hits = atomicExch(&slots.hits[slot], 0u);
+                    __threadfence();
+                    atomicSub(slots.active, 1u);
+                    atomicExch(&slots.nblk[slot], 0u);  // free
+                }
+            }
+        }
+        if (last) {
+            if (tile_pairs && threadIdx.x == 0) tile_pairs[tile] = hits;
+            write_tile<false, ROWS>(view, tp, q, nullptr);
+        }
+        if (!helper) return;
+    }
+}
+
 // Dense reference of the same rasterization: every pixel of a tile against
 // every triangle of the scene, with no binning and no cull.  As in the
 // oracle, the miter distance is evaluated first: a triangle whose enlarged
@@ -558,27 +801,14 @@ __global__ void __launch_bounds__(RT, VSR_RASTER_CTAS_PER_SM) raster_pool_kernel
 __global__ void __launch_bounds__(RT) raster_dense_kernel(RasterView view, int* __restrict__ status)
 {
     __shared__ Stage st;
-    const int tile = blockIdx.x;
-    const int W = view.W, H = view.H, T = view.T;
-    const int tx = tile % view.tiles_x, ty = tile / view.tiles_x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int px = tx * TILE + (warp & 1) * 8 + (lane & 7);
-    const int py0 = ty * TILE + (warp >> 1) * 8 + (lane >> 3);
-    const Cone tc = view.tiles[tile];
+    const int T = view.T;
+    const TilePos tp(blockIdx.x, view.tiles_x);
+    const Cone tc = view.tiles[blockIdx.x];
     const float ax = tc.c0.x, ay = tc.c0.y, az = tc.c0.z;
     PixPair q;
-    bool inimg[PPT];
-    {
-        float4 g[PPT];
-#pragma unroll
-        for (int p = 0; p < PPT; ++p) {
-            const int py = py0 + 4 * p;
-            inimg[p] = px < W && py < H;
-            g[p] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (inimg[p]) g[p] = view.map[(size_t)py * W + px];
-        }
-        pix_pair(q, g[0], g[1], ax, ay, az);
-    }
+    float4 g[PPT];
+    load_pixels(view, tp, g);
+    pix_pair(q, g[0], g[1], ax, ay, az);
     const bool active = tc.c1.z > 0.0f;
     const size_t TT = (size_t)T;
     uint32_t unused = 0;
@@ -604,15 +834,8 @@ __global__ void __launch_bounds__(RT) raster_dense_kernel(RasterView view, int* 
         }
     }
 #pragma unroll
-    for (int p = 0; p < PPT; ++p) {
-        if (!inimg[p]) continue;
-        const size_t o = (size_t)(py0 + 4 * p) * W + px;
-        const uint32_t acc = final_acc(q, p);
-        const bool hit = q.key[p] != KEY_NONE;
-        if (view.out_id) view.out_id[o] = hit ? (uint32_t)(q.key[p] & 0xffffffffull) : 0xffffffffu;
-        if (view.out_depth) view.out_depth[o] = hit ? __uint_as_float((uint32_t)(q.key[p] >> 32) + 1u) : INFINITY;
-        if (view.out_cov) view.out_cov[o] = (float)acc * (1.0f / (float)COV_ONE);
-    }
+    for (int p = 0; p < PPT; ++p) q.acc[p] = final_acc(q, p);
+    write_tile<false, false>(view, tp, q, nullptr);
 }
 
 // Work items per tile: ceil(bin / split_max) when a split slot and room in
@@ -705,6 +928,63 @@ vsr_status launch_raster_items(const RasterView& view, const uint32_t* offsets, 
     auto kern = host_out ? raster_items_kernel<true> : raster_items_kernel<false>;
     kern<<<n_tiles + extra_cap, RT, 0, st>>>(view, n_tiles, w.nsplit_of, w.split_slot, w.extra, w.counters + 1,
                                              split_max, SplitAcc{w.acc, w.key, w.done}, status);
+    VSR_CUDA_TRY(cudaGetLastError());
+    return VSR_OK;
+}
+
+vsr_status walk_work_alloc(WalkWork* w, cudaStream_t st)
+{
+    if (w->mem) return VSR_OK;
+    // accumulators | keys | claims | done | nblk | hits | hint, active
+    const size_t pix = sizeof(unsigned long long) * TILE_PIX * (size_t)WALK_SLOTS;
+    const size_t rest = sizeof(unsigned long long) * WALK_SLOTS + 3 * sizeof(uint32_t) * WALK_SLOTS + 2 * sizeof(uint32_t);
+    char* m = nullptr;
+    if (cudaMalloc((void**)&m, 2 * pix + rest) != cudaSuccess) {
+        cudaGetLastError();
+        return VSR_ERR_OOM;
+    }
+    if (cudaMemsetAsync(m, 0, pix, st) != cudaSuccess || cudaMemsetAsync(m + pix, 0xff, pix, st) != cudaSuccess ||
+        cudaMemsetAsync(m + 2 * pix, 0, rest, st) != cudaSuccess) {
+        cudaFree(m);
+        return VSR_ERR_CUDA;
+    }
+    w->mem = m;
+    return VSR_OK;
+}
+
+void walk_work_free(WalkWork* w)
+{
+    cudaFree(w->mem);
+    w->mem = nullptr;
+}
+
+vsr_status launch_raster_walk(const RasterView& view, const WalkIndex& wi, const float4* geom, const WalkWork& work,
+                              uint32_t* tile_pairs, int* status, cudaStream_t st, bool host_out)
+{
+    const int ntiles = view.tiles_x * ((view.H + TILE - 1) / TILE);
+    if (ntiles == 0) return VSR_OK;
+    const int sms = sm_count();
+    if (sms < 0) return VSR_ERR_CUDA;
+    const size_t pix = (size_t)TILE_PIX * WALK_SLOTS;
+    WalkSlots sl;
+    sl.split.acc = (unsigned long long*)work.mem;
+    sl.split.key = sl.split.acc + pix;
+    sl.claim = sl.split.key + pix;
+    sl.split.done = (uint32_t*)(sl.claim + WALK_SLOTS);
+    sl.nblk = sl.split.done + WALK_SLOTS;
+    sl.hits = sl.nblk + WALK_SLOTS;
+    sl.hint = sl.hits + WALK_SLOTS;
+    sl.active = sl.hint + 1;
+    // helpers only where a tile can have enough candidates; few tiles: smaller
+    // blocks, handed out from the second on
+    const int wave = sms * VSR_RASTER_CTAS_PER_SM;
+    const bool few = ntiles < wave;
+    const int block = few ? WALK_BLOCK / 4 : WALK_BLOCK;
+    const int split = few ? 2 : (int)WALK_SPLIT_BLOCKS;
+    const int helpers = view.T > split * block ? wave : 0;
+    auto kern = host_out ? raster_walk_kernel<true> : raster_walk_kernel<false>;
+    kern<<<ntiles + helpers, RT, 0, st>>>(view, wi, geom, ntiles, (uint32_t)block, (uint32_t)split, few ? 40 : 0, sl,
+                                          tile_pairs, status);
     VSR_CUDA_TRY(cudaGetLastError());
     return VSR_OK;
 }

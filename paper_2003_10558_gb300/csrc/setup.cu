@@ -24,7 +24,7 @@
 // is placed to ~1e-6 of a pixel.
 #include "df.cuh"
 #include "df2.cuh"
-#include "vsr_internal.cuh"
+#include "walk.cuh"
 
 namespace {
 
@@ -73,22 +73,45 @@ __device__ __forceinline__ unsigned first_positive_c(float x, float y, float z)
     return z > 0.0f;
 }
 
-// VIEWS: blockIdx.y is a view; its camera is read from cams_dev (12 floats)
-// and its records go to rec + view * REC_F * T.
-template <bool VIEWS>
+// A triangle's cell of the grid: the finest level whose cells are at least as
+// tall as the cap radius (twice the height in the coarsest; by the sine, which
+// is accurate for small caps), else the list.  sr: sin of the cap radius, 0
+// for no cap; smax: per level, the float bits of the largest one.
+__device__ __forceinline__ uint32_t grid_cell(float x, float y, float z, float cr, float sr,
+                                              unsigned (&smax)[GRID_LEVELS])
+{
+    static_assert(grid_nlat(0) == 192 && grid_nlat(1) == 96 && grid_nlat(2) == 48 && grid_nlat(3) == 12, "bounds");
+    // sin of pi/192, pi/96, pi/48, 2 pi/12, rounded down
+    constexpr float S0 = 0.0163617f, S1 = 0.0327190f, S2 = 0.0654031f, S3 = 0.5f;
+    if (!(sr > 0.0f)) return 0xffffffffu;
+    if (!(cr > 0.0f) || sr > S3) return GRID_LIST;
+    const int l = (sr > S0) + (sr > S1) + (sr > S2);
+#pragma unroll
+    for (int q = 0; q < GRID_LEVELS; ++q)
+        if (q == l) smax[q] = max(smax[q], __float_as_uint(sr));  // positive floats order as their bits
+    const int nlat = grid_nlat_of(l);
+    const int row = grid_row(grid_lat(y), nlat);
+    const int ncol = grid_ncol(nlat, row);
+    const int col = (int)floorf((grid_lon(x, z) + IDX_PI) * ((float)ncol * (0.5f / IDX_PI)));
+    return (uint32_t)(grid_base_of(l) + row * (2 * nlat + 1) + min(ncol - 1, max(0, col)));
+}
+
+// VIEW: the camera is read from cams_dev (12 floats).  grid.counts != NULL:
+// the triangles' cells are counted for launch_grid_file.
+template <bool VIEW>
 __global__ void __launch_bounds__(128, VSR_SETUP_PAIR_CTAS) setup_pair_kernel(const float* __restrict__ tris, int T,
                                                                              Cam cam, const float* __restrict__ cams_dev,
-                                                                             float4* __restrict__ rec)
+                                                                             float4* __restrict__ rec, TriGrid grid)
 {
     const int t0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+    const unsigned am = __ballot_sync(0xffffffffu, t0 < T);  // the lanes that go on
     if (t0 >= T) return;
-    if (VIEWS) {
-        const float* cv = cams_dev + 12 * blockIdx.y;
+    if (VIEW) {
+        const float* cv = cams_dev;
 #pragma unroll
         for (int q = 0; q < 3; ++q) cam.O[q] = cv[q];
 #pragma unroll
         for (int q = 0; q < 9; ++q) cam.M[q] = cv[3 + q];
-        rec += (size_t)blockIdx.y * REC_F * (size_t)T;
     }
     const bool has1 = t0 + 1 < T;
     const int t1 = has1 ? t0 + 1 : t0;
@@ -164,6 +187,22 @@ __global__ void __launch_bounds__(128, VSR_SETUP_PAIR_CTAS) setup_pair_kernel(co
     const df3_2 Nh = normalize3_2(N);
     const df2 dN = df2_dot(V[0], Nh);
 
+    if (grid.counts) {
+        unsigned smax[GRID_LEVELS] = {};
+        const uint32_t w0 = grid_cell(Sh.x.hi.x, Sh.y.hi.x, Sh.z.hi.x, slen.hi.x, bad0 ? 0.0f : sr.hi.x, smax);
+        const uint32_t w1 =
+            grid_cell(Sh.x.hi.y, Sh.y.hi.y, Sh.z.hi.y, slen.hi.y, bad1 || !has1 ? 0.0f : sr.hi.y, smax);
+        if (w0 != 0xffffffffu) atomicAdd(&grid.counts[w0], 1u);
+        if (w1 != 0xffffffffu) atomicAdd(&grid.counts[w1], 1u);
+        grid.where[t0] = w0;
+        if (has1) grid.where[t1] = w1;
+#pragma unroll
+        for (int q = 0; q < GRID_LEVELS; ++q) {
+            const unsigned m = __reduce_max_sync(am, smax[q]);
+            if (m && (threadIdx.x & 31) == 0) atomicMax(&grid.hdr[GRID_H_BUILD + q], m);
+        }
+    }
+
     const size_t TT = (size_t)T;
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
@@ -200,25 +239,26 @@ __global__ void __launch_bounds__(128, VSR_SETUP_PAIR_CTAS) setup_pair_kernel(co
 
 }  // namespace
 
-vsr_status launch_setup(const float* tris, int T, const float cam[12], float4* rec, cudaStream_t st)
+vsr_status launch_setup(const float* tris, int T, const float cam[12], float4* rec, const TriGrid* grid,
+                        cudaStream_t st)
 {
     if (T == 0) return VSR_OK;
     Cam c;
     for (int q = 0; q < 3; ++q) c.O[q] = cam[q];
     for (int q = 0; q < 9; ++q) c.M[q] = cam[3 + q];
     const int pairs = (T + 1) / 2;
-    setup_pair_kernel<false><<<(pairs + 127) / 128, 128, 0, st>>>(tris, T, c, nullptr, rec);
+    setup_pair_kernel<false><<<(pairs + 127) / 128, 128, 0, st>>>(tris, T, c, nullptr, rec, grid ? *grid : TriGrid{});
     VSR_CUDA_TRY(cudaGetLastError());
     return VSR_OK;
 }
 
-vsr_status launch_setup_views(const float* tris, int T, const float* cams_dev, int nviews, float4* rec,
-                              cudaStream_t st)
+vsr_status launch_setup_view(const float* tris, int T, const float* cam_dev, float4* rec, const TriGrid* grid,
+                             cudaStream_t st)
 {
-    if (T == 0 || nviews == 0) return VSR_OK;
-    Cam c = {};
+    if (T == 0) return VSR_OK;
     const int pairs = (T + 1) / 2;
-    setup_pair_kernel<true><<<dim3((pairs + 127) / 128, nviews), 128, 0, st>>>(tris, T, c, cams_dev, rec);
+    setup_pair_kernel<true><<<(pairs + 127) / 128, 128, 0, st>>>(tris, T, Cam{}, cam_dev, rec,
+                                                                 grid ? *grid : TriGrid{});
     VSR_CUDA_TRY(cudaGetLastError());
     return VSR_OK;
 }

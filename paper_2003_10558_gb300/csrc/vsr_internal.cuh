@@ -153,7 +153,10 @@ vsr_status launch_map_cones(const float4* map, int W, int H, Cone* tiles, float4
 // deriv (optional): 2 float4 per pixel, (d_i G, d_j G) for the pixel step
 vsr_status launch_map_spec(const vsr_map_spec& spec, float4* map, Cone* tiles, float4* geom, float4* deriv,
                            unsigned long long* h_gen, uint32_t gen, cudaStream_t st);
-vsr_status launch_setup(const float* tris, int T, const float cam[12], float4* rec, cudaStream_t st);
+struct TriGrid;
+// grid: count the triangles' cells for launch_grid_file (NULL: no grid)
+vsr_status launch_setup(const float* tris, int T, const float cam[12], float4* rec, const TriGrid* grid,
+                        cudaStream_t st);
 
 // Device memory of a tile index (sized for IDX_CELLS_MAX cells, ntiles tiles).
 // The cones of the small tiles are stored sorted by home cell, so the cells
@@ -215,81 +218,93 @@ __device__ __forceinline__ Cone index_entry(const Cone& c, int i)
     e.c1 = make_float4(c.c1.x, c.c1.y, __uint_as_float((uint32_t)i), 0.0f);
     return e;
 }
-// binning of one frame: counts and cursor zeroed by the caller ->
-// launch_bin_count (records (tile, triangle) into pairs[0, pair_cap)
-// and counts them in *cursor; pairs may be NULL) -> launch_scan(counts,
-// NULL) -> launch_bin_fill (a map over the pairs when *cursor <= pair_cap,
-// else a second search; pass the count pass's pairs / pair_cap, or NULL)
-vsr_status launch_bin_count(const float4* rec, int T, TileIndex idx, uint32_t* counts, uint32_t* cursor,
-                            uint2* pairs, uint32_t pair_cap, cudaStream_t st, int pstep = 0);
-// total_host (optional): the device address of a pinned host word that
-// also receives the total
-vsr_status launch_scan(const uint32_t* counts, const uint32_t* extra, int n, const int* n_dev, uint32_t* offsets,
-                       cudaStream_t st, uint32_t* total_host = nullptr);
+// triangle-major binning of one frame (vsr_raster_noalloc): counts zeroed by
+// the caller -> launch_bin_count -> launch_scan -> launch_bin_fill (a second
+// search)
+vsr_status launch_bin_count(const float4* rec, int T, TileIndex idx, uint32_t* counts, cudaStream_t st);
+vsr_status launch_scan(const uint32_t* counts, int n, uint32_t* offsets, cudaStream_t st);
 vsr_status launch_bin_fill(const float4* rec, int T, TileIndex idx, const uint32_t* offsets, uint32_t* counts,
-                           const uint32_t* cursor, const uint2* pairs, uint32_t pair_cap, uint32_t* ids, uint32_t cap,
-                           int* status, cudaStream_t st, int pstep = 0);
+                           uint32_t* ids, uint32_t cap, int* status, cudaStream_t st);
 
 // ---------------------------------------------------------------------------
-// Tile-major binning.  The frame's triangles are filed by the cell of their
-// cap centre on one of two latitude-longitude grids of the view sphere (the
-// same latitude / longitude as the tile index): caps of enlarged radius up to
-// two cells of the fine grid (pi / TRI_NLAT0) in its cells, TRI_K0 per cell,
-// a triangle that does not fit (a larger cap or a full cell) in the coarse
-// grid (pi / TRI_NLAT1, TRI_K1 per cell) if its cap is at most two of its
-// cells, and the rest in one list.  Every tile then tests only the triangles
-// of the cells within its half-angle plus each grid's largest cap radius of
-// its axis, and the list: one warp per tile, the same cap / cone test as the
-// triangle-major search.  One pass: the warp stages its hits in shared
-// memory, takes its range of the bins with one atomic, and writes them, so
-// the bins of tile u are ids[starts[u] .. ends[u]) (not ordered by tile);
-// starts[ntiles] receives the total.
-constexpr int TRI_NLAT0 = 128, TRI_NLON0 = 2 * TRI_NLAT0, TRI_K0 = 64;
-constexpr int TRI_NLAT1 = 16, TRI_NLON1 = 2 * TRI_NLAT1, TRI_K1 = 512;
-constexpr int TRI_CELLS0 = TRI_NLAT0 * TRI_NLON0;
-constexpr int TRI_CELLS1 = TRI_NLAT1 * TRI_NLON1;
-constexpr int TRI_LARGE = TRI_CELLS0 + TRI_CELLS1;  // the counter of the list
-constexpr int TRI_CELLS = TRI_LARGE + 1;
-// entry numbers: fine cells, coarse cells, then the list
-constexpr uint32_t TRI_E1 = (uint32_t)TRI_CELLS0 * TRI_K0;
-constexpr uint32_t TRI_E2 = TRI_E1 + (uint32_t)TRI_CELLS1 * TRI_K1;
-
-// Device memory of a triangle index (per scene, up to T triangles and
-// ntiles tiles).  The counters and the header are zero between binnings:
-// the last kernel of a binning clears them for the next one, so the
-// launches are the same every time and can be captured in a graph (after a
-// failed launch the next binning clears them first).
-constexpr int TRI_HDR = TRI_CELLS;  // header words after the cell counters:
-constexpr int TRI_H_CURSOR = 2;     //   [0..1] largest enlarged cap radius of the fine / coarse grid (float bits),
-constexpr int TRI_H_DONE = 3;       //   bin cursor, finished CTAs of the tile pass,
-constexpr int TRI_H_HEAVY = 4;      //   heavy tiles listed,
-constexpr int TRI_H_NEXT = 5;       //   heavy tiles taken,
-constexpr int TRI_H_DONE2 = 6;      //   finished CTAs of the heavy-tile pass
-constexpr int TRI_WORDS = TRI_CELLS + 7;
-struct TriIndex {
-    // TRI_WORDS: triangles filed per cell (may exceed the cell's capacity)
-    // and the list length, then the header
-    uint32_t* counts;
-    uint32_t* heavy;  // ntiles: tiles binned by a whole CTA (more than BIN_STAGE_HITS entries)
-    float4* cap;      // TRI_E2 + T entries: (S-hat xyz, cos beta)
-    float2* cs;       // TRI_E2 + T entries: (sin beta, triangle bits)
-    int64_t T;        // capacity of the list
-    int ntiles;       // capacity of the heavy list
-    bool dirty;       // host side: a binning may have left the counters behind
+// Triangle grid: the triangles of a set-up by the place of their caps on the
+// view sphere, built with the set-up (it does not depend on the map) and
+// walked by every tile of a raster or binning (walk.cuh).
+//
+// GRID_LEVELS latitude-longitude grids (latitude = asin(y), longitude =
+// atan2(x, z)), 192 rows in the finest; a triangle is filed by its cap's
+// centre in the finest level whose cells are at least as tall as its cap
+// radius (twice the height in the coarsest), and in a list beyond that.  Rows
+// near the poles have fewer cells (grid_ncol), so cells are of about equal
+// area.  The triangles of a row's cells are consecutive entries in cell order,
+// so a window of a row is one range of entries (two where it wraps), and the
+// levels' largest radii bound how far a tile has to look.  The entries are
+// sorted by counting (cell counts in the set-up kernel, row starts, entries),
+// so there is no capacity per cell.
+// The levels by a model of the candidates per tile (window area x density) on
+// the 1080p frame, a 4096 x 2176 frame, a view inside a cloud and smaller
+// ones: 2.4 - 4.2 per triangle whose cap reaches the tile, against 2.4 - 4.3
+// with levels of 192, 48, 12 rows and 3.0 - 7.5 with 128, 16; levels of 256
+// and 512 rows save up to a fifth of the candidates but double the ranges.
+constexpr int GRID_LEVELS = 4;
+__host__ __device__ constexpr int grid_nlat(int l) { return l == 0 ? 192 : (l == 1 ? 96 : (l == 2 ? 48 : 12)); }
+__host__ __device__ constexpr int grid_stride(int l) { return 2 * grid_nlat(l) + 1; }  // words per row: cells, end
+__host__ __device__ constexpr int grid_base(int l)
+{
+    int b = 0;
+    for (int q = 0; q < l; ++q) b += grid_nlat(q) * grid_stride(q);
+    return b;
+}
+constexpr int GRID_LIST = grid_base(GRID_LEVELS);  // the list: its start, its end
+constexpr int GRID_WORDS = GRID_LIST + 2;
+constexpr int GRID_ROWS = grid_nlat(0) + grid_nlat(1) + grid_nlat(2) + grid_nlat(3);
+// header words
+constexpr int GRID_H_BUILD = 0;   // [0 .. 3] per level: float bits of the largest sin(cap radius), while filing
+constexpr int GRID_H_CURSOR = 4;  // entries given to rows, while filing
+constexpr int GRID_H_MAX = 8;     // [8 .. 11] the filed triangles' largest sin(cap radius) per level, 0: level empty
+constexpr int GRID_H_N = 12;      // entries
+constexpr int GRID_HDR = 16;
+// scenes of up to this many triangles have no grid: every tile tests them
+// all, two steps of a CTA (the two filing launches cost more, ~5 us)
+constexpr int GRID_DIRECT = 256;
+struct TriGrid {
+    uint32_t* counts = nullptr;  // GRID_WORDS: triangles counted per cell, then left to place; zero between set-ups
+    uint32_t* start = nullptr;   // GRID_WORDS: first entry of each cell, each row closed by its end
+    uint32_t* hdr = nullptr;     // GRID_HDR
+    uint32_t* where = nullptr;   // T: cell word, or ~0 without a cap
+    float4* ent = nullptr;       // T entries: (S-hat xyz, cos rho)
+    float2* ent2 = nullptr;      // (sin rho, triangle bits)
+    int64_t T = 0;               // capacity
+    bool dirty = false;          // host side: a failed set-up may have left counters behind
 };
-vsr_status tri_index_alloc(TriIndex* ti, int64_t T, int ntiles);
-void tri_index_free(TriIndex* ti);
-size_t tri_index_bytes(int64_t T, int ntiles);
-// binning of one frame, tile-major: the triangle index of rec, then every
-// tile of the map.  idx: the map's tile index (its header's
-// widest ramp and each tile's geometry); tiles: the map's ntiles cones;
-// starts / ends: ntiles + 1 / ntiles words; T <= ti->T.  With more pairs
-// than cap the bins are cut at cap and VSR_ERR_BIN_OVERFLOW is raised;
-// total_host (optional): the device address of a pinned host word that
+vsr_status grid_alloc(TriGrid* g, int64_t T);
+void grid_free(TriGrid* g);
+size_t grid_bytes(int64_t T);
+// row starts and entries from the cells and counts of the set-up kernel
+vsr_status launch_grid_file(const float4* rec, int T, const TriGrid& g, cudaStream_t st);
+// what the walk reads: a grid, or (direct) the caps of all T triangles
+struct WalkIndex {
+    const uint32_t* start;
+    const uint32_t* hdr;
+    const float4* ent;
+    const float2* ent2;
+    int direct;
+    int pstep;  // caps of the per-fragment pixel step
+};
+inline bool grid_used(int64_t T) { return T > GRID_DIRECT; }
+inline WalkIndex walk_index(const TriGrid& g, int64_t T, int pstep = 0)
+{
+    return WalkIndex{g.start, g.hdr, g.ent, g.ent2, grid_used(T) ? 0 : 1, pstep};
+}
+// binning by the walk: every tile's bin, in one launch.  starts / ends: ntiles
+// + 1 / ntiles words, tile u's ids at [starts[u], ends[u]) in no order of
+// tiles, starts[ntiles] the total; ctr: two words, zero between binnings.
+// With more pairs than cap the bins are cut at cap and VSR_ERR_BIN_OVERFLOW is
+// raised; total_host (optional): the device address of a pinned host word that
 // also receives the total.
-vsr_status launch_bin_tiles(const float4* rec, int T, const TileIndex& idx, const Cone* tiles, int ntiles,
-                            TriIndex& ti, uint32_t* starts, uint32_t* ends, uint32_t* ids, uint32_t cap, int* status,
-                            uint32_t* total_host, cudaStream_t st, int pstep = 0);
+vsr_status launch_bin_walk(const float4* rec, int T, const WalkIndex& wi, const float4* geom, const Cone* tiles,
+                           int ntiles, uint32_t* ctr, uint32_t* starts, uint32_t* ends, uint32_t* ids, uint32_t cap,
+                           int* status, uint32_t* total_host, cudaStream_t st);
 // One view as the raster kernel sees it: its map, tile cones, set-up
 // records, bin offsets (indexed by the view's own tile number), bin ids and
 // outputs.
@@ -306,8 +321,8 @@ struct RasterView {
     uint32_t* out_id;
     float* out_depth;
     float* out_cov;
-    // bins of the tile-major binner: tile u's bin ends at ends[u] (NULL:
-    // bins in tile order, tile u's ending at offsets[u + 1])
+    // stored bins of the walk: tile u's bin ends at ends[u] (NULL: bins in
+    // tile order, tile u's ending at offsets[u + 1])
     const uint32_t* ends = nullptr;
 };
 
@@ -321,10 +336,6 @@ struct BinView {
     const float4* rec;
     uint32_t* counts;
     const uint32_t* offsets;
-    uint2* pairs;       // (tile, triangle) of every hit, or NULL
-    uint32_t pair_cap;
-    uint32_t* cursor;   // hits recorded (may exceed pair_cap: the list is then incomplete)
-    int pstep;          // bins for the per-fragment pixel step (wider caps, see pstep_cap)
     uint32_t ntiles;    // tiles of the map: every index read from the tile index is clamped to it
 };
 
@@ -396,6 +407,21 @@ vsr_status launch_raster_pool(const PoolView* views_dev, const uint32_t* item_st
 // host_out: the outputs are pinned host memory (written in whole tile rows)
 vsr_status launch_raster_items(const RasterView& view, const uint32_t* offsets, uint32_t n_tiles, uint32_t cap,
                                RasterWork w, int split_max, int* status, cudaStream_t st, bool host_out = false);
+// binning and raster in one launch over the grid (raster_walk_kernel): the
+// slots in which the parts of a tile with many candidates merge
+constexpr int WALK_SLOTS = 1024;
+constexpr uint32_t WALK_SPLIT_BLOCKS = 3;  // blocks of candidates up to which a tile is one CTA's
+struct WalkWork {
+    char* mem = nullptr;
+};
+// (cleared on st; a launch leaves the slots as it found them)
+vsr_status walk_work_alloc(WalkWork* w, cudaStream_t st);
+void walk_work_free(WalkWork* w);
+constexpr size_t WALK_WORK_BYTES = (size_t)WALK_SLOTS * (16 * TILE_PIX + 20) + 8;
+// view: no bins needed; tile_pairs (optional): the triangles found per tile;
+// host_out: as launch_raster_items
+vsr_status launch_raster_walk(const RasterView& view, const WalkIndex& wi, const float4* geom, const WalkWork& work,
+                              uint32_t* tile_pairs, int* status, cudaStream_t st, bool host_out = false);
 // the dense reference: every pixel against every triangle, no bins
 vsr_status launch_raster_dense(const RasterView& view, int* status, cudaStream_t st);
 // allocate / free a RasterWork for up to n_tiles tiles (accumulators
@@ -403,15 +429,12 @@ vsr_status launch_raster_dense(const RasterView& view, int* status, cudaStream_t
 vsr_status raster_work_alloc(RasterWork* w, uint32_t n_tiles);
 void raster_work_free(RasterWork* w);
 int raster_threads_per_cta();
-// set-up of nviews views (grid.y = view) with the cameras in device memory
-// (12 floats each: O xyz, M 3x3 row-major); view v's records at
-// rec + v * REC_F * T
-vsr_status launch_setup_views(const float* tris, int T, const float* cams_dev, int nviews, float4* rec,
+// the same with the camera in device memory (12 floats: O xyz, M 3x3 row-major)
+vsr_status launch_setup_view(const float* tris, int T, const float* cam_dev, float4* rec, const TriGrid* grid,
                               cudaStream_t st);
-// exclusive scan of counts (+ extra) for large n (multi-CTA); `partials`
-// needs 2 * ceil(n / 4096) + 2 words
-vsr_status launch_scan_large(const uint32_t* counts, const uint32_t* extra, int n, uint32_t* partials,
-                             uint32_t* offsets, cudaStream_t st);
+// exclusive scan of counts for large n (multi-CTA); `partials` needs
+// 2 * ceil(n / 4096) + 2 words
+vsr_status launch_scan_large(const uint32_t* counts, int n, uint32_t* partials, uint32_t* offsets, cudaStream_t st);
 
 vsr_status launch_raster(const float4* map, int W, int H, const Cone* tiles, const float4* rec, int T,
                          const uint32_t* offsets, const uint32_t* ids, uint32_t cap, uint32_t* id, float* depth,
