@@ -640,7 +640,7 @@ static vsr_status raster_tiles(vsr_map m, vsr_scene sc, uint32_t* id_dev, float*
         if (ntiles > sc->work_tiles) {
             raster_work_free(&sc->work);
             sc->work_tiles = 0;
-            vsr_status s = raster_work_alloc(&sc->work, ntiles);
+            vsr_status s = raster_work_alloc(&sc->work, ntiles, (cudaStream_t)stream);
             if (s != VSR_OK) return s;
             sc->work_tiles = ntiles;
         }
@@ -1111,7 +1111,7 @@ vsr_status batch_view_alloc(BatchView& v, int64_t T, int tiles, bool pooled, cud
         v.tiles = 0;
         if ((s = dalloc(&v.offsets, (size_t)tiles + 1)) != VSR_OK) return s;
         if ((s = dalloc(&v.ends, (size_t)tiles)) != VSR_OK) return s;
-        if ((s = raster_work_alloc(&v.work, (uint32_t)tiles)) != VSR_OK) return s;
+        if ((s = raster_work_alloc(&v.work, (uint32_t)tiles, st)) != VSR_OK) return s;
         v.tiles = tiles;
     }
     return VSR_OK;

@@ -1000,27 +1000,30 @@ vsr_status launch_raster_dense(const RasterView& view, int* status, cudaStream_t
 
 int raster_threads_per_cta() { return RT; }
 
-vsr_status raster_work_alloc(RasterWork* w, uint32_t n_tiles)
+vsr_status raster_work_alloc(RasterWork* w, uint32_t n_tiles, cudaStream_t st)
 {
     *w = RasterWork{};
-    const uint32_t cap = n_tiles < SPLIT_SLOTS ? n_tiles : SPLIT_SLOTS;
-    const uint32_t xcap = EXTRA_ITEMS;
-    if (cudaMalloc((void**)&w->nsplit_of, sizeof(uint32_t) * (n_tiles + 1)) != cudaSuccess ||
-        cudaMalloc((void**)&w->split_slot, sizeof(int32_t) * (n_tiles + 1)) != cudaSuccess ||
-        cudaMalloc((void**)&w->counters, sizeof(uint32_t) * 2) != cudaSuccess ||
-        cudaMalloc((void**)&w->extra, sizeof(uint2) * xcap) != cudaSuccess ||
-        cudaMalloc((void**)&w->acc, sizeof(unsigned long long) * TILE_PIX * ((size_t)cap + 1)) != cudaSuccess ||
-        cudaMalloc((void**)&w->key, sizeof(unsigned long long) * TILE_PIX * ((size_t)cap + 1)) != cudaSuccess ||
-        cudaMalloc((void**)&w->done, sizeof(uint32_t) * ((size_t)cap + 1)) != cudaSuccess) {
+    const size_t cap = n_tiles < SPLIT_SLOTS ? n_tiles : SPLIT_SLOTS;
+    // one allocation: accumulators | keys | extra items | done | items and slots per tile | counters
+    const size_t pix = sizeof(unsigned long long) * TILE_PIX * (cap + 1);
+    const size_t extra = sizeof(uint2) * EXTRA_ITEMS, done = sizeof(uint32_t) * (cap + 1);
+    const size_t tiles = sizeof(uint32_t) * ((size_t)n_tiles + 1);
+    char* m = nullptr;
+    if (cudaMalloc((void**)&m, 2 * pix + extra + done + 2 * tiles + 2 * sizeof(uint32_t)) != cudaSuccess) {
         cudaGetLastError();
-        raster_work_free(w);
         return VSR_ERR_OOM;
     }
-    w->split_cap = cap;
-    w->extra_cap = xcap;
-    if (cudaMemset(w->acc, 0, sizeof(unsigned long long) * TILE_PIX * ((size_t)cap + 1)) != cudaSuccess ||
-        cudaMemset(w->key, 0xff, sizeof(unsigned long long) * TILE_PIX * ((size_t)cap + 1)) != cudaSuccess ||
-        cudaMemset(w->done, 0, sizeof(uint32_t) * ((size_t)cap + 1)) != cudaSuccess) {
+    w->acc = (unsigned long long*)m;
+    w->key = (unsigned long long*)(m + pix);
+    w->extra = (uint2*)(m + 2 * pix);
+    w->done = (uint32_t*)(m + 2 * pix + extra);
+    w->nsplit_of = (uint32_t*)(m + 2 * pix + extra + done);
+    w->split_slot = (int32_t*)(m + 2 * pix + extra + done + tiles);
+    w->counters = (uint32_t*)(m + 2 * pix + extra + done + 2 * tiles);
+    w->split_cap = (uint32_t)cap;
+    w->extra_cap = EXTRA_ITEMS;
+    if (cudaMemsetAsync(w->acc, 0, pix, st) != cudaSuccess || cudaMemsetAsync(w->key, 0xff, pix, st) != cudaSuccess ||
+        cudaMemsetAsync(w->done, 0, done, st) != cudaSuccess) {
         raster_work_free(w);
         return VSR_ERR_CUDA;
     }
@@ -1029,12 +1032,6 @@ vsr_status raster_work_alloc(RasterWork* w, uint32_t n_tiles)
 
 void raster_work_free(RasterWork* w)
 {
-    cudaFree(w->nsplit_of);
-    cudaFree(w->split_slot);
-    cudaFree(w->counters);
-    cudaFree(w->extra);
     cudaFree(w->acc);
-    cudaFree(w->key);
-    cudaFree(w->done);
     *w = RasterWork{};
 }

@@ -425,8 +425,9 @@ vsr_status launch_raster_walk(const RasterView& view, const WalkIndex& wi, const
 // the dense reference: every pixel against every triangle, no bins
 vsr_status launch_raster_dense(const RasterView& view, int* status, cudaStream_t st);
 // allocate / free a RasterWork for up to n_tiles tiles (accumulators
-// initialised)
-vsr_status raster_work_alloc(RasterWork* w, uint32_t n_tiles);
+// initialised on st, before the launches that follow there: a clear on another
+// stream would race with them)
+vsr_status raster_work_alloc(RasterWork* w, uint32_t n_tiles, cudaStream_t st);
 void raster_work_free(RasterWork* w);
 int raster_threads_per_cta();
 // the same with the camera in device memory (12 floats: O xyz, M 3x3 row-major)
