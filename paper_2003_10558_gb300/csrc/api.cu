@@ -74,7 +74,6 @@ vsr_status map_alloc(vsr_map m, int W, int H)
     if ((st = dalloc(&m->idx.geom, nt)) != VSR_OK) return st;
     m->idx.ntiles = (uint32_t)nt;
     m->idx_built = false;
-    m->hgen = 0;  // the first generation clears the widest-ramp word
     if ((m->spec.flags & VSR_MAP_DERIVATIVES) && (st = dalloc(&m->deriv, 2 * (size_t)W * H)) != VSR_OK) return st;
     return VSR_OK;
 }
@@ -138,31 +137,18 @@ void set_universal_spec(vsr_map m)
     m->lens_grad = true;
 }
 
-// the next generation of the map's widest-ramp word: the first one (of
-// new memory, or after 2^32 - 1 of them) clears the word on st first
-vsr_status next_hgen(vsr_map m, cudaStream_t st)
-{
-    if (m->hgen == 0 || m->hgen == 0xffffffffu) {
-        VSR_CUDA_TRY(cudaMemsetAsync(&m->idx.hdr->h_gen, 0, sizeof(unsigned long long), st));
-        m->hgen = 0;
-    }
-    ++m->hgen;
-    return VSR_OK;
-}
-
 // One generation of the map: the map kernel writes the map, the tile cones
-// and geometry and the widest ramp, all the tile-major binner needs; the
-// tile index of the triangle-major search is left to its first use.
+// and their geometry; the tile index of the triangle-major search is left to
+// its first use.
 vsr_status map_generate(vsr_map m, cudaStream_t st)
 {
     bool plain = m->spec.kind == VSR_MAP_UNIVERSAL && !m->deriv;
     for (int q = 0; q < 6; ++q) plain = plain && m->spec.distortion[q] == 0.0f;
     m->idx_built = false;
-    vsr_status s = next_hgen(m, st);
-    if (s != VSR_OK) return s;
-    s = plain ? launch_map(m->p.W, m->p.H, m->p.aov, m->p.k, m->p.l, m->p.s, m->p.omega_deg, m->map, m->tiles,
-                           m->idx.geom, &m->idx.hdr->h_gen, m->hgen, st)
-              : launch_map_spec(m->spec, m->map, m->tiles, m->idx.geom, m->deriv, &m->idx.hdr->h_gen, m->hgen, st);
+    const vsr_status s =
+        plain ? launch_map(m->p.W, m->p.H, m->p.aov, m->p.k, m->p.l, m->p.s, m->p.omega_deg, m->map, m->tiles,
+                           m->idx.geom, st)
+              : launch_map_spec(m->spec, m->map, m->tiles, m->idx.geom, m->deriv, st);
     m->gen = g_gen.fetch_add(1);
     return s;
 }
@@ -229,22 +215,22 @@ vsr_status bins_realloc(vsr_scene sc, uint32_t want)
 
 vsr_status ensure_ws(vsr_scene sc, int ntiles, cudaStream_t st)
 {
-    vsr_status s;
-    if (!sc->bin_ctr) {
-        if ((s = dalloc(&sc->bin_ctr, 2)) != VSR_OK) return s;
-        VSR_CUDA_TRY(cudaMemsetAsync(sc->bin_ctr, 0, 2 * sizeof(uint32_t), st));
-    }
     if (ntiles <= sc->ws_tiles) return VSR_OK;
-    cudaFree(sc->ends);
+    // one allocation: offsets | ends | tile_pairs | bin_ctr
+    const size_t n = (size_t)ntiles;
     cudaFree(sc->offsets);
-    cudaFree(sc->tile_pairs);
-    sc->ends = sc->offsets = sc->tile_pairs = nullptr;
+    sc->offsets = sc->ends = sc->tile_pairs = sc->bin_ctr = nullptr;
     sc->ws_tiles = 0;
-    if ((s = dalloc(&sc->ends, (size_t)ntiles)) != VSR_OK) return s;
-    if ((s = dalloc(&sc->offsets, (size_t)ntiles + 1)) != VSR_OK) return s;
-    if ((s = dalloc(&sc->tile_pairs, (size_t)ntiles)) != VSR_OK) return s;
+    vsr_status s = dalloc(&sc->offsets, 3 * n + 3);
+    if (s != VSR_OK) return s;
+    sc->ends = sc->offsets + n + 1;
+    sc->tile_pairs = sc->ends + n;
+    sc->bin_ctr = sc->tile_pairs + n;
+    VSR_CUDA_TRY(cudaMemsetAsync(sc->bin_ctr, 0, 2 * sizeof(uint32_t), st));
     sc->ws_tiles = ntiles;
     sc->sized_shape = 0;
+    // (the bins' places went with the old arrays)
+    sc->binned_map = sc->binned_scene = 0;
     return VSR_OK;
 }
 
@@ -402,8 +388,7 @@ vsr_status vsr_map_from_device(const float* xyzd_dev, int W, int H, void* stream
     if (s == VSR_OK && cudaMemcpyAsync(m->map, xyzd_dev, sizeof(float4) * (size_t)W * H, cudaMemcpyDeviceToDevice,
                                        st) != cudaSuccess)
         s = VSR_ERR_CUDA;
-    if (s == VSR_OK) s = next_hgen(m, st);
-    if (s == VSR_OK) s = launch_map_cones(m->map, W, H, m->tiles, m->idx.geom, &m->idx.hdr->h_gen, m->hgen, st);
+    if (s == VSR_OK) s = launch_map_cones(m->map, W, H, m->tiles, m->idx.geom, st);
     if (s != VSR_OK) {
         map_release(m);
         delete m;
@@ -514,10 +499,7 @@ void vsr_scene_free(vsr_scene sc)
 {
     if (!sc) return;
     cudaFree(sc->rec);
-    cudaFree(sc->ends);
     cudaFree(sc->offsets);
-    cudaFree(sc->tile_pairs);
-    cudaFree(sc->bin_ctr);
     cudaFree(sc->ids);
     grid_free(&sc->grid);
     walk_work_free(&sc->walk);
@@ -1041,9 +1023,7 @@ void batch_view_free(BatchView& v)
     cudaFree(v.rec);
     grid_free(&v.grid);
     walk_work_free(&v.walk);
-    cudaFree(v.ctr);
     cudaFree(v.offsets);
-    cudaFree(v.ends);
     cudaFree(v.ids);
     raster_work_free(&v.work);
     v = BatchView{};
@@ -1099,18 +1079,15 @@ vsr_status batch_view_alloc(BatchView& v, int64_t T, int tiles, bool pooled, cud
     }
     if ((s = walk_work_alloc(&v.walk, st)) != VSR_OK) return s;
     if (!pooled) return VSR_OK;
-    if (!v.ctr) {
-        if ((s = dalloc(&v.ctr, 2)) != VSR_OK) return s;
-        VSR_CUDA_TRY(cudaMemsetAsync(v.ctr, 0, 2 * sizeof(uint32_t), st));
-    }
     if (tiles > v.tiles) {
         cudaFree(v.offsets);
-        cudaFree(v.ends);
         raster_work_free(&v.work);
-        v.offsets = v.ends = nullptr;
+        v.offsets = v.ends = v.ctr = nullptr;
         v.tiles = 0;
-        if ((s = dalloc(&v.offsets, (size_t)tiles + 1)) != VSR_OK) return s;
-        if ((s = dalloc(&v.ends, (size_t)tiles)) != VSR_OK) return s;
+        if ((s = dalloc(&v.offsets, 2 * (size_t)tiles + 3)) != VSR_OK) return s;
+        v.ends = v.offsets + tiles + 1;
+        v.ctr = v.ends + tiles;
+        VSR_CUDA_TRY(cudaMemsetAsync(v.ctr, 0, 2 * sizeof(uint32_t), st));
         if ((s = raster_work_alloc(&v.work, (uint32_t)tiles, st)) != VSR_OK) return s;
         v.tiles = tiles;
     }

@@ -139,10 +139,7 @@ __global__ void __launch_bounds__(IDX_FUSED_THREADS) idx_fused_kernel(const Cone
     __shared__ TileIndexHdr s_h;
     __shared__ uint32_t s_wsum[IDX_FUSED_THREADS / 32];
     const int tid = threadIdx.x, lane = tid & 31;
-    if (tid == 0) {
-        s_h = TileIndexHdr{};
-        s_h.h_gen = hdr->h_gen;  // the map kernels' word, kept
-    }
+    if (tid == 0) s_h = TileIndexHdr{};
     __syncthreads();
     // 1. histogram of half-angles (one add per group of equal bins in a
     // warp), valid tiles, widest ramp (one atomic per warp)

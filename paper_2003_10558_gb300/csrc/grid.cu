@@ -182,25 +182,28 @@ vsr_status grid_alloc(TriGrid* g, int64_t T)
 {
     if (!g->counts) {
         // counters and header in one allocation, cleared by the first set-up
-        VSR_CUDA_TRY(cudaMalloc((void**)&g->counts, sizeof(uint32_t) * (2 * (size_t)GRID_WORDS + GRID_HDR)));
+        if (cudaMalloc((void**)&g->counts, sizeof(uint32_t) * (2 * (size_t)GRID_WORDS + GRID_HDR)) != cudaSuccess) {
+            cudaGetLastError();
+            g->counts = nullptr;
+            return VSR_ERR_OOM;
+        }
         g->hdr = g->counts + GRID_WORDS;
         g->start = g->hdr + GRID_HDR;
         g->dirty = true;
     }
     if (T > g->T) {
-        cudaFree(g->where);
         cudaFree(g->ent);
-        cudaFree(g->ent2);
         g->where = nullptr;
         g->ent = nullptr;
         g->ent2 = nullptr;
         g->T = 0;
-        if (cudaMalloc((void**)&g->where, sizeof(uint32_t) * (size_t)T) != cudaSuccess ||
-            cudaMalloc((void**)&g->ent, sizeof(float4) * (size_t)T) != cudaSuccess ||
-            cudaMalloc((void**)&g->ent2, sizeof(float2) * (size_t)T) != cudaSuccess) {
+        if (cudaMalloc((void**)&g->ent, (sizeof(float4) + sizeof(float2) + sizeof(uint32_t)) * (size_t)T) !=
+            cudaSuccess) {
             cudaGetLastError();
             return VSR_ERR_OOM;
         }
+        g->ent2 = (float2*)(g->ent + T);
+        g->where = (uint32_t*)(g->ent2 + T);
         g->T = T;
     }
     return VSR_OK;
@@ -209,9 +212,7 @@ vsr_status grid_alloc(TriGrid* g, int64_t T)
 void grid_free(TriGrid* g)
 {
     cudaFree(g->counts);
-    cudaFree(g->where);
     cudaFree(g->ent);
-    cudaFree(g->ent2);
     *g = TriGrid{};
 }
 

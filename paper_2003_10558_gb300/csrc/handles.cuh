@@ -36,7 +36,6 @@ struct vsr_map_s {
     // (vsr_raster_noalloc)
     TileIndex idx = {};
     bool idx_built = false;
-    uint32_t hgen = 0;  // generation of the widest-ramp word (idx.hdr->h_gen)
     int tx = 0, ty = 0;
     uint64_t gen = 0;
 };

@@ -85,17 +85,12 @@ struct Cone {
 // latitude/longitude window of cells.  Grid size and alpha_cut are chosen on
 // the device from the distribution of tile half-angles.  The index serves
 // the triangle-major search of the fixed-array path and is built on its
-// first use after each generation of the map; the header's first word, the
-// widest ramp, is kept by the map kernels for every generation.
+// first use after each generation of the map.
 constexpr int IDX_NLAT_MAX = 128;
 constexpr int IDX_CELLS_MAX = IDX_NLAT_MAX * 2 * IDX_NLAT_MAX;
 constexpr int IDX_HIST = 64;
 
 struct TileIndexHdr {
-    // (generation << 32) | float bits of the largest ramp half-width of the
-    // map's latest generation: raised by the map kernels with a 64-bit
-    // maximum, so the widest ramp is known without the rest of the index
-    unsigned long long h_gen;
     int nlat, nlon;             // grid: nlon = 2 nlat, square cells of `cell` radians
     int ncell;                  // nlat * nlon
     float cell;
@@ -142,17 +137,14 @@ __device__ __forceinline__ bool cap_hits_cone(float3 S, float cos_rho, float sin
     } while (0)
 
 // Kernel launchers (defined in the .cu files, called by the host library).
-// The map kernels write the tile cones and geometry and raise the map's
-// widest-ramp word h_gen (TileIndexHdr::h_gen) with generation gen, which
-// must exceed every generation the word has seen.
+// The map kernels write the map, the tile cones and their geometry.
 vsr_status launch_map(int W, int H, int aov, float k, float l, float s, float omega_deg, float4* map, Cone* tiles,
-                      float4* geom, unsigned long long* h_gen, uint32_t gen, cudaStream_t st);
-vsr_status launch_map_cones(const float4* map, int W, int H, Cone* tiles, float4* geom, unsigned long long* h_gen,
-                            uint32_t gen, cudaStream_t st);
+                      float4* geom, cudaStream_t st);
+vsr_status launch_map_cones(const float4* map, int W, int H, Cone* tiles, float4* geom, cudaStream_t st);
 // a map of any vsr_map_kind (param after limits for the Universal kind);
 // deriv (optional): 2 float4 per pixel, (d_i G, d_j G) for the pixel step
 vsr_status launch_map_spec(const vsr_map_spec& spec, float4* map, Cone* tiles, float4* geom, float4* deriv,
-                           unsigned long long* h_gen, uint32_t gen, cudaStream_t st);
+                           cudaStream_t st);
 struct TriGrid;
 // grid: count the triangles' cells for launch_grid_file (NULL: no grid)
 vsr_status launch_setup(const float* tris, int T, const float cam[12], float4* rec, const TriGrid* grid,
