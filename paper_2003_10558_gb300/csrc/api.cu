@@ -234,11 +234,18 @@ vsr_status ensure_ws(vsr_scene sc, int ntiles, cudaStream_t st)
     return VSR_OK;
 }
 
-// the bins' sizes depend on the map, the scene and the step's cap width
-uint64_t bin_shape_of(vsr_map m, vsr_scene sc, int pstep)
+// The bins' sizes depend on the map, the scene and the step's cap width: are
+// they sized for this shape?  (Those of the pixel step's wider caps hold the
+// global step's too.)
+uint64_t bin_shape_of(vsr_map m, vsr_scene sc) { return ((uint64_t)(m->tx * m->ty) << 32) ^ (uint64_t)sc->T; }
+bool bins_sized(vsr_map m, vsr_scene sc, int pstep)
 {
-    return ((uint64_t)(m->tx * m->ty) << 32) ^ (uint64_t)sc->T ^ ((uint64_t)(pstep != 0) << 63);
+    if (sc->cap == 0) return false;
+    return sc->async_sizing || (sc->sized_shape == bin_shape_of(m, sc) && (!pstep || sc->sized_pstep));
 }
+
+// the scene's workspace of a walking raster, and its bookkeeping
+vsr_status walk_begin(vsr_map m, vsr_scene sc, cudaStream_t st);
 
 }  // namespace
 
@@ -536,11 +543,14 @@ vsr_status vsr_raster_pstep(vsr_map m, vsr_scene sc, uint32_t* id_dev, float* de
 {
     if (!m || !sc || !m->deriv) return VSR_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    vsr_status s = bin_scene(m, sc, 1, st);
-    if (s != VSR_OK) return s;
-    const RasterView v{m->map,  m->p.W, m->p.H, m->tiles, m->tx,     sc->rec,   (int)sc->T, sc->offsets,
-                       sc->ids, sc->cap, id_dev, depth_dev, cov_dev, sc->ends};
-    s = launch_raster_pstep(v, m->deriv, scene_status(sc), st);
+    vsr_status s;
+    // the first frame of a shape also sizes and fills the stored bins (see raster_frame)
+    if (!bins_sized(m, sc, 1) && (s = bin_scene(m, sc, 1, st)) != VSR_OK) return s;
+    if ((s = walk_begin(m, sc, st)) != VSR_OK) return s;
+    const RasterView v{m->map,  m->p.W, m->p.H, m->tiles, m->tx,    sc->rec,  (int)sc->T,
+                       nullptr, nullptr, 0u,    id_dev,   depth_dev, cov_dev};
+    s = launch_raster_pstep(v, m->deriv, walk_index(sc->grid, sc->T, 1), m->idx.geom, sc->walk, sc->tile_pairs,
+                            scene_status(sc), st);
     return s == VSR_OK ? scene_used(sc, st) : s;
 }
 
@@ -559,8 +569,7 @@ static vsr_status bin_scene(vsr_map m, vsr_scene sc, int pstep, cudaStream_t st)
     // (copied to pinned memory, read only once its event has completed, never
     // waited for) grows the capacity ahead of need, and the binning kernels
     // report any overflow in the status word.
-    const uint64_t shape = bin_shape_of(m, sc, pstep);
-    const bool resize = sc->cap == 0 || (!sc->async_sizing && sc->sized_shape != shape);
+    const bool resize = !bins_sized(m, sc, pstep);
     if (!resize && sc->total_pending && cudaEventQuery(sc->total_event) == cudaSuccess) {
         sc->total_pending = false;
         const uint64_t last = *sc->h_total;
@@ -597,7 +606,8 @@ static vsr_status bin_scene(vsr_map m, vsr_scene sc, int pstep, cudaStream_t st)
             if ((s = bins_realloc(sc, (uint32_t)want)) != VSR_OK) return s;
             if ((s = walk(scene_status(sc), nullptr)) != VSR_OK) return s;
         }
-        sc->sized_shape = shape;
+        sc->sized_shape = bin_shape_of(m, sc);
+        sc->sized_pstep = pstep != 0;
     }
     sc->binned_map = m->gen;
     sc->binned_scene = sc->gen;
@@ -641,6 +651,20 @@ static vsr_status raster_tiles(vsr_map m, vsr_scene sc, uint32_t* id_dev, float*
     return s == VSR_OK ? scene_used(sc, (cudaStream_t)stream) : s;
 }
 
+namespace {
+vsr_status walk_begin(vsr_map m, vsr_scene sc, cudaStream_t st)
+{
+    const int ntiles = m->tx * m->ty;
+    vsr_status s;
+    if ((s = ensure_ws(sc, ntiles, st)) != VSR_OK || (s = walk_work_alloc(&sc->walk, st)) != VSR_OK) return s;
+    sc->last_ntiles = ntiles;
+    sc->walked_map = m->gen;
+    sc->walked_scene = sc->gen;
+    sc->walked_last = true;
+    return VSR_OK;
+}
+}  // namespace
+
 // One frame of (m, s) without statistics.  The walking raster needs no bins
 // (1920x1080, 220k triangles: see the figures at raster_walk_kernel), but the
 // first frame of a shape goes through stored ones, as does every frame of a
@@ -652,21 +676,16 @@ static vsr_status raster_frame(vsr_map m, vsr_scene sc, uint32_t* id_dev, float*
 {
     if (!m || !sc) return VSR_ERR_INVALID_ARG;
     vsr_status s;
-    if (sc->async_sizing || sc->cap == 0 || sc->sized_shape != bin_shape_of(m, sc, 0)) {
+    if (sc->async_sizing || !bins_sized(m, sc, 0)) {
         if ((s = bin_scene(m, sc, 0, st)) != VSR_OK) return s;
         return raster_tiles(m, sc, id_dev, depth_dev, cov_dev, nullptr, st, host_out);
     }
-    const int ntiles = m->tx * m->ty;
-    if ((s = ensure_ws(sc, ntiles, st)) != VSR_OK || (s = walk_work_alloc(&sc->walk, st)) != VSR_OK) return s;
+    if ((s = walk_begin(m, sc, st)) != VSR_OK) return s;
     const RasterView v{m->map, m->p.W, m->p.H, m->tiles, m->tx,   sc->rec,   (int)sc->T,
                        nullptr, nullptr, 0u,   id_dev,   depth_dev, cov_dev};
     if ((s = launch_raster_walk(v, walk_index(sc->grid, sc->T), m->idx.geom, sc->walk, sc->tile_pairs,
                                 scene_status(sc), st, host_out)) != VSR_OK)
         return s;
-    sc->last_ntiles = ntiles;
-    sc->walked_map = m->gen;
-    sc->walked_scene = sc->gen;
-    sc->walked_last = true;
     return scene_used(sc, st);
 }
 

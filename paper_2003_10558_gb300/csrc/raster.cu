@@ -37,37 +37,9 @@
 // order-free, so the result does not depend on the cull.
 #include <type_traits>
 
-#include "stage.cuh"
-#include "walk.cuh"
+#include "raster_walk.cuh"
 
 namespace {
-
-constexpr int RT = 128;          // threads per CTA (one 16x16 tile)
-constexpr int PPT = 2;           // pixels per thread: (x, y) and (x, y + 4) of the warp's 8x8 block
-constexpr int CHUNK = RT;        // triangles staged per pass
-static_assert(CHUNK == STAGE_CHUNK, "one staging slot per thread");
-static_assert(RT * PPT == TILE_PIX, "one CTA covers one tile");
-// resident CTAs per SM the timed kernel is compiled for (its register cap)
-#ifndef VSR_RASTER_CTAS_PER_SM
-#define VSR_RASTER_CTAS_PER_SM 8
-#endif
-
-// One 16x16 tile of one view.  Called by every thread of a CTA of RT
-// threads; `st` is the CTA's staging area (reusable across calls: every use
-// is fenced by the barriers of the chunk loop).
-// Split tiles: a tile whose bin is longer than split_max triangles (a
-// multiple of CHUNK) is processed as several work items of at most
-// split_max triangles each.  The
-// items of one tile add their coverage (2^-22 fixed point) and take the
-// minimum of their visibility keys in the tile's accumulator slot with
-// atomics -- both are order-free, so the result is exactly that of one item
-// -- and the item that arrives last (atomic counter, nothing waits) writes
-// the outputs and clears the slot for the next frame.
-struct SplitAcc {
-    unsigned long long* acc;  // [slot][TILE_PIX], zero between frames (64 bits: many partials)
-    unsigned long long* key;  // [slot][TILE_PIX], ~0 between frames
-    uint32_t* done;           // [slot], zero between frames
-};
 
 // A cone (axis, cos, sin, widest ramp half-width) may hold a fragment of the
 // staged triangle (cap a, b; edge normals n1..n3): the cap test, and unless
@@ -86,50 +58,6 @@ __device__ __forceinline__ bool cone_may_hit(const float4& a, const float4& b, c
                                   fmaf(c0.x, n3.x, fmaf(c0.y, n3.y, c0.z * n3.z)) > lim));
 }
 
-// View cone of the warp's 8x8 block from its valid pixels: axis = normalised
-// sum, cos alpha = min G.axis less a margin, h = the widest ramp half-width;
-// a block without a valid pixel gets valid = 0, a degenerate sum the whole
-// sphere.  The cone only culls, so the sums may be taken in any order: the
-// axis by shuffles, the two extrema by the integer reductions of sm_80+
-// (non-negative floats order as their bits; the minimum of G.axis <= 1 + a
-// few ulp as the maximum of 2 - G.axis, whose rounding of 1.2e-7 the margin
-// covers).
-__device__ __forceinline__ void block_cone(const float* gx, const float* gy, const float* gz, const float* h,
-                                           const bool* pv, float4& c0, float4& c1)
-{
-    const unsigned FULL = 0xffffffffu;
-    const int cn = __popc(__ballot_sync(FULL, pv[0])) + __popc(__ballot_sync(FULL, pv[1]));
-    float sx = 0.0f, sy = 0.0f, sz = 0.0f, hw = 0.0f;
-#pragma unroll
-    for (int p = 0; p < PPT; ++p)
-        if (pv[p]) {
-            sx += gx[p];
-            sy += gy[p];
-            sz += gz[p];
-            hw = fmaxf(hw, h[p]);
-        }
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        sx += __shfl_xor_sync(FULL, sx, o);
-        sy += __shfl_xor_sync(FULL, sy, o);
-        sz += __shfl_xor_sync(FULL, sz, o);
-    }
-    hw = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(hw)));
-    const float len2 = fmaf(sx, sx, fmaf(sy, sy, sz * sz));
-    const bool deg = !(len2 > 1e-12f * (float)(cn * cn));
-    const float inv = rsqrtf(len2);
-    const float ax = deg ? 0.0f : sx * inv, ay = deg ? 0.0f : sy * inv, az = deg ? 1.0f : sz * inv;
-    float away = 0.0f;
-#pragma unroll
-    for (int p = 0; p < PPT; ++p)
-        if (pv[p]) away = fmaxf(away, 2.0f - fmaf(gx[p], ax, fmaf(gy[p], ay, gz[p] * az)));
-    const float cm = 2.0f - __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(away)));
-    float cs = fmaxf(-1.0f, fminf(1.0f, cm - 2e-6f));
-    if (deg) cs = -1.0f;
-    c0 = make_float4(ax, ay, az, cs);
-    c1 = make_float4(sqrtf(fmaxf(0.0f, 1.0f - cs * cs)), hw, cn > 0 ? 1.0f : 0.0f, 0.0f);
-}
-
 // One lane's two pixels as the evaluation sees them.
 struct PixPair {
     float2 dgx, dgy, dgz;  // G - a (tile axis) of both pixels; 0 at an invalid pixel
@@ -140,21 +68,6 @@ struct PixPair {
     unsigned long long key[PPT];  // ((bits(r) - 1) << 32) | t of the nearest centre-inside fragment, or KEY_NONE
     int32_t cnt_in[PPT];   // centre-inside fragments (statistics)
 };
-// A depth 0 < r < inf has bits(r) - 1 < DEPTH_LIM (unsigned; NaN, zeros and
-// negative numbers do not), so a key below KEY_NONE is a valid depth's.
-constexpr uint32_t DEPTH_LIM = 0x7f7fffffu;
-constexpr unsigned long long KEY_NONE = (unsigned long long)DEPTH_LIM << 32;
-
-// 1/x to the precision of the hardware's reciprocal; x neither denormal nor
-// above 2^126: the quotient a * rcp_fast(x) is then __fdividef(a, x) bit for
-// bit, without the instructions that scale its operands.
-__device__ __forceinline__ float rcp_fast(float x)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
 // Evaluate staged slot j at the lane's two pixels and merge the fragments into the pixels' coverage and keys.
 // Called by all 32 lanes of a warp together (warp votes).
 //
@@ -258,40 +171,6 @@ __device__ __forceinline__ uint32_t final_acc(const PixPair& q, int p)
     return q.lim[p] < INFINITY ? min(q.acc[p], COV_ONE) : 0u;
 }
 
-// A thread's place in its tile: warp w covers the 8x8 block (w & 1, w >> 1),
-// a lane the pixels (lx, ly) and (lx, ly + 4).
-struct TilePos {
-    int tx, ty, lx, ly, px, py;
-    __device__ __forceinline__ TilePos(int tile, int tiles_x)
-    {
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        tx = tile % tiles_x;
-        ty = tile / tiles_x;
-        lx = (warp & 1) * 8 + (lane & 7);
-        ly = (warp >> 1) * 8 + (lane >> 3);
-        px = tx * TILE + lx;
-        py = ty * TILE + ly;
-    }
-};
-
-// The lane's pixels from the map (zero outside the picture).
-__device__ __forceinline__ void load_pixels(const RasterView& view, const TilePos& tp, float4 (&g)[PPT])
-{
-#pragma unroll
-    for (int p = 0; p < PPT; ++p) {
-        const int y = tp.py + 4 * p;
-        g[p] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (tp.px < view.W && y < view.H) g[p] = view.map[(size_t)y * view.W + tp.px];
-    }
-}
-
-// The warps' view cones (their 8x8 pixels; block_cone), in shared memory: the
-// cull reads them once per 32 triangles, and held in registers they would
-// spill others out of the evaluation loop.
-struct WarpCones {
-    float4 c[RT / 32][2];
-};
-
 // The pixels' loop state, and the warp's own view cone; returns whether the
 // warp has a valid pixel.
 __device__ __forceinline__ bool start_pixels(const float4 (&g)[PPT], const float4& axis, PixPair& q, WarpCones& wc)
@@ -308,19 +187,6 @@ __device__ __forceinline__ bool start_pixels(const float4 (&g)[PPT], const float
     }
     __syncwarp();
     return c1.z > 0.0f;
-}
-
-// Stage triangle t into slot j (an index beyond the records -- never left by a
-// completed binning or grid -- empties the slot and raises the status).
-__device__ __forceinline__ void stage_checked(const float4* __restrict__ rec, int T, uint32_t t, const float4& axis,
-                                              Stage& st, int j, int* status)
-{
-    if (t >= (uint32_t)T) {
-        raise_status(status, VSR_ERR_BIN_OVERFLOW);
-        st.s6[j] = make_float4(0.0f, 0.0f, 0.0f, __uint_as_float(STAGE_EMPTY));
-    } else {
-        stage_triangle(rec, (size_t)T, t, axis.x, axis.y, axis.z, st, j);
-    }
 }
 
 // The n staged triangles of a chunk at the warp's pixels: a lane-parallel cull
@@ -347,81 +213,34 @@ __device__ __forceinline__ void eval_chunk(const Stage& st, int n, const WarpCon
     }
 }
 
-// Merge the lane's pixels into accumulator slot `slot` of a tile processed in
-// several parts; the part that brings the count of `done` units to `target`
-// gets the tile's result in q, clears the slot and returns true.  Called by
-// every thread of the CTA.
-__device__ __forceinline__ bool merge_slot(const SplitAcc& split, int slot, const TilePos& tp, PixPair& q,
-                                           uint32_t units, uint32_t target)
-{
-    __shared__ int s_last;
-    const int lp0 = tp.lx + TILE * tp.ly;
-    unsigned long long* __restrict__ sacc = split.acc + (size_t)slot * TILE_PIX;
-    unsigned long long* __restrict__ skey = split.key + (size_t)slot * TILE_PIX;
-#pragma unroll
-    for (int p = 0; p < PPT; ++p) {
-        if (q.acc[p]) atomicAdd(&sacc[lp0 + TILE * 4 * p], (unsigned long long)q.acc[p]);
-        if (q.key[p] != KEY_NONE) atomicMin(&skey[lp0 + TILE * 4 * p], q.key[p]);
+// The global step for the walking raster.
+struct GlobalStep {
+    static constexpr int CTAS = VSR_RASTER_CTAS_PER_SM;
+    using Pix = PixPair;
+    using Cones = WarpCones;
+    struct In {};
+    struct Raw {
+        float4 g[PPT];
+    };
+    __device__ __forceinline__ static void load(const RasterView& view, const In&, const TilePos& tp, Raw& r)
+    {
+        load_pixels(view, tp, r.g);
     }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(&split.done[slot], units) + units == target;
-    __syncthreads();
-    if (!s_last) return false;
-    __threadfence();
-#pragma unroll
-    for (int p = 0; p < PPT; ++p) {
-        q.acc[p] = (uint32_t)min(atomicExch(&sacc[lp0 + TILE * 4 * p], 0ull), (unsigned long long)COV_ONE);
-        q.key[p] = min(atomicExch(&skey[lp0 + TILE * 4 * p], ~0ull), KEY_NONE);
+    __device__ __forceinline__ static bool start(const Raw& r, const float4& axis, Pix& q, Cones& wc)
+    {
+        return start_pixels(r.g, axis, q, wc);
     }
-    if (threadIdx.x == 0) split.done[slot] = 0u;
-    return true;
-}
-
-// ROWS: the outputs go through shared memory and leave in whole tile rows
-// (pinned host outputs written in place over the host link).
-template <bool STATS, bool ROWS>
-__device__ __forceinline__ void write_tile(const RasterView& view, const TilePos& tp, const PixPair& q,
-                                           int32_t* __restrict__ n_inside)
-{
-    const int W = view.W, H = view.H;
-    if constexpr (!ROWS) {
-#pragma unroll
-        for (int p = 0; p < PPT; ++p) {
-            if (tp.px >= W || tp.py + 4 * p >= H) continue;
-            const size_t o = (size_t)(tp.py + 4 * p) * W + tp.px;
-            const bool hit = q.key[p] != KEY_NONE;
-            if (view.out_id) view.out_id[o] = hit ? (uint32_t)(q.key[p] & 0xffffffffull) : 0xffffffffu;
-            if (view.out_depth) view.out_depth[o] = hit ? __uint_as_float((uint32_t)(q.key[p] >> 32) + 1u) : INFINITY;
-            if (view.out_cov) view.out_cov[o] = (float)q.acc[p] * (1.0f / (float)COV_ONE);
-            if (STATS && n_inside) n_inside[o] = q.cnt_in[p];
-        }
-    } else {
-        // Through shared memory, so that each warp store covers two whole tile
-        // rows (16 pixels, 64 B each) instead of four 8-pixel pieces: over the
-        // host link 32-byte pieces cost about a quarter of its bandwidth.
-        __shared__ uint32_t s_out[3][TILE_PIX];
-#pragma unroll
-        for (int p = 0; p < PPT; ++p) {
-            const int lp = tp.lx + TILE * (tp.ly + 4 * p);
-            const bool hit = q.key[p] != KEY_NONE;
-            s_out[0][lp] = hit ? (uint32_t)(q.key[p] & 0xffffffffull) : 0xffffffffu;
-            s_out[1][lp] = hit ? (uint32_t)(q.key[p] >> 32) + 1u : __float_as_uint(INFINITY);
-            s_out[2][lp] = __float_as_uint((float)q.acc[p] * (1.0f / (float)COV_ONE));
-        }
-        __syncthreads();
-#pragma unroll
-        for (int i = threadIdx.x; i < TILE_PIX; i += RT) {
-            const int ox = tp.tx * TILE + (i % TILE), oy = tp.ty * TILE + i / TILE;
-            if (ox >= W || oy >= H) continue;
-            const size_t o = (size_t)oy * W + ox;
-            if (view.out_id) view.out_id[o] = s_out[0][i];
-            if (view.out_depth) view.out_depth[o] = __uint_as_float(s_out[1][i]);
-            if (view.out_cov) view.out_cov[o] = __uint_as_float(s_out[2][i]);
-        }
-        __syncthreads();  // read before the CTA's next tile writes it
+    __device__ __forceinline__ static bool cull(const Stage& st, int j, const Cones& wc, int warp)
+    {
+        return cone_may_hit(st.s0[j], st.s1[j], st.s2[j], st.s3[j], st.s4[j], wc.c[warp][0], wc.c[warp][1], false);
     }
-}
+    __device__ __forceinline__ static void eval(const Stage& st, int j, Pix& q)
+    {
+        uint32_t unused = 0;
+        eval_slot<false>(st, j, q, unused);
+    }
+    __device__ __forceinline__ static uint32_t final_acc(const Pix& q, int p) { return ::final_acc(q, p); }
+};
 
 template <bool STATS, bool ROWS = false>
 __device__ __forceinline__ void raster_tile(const RasterView& view, int tile, Stage& st, bool count_alg,
@@ -470,7 +289,13 @@ __device__ __forceinline__ void raster_tile(const RasterView& view, int tile, St
 #pragma unroll
     for (int p = 0; p < PPT; ++p) q.acc[p] = final_acc(q, p);
     if (split_slot >= 0 && !merge_slot(split, split_slot, tp, q, 1u, (uint32_t)nsplit)) return;
-    write_tile<STATS, ROWS>(view, tp, q, n_inside);
+    write_tile<ROWS>(view, tp, q);
+    if (STATS && n_inside) {
+#pragma unroll
+        for (int p = 0; p < PPT; ++p)
+            if (tp.px < view.W && tp.py + 4 * p < view.H)
+                n_inside[(size_t)(tp.py + 4 * p) * view.W + tp.px] = q.cnt_in[p];
+    }
 }
 
 template <bool STATS>
@@ -592,205 +417,6 @@ __global__ void __launch_bounds__(RT, VSR_RASTER_CTAS_PER_SM) raster_pool_kernel
     }
 }
 
-// Binning and raster in one launch: every tile's CTA walks its candidates
-// (walk.cuh) WALK_BLOCK at a time, lists the hits in shared memory and
-// rasterizes them, so the bins are never stored and no pass over the tiles
-// runs before.  Against the tile pass, the heavy-tile pass, the work-item pass
-// and the raster over stored bins (four launches), the walk's latency is
-// hidden by the other CTAs' evaluation (see the measured figures at
-// vsr_raster).
-//
-// A tile with many candidates is processed by several CTAs that merge in an
-// accumulator slot (merge_slot): the tile's own CTA takes a free slot and
-// publishes the tile there, the CTAs past the tiles (helpers) look for such
-// tiles, and each block of candidates goes to whoever adds 1 to the slot's
-// claim word next, (tile << 32) | blocks claimed.  An owner without a slot
-// works alone, a helper that finds nothing ends, and the part that finishes
-// the last block writes the tile and frees the slot.  A claim names its tile,
-// so one made on a slot that has changed hands is still a claim of the slot's
-// present tile; a claim past the tile's last block is no block.  While a part
-// holds unmerged blocks its slot cannot be freed.  Nobody waits for another,
-// but that helpers which start together with the tiles (fewer tiles than
-// resident CTAs) look again for about 10 us before they give up.
-struct WalkSlots {
-    SplitAcc split;             // WALK_SLOTS accumulators
-    unsigned long long* claim;  // WALK_SLOTS: (tile << 32) | blocks claimed
-    uint32_t* nblk;             // WALK_SLOTS: blocks of the slot's tile; 0 free, ~0 being set up
-    uint32_t* hits;             // WALK_SLOTS: hits of the parts merged so far
-    uint32_t* hint;             // where the next owner looks first
-    uint32_t* active;           // published tiles
-};
-
-// What a CTA knows of its tile, in shared memory: uniform, and needed only
-// between the evaluations, whose loop has no registers to spare.
-struct WalkTile {
-    Cone cone;
-    uint32_t nblk, next;  // blocks of the tile, this CTA's next one
-    uint32_t units, hits;  // blocks done and hits found by this CTA
-    int tile, slot;        // slot: -1 unless the tile is shared
-    uint32_t n;            // hits of the current block
-};
-
-template <bool ROWS>
-__global__ void __launch_bounds__(RT, VSR_RASTER_CTAS_PER_SM) raster_walk_kernel(RasterView view, WalkIndex wi,
-                                                                                 const float4* __restrict__ geom,
-                                                                                 int ntiles, uint32_t block,
-                                                                                 uint32_t split_blocks, int looks,
-                                                                                 WalkSlots slots,
-                                                                                 uint32_t* __restrict__ tile_pairs,
-                                                                                 int* __restrict__ status)
-{
-    __shared__ Stage st;
-    __shared__ WalkShared ws;
-    __shared__ WarpCones wc;
-    __shared__ WalkTile wt;
-    __shared__ uint32_t s_ids[WALK_BLOCK];
-    static_assert(RT == WALK_THREADS, "the walk's CTA");
-    const unsigned FULL = 0xffffffffu;
-    const bool helper = blockIdx.x >= (uint32_t)ntiles;
-    for (;;) {
-        PixPair q;
-        bool warp_active;
-        {
-            int tile = (int)blockIdx.x, slot = -1;
-            uint32_t first = 0u;
-            if (helper) {
-                // a published tile with blocks left: the lowest such slot from
-                // a start of this CTA's own
-                __syncthreads();
-                if (threadIdx.x == 0) {
-                    while (!*(volatile uint32_t*)slots.active && looks > 0) {
-                        --looks;
-                        __nanosleep(250);
-                    }
-                    wt.slot = *(volatile uint32_t*)slots.active ? WALK_SLOTS : -1;
-                }
-                __syncthreads();
-                if (wt.slot < 0) return;
-                const int from = (int)((blockIdx.x * 37u) % WALK_SLOTS);
-                int mine = WALK_SLOTS;
-                for (int i = threadIdx.x; i < WALK_SLOTS && mine == WALK_SLOTS; i += RT) {
-                    const int c = (from + i) % WALK_SLOTS;
-                    const uint32_t nb = *(volatile uint32_t*)&slots.nblk[c];
-                    if (nb != 0u && nb != 0xffffffffu &&
-                        (uint32_t)*(volatile unsigned long long*)&slots.claim[c] < nb)
-                        mine = i;
-                }
-                if (mine < WALK_SLOTS) atomicMin(&wt.slot, mine);
-                __syncthreads();
-                slot = wt.slot;
-                if (slot == WALK_SLOTS) return;
-                slot = (from + slot) % WALK_SLOTS;
-                if (threadIdx.x == 0) {
-                    const unsigned long long c = atomicAdd(&slots.claim[slot], 1ull);
-                    wt.tile = (int)(c >> 32);
-                    wt.next = (uint32_t)c;
-                }
-                __syncthreads();
-                tile = wt.tile;
-                first = wt.next;
-                if (tile >= ntiles) return;
-            }
-            const float4 axis = view.tiles[tile].c0;
-            float4 g[PPT];
-            load_pixels(view, TilePos(tile, view.tiles_x), g);  // in flight while the first warp finds the ranges
-            if (threadIdx.x == RT - 1) wt.cone = view.tiles[tile];
-            if (threadIdx.x < 32) walk_ranges(wi, view.T, geom[tile], axis.y, ws);
-            if (threadIdx.x == 0) {
-                const uint32_t nblk = (ws.total + block - 1) / block;
-                if (!helper && nblk > split_blocks) {
-                    const uint32_t from = atomicAdd(slots.hint, 1u);
-                    for (uint32_t i = 0; i < 8u && slot < 0; ++i) {
-                        const uint32_t c = (from + i) % WALK_SLOTS;
-                        if (atomicCAS(&slots.nblk[c], 0u, 0xffffffffu) == 0u) {
-                            atomicExch(&slots.claim[c], (unsigned long long)(uint32_t)tile << 32 | 1ull);
-                            __threadfence();
-                            atomicExch(&slots.nblk[c], nblk);
-                            atomicAdd(slots.active, 1u);
-                            slot = (int)c;
-                        }
-                    }
-                }
-                wt.tile = tile;
-                wt.slot = slot;
-                wt.nblk = nblk;
-                wt.next = first;
-                wt.units = wt.hits = wt.n = 0u;
-            }
-            warp_active = start_pixels(g, axis, q, wc);
-            __syncthreads();
-            if (helper && first >= wt.nblk) continue;  // finished meanwhile
-        }
-        while (wt.next < wt.nblk) {
-            {
-                Walk w;
-                w.init(wi, wt.cone, ws);
-                const uint32_t e0 = wt.next * block, e1 = min(ws.total, e0 + block);
-                const int lane = threadIdx.x & 31;
-                for (uint32_t i0 = e0; i0 < e1; i0 += RT) {
-                    const uint32_t idx = i0 + threadIdx.x;
-                    uint32_t t;
-                    const bool hit = w.test(wi, view.rec, view.T, ws, idx, idx < e1, t);
-                    const unsigned m = __ballot_sync(FULL, hit);
-                    if (!m) continue;
-                    uint32_t base = 0;
-                    if (lane == 0) base = atomicAdd(&wt.n, (uint32_t)__popc(m));
-                    base = __shfl_sync(FULL, base, 0);
-                    if (hit) s_ids[base + (uint32_t)__popc(m & ((1u << lane) - 1u))] = t;
-                }
-            }
-            __syncthreads();
-            for (uint32_t base = 0; base < wt.n; base += CHUNK) {
-                const int nc = (int)min((uint32_t)CHUNK, wt.n - base);
-#pragma unroll
-                for (int p = 0; p < PPT; ++p) q.acc[p] = min(q.acc[p], COV_ONE);
-                if (base) __syncthreads();
-                if ((int)threadIdx.x < nc)
-                    stage_checked(view.rec, view.T, s_ids[base + threadIdx.x], wt.cone.c0, st, threadIdx.x, status);
-                __syncthreads();
-                uint32_t ca = 0, ce = 0;
-                if (warp_active) eval_chunk<false>(st, nc, wc, false, q, ca, ce);
-            }
-            // the only block of a tile that is not shared (almost every tile):
-            // no one waits for the others' evaluation
-            if (wt.nblk == 1u && wt.slot < 0) break;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                wt.hits += wt.n;
-                wt.n = 0u;
-                ++wt.units;
-                wt.next = wt.slot >= 0 ? (uint32_t)atomicAdd(&slots.claim[wt.slot], 1ull) : wt.next + 1u;
-            }
-            __syncthreads();
-        }
-#pragma unroll
-        for (int p = 0; p < PPT; ++p) q.acc[p] = final_acc(q, p);
-        const int tile = wt.tile, slot = wt.slot;
-        const TilePos tp(tile, view.tiles_x);
-        uint32_t hits = wt.hits + wt.n;
-        bool last = true;
-        if (slot >= 0) {
-            if (threadIdx.x == 0 && hits) atomicAdd(&slots.hits[slot], hits);
-            last = merge_slot(slots.split, slot, tp, q, wt.units, wt.nblk);
-            if (last) {
-                __threadfence();
-                __syncthreads();
-                if (threadIdx.x == 0) {
-                    hits = atomicExch(&slots.hits[slot], 0u);
-                    __threadfence();
-                    atomicSub(slots.active, 1u);
-                    atomicExch(&slots.nblk[slot], 0u);  // free
-                }
-            }
-        }
-        if (last) {
-            if (tile_pairs && threadIdx.x == 0) tile_pairs[tile] = hits;
-            write_tile<false, ROWS>(view, tp, q, nullptr);
-        }
-        if (!helper) return;
-    }
-}
-
 // Dense reference of the same rasterization: every pixel of a tile against
 // every triangle of the scene, with no binning and no cull.  As in the
 // oracle, the miter distance is evaluated first: a triangle whose enlarged
@@ -835,7 +461,7 @@ __global__ void __launch_bounds__(RT) raster_dense_kernel(RasterView view, int* 
     }
 #pragma unroll
     for (int p = 0; p < PPT; ++p) q.acc[p] = final_acc(q, p);
-    write_tile<false, false>(view, tp, q, nullptr);
+    write_tile<false>(view, tp, q);
 }
 
 // Work items per tile: ceil(bin / split_max) when a split slot and room in
@@ -961,32 +587,7 @@ void walk_work_free(WalkWork* w)
 vsr_status launch_raster_walk(const RasterView& view, const WalkIndex& wi, const float4* geom, const WalkWork& work,
                               uint32_t* tile_pairs, int* status, cudaStream_t st, bool host_out)
 {
-    const int ntiles = view.tiles_x * ((view.H + TILE - 1) / TILE);
-    if (ntiles == 0) return VSR_OK;
-    const int sms = sm_count();
-    if (sms < 0) return VSR_ERR_CUDA;
-    const size_t pix = (size_t)TILE_PIX * WALK_SLOTS;
-    WalkSlots sl;
-    sl.split.acc = (unsigned long long*)work.mem;
-    sl.split.key = sl.split.acc + pix;
-    sl.claim = sl.split.key + pix;
-    sl.split.done = (uint32_t*)(sl.claim + WALK_SLOTS);
-    sl.nblk = sl.split.done + WALK_SLOTS;
-    sl.hits = sl.nblk + WALK_SLOTS;
-    sl.hint = sl.hits + WALK_SLOTS;
-    sl.active = sl.hint + 1;
-    // helpers only where a tile can have enough candidates; few tiles: smaller
-    // blocks, handed out from the second on
-    const int wave = sms * VSR_RASTER_CTAS_PER_SM;
-    const bool few = ntiles < wave;
-    const int block = few ? WALK_BLOCK / 4 : WALK_BLOCK;
-    const int split = few ? 2 : (int)WALK_SPLIT_BLOCKS;
-    const int helpers = view.T > split * block ? wave : 0;
-    auto kern = host_out ? raster_walk_kernel<true> : raster_walk_kernel<false>;
-    kern<<<ntiles + helpers, RT, 0, st>>>(view, wi, geom, ntiles, (uint32_t)block, (uint32_t)split, few ? 40 : 0, sl,
-                                          tile_pairs, status);
-    VSR_CUDA_TRY(cudaGetLastError());
-    return VSR_OK;
+    return launch_walk<GlobalStep>(view, GlobalStep::In{}, wi, geom, work, tile_pairs, status, st, host_out);
 }
 
 vsr_status launch_raster_dense(const RasterView& view, int* status, cudaStream_t st)

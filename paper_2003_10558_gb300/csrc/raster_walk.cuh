@@ -1,0 +1,264 @@
+// raster_walk.cuh -- the raster that needs no stored bins (see walk.cuh for
+// the candidates of a tile), for any pixel step.
+#pragma once
+
+#include "tile.cuh"
+#include "walk.cuh"
+
+namespace {
+
+// Binning and raster in one launch: every tile's CTA walks its candidates
+// (walk.cuh) WALK_BLOCK at a time, lists the hits in shared memory and
+// rasterizes them, so the bins are never stored and no pass over the tiles
+// runs before.  Against the tile pass, the heavy-tile pass, the work-item pass
+// and the raster over stored bins (four launches), the walk's latency is
+// hidden by the other CTAs' evaluation (see the measured figures at
+// vsr_raster).
+//
+// A tile with many candidates is processed by several CTAs that merge in an
+// accumulator slot (merge_slot): the tile's own CTA takes a free slot and
+// publishes the tile there, the CTAs past the tiles (helpers) look for such
+// tiles, and each block of candidates goes to whoever adds 1 to the slot's
+// claim word next, (tile << 32) | blocks claimed.  An owner without a slot
+// works alone, a helper that finds nothing ends, and the part that finishes
+// the last block writes the tile and frees the slot.  A claim names its tile,
+// so one made on a slot that has changed hands is still a claim of the slot's
+// present tile; a claim past the tile's last block is no block.  While a part
+// holds unmerged blocks its slot cannot be freed.  Nobody waits for another,
+// but that helpers which start together with the tiles (fewer tiles than
+// resident CTAs) look again for about 10 us before they give up.
+struct WalkSlots {
+    SplitAcc split;             // WALK_SLOTS accumulators
+    unsigned long long* claim;  // WALK_SLOTS: (tile << 32) | blocks claimed
+    uint32_t* nblk;             // WALK_SLOTS: blocks of the slot's tile; 0 free, ~0 being set up
+    uint32_t* hits;             // WALK_SLOTS: hits of the parts merged so far
+    uint32_t* hint;             // where the next owner looks first
+    uint32_t* active;           // published tiles
+};
+
+// What a CTA knows of its tile, in shared memory: uniform, and needed only
+// between the evaluations, whose loop has no registers to spare.
+struct WalkTile {
+    Cone cone;
+    uint32_t nblk, next;  // blocks of the tile, this CTA's next one
+    uint32_t units, hits;  // blocks done and hits found by this CTA
+    int tile, slot;        // slot: -1 unless the tile is shared
+    uint32_t n;            // hits of the current block
+};
+
+// The n staged triangles of a chunk at the warp's pixels: a lane-parallel cull
+// of 32 triangles at a time against the warp's cone, then the survivors one by
+// one.
+template <class Step>
+__device__ __forceinline__ void walk_eval(const Stage& st, int n, const typename Step::Cones& wc,
+                                          typename Step::Pix& q)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int gbase = 0; gbase < n; gbase += 32) {
+        bool keep = false;
+        const int jj = gbase + lane;
+        if (jj < n && __float_as_uint(st.s6[jj].w) != STAGE_EMPTY) keep = Step::cull(st, jj, wc, warp);
+        unsigned mask = __ballot_sync(0xffffffffu, keep);
+        while (mask) {
+            const int k = 31 - __clz(mask);  // any order: from the top, one instruction less than from the bottom
+            mask ^= 1u << k;
+            Step::eval(st, gbase + k, q);
+        }
+    }
+}
+
+// Step: how pixels are loaded, culled against and evaluated (the global step
+// of raster.cu, the per-fragment step of pstep.cu).
+template <class Step, bool ROWS>
+__global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView view, typename Step::In in, WalkIndex wi,
+                                                                     const float4* __restrict__ geom, int ntiles,
+                                                                     uint32_t block, uint32_t split_blocks, int looks,
+                                                                     WalkSlots slots,
+                                                                     uint32_t* __restrict__ tile_pairs,
+                                                                     int* __restrict__ status)
+{
+    __shared__ Stage st;
+    __shared__ WalkShared ws;
+    __shared__ typename Step::Cones wc;
+    __shared__ WalkTile wt;
+    __shared__ uint32_t s_ids[WALK_BLOCK];
+    static_assert(RT == WALK_THREADS, "the walk's CTA");
+    const unsigned FULL = 0xffffffffu;
+    const bool helper = blockIdx.x >= (uint32_t)ntiles;
+    for (;;) {
+        typename Step::Pix q;
+        bool warp_active;
+        {
+            int tile = (int)blockIdx.x, slot = -1;
+            uint32_t first = 0u;
+            if (helper) {
+                // a published tile with blocks left: the lowest such slot from
+                // a start of this CTA's own
+                __syncthreads();
+                if (threadIdx.x == 0) {
+                    while (!*(volatile uint32_t*)slots.active && looks > 0) {
+                        --looks;
+                        __nanosleep(250);
+                    }
+                    wt.slot = *(volatile uint32_t*)slots.active ? WALK_SLOTS : -1;
+                }
+                __syncthreads();
+                if (wt.slot < 0) return;
+                const int from = (int)((blockIdx.x * 37u) % WALK_SLOTS);
+                int mine = WALK_SLOTS;
+                for (int i = threadIdx.x; i < WALK_SLOTS && mine == WALK_SLOTS; i += RT) {
+                    const int c = (from + i) % WALK_SLOTS;
+                    const uint32_t nb = *(volatile uint32_t*)&slots.nblk[c];
+                    if (nb != 0u && nb != 0xffffffffu &&
+                        (uint32_t)*(volatile unsigned long long*)&slots.claim[c] < nb)
+                        mine = i;
+                }
+                if (mine < WALK_SLOTS) atomicMin(&wt.slot, mine);
+                __syncthreads();
+                slot = wt.slot;
+                if (slot == WALK_SLOTS) return;
+                slot = (from + slot) % WALK_SLOTS;
+                if (threadIdx.x == 0) {
+                    const unsigned long long c = atomicAdd(&slots.claim[slot], 1ull);
+                    wt.tile = (int)(c >> 32);
+                    wt.next = (uint32_t)c;
+                }
+                __syncthreads();
+                tile = wt.tile;
+                first = wt.next;
+                if (tile >= ntiles) return;
+            }
+            const float4 axis = view.tiles[tile].c0;
+            typename Step::Raw g;
+            Step::load(view, in, TilePos(tile, view.tiles_x), g);  // in flight while the first warp finds the ranges
+            if (threadIdx.x == RT - 1) wt.cone = view.tiles[tile];
+            if (threadIdx.x < 32) walk_ranges(wi, view.T, geom[tile], axis.y, ws);
+            if (threadIdx.x == 0) {
+                const uint32_t nblk = (ws.total + block - 1) / block;
+                if (!helper && nblk > split_blocks) {
+                    const uint32_t from = atomicAdd(slots.hint, 1u);
+                    for (uint32_t i = 0; i < 8u && slot < 0; ++i) {
+                        const uint32_t c = (from + i) % WALK_SLOTS;
+                        if (atomicCAS(&slots.nblk[c], 0u, 0xffffffffu) == 0u) {
+                            atomicExch(&slots.claim[c], (unsigned long long)(uint32_t)tile << 32 | 1ull);
+                            __threadfence();
+                            atomicExch(&slots.nblk[c], nblk);
+                            atomicAdd(slots.active, 1u);
+                            slot = (int)c;
+                        }
+                    }
+                }
+                wt.tile = tile;
+                wt.slot = slot;
+                wt.nblk = nblk;
+                wt.next = first;
+                wt.units = wt.hits = wt.n = 0u;
+            }
+            warp_active = Step::start(g, axis, q, wc);
+            __syncthreads();
+            if (helper && first >= wt.nblk) continue;  // finished meanwhile
+        }
+        while (wt.next < wt.nblk) {
+            {
+                Walk w;
+                w.init(wi, wt.cone, ws);
+                const uint32_t e0 = wt.next * block, e1 = min(ws.total, e0 + block);
+                const int lane = threadIdx.x & 31;
+                for (uint32_t i0 = e0; i0 < e1; i0 += RT) {
+                    const uint32_t idx = i0 + threadIdx.x;
+                    uint32_t t;
+                    const bool hit = w.test(wi, view.rec, view.T, ws, idx, idx < e1, t);
+                    const unsigned m = __ballot_sync(FULL, hit);
+                    if (!m) continue;
+                    uint32_t base = 0;
+                    if (lane == 0) base = atomicAdd(&wt.n, (uint32_t)__popc(m));
+                    base = __shfl_sync(FULL, base, 0);
+                    if (hit) s_ids[base + (uint32_t)__popc(m & ((1u << lane) - 1u))] = t;
+                }
+            }
+            __syncthreads();
+            for (uint32_t base = 0; base < wt.n; base += CHUNK) {
+                const int nc = (int)min((uint32_t)CHUNK, wt.n - base);
+#pragma unroll
+                for (int p = 0; p < PPT; ++p) q.acc[p] = min(q.acc[p], COV_ONE);
+                if (base) __syncthreads();
+                if ((int)threadIdx.x < nc)
+                    stage_checked(view.rec, view.T, s_ids[base + threadIdx.x], wt.cone.c0, st, threadIdx.x, status);
+                __syncthreads();
+                if (warp_active) walk_eval<Step>(st, nc, wc, q);
+            }
+            // the only block of a tile that is not shared (almost every tile):
+            // no one waits for the others' evaluation
+            if (wt.nblk == 1u && wt.slot < 0) break;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                wt.hits += wt.n;
+                wt.n = 0u;
+                ++wt.units;
+                wt.next = wt.slot >= 0 ? (uint32_t)atomicAdd(&slots.claim[wt.slot], 1ull) : wt.next + 1u;
+            }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int p = 0; p < PPT; ++p) q.acc[p] = Step::final_acc(q, p);
+        const int tile = wt.tile, slot = wt.slot;
+        const TilePos tp(tile, view.tiles_x);
+        uint32_t hits = wt.hits + wt.n;
+        bool last = true;
+        if (slot >= 0) {
+            if (threadIdx.x == 0 && hits) atomicAdd(&slots.hits[slot], hits);
+            last = merge_slot(slots.split, slot, tp, q, wt.units, wt.nblk);
+            if (last) {
+                __threadfence();
+                __syncthreads();
+                if (threadIdx.x == 0) {
+                    hits = atomicExch(&slots.hits[slot], 0u);
+                    __threadfence();
+                    atomicSub(slots.active, 1u);
+                    atomicExch(&slots.nblk[slot], 0u);  // free
+                }
+            }
+        }
+        if (last) {
+            if (tile_pairs && threadIdx.x == 0) tile_pairs[tile] = hits;
+            write_tile<ROWS>(view, tp, q);
+        }
+        if (!helper) return;
+    }
+}
+
+// grid and arguments of a walking raster over `work`'s slots
+template <class Step>
+inline vsr_status launch_walk(const RasterView& view, const typename Step::In& in, const WalkIndex& wi,
+                              const float4* geom, const WalkWork& work, uint32_t* tile_pairs, int* status,
+                              cudaStream_t st, bool host_out)
+{
+    const int ntiles = view.tiles_x * ((view.H + TILE - 1) / TILE);
+    if (ntiles == 0) return VSR_OK;
+    const int sms = sm_count();
+    if (sms < 0) return VSR_ERR_CUDA;
+    const size_t pix = (size_t)TILE_PIX * WALK_SLOTS;
+    WalkSlots sl;
+    sl.split.acc = (unsigned long long*)work.mem;
+    sl.split.key = sl.split.acc + pix;
+    sl.claim = sl.split.key + pix;
+    sl.split.done = (uint32_t*)(sl.claim + WALK_SLOTS);
+    sl.nblk = sl.split.done + WALK_SLOTS;
+    sl.hits = sl.nblk + WALK_SLOTS;
+    sl.hint = sl.hits + WALK_SLOTS;
+    sl.active = sl.hint + 1;
+    // helpers only where a tile can have enough candidates; few tiles: smaller
+    // blocks, handed out from the second on
+    const int wave = sms * Step::CTAS;
+    const bool few = ntiles < wave;
+    const int block = few ? WALK_BLOCK / 4 : WALK_BLOCK;
+    const int split = few ? 2 : (int)WALK_SPLIT_BLOCKS;
+    const int helpers = view.T > split * block ? wave : 0;
+    auto kern = host_out ? raster_walk_kernel<Step, true> : raster_walk_kernel<Step, false>;
+    kern<<<ntiles + helpers, RT, 0, st>>>(view, in, wi, geom, ntiles, (uint32_t)block, (uint32_t)split, few ? 40 : 0,
+                                          sl, tile_pairs, status);
+    VSR_CUDA_TRY(cudaGetLastError());
+    return VSR_OK;
+}
+
+}  // namespace

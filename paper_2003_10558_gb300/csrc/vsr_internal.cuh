@@ -477,6 +477,8 @@ size_t map_backward_partials(int W, int H);
 vsr_status launch_map_backward(int W, int H, int aov, float k, float l, float s, float omega_deg,
                                const float4* dmap, float* partials, double* dlens, cudaStream_t st);
 
-// rasterization with the per-fragment pixel step (pstep.cu): one CTA per
-// tile over whole bins; deriv: 2 float4 per pixel from launch_map_spec
-vsr_status launch_raster_pstep(const RasterView& view, const float4* deriv, int* status, cudaStream_t st);
+// rasterization with the per-fragment pixel step (pstep.cu), as
+// launch_raster_walk with a pstep index; deriv: 2 float4 per pixel from
+// launch_map_spec
+vsr_status launch_raster_pstep(const RasterView& view, const float4* deriv, const WalkIndex& wi, const float4* geom,
+                               const WalkWork& work, uint32_t* tile_pairs, int* status, cudaStream_t st);
