@@ -142,6 +142,10 @@ __device__ __forceinline__ df3_2 df3_2_add(df3_2 a, df3_2 b)
     return {df2_add(a.x, b.x), df2_add(a.y, b.y), df2_add(a.z, b.z)};
 }
 __device__ __forceinline__ df3_2 df3_2_scale(df3_2 a, df2 s) { return {df2_mul(a.x, s), df2_mul(a.y, s), df2_mul(a.z, s)}; }
+// a / 2: exact in both parts (barring underflow), the product by the
+// double-word 1/2 bit for bit
+__device__ __forceinline__ df2 df2_half(df2 a) { return {mul2(a.hi, f2(0.5f)), mul2(a.lo, f2(0.5f))}; }
+__device__ __forceinline__ df3_2 df3_2_half(df3_2 a) { return {df2_half(a.x), df2_half(a.y), df2_half(a.z)}; }
 __device__ __forceinline__ df3_2 df3_2_neg(df3_2 a) { return {df2_neg(a.x), df2_neg(a.y), df2_neg(a.z)}; }
 __device__ __forceinline__ df3_2 df3_2_sel(bool cx, bool cy, df3_2 a, df3_2 b)
 {

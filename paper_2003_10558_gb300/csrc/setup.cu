@@ -33,6 +33,14 @@ struct Cam {
     float M[9];
 };
 
+__host__ __device__ __forceinline__ bool identity(const Cam& c)
+{
+    bool i = true;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) i = i && c.M[q] == ((q % 4 == 0) ? 1.0f : 0.0f);
+    return i;
+}
+
 __device__ __forceinline__ bool vless(const float* P, const float* Q)
 {
     for (int c = 0; c < 3; ++c) {
@@ -41,11 +49,6 @@ __device__ __forceinline__ bool vless(const float* P, const float* Q)
     }
     return false;
 }
-
-// resident CTAs per SM the pair kernel is compiled for (its register cap)
-#ifndef VSR_SETUP_PAIR_CTAS
-#define VSR_SETUP_PAIR_CTAS 1
-#endif
 
 // The set-up of two triangles per thread, every double-word step in packed
 // FP32x2 arithmetic (component x: triangle t0, y: t1 = t0 + 1; df2.cuh), so
@@ -96,17 +99,25 @@ __device__ __forceinline__ uint32_t grid_cell(float x, float y, float z, float c
     return (uint32_t)(grid_base_of(l) + row * (2 * nlat + 1) + min(ncol - 1, max(0, col)));
 }
 
-// VIEW: the camera is read from cams_dev (12 floats).  grid.counts != NULL:
-// the triangles' cells are counted for launch_grid_file.
-template <bool VIEW>
-__global__ void __launch_bounds__(128, VSR_SETUP_PAIR_CTAS) setup_pair_kernel(const float* __restrict__ tris, int T,
-                                                                             Cam cam, const float* __restrict__ cams_dev,
-                                                                             float4* __restrict__ rec, TriGrid grid)
+// CAM_IDENT: the camera (an argument) has the identity rotation, the common
+// one; CAM_ROTATED: any other; CAM_DEVICE: it is read from cams_dev (12
+// floats).  grid.counts != NULL: the triangles' cells are counted for
+// launch_grid_file.
+// Resident CTAs per SM (the register cap): 3 (166 registers), but 2 for a
+// rotated camera, whose transform wants the registers: 220k triangles, identity
+// 33.2 -> 30.3 us at 3; 1M triangles, rotated 141.6 us at 2, 144.2 us at 3.
+enum { CAM_IDENT, CAM_ROTATED, CAM_DEVICE };
+template <int CAM>
+__global__ void __launch_bounds__(128, CAM == CAM_ROTATED ? 2 : 3) setup_pair_kernel(const float* __restrict__ tris,
+                                                                                   int T, Cam cam,
+                                                                                   const float* __restrict__ cams_dev,
+                                                                                   float4* __restrict__ rec,
+                                                                                   TriGrid grid)
 {
     const int t0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     const unsigned am = __ballot_sync(0xffffffffu, t0 < T);  // the lanes that go on
     if (t0 >= T) return;
-    if (VIEW) {
+    if (CAM == CAM_DEVICE) {
         const float* cv = cams_dev;
 #pragma unroll
         for (int q = 0; q < 3; ++q) cam.O[q] = cv[q];
@@ -124,9 +135,7 @@ __global__ void __launch_bounds__(128, VSR_SETUP_PAIR_CTAS) setup_pair_kernel(co
     // an identity rotation (the common camera) needs only the exact
     // differences A - O: the pair products by 1 and sums with 0 of the
     // general transform return those pairs unchanged
-    bool ident = true;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) ident = ident && cam.M[q] == ((q % 4 == 0) ? 1.0f : 0.0f);
+    const bool ident = CAM == CAM_IDENT || (CAM == CAM_DEVICE && identity(cam));
     df3_2 V[3];
     bool eye0 = false, eye1 = false;
 #pragma unroll
@@ -161,15 +170,19 @@ __global__ void __launch_bounds__(128, VSR_SETUP_PAIR_CTAS) setup_pair_kernel(co
     const df2 Os = df2_mul(a2, df2_sub(df2_add(b2, c2), a2));
     const df2 Ot = df2_mul(b2, df2_sub(df2_add(c2, a2), b2));
     const df2 Op = df2_mul(c2, df2_sub(df2_add(a2, b2), c2));
-    const df2 half = df2_make(f2(0.5f));
     const df3_2 num = df3_2_add(df3_2_add(df3_2_scale(U0, Os), df3_2_scale(U1, Ot)), df3_2_scale(U2, Op));
-    df3_2 S = df3_2_scale(num, df2_recip(df2_add(df2_add(Os, Ot), Op)));
-    const bool p0 = Op.hi.x <= 0.0f, p1 = Op.hi.y <= 0.0f;
-    S = df3_2_sel(p0, p1, df3_2_scale(df3_2_add(U0, U1), half), S);
-    const bool q0 = Ot.hi.x <= 0.0f, q1 = Ot.hi.y <= 0.0f;
-    S = df3_2_sel(q0, q1, df3_2_scale(df3_2_add(U2, U0), half), S);
+    const df3_2 circ = df3_2_scale(num, df2_recip(df2_add(df2_add(Os, Ot), Op)));
+    // the midpoint opposite the first non-positive O of Os, Ot, Op: its two
+    // vertices are selected, so one sum is formed instead of three (the kernel
+    // is bound by the packed FP32x2 pipe: 12 % of its operations); the half is
+    // exact in both parts
     const bool r0 = Os.hi.x <= 0.0f, r1 = Os.hi.y <= 0.0f;
-    S = df3_2_sel(r0, r1, df3_2_scale(df3_2_add(U1, U2), half), S);
+    const bool q0 = Ot.hi.x <= 0.0f, q1 = Ot.hi.y <= 0.0f;
+    const bool p0 = Op.hi.x <= 0.0f, p1 = Op.hi.y <= 0.0f;
+    const df3_2 ma = df3_2_sel(r0, r1, U1, df3_2_sel(q0, q1, U2, U0));
+    const df3_2 mb = df3_2_sel(r0, r1, U2, df3_2_sel(q0, q1, U0, U1));
+    const df3_2 mid = df3_2_half(df3_2_add(ma, mb));
+    const df3_2 S = df3_2_sel(r0 || q0 || p0, r1 || q1 || p1, mid, circ);
     const df2 s2len = df2_dot(S, S);
     const df2 rs = df2_rsqrt(s2len);
     const df2 slen = df2_mul(s2len, rs);
@@ -247,7 +260,8 @@ vsr_status launch_setup(const float* tris, int T, const float cam[12], float4* r
     for (int q = 0; q < 3; ++q) c.O[q] = cam[q];
     for (int q = 0; q < 9; ++q) c.M[q] = cam[3 + q];
     const int pairs = (T + 1) / 2;
-    setup_pair_kernel<false><<<(pairs + 127) / 128, 128, 0, st>>>(tris, T, c, nullptr, rec, grid ? *grid : TriGrid{});
+    auto kern = identity(c) ? setup_pair_kernel<CAM_IDENT> : setup_pair_kernel<CAM_ROTATED>;
+    kern<<<(pairs + 127) / 128, 128, 0, st>>>(tris, T, c, nullptr, rec, grid ? *grid : TriGrid{});
     VSR_CUDA_TRY(cudaGetLastError());
     return VSR_OK;
 }
@@ -257,8 +271,8 @@ vsr_status launch_setup_view(const float* tris, int T, const float* cam_dev, flo
 {
     if (T == 0) return VSR_OK;
     const int pairs = (T + 1) / 2;
-    setup_pair_kernel<true><<<(pairs + 127) / 128, 128, 0, st>>>(tris, T, Cam{}, cam_dev, rec,
-                                                                 grid ? *grid : TriGrid{});
+    setup_pair_kernel<CAM_DEVICE><<<(pairs + 127) / 128, 128, 0, st>>>(tris, T, Cam{}, cam_dev, rec,
+                                                                      grid ? *grid : TriGrid{});
     VSR_CUDA_TRY(cudaGetLastError());
     return VSR_OK;
 }
