@@ -665,6 +665,13 @@ vsr_status walk_begin(vsr_map m, vsr_scene sc, cudaStream_t st)
 }
 }  // namespace
 
+vsr_status scene_walk_begin(vsr_map m, vsr_scene sc, cudaStream_t st)
+{
+    vsr_status s;
+    if (!bins_sized(m, sc, 0) && (s = bin_scene(m, sc, 0, st)) != VSR_OK) return s;
+    return walk_begin(m, sc, st);
+}
+
 // One frame of (m, s) without statistics.  The walking raster needs no bins
 // (1920x1080, 220k triangles: see the figures at raster_walk_kernel), but the
 // first frame of a shape goes through stored ones, as does every frame of a

@@ -605,75 +605,3 @@ vsr_status launch_bin_fill(const float4* rec, int T, TileIndex idx, const uint32
     VSR_CUDA_TRY(cudaGetLastError());
     return VSR_OK;
 }
-
-// ---- large exclusive scan (multi-CTA) ---------------------------------------
-// pass 1: per 4096-element block sums; pass 2: one CTA scans the block sums
-// (partials[nb] = total); pass 3: per block, local scan plus the block's base.
-
-__global__ void __launch_bounds__(1024) scan_block_sums(const uint32_t* __restrict__ counts, int n,
-                                                         uint32_t* __restrict__ partials)
-{
-    __shared__ uint32_t ws[32];
-    const int b = blockIdx.x * 4096 + 4 * threadIdx.x;
-    uint32_t v = 0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-        if (b + q < n) v += counts[b + q];
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        uint32_t w = ws[threadIdx.x];
-        for (int o = 16; o; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-        if (threadIdx.x == 0) partials[blockIdx.x] = w;
-    }
-}
-
-__global__ void __launch_bounds__(1024) scan_blocks_apply(const uint32_t* __restrict__ counts, int n,
-                                                           const uint32_t* __restrict__ bases,
-                                                           uint32_t* __restrict__ offsets)
-{
-    __shared__ uint32_t warp_sums[32];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int b = blockIdx.x * 4096 + 4 * tid;
-    uint32_t v[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) v[q] = b + q < n ? counts[b + q] : 0u;
-    const uint32_t local = v[0] + v[1] + v[2] + v[3];
-    uint32_t x = local;
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) warp_sums[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-        uint32_t s = warp_sums[lane];
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += y;
-        }
-        warp_sums[lane] = s;
-    }
-    __syncthreads();
-    uint32_t run = bases[blockIdx.x] + x - local + (warp > 0 ? warp_sums[warp - 1] : 0u);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        if (b + q < n) offsets[b + q] = run;
-        run += v[q];
-    }
-    if (blockIdx.x == gridDim.x - 1 && tid == 0) offsets[n] = bases[gridDim.x];
-}
-
-vsr_status launch_scan_large(const uint32_t* counts, int n, uint32_t* partials, uint32_t* offsets, cudaStream_t st)
-{
-    const int nb = (n + 4095) / 4096;
-    if (nb <= 1) return launch_scan(counts, n, offsets, st);
-    scan_block_sums<<<nb, 1024, 0, st>>>(counts, n, partials);
-    // scan the nb block sums in place into partials[nb + 1 ...]: reuse the one-CTA scan
-    vsr_status s = launch_scan(partials, nb, partials + nb + 1, st);
-    if (s != VSR_OK) return s;
-    scan_blocks_apply<<<nb, 1024, 0, st>>>(counts, n, partials + nb + 1, offsets);
-    VSR_CUDA_TRY(cudaGetLastError());
-    return VSR_OK;
-}

@@ -7,11 +7,17 @@
 //   over the fragments of a pixel in ascending (r, t):
 //     m^fc = min(m^f, 1 - m^b);  I += m^fc shade;  m^b += m^fc
 // Unlike coverage, the image depends on the order, so every fragment is
-// kept: a count pass and a fill pass over the tile bins (the same template,
-// so both see exactly the same fragments), an exclusive scan of the
-// per-pixel counts in between, and each thread sorts and merges its own
-// pixels' lists after the fill.  A fragment record is the float4
-// (r, t, m^f, shade).
+// kept, as the float4 (r, t, m^f, shade), sorted per pixel.  Two launches:
+//  * frag_count_kernel walks the triangle grid (walk.cuh), evaluates every
+//    pixel x triangle pair, counts each pixel's fragments, takes the tile's
+//    range of the lists with one atomic (so no scan over the pixels runs) and
+//    keeps what the second launch needs: the tile's triangles and, per pixel,
+//    a bit for each that is a fragment.  Ids and depths are final here.
+//  * frag_fill_kernel, after the host has read the total, evaluates only the
+//    triangles with a fragment in the warp's block, sorts each pixel's
+//    fragments on their way in (shared memory), writes and merges them.
+// A tile with more than FRAG_LIST triangles keeps no list: the fill walks and
+// evaluates it again.
 //
 // Backward (vsr_raster_backward).  Per pixel, with upstream gradients dI,
 // dcov, ddepth: the merge takes m^fc = m^f until the first fragment f* with
@@ -27,250 +33,389 @@
 // per-triangle record gradients accumulate with float4 atomics; the
 // per-pixel (dG, d delta) go to the map adjoint (map.cu), and the set-up
 // adjoint below takes the record gradients to the world vertices.
-#include "stage.cuh"
+#include "tile.cuh"
+#include "walk.cuh"
 
 namespace {
 
-constexpr int FT = 128;  // threads of a fragment-kernel CTA: one 16x16 tile, two pixels per thread
-constexpr int PPT = 2;
-static_assert(FT == STAGE_CHUNK && FT * PPT == TILE_PIX, "tile layout");
-
-struct FragView {
-    const float4* map;
-    int W, H;
-    const Cone* tiles;
-    int tiles_x;
-    const float4* rec;
-    int T;
-    const uint32_t* offsets;  // tile bins
-    const uint32_t* ids;
-    uint32_t cap;
-    const float* colors;      // per triangle, NULL = 1
-    uint32_t* counts;         // count pass: fragments per pixel
-    const uint32_t* foff;     // fill pass: first fragment of each pixel (W*H + 1, exclusive scan)
-    float4* frags;            // fill pass: (r, t bits, m^f, shade)
-    uint32_t fcap;
-    float* image;
-    float* cov;
-    uint32_t* out_id;
-    float* out_depth;
-    const uint32_t* ends;     // as RasterView::ends
-};
+static_assert(FRAG_LIST == STAGE_CHUNK && FRAG_LIST == 128, "a tile's list is one chunk, a pixel's bits four words");
 
 __device__ __forceinline__ bool frag_less(const float4& a, const float4& b)
 {
     return a.x < b.x || (a.x == b.x && __float_as_uint(a.y) < __float_as_uint(b.y));
 }
 
-template <bool FILL>
-__global__ void __launch_bounds__(FT) frag_kernel(FragView v, int* __restrict__ status)
+// A lane's two pixels as the fragment kernels see them.
+struct FragPix {
+    float2 dgx, dgy, dgz, eg;  // G - a, |G|^2 - 1; 0 at an invalid pixel
+    float delta[PPT], lim[PPT];  // as PixPair of raster.cu
+};
+
+__device__ __forceinline__ bool frag_start(const FragArgs& v, const TilePos& tp, const float4& axis, FragPix& q,
+                                           WarpCones& wc)
 {
-    __shared__ Stage st;
-    __shared__ float scol[STAGE_CHUNK];
-    const int tile = blockIdx.x;
-    const int W = v.W, H = v.H, T = v.T;
-    const size_t TT = (size_t)T;
-    const int tx = tile % v.tiles_x, ty = tile / v.tiles_x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int px = tx * TILE + (warp & 1) * 8 + (lane & 7);
-    const int py0 = ty * TILE + (warp >> 1) * 8 + (lane >> 3);
-
-    const Cone tc = v.tiles[tile];
-    const float ax = tc.c0.x, ay = tc.c0.y, az = tc.c0.z;
-
-    float gx[PPT], gy[PPT], gz[PPT], dgx[PPT], dgy[PPT], dgz[PPT], delta[PPT], h[PPT], eg[PPT];
-    bool pv[PPT], inimg[PPT];
-    uint32_t cnt[PPT], room[PPT];
-    size_t fbase[PPT];
-    unsigned long long key[PPT];
+    float gx[PPT], gy[PPT], gz[PPT], h[PPT];
+    bool pv[PPT];
 #pragma unroll
     for (int p = 0; p < PPT; ++p) {
-        const int py = py0 + 4 * p;
-        inimg[p] = px < W && py < H;
-        const size_t o = (size_t)py * W + px;
+        const int y = tp.py + 4 * p;
         float4 g = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (inimg[p]) g = v.map[o];
+        if (tp.px < v.W && y < v.H) g = v.map[(size_t)y * v.W + tp.px];
         pv[p] = g.w > 0.0f;
         gx[p] = g.x;
         gy[p] = g.y;
         gz[p] = g.z;
-        delta[p] = g.w;
         h[p] = pv[p] ? 0.5f / g.w : 0.0f;
-        eg[p] = pv[p] ? norm2_minus_one(g.x, g.y, g.z) : 0.0f;
-        dgx[p] = g.x - ax;
-        dgy[p] = g.y - ay;
-        dgz[p] = g.z - az;
-        cnt[p] = 0u;
-        key[p] = ~0ull;
-        fbase[p] = 0;
-        room[p] = 0u;
-        if (FILL && inimg[p]) {
-            fbase[p] = v.foff[o];
-            room[p] = v.foff[o + 1] - v.foff[o];
-        }
+        q.delta[p] = g.w;
+        q.lim[p] = pv[p] ? -h[p] : INFINITY;
     }
-
-    // the warp's own view cone (its 8x8 pixels), as in the coverage kernel
-    float sx = 0.0f, sy = 0.0f, sz = 0.0f, cn = 0.0f, hw = 0.0f;
-#pragma unroll
-    for (int p = 0; p < PPT; ++p)
-        if (pv[p]) {
-            sx += gx[p];
-            sy += gy[p];
-            sz += gz[p];
-            cn += 1.0f;
-            hw = fmaxf(hw, h[p]);
-        }
-    sx = warp_sum(sx);
-    sy = warp_sum(sy);
-    sz = warp_sum(sz);
-    const float wcnt = warp_sum(cn);
-    const float wh = warp_max(hw);
-    const float wl = sqrtf(sx * sx + sy * sy + sz * sz);
-    const bool wdeg = !(wl > 1e-6f * fmaxf(wcnt, 1.0f));
-    const float wax = wdeg ? 0.0f : sx / wl, way = wdeg ? 0.0f : sy / wl, waz = wdeg ? 1.0f : sz / wl;
-    float cm = 2.0f;
-#pragma unroll
-    for (int p = 0; p < PPT; ++p)
-        if (pv[p]) cm = fminf(cm, gx[p] * wax + gy[p] * way + gz[p] * waz);
-    float wcos = fmaxf(-1.0f, fminf(1.0f, warp_min(cm) - 2e-6f));
-    if (wdeg) wcos = -1.0f;
-    const float wsin = sqrtf(fmaxf(0.0f, 1.0f - wcos * wcos));
-    const bool warp_active = wcnt > 0.0f;
-
-    uint32_t b0 = 0, b1 = 0;
-    if (tc.c1.z > 0.0f) {
-        b0 = v.offsets[tile];
-        b1 = v.ends ? v.ends[tile] : v.offsets[tile + 1];
-        if (b1 > v.cap) {
-            if (threadIdx.x == 0) raise_status(status, VSR_ERR_BIN_OVERFLOW);
-            b1 = v.cap;
-            b0 = min(b0, v.cap);
-        }
+    q.dgx = make_float2(pv[0] ? gx[0] - axis.x : 0.0f, pv[1] ? gx[1] - axis.x : 0.0f);
+    q.dgy = make_float2(pv[0] ? gy[0] - axis.y : 0.0f, pv[1] ? gy[1] - axis.y : 0.0f);
+    q.dgz = make_float2(pv[0] ? gz[0] - axis.z : 0.0f, pv[1] ? gz[1] - axis.z : 0.0f);
+    const float2 eg = norm2_minus_one2(make_float2(gx[0], gx[1]), make_float2(gy[0], gy[1]), make_float2(gz[0], gz[1]));
+    q.eg = make_float2(pv[0] ? eg.x : 0.0f, pv[1] ? eg.y : 0.0f);
+    float4 c0, c1;
+    block_cone(gx, gy, gz, h, pv, c0, c1);
+    if ((threadIdx.x & 31) == 0) {
+        wc.c[threadIdx.x >> 5][0] = c0;
+        wc.c[threadIdx.x >> 5][1] = c1;
     }
-    // the thread's two pixels side by side for the packed FP32x2 distances
-    // (bit for bit the scalar ones, so the classification is the coverage
-    // kernel's)
-    static_assert(PPT == 2, "packed pairs hold the thread's two pixels");
-    const float2 dgx2 = make_float2(dgx[0], dgx[1]), dgy2 = make_float2(dgy[0], dgy[1]),
-                 dgz2 = make_float2(dgz[0], dgz[1]), eg2 = make_float2(eg[0], eg[1]);
+    __syncwarp();
+    return c1.z > 0.0f;
+}
 
-    for (uint32_t base = b0; base < b1; base += STAGE_CHUNK) {
-        const int n = (int)min((uint32_t)STAGE_CHUNK, b1 - base);
+// One staged triangle at the lane's pixels: the coverage kernel's distances
+// and classification.
+struct FragEval {
+    float gm[PPT], r[PPT], D[PPT];
+    bool f[PPT], in[PPT];
+};
+// false (for the whole warp): no fragment
+__device__ __forceinline__ bool frag_eval(const Stage& st, int j, const FragPix& q, FragEval& o)
+{
+    const float4 b = st.s1[j], e = st.s6[j];
+    const float2 g4 = miter_distance2(q.dgx, q.dgy, q.dgz, e, b, q.eg);
+    const float2 g1 = plane_distance2(q.dgx, q.dgy, q.dgz, st.s2[j]);
+    const float2 g2 = plane_distance2(q.dgx, q.dgy, q.dgz, st.s3[j]);
+    const float2 g3 = plane_distance2(q.dgx, q.dgy, q.dgz, st.s4[j]);
+    const float g3m[PPT] = {fminf(fminf(g1.x, g2.x), g3.x), fminf(fminf(g1.y, g2.y), g3.y)};
+    o.gm[0] = fminf(g3m[0], g4.x);
+    o.gm[1] = fminf(g3m[1], g4.y);
+    const bool f0 = o.gm[0] > q.lim[0], f1 = o.gm[1] > q.lim[1];
+    if (!__any_sync(0xffffffffu, f0 || f1)) return false;
+    const float2 Dp = plane_distance2(q.dgx, q.dgy, q.dgz, st.s5[j]);
+    o.D[0] = Dp.x;
+    o.D[1] = Dp.y;
+    const unsigned ties = __float_as_uint(st.s0[j].w);
+#pragma unroll
+    for (int p = 0; p < PPT; ++p) {
+        o.r[p] = __fdividef(b.w, o.D[p]);
+        o.f[p] = (p ? f1 : f0) && __float_as_uint(o.r[p]) - 1u < DEPTH_LIM;  // 0 < r < inf
+        o.in[p] = o.f[p] && centre_inside(p ? g1.y : g1.x, p ? g2.y : g2.x, p ? g3.y : g3.x, g3m[p], ties);
+    }
+    return true;
+}
+
+__device__ __forceinline__ float4 frag_record(const FragEval& o, const FragPix& q, int p, uint32_t t, float colour)
+{
+    return make_float4(o.r[p], __uint_as_float(t), __saturatef(fmaf(o.gm[p], q.delta[p], 0.5f)),
+                       colour * fabsf(o.D[p]));
+}
+
+struct FragShared {
+    Stage st;
+    WalkShared ws;
+    WarpCones wc;
+    uint32_t ids[WALK_BLOCK];
+    uint32_t n;
+};
+
+// The tile's triangles, walked block by block and staged chunk by chunk; each
+// survivor of the warp's cull goes to each(j, group, k): staged slot j = 32
+// group + k.  Called by every thread of the CTA after walk_ranges, frag_start
+// and a barrier; staged(t, j) runs in the thread that stages triangle t.
+template <class Stage1, class Each>
+__device__ __forceinline__ void frag_walk(const FragArgs& v, const Cone& tc, FragShared& s, bool active, Stage1 staged,
+                                          Each each)
+{
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (uint32_t e0 = 0; e0 < s.ws.total; e0 += WALK_BLOCK) {
+        if (e0) {
+            __syncthreads();
+            if (threadIdx.x == 0) s.n = 0u;
+            __syncthreads();
+        }
+        const uint32_t e1 = min(s.ws.total, e0 + (uint32_t)WALK_BLOCK);
+        Walk w;
+        w.init(v.wi, tc, s.ws);
+        for (uint32_t i0 = e0; i0 < e1; i0 += WALK_THREADS) {
+            const uint32_t idx = i0 + threadIdx.x;
+            uint32_t t;
+            const bool hit = w.test(v.wi, v.rec, v.T, s.ws, idx, idx < e1, t);
+            const unsigned m = __ballot_sync(FULL, hit);
+            if (!m) continue;
+            uint32_t base = 0;
+            if (lane == 0) base = atomicAdd(&s.n, (uint32_t)__popc(m));
+            base = __shfl_sync(FULL, base, 0);
+            if (hit) s.ids[base + (uint32_t)__popc(m & ((1u << lane) - 1u))] = t;
+        }
         __syncthreads();
-        if ((int)threadIdx.x < n) {
-            const uint32_t t = v.ids[base + threadIdx.x];
-            if (t >= (uint32_t)T) {
-                raise_status(status, VSR_ERR_BIN_OVERFLOW);
-                st.s6[threadIdx.x] = make_float4(0.0f, 0.0f, 0.0f, __uint_as_float(STAGE_EMPTY));
-            } else {
-                stage_triangle(v.rec, TT, t, ax, ay, az, st, threadIdx.x);
-                scol[threadIdx.x] = v.colors ? v.colors[t] : 1.0f;
+        const uint32_t n = s.n;
+        for (uint32_t base = 0; base < n; base += STAGE_CHUNK) {
+            const int nc = (int)min((uint32_t)STAGE_CHUNK, n - base);
+            if (base) __syncthreads();
+            if ((int)threadIdx.x < nc) {
+                const uint32_t t = s.ids[base + threadIdx.x];
+                stage_checked(v.rec, v.T, t, tc.c0, s.st, threadIdx.x, v.status);
+                staged(t, (int)threadIdx.x);
+            }
+            __syncthreads();
+            if (!active) continue;
+#pragma unroll
+            for (int g = 0; g < STAGE_CHUNK / 32; ++g) {
+                const int jj = 32 * g + lane;
+                if (32 * g >= nc) break;
+                bool keep = false;
+                if (jj < nc && __float_as_uint(s.st.s6[jj].w) != STAGE_EMPTY)
+                    keep = cone_may_hit(s.st.s0[jj], s.st.s1[jj], s.st.s2[jj], s.st.s3[jj], s.st.s4[jj],
+                                        s.wc.c[warp][0], s.wc.c[warp][1], false);
+                unsigned mask = __ballot_sync(FULL, keep);
+                while (mask) {
+                    const int k = 31 - __clz(mask);
+                    mask ^= 1u << k;
+                    each(32 * g + k, g, k);
+                }
             }
         }
-        __syncthreads();
-        if (!warp_active) continue;
-        for (int gbase = 0; gbase < n; gbase += 32) {
-            bool keep = false;
-            const int jj = gbase + lane;
-            if (jj < n && __float_as_uint(st.s6[jj].w) != STAGE_EMPTY) {
-                const float4 a = st.s0[jj];
-                const float4 b = st.s1[jj];
-                keep = cap_hits_cone(make_float3(a.x, a.y, a.z), 1.0f - 0.5f * b.y, b.x, make_float3(wax, way, waz),
-                                     wcos, wsin, wh);
-                const float lim = -(wh + wsin + (1.0f - wcos) + 1e-6f);
-                const float4 n1 = st.s2[jj], n2 = st.s3[jj], n3 = st.s4[jj];
-                keep = keep && fmaf(wax, n1.x, fmaf(way, n1.y, waz * n1.z)) > lim &&
-                       fmaf(wax, n2.x, fmaf(way, n2.y, waz * n2.z)) > lim &&
-                       fmaf(wax, n3.x, fmaf(way, n3.y, waz * n3.z)) > lim;
+    }
+}
+
+__global__ void __launch_bounds__(RT, 6) frag_count_kernel(FragArgs v)
+{
+    __shared__ FragShared s;
+    __shared__ uint32_t s_sum[RT / 32], s_base;
+    const unsigned FULL = 0xffffffffu;
+    const int tile = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const TilePos tp(tile, v.tiles_x);
+    const Cone tc = v.tiles[tile];
+    if (threadIdx.x < 32) walk_ranges(v.wi, v.T, v.geom[tile], tc.c0.y, s.ws);
+    if (threadIdx.x == 0) s.n = 0u;
+    FragPix q;
+    const bool active = frag_start(v, tp, tc.c0, q, s.wc);
+    uint32_t cnt[PPT] = {0u, 0u}, bits[PPT][4] = {};
+    unsigned long long key[PPT] = {~0ull, ~0ull};
+    __syncthreads();
+    frag_walk(
+        v, tc, s, active, [](uint32_t, int) {},
+        [&](int j, int g, int k) {
+            FragEval o;
+            if (!frag_eval(s.st, j, q, o)) return;
+            const uint32_t t = __float_as_uint(s.st.s6[j].w);
+#pragma unroll
+            for (int p = 0; p < PPT; ++p) {
+                cnt[p] += o.f[p];
+                // (g is a constant of the unrolled loop: bits stay in registers)
+                bits[p][g] |= (o.f[p] ? 1u : 0u) << k;
+                const unsigned long long kk = ((unsigned long long)__float_as_uint(o.r[p]) << 32) | t;
+                if (o.in[p] && kk < key[p]) key[p] = kk;
             }
-            unsigned mask = __ballot_sync(0xffffffffu, keep);
-            while (mask) {
-                const int j = gbase + __ffs(mask) - 1;
-                mask &= mask - 1;
-                const float4 a = st.s0[j];
-                const float4 b = st.s1[j];
-                const float4 e = st.s6[j];
-                const float2 g4p = miter_distance2(dgx2, dgy2, dgz2, e, b, eg2);
-                const float g4[PPT] = {g4p.x, g4p.y};
-                bool p4[PPT], any4 = false;
+        });
+    // the tile's range of the lists, its pixels in thread order
+    const uint32_t mine = cnt[0] + cnt[1];
+    uint32_t incl = mine;
 #pragma unroll
-                for (int p = 0; p < PPT; ++p) {
-                    p4[p] = pv[p] && g4[p] > -h[p];
-                    any4 |= p4[p];
-                }
-                if (!__any_sync(0xffffffffu, any4)) continue;
-                const float2 g1p = plane_distance2(dgx2, dgy2, dgz2, st.s2[j]);
-                const float2 g2p = plane_distance2(dgx2, dgy2, dgz2, st.s3[j]);
-                const float2 g3p = plane_distance2(dgx2, dgy2, dgz2, st.s4[j]);
-                const float g1[PPT] = {g1p.x, g1p.y}, g2[PPT] = {g2p.x, g2p.y}, g3[PPT] = {g3p.x, g3p.y};
-                float g3m[PPT], gm[PPT];
-                bool frag[PPT], anyf = false;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) s_sum[warp] = incl;
+    __syncthreads();
+    uint32_t before = 0, total = 0;
 #pragma unroll
-                for (int p = 0; p < PPT; ++p) {
-                    g3m[p] = fminf(fminf(g1[p], g2[p]), g3[p]);
-                    gm[p] = fminf(g3m[p], g4[p]);
-                    frag[p] = p4[p] && gm[p] > -h[p];
-                    anyf |= frag[p];
-                }
-                if (!__any_sync(0xffffffffu, anyf)) continue;
-                const float2 Dp = plane_distance2(dgx2, dgy2, dgz2, st.s5[j]);
-                const float D2[PPT] = {Dp.x, Dp.y};
-                const unsigned ties = __float_as_uint(a.w);
-                const uint32_t t = __float_as_uint(e.w);
+    for (int w = 0; w < RT / 32; ++w) {
+        if (w < warp) before += s_sum[w];
+        total += s_sum[w];
+    }
+    const bool list = s.ws.total <= (uint32_t)WALK_BLOCK && s.n <= (uint32_t)FRAG_LIST;
+    if (threadIdx.x == 0) {
+        s_base = total ? atomicAdd(v.cursor, total) : 0u;
+        v.tile_n[tile] = list ? s.n : 0xffffffffu;
+    }
+    if (list && threadIdx.x < s.n) v.tile_ids[(size_t)tile * FRAG_LIST + threadIdx.x] = s.ids[threadIdx.x];
+    __syncthreads();
+    uint32_t off = s_base + before + incl - mine;
 #pragma unroll
-                for (int p = 0; p < PPT; ++p) {
-                    const float D = D2[p];
-                    const float r = __fdividef(b.w, D);
-                    const bool f = frag[p] && __float_as_uint(r) - 1u < 0x7f7fffffu;  // 0 < r < inf
-                    if (!f) continue;
-                    if (FILL) {
-                        const float m = __saturatef(fmaf(gm[p], delta[p], 0.5f));
-                        if (cnt[p] < room[p])
-                            v.frags[fbase[p] + cnt[p]] =
-                                make_float4(r, __uint_as_float(t), m, scol[j] * fabsf(D));
-                        const unsigned long long k = ((unsigned long long)__float_as_uint(r) << 32) | t;
-                        if (centre_inside(g1[p], g2[p], g3[p], g3m[p], ties) && k < key[p]) key[p] = k;
+    for (int p = 0; p < PPT; ++p) {
+        if (tp.px < v.W && tp.py + 4 * p < v.H) {
+            const size_t o = (size_t)(tp.py + 4 * p) * v.W + tp.px;
+            v.span[o] = make_uint2(off, cnt[p]);
+            if (list) v.bits[o] = make_uint4(bits[p][0], bits[p][1], bits[p][2], bits[p][3]);
+            const bool hit = key[p] != ~0ull;
+            if (v.out_id) v.out_id[o] = hit ? (uint32_t)(key[p] & 0xffffffffull) : 0xffffffffu;
+            if (v.out_depth) v.out_depth[o] = hit ? __uint_as_float((uint32_t)(key[p] >> 32)) : INFINITY;
+        }
+        off += cnt[p];
+    }
+}
+
+// fragments of a pixel sorted in shared memory; a longer list is sorted where
+// it is stored
+constexpr uint32_t FRAG_SORT = 8;
+
+__global__ void __launch_bounds__(RT, 5) frag_fill_kernel(FragArgs v)
+{
+    __shared__ union {
+        FragShared walk;
+        struct {
+            Stage st;
+            float4 rec[FRAG_SORT][RT];
+        } list;
+    } s;
+    __shared__ float scol[STAGE_CHUNK];
+    const unsigned FULL = 0xffffffffu;
+    const int tile = blockIdx.x;
+    const TilePos tp(tile, v.tiles_x);
+    const Cone tc = v.tiles[tile];
+    if (tile == 0 && threadIdx.x == 0) *v.cursor = 0u;  // for the next frame
+    const uint32_t n = v.tile_n[tile];
+    FragPix q;
+    uint2 span[PPT] = {};
+    bool inimg[PPT];
+#pragma unroll
+    for (int p = 0; p < PPT; ++p) {
+        inimg[p] = tp.px < v.W && tp.py + 4 * p < v.H;
+        if (inimg[p]) span[p] = v.span[(size_t)(tp.py + 4 * p) * v.W + tp.px];
+    }
+    // (room beyond the buffer is never given out once the host has sized it)
+    const bool fits = (uint64_t)span[0].x + span[0].y <= v.fcap && (uint64_t)span[1].x + span[1].y <= v.fcap;
+    if (!fits) {
+        raise_status(v.status, VSR_ERR_FRAG_OVERFLOW);
+        span[0].y = span[1].y = 0u;
+    }
+    uint32_t cnt[PPT] = {0u, 0u};
+    bool sorted[PPT] = {false, false};
+    auto put = [&](const FragEval& o, int p, uint32_t t, float colour) {
+        // append (lists that are not sorted on their way in)
+        if (cnt[p] < span[p].y) v.frags[(size_t)span[p].x + cnt[p]] = frag_record(o, q, p, t, colour);
+        ++cnt[p];
+    };
+    if (n <= (uint32_t)FRAG_LIST) {
+        __shared__ WarpCones wc;
+        if (threadIdx.x < n) {
+            const uint32_t t = v.tile_ids[(size_t)tile * FRAG_LIST + threadIdx.x];
+            stage_checked(v.rec, v.T, t, tc.c0, s.list.st, threadIdx.x, v.status);
+            scol[threadIdx.x] = v.colors && t < (uint32_t)v.T ? v.colors[t] : 1.0f;
+        }
+        frag_start(v, tp, tc.c0, q, wc);
+        uint4 bits[PPT];
+#pragma unroll
+        for (int p = 0; p < PPT; ++p) {
+            bits[p] = make_uint4(0u, 0u, 0u, 0u);
+            if (inimg[p] && span[p].y) bits[p] = v.bits[(size_t)(tp.py + 4 * p) * v.W + tp.px];
+            sorted[p] = span[p].y <= FRAG_SORT;
+        }
+        __syncthreads();
+        // (one pixel's list at a time in shared memory: the first pixels of
+        // the lanes, then the second)
+#pragma unroll
+        for (int p = 0; p < PPT; ++p) {
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                const uint32_t b = g == 0 ? bits[p].x : (g == 1 ? bits[p].y : (g == 2 ? bits[p].z : bits[p].w));
+                unsigned any = __reduce_or_sync(FULL, b);
+                while (any) {
+                    const int k = 31 - __clz(any);
+                    any ^= 1u << k;
+                    const int j = 32 * g + k;
+                    if (!(b >> k & 1u)) continue;
+                    // this pixel's distances in scalar form (bit for bit the packed ones)
+                    const float dx = p ? q.dgx.y : q.dgx.x, dy = p ? q.dgy.y : q.dgy.x, dz = p ? q.dgz.y : q.dgz.x;
+                    const float4 c = s.list.st.s1[j], e = s.list.st.s6[j];
+                    const float g4 = miter_distance(dx, dy, dz, e, c, p ? q.eg.y : q.eg.x);
+                    const float g3m = fminf(fminf(plane_distance(dx, dy, dz, s.list.st.s2[j]),
+                                                  plane_distance(dx, dy, dz, s.list.st.s3[j])),
+                                            plane_distance(dx, dy, dz, s.list.st.s4[j]));
+                    const float D = plane_distance(dx, dy, dz, s.list.st.s5[j]);
+                    const float4 x = make_float4(__fdividef(c.w, D), e.w,
+                                                 __saturatef(fmaf(fminf(g3m, g4), q.delta[p], 0.5f)),
+                                                 scol[j] * fabsf(D));
+                    if (cnt[p] >= span[p].y) {
+                        ++cnt[p];  // spans of another frame: reported below
+                    } else if (sorted[p]) {
+                        uint32_t u = cnt[p];
+                        while (u > 0 && frag_less(x, s.list.rec[u - 1][threadIdx.x])) {
+                            s.list.rec[u][threadIdx.x] = s.list.rec[u - 1][threadIdx.x];
+                            --u;
+                        }
+                        s.list.rec[u][threadIdx.x] = x;
+                        ++cnt[p];
+                    } else {
+                        v.frags[(size_t)span[p].x + cnt[p]] = x;
+                        ++cnt[p];
                     }
-                    ++cnt[p];
                 }
             }
+            if (!sorted[p] || !inimg[p]) continue;
+            // the pixel's merge, and its list
+            float mb = 0.0f, img = 0.0f;
+            for (uint32_t u = 0; u < min(cnt[p], span[p].y); ++u) {
+                const float4 x = s.list.rec[u][threadIdx.x];
+                v.frags[(size_t)span[p].x + u] = x;
+                if (mb < 1.0f) {
+                    const float mfc = fminf(x.z, 1.0f - mb);
+                    img = fmaf(mfc, x.w, img);
+                    mb += mfc;
+                }
+            }
+            const size_t o = (size_t)(tp.py + 4 * p) * v.W + tp.px;
+            if (v.image) v.image[o] = img;
+            if (v.cov) v.cov[o] = mb;
         }
+    } else {
+        if (threadIdx.x < 32) walk_ranges(v.wi, v.T, v.geom[tile], tc.c0.y, s.walk.ws);
+        if (threadIdx.x == 0) s.walk.n = 0u;
+        const bool active = frag_start(v, tp, tc.c0, q, s.walk.wc);
+        __syncthreads();
+        frag_walk(
+            v, tc, s.walk, active,
+            [&](uint32_t t, int j) { scol[j] = v.colors && t < (uint32_t)v.T ? v.colors[t] : 1.0f; },
+            [&](int j, int, int) {
+                FragEval o;
+                if (!frag_eval(s.walk.st, j, q, o)) return;
+                const uint32_t t = __float_as_uint(s.walk.st.s6[j].w);
+#pragma unroll
+                for (int p = 0; p < PPT; ++p)
+                    if (o.f[p]) put(o, p, t, scol[j]);
+            });
     }
-
 #pragma unroll
     for (int p = 0; p < PPT; ++p) {
         if (!inimg[p]) continue;
-        const size_t o = (size_t)(py0 + 4 * p) * W + px;
-        if (!FILL) {
-            v.counts[o] = cnt[p];
-            continue;
-        }
-        if (cnt[p] != room[p]) raise_status(status, VSR_ERR_FRAG_OVERFLOW);  // counts of another frame
-        const uint32_t n = min(cnt[p], room[p]);
-        float4* F = v.frags + fbase[p];
-        // insertion sort by (r, t): lists are a few fragments long
-        for (uint32_t q = 1; q < n; ++q) {
-            const float4 x = F[q];
-            uint32_t u = q;
-            while (u > 0 && frag_less(x, F[u - 1])) {
-                F[u] = F[u - 1];
-                --u;
+        if (fits && cnt[p] != span[p].y) raise_status(v.status, VSR_ERR_FRAG_OVERFLOW);  // spans of another frame
+        if (sorted[p]) continue;
+        const size_t o = (size_t)(tp.py + 4 * p) * v.W + tp.px;
+        const uint32_t m = min(cnt[p], span[p].y);
+        float4* F = v.frags + span[p].x;
+        // insertion sort by (r, t)
+        for (uint32_t u = 1; u < m; ++u) {
+            const float4 x = F[u];
+            uint32_t w = u;
+            while (w > 0 && frag_less(x, F[w - 1])) {
+                F[w] = F[w - 1];
+                --w;
             }
-            F[u] = x;
+            F[w] = x;
         }
         float mb = 0.0f, img = 0.0f;
-        for (uint32_t q = 0; q < n && mb < 1.0f; ++q) {
-            const float4 x = F[q];
+        for (uint32_t u = 0; u < m && mb < 1.0f; ++u) {
+            const float4 x = F[u];
             const float mfc = fminf(x.z, 1.0f - mb);
             img = fmaf(mfc, x.w, img);
             mb += mfc;
         }
-        const bool hit = key[p] != ~0ull;
         if (v.image) v.image[o] = img;
         if (v.cov) v.cov[o] = mb;
-        if (v.out_id) v.out_id[o] = hit ? (uint32_t)(key[p] & 0xffffffffull) : 0xffffffffu;
-        if (v.out_depth) v.out_depth[o] = hit ? __uint_as_float((uint32_t)(key[p] >> 32)) : INFINITY;
     }
 }
 
@@ -283,7 +428,7 @@ struct BackView {
     const float4* rec;
     int T;
     const float* colors;
-    const uint32_t* foff;
+    const uint2* span;
     const float4* frags;
     const uint32_t* id;
     const float* dimage;
@@ -314,8 +459,9 @@ __global__ void __launch_bounds__(TILE_PIX) frag_backward_kernel(BackView v)
     const float dI = v.dimage ? v.dimage[o] : 0.0f;
     const float dC = v.dcov ? v.dcov[o] : 0.0f;
     const float dD = v.ddepth ? v.ddepth[o] : 0.0f;
-    const uint32_t b0 = v.foff[o], n = v.foff[o + 1] - b0;
-    const float4* __restrict__ F = v.frags + b0;
+    const uint2 span = v.span[o];
+    const uint32_t n = span.y;
+    const float4* __restrict__ F = v.frags + span.x;
 
     // the saturating fragment, replaying the forward merge's arithmetic
     uint32_t fstar = n;
@@ -557,20 +703,14 @@ __global__ void __launch_bounds__(128) setup_backward_kernel(const float* __rest
 
 vsr_status launch_frag_count(const FragArgs& a, cudaStream_t st)
 {
-    const int tx = (a.W + TILE - 1) / TILE, ty = (a.H + TILE - 1) / TILE;
-    FragView v{a.map, a.W, a.H, a.tiles, tx, a.rec, a.T, a.offsets, a.ids, a.cap, a.colors, a.counts,
-               nullptr, nullptr, 0u, nullptr, nullptr, nullptr, nullptr, a.ends};
-    frag_kernel<false><<<tx * ty, FT, 0, st>>>(v, a.status);
+    frag_count_kernel<<<a.tiles_x * ((a.H + TILE - 1) / TILE), RT, 0, st>>>(a);
     VSR_CUDA_TRY(cudaGetLastError());
     return VSR_OK;
 }
 
 vsr_status launch_frag_fill(const FragArgs& a, cudaStream_t st)
 {
-    const int tx = (a.W + TILE - 1) / TILE, ty = (a.H + TILE - 1) / TILE;
-    FragView v{a.map,    a.W,   a.H,     a.tiles, tx,    a.rec,   a.T,      a.offsets, a.ids, a.cap,
-               a.colors, nullptr, a.foff, a.frags, a.fcap, a.image, a.cov, a.out_id, a.out_depth, a.ends};
-    frag_kernel<true><<<tx * ty, FT, 0, st>>>(v, a.status);
+    frag_fill_kernel<<<a.tiles_x * ((a.H + TILE - 1) / TILE), RT, 0, st>>>(a);
     VSR_CUDA_TRY(cudaGetLastError());
     return VSR_OK;
 }
@@ -578,7 +718,7 @@ vsr_status launch_frag_fill(const FragArgs& a, cudaStream_t st)
 vsr_status launch_frag_backward(const FragArgs& a, const uint32_t* id, const float* dimage, const float* dcov,
                                 const float* ddepth, float4* grad, float4* dmap, cudaStream_t st)
 {
-    BackView v{a.map, a.W, a.H, a.rec, a.T, a.colors, a.foff, a.frags, id, dimage, dcov, ddepth, grad, dmap};
+    BackView v{a.map, a.W, a.H, a.rec, a.T, a.colors, a.span, a.frags, id, dimage, dcov, ddepth, grad, dmap};
     dim3 grid((a.W + TILE - 1) / TILE, (a.H + TILE - 1) / TILE);
     frag_backward_kernel<<<grid, TILE_PIX, 0, st>>>(v);
     VSR_CUDA_TRY(cudaGetLastError());

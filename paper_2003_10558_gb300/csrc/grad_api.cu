@@ -6,10 +6,13 @@
 #include "handles.cuh"
 
 struct vsr_frags_s {
-    size_t npix = 0;            // per-pixel buffers sized for this many pixels
-    uint32_t* counts = nullptr;  // npix
-    uint32_t* foff = nullptr;    // npix + 1
-    uint32_t* scan_part = nullptr;
+    size_t npix = 0, ntiles = 0;  // per-pixel and per-tile buffers sized for these
+    uint2* span = nullptr;        // npix
+    uint4* bits = nullptr;        // npix
+    uint32_t* tile_n = nullptr;   // ntiles
+    uint32_t* tile_ids = nullptr; // ntiles x FRAG_LIST
+    uint32_t* cursor = nullptr;
+    bool dirty = true;            // the cursor is not known to be zero
     float4* frags = nullptr;
     uint32_t fcap = 0;
     uint32_t* h_total = nullptr;  // pinned
@@ -27,31 +30,35 @@ namespace {
 
 void frags_release_pixels(vsr_frags f)
 {
-    cudaFree(f->counts);
-    cudaFree(f->foff);
-    cudaFree(f->scan_part);
+    cudaFree(f->span);
+    cudaFree(f->bits);
+    cudaFree(f->tile_n);
+    cudaFree(f->tile_ids);
     cudaFree(f->dmap);
     cudaFree(f->lens_part);
-    f->counts = f->foff = f->scan_part = nullptr;
+    f->span = nullptr;
+    f->bits = nullptr;
+    f->tile_n = f->tile_ids = nullptr;
     f->dmap = nullptr;
     f->lens_part = nullptr;
-    f->npix = 0;
+    f->npix = f->ntiles = 0;
 }
 
-vsr_status frags_ensure_pixels(vsr_frags f, int W, int H)
+vsr_status frags_ensure_pixels(vsr_frags f, int W, int H, size_t ntiles)
 {
     const size_t n = (size_t)W * H;
-    if (n <= f->npix) return VSR_OK;
-    frags_release_pixels(f);
     vsr_status s;
-    const size_t nb = (n + 4095) / 4096;
-    if ((s = dalloc(&f->counts, n)) != VSR_OK || (s = dalloc(&f->foff, n + 1)) != VSR_OK ||
-        (s = dalloc(&f->scan_part, 2 * nb + 2)) != VSR_OK || (s = dalloc(&f->dmap, n)) != VSR_OK ||
-        (s = dalloc(&f->lens_part, map_backward_partials(W, H) + (size_t)W * 4)) != VSR_OK) {
+    if (!f->cursor && (s = dalloc(&f->cursor, 1)) != VSR_OK) return s;
+    if (n <= f->npix && ntiles <= f->ntiles) return VSR_OK;
+    frags_release_pixels(f);
+    if ((s = dalloc(&f->span, n)) != VSR_OK || (s = dalloc(&f->bits, n)) != VSR_OK ||
+        (s = dalloc(&f->tile_n, ntiles)) != VSR_OK || (s = dalloc(&f->tile_ids, ntiles * FRAG_LIST)) != VSR_OK ||
+        (s = dalloc(&f->dmap, n)) != VSR_OK || (s = dalloc(&f->lens_part, 4 * ntiles)) != VSR_OK) {
         frags_release_pixels(f);
         return s;
     }
     f->npix = n;
+    f->ntiles = ntiles;
     return VSR_OK;
 }
 
@@ -61,16 +68,18 @@ FragArgs frag_args(vsr_map m, vsr_scene sc, const float* colors, vsr_frags f)
     a.map = m->map;
     a.W = m->p.W;
     a.H = m->p.H;
+    a.tiles_x = m->tx;
     a.tiles = m->tiles;
+    a.geom = m->idx.geom;
     a.rec = sc->rec;
     a.T = (int)sc->T;
-    a.offsets = sc->offsets;
-    a.ends = sc->ends;
-    a.ids = sc->ids;
-    a.cap = sc->cap;
+    a.wi = walk_index(sc->grid, sc->T);
     a.colors = colors;
-    a.counts = f->counts;
-    a.foff = f->foff;
+    a.cursor = f->cursor;
+    a.tile_n = f->tile_n;
+    a.tile_ids = f->tile_ids;
+    a.span = f->span;
+    a.bits = f->bits;
     a.frags = f->frags;
     a.fcap = f->fcap;
     a.status = scene_status(sc);
@@ -100,6 +109,7 @@ void vsr_frags_free(vsr_frags f)
 {
     if (!f) return;
     frags_release_pixels(f);
+    cudaFree(f->cursor);
     cudaFree(f->frags);
     cudaFree(f->grad);
     if (f->h_total) cudaFreeHost(f->h_total);
@@ -112,15 +122,18 @@ vsr_status vsr_raster_shaded(vsr_map m, vsr_scene sc, const float* colors_dev, v
     if (!m || !sc || !f) return VSR_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
     f->valid = false;
-    vsr_status s = vsr_bin(m, sc, stream);
-    if (s != VSR_OK) return s;
+    vsr_status s;
+    // the first frame of a shape also sizes the stored bins (see raster_frame)
+    if ((s = scene_walk_begin(m, sc, st)) != VSR_OK) return s;
     const int W = m->p.W, H = m->p.H;
-    if ((s = frags_ensure_pixels(f, W, H)) != VSR_OK) return s;
+    if ((s = frags_ensure_pixels(f, W, H, (size_t)m->tx * m->ty)) != VSR_OK) return s;
     FragArgs a = frag_args(m, sc, colors_dev, f);
+    a.out_id = id_dev;
+    a.out_depth = depth_dev;
+    if (f->dirty) VSR_CUDA_TRY(cudaMemsetAsync(f->cursor, 0, sizeof(uint32_t), st));
+    f->dirty = true;  // until the fill, which clears it, is queued
     if ((s = launch_frag_count(a, st)) != VSR_OK) return s;
-    const int npix = W * H;
-    if ((s = launch_scan_large(f->counts, npix, f->scan_part, f->foff, st)) != VSR_OK) return s;
-    VSR_CUDA_TRY(cudaMemcpyAsync(f->h_total, f->foff + npix, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+    VSR_CUDA_TRY(cudaMemcpyAsync(f->h_total, f->cursor, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
     VSR_CUDA_TRY(cudaStreamSynchronize(st));
     const uint32_t total = *f->h_total;
     if (total > f->fcap) {
@@ -136,9 +149,8 @@ vsr_status vsr_raster_shaded(vsr_map m, vsr_scene sc, const float* colors_dev, v
     a.fcap = f->fcap;
     a.image = image_dev;
     a.cov = cov_dev;
-    a.out_id = id_dev;
-    a.out_depth = depth_dev;
     if ((s = launch_frag_fill(a, st)) != VSR_OK) return s;
+    f->dirty = false;
     f->map_gen = m->gen;
     f->scene_gen = sc->gen;
     f->W = W;

@@ -107,6 +107,11 @@ struct vsr_scene_s {
 
 inline int* scene_status(const vsr_scene_s* s) { return s->status ? s->status : status_word(); }
 
+// A launch that walks the scene's grid follows on st: its workspace and
+// bookkeeping; the first frame of a shape goes through stored bins first, so
+// that they are sized (see raster_frame in api.cu).
+vsr_status scene_walk_begin(vsr_map m, vsr_scene sc, cudaStream_t st);
+
 // Note a use of the scene's buffers queued on st (see use_event).
 inline vsr_status scene_used(vsr_scene_s* s, cudaStream_t st)
 {

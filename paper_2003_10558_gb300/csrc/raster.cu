@@ -41,23 +41,6 @@
 
 namespace {
 
-// A cone (axis, cos, sin, widest ramp half-width) may hold a fragment of the
-// staged triangle (cap a, b; edge normals n1..n3): the cap test, and unless
-// counting algorithmic tests (defined by the cap alone) the edge planes.
-// Every pixel G of the cone is within alpha of the axis c, so
-// G.n <= c.n + sin(alpha) + (1 - cos(alpha)) for a unit normal n; a triangle
-// with some edge plane below -h there has no fragment.
-__device__ __forceinline__ bool cone_may_hit(const float4& a, const float4& b, const float4& n1, const float4& n2,
-                                             const float4& n3, const float4& c0, const float4& c1, bool count_alg)
-{
-    bool keep = cap_hits_cone(make_float3(a.x, a.y, a.z), 1.0f - 0.5f * b.y, b.x, make_float3(c0.x, c0.y, c0.z),
-                              c0.w, c1.x, c1.y);
-    const float lim = -(c1.y + c1.x + (1.0f - c0.w) + 1e-6f);
-    return keep && (count_alg || (fmaf(c0.x, n1.x, fmaf(c0.y, n1.y, c0.z * n1.z)) > lim &&
-                                  fmaf(c0.x, n2.x, fmaf(c0.y, n2.y, c0.z * n2.z)) > lim &&
-                                  fmaf(c0.x, n3.x, fmaf(c0.y, n3.y, c0.z * n3.z)) > lim));
-}
-
 // One lane's two pixels as the evaluation sees them.
 struct PixPair {
     float2 dgx, dgy, dgz;  // G - a (tile axis) of both pixels; 0 at an invalid pixel

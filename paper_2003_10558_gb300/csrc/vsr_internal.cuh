@@ -425,10 +425,6 @@ int raster_threads_per_cta();
 // the same with the camera in device memory (12 floats: O xyz, M 3x3 row-major)
 vsr_status launch_setup_view(const float* tris, int T, const float* cam_dev, float4* rec, const TriGrid* grid,
                               cudaStream_t st);
-// exclusive scan of counts for large n (multi-CTA); `partials` needs
-// 2 * ceil(n / 4096) + 2 words
-vsr_status launch_scan_large(const uint32_t* counts, int n, uint32_t* partials, uint32_t* offsets, cudaStream_t st);
-
 vsr_status launch_raster(const float4* map, int W, int H, const Cone* tiles, const float4* rec, int T,
                          const uint32_t* offsets, const uint32_t* ids, uint32_t cap, uint32_t* id, float* depth,
                          float* cov, unsigned long long* n_alg, unsigned long long* n_exec, int32_t* n_inside,
@@ -446,26 +442,28 @@ enum {
     GF_D = 5,    // d/d (A'.N-hat), 0, 0, 0
     GF_COUNT = 6
 };
+constexpr int FRAG_LIST = 128;  // triangles of a tile whose fragment bits the count pass keeps
 struct FragArgs {
     const float4* map;
-    int W, H;
+    int W, H, tiles_x;
     const Cone* tiles;
+    const float4* geom;
     const float4* rec;
     int T;
-    const uint32_t* offsets;  // tile bins
-    const uint32_t* ids;
-    uint32_t cap;
-    const float* colors;      // per triangle, NULL = 1
-    uint32_t* counts;         // W*H fragments per pixel (count pass)
-    const uint32_t* foff;     // W*H + 1 exclusive scan of counts
-    float4* frags;            // fragment records (r, t, m^f, shade)
+    WalkIndex wi;
+    const float* colors;  // per triangle, NULL = 1
+    uint32_t* cursor;     // fragments given out (zero before the count, cleared by the fill)
+    uint32_t* tile_n;     // per tile: its triangles, or ~0 (more than FRAG_LIST)
+    uint32_t* tile_ids;   // per tile: FRAG_LIST of them
+    uint2* span;          // per pixel: (first fragment, fragments)
+    uint4* bits;          // per pixel: a bit per triangle of the tile's list that is a fragment
+    float4* frags;        // fragment records (r, t, m^f, shade)
     uint32_t fcap;
     float* image;
     float* cov;
     uint32_t* out_id;
     float* out_depth;
     int* status;
-    const uint32_t* ends = nullptr;  // as RasterView::ends
 };
 vsr_status launch_frag_count(const FragArgs& a, cudaStream_t st);
 vsr_status launch_frag_fill(const FragArgs& a, cudaStream_t st);
