@@ -44,7 +44,7 @@ void frags_release_pixels(vsr_frags f)
     f->npix = f->ntiles = 0;
 }
 
-vsr_status frags_ensure_pixels(vsr_frags f, int W, int H, size_t ntiles)
+vsr_status frags_ensure_pixels(vsr_frags f, int W, int H, size_t ntiles, cudaStream_t st)
 {
     const size_t n = (size_t)W * H;
     vsr_status s;
@@ -53,9 +53,13 @@ vsr_status frags_ensure_pixels(vsr_frags f, int W, int H, size_t ntiles)
     frags_release_pixels(f);
     if ((s = dalloc(&f->span, n)) != VSR_OK || (s = dalloc(&f->bits, n)) != VSR_OK ||
         (s = dalloc(&f->tile_n, ntiles)) != VSR_OK || (s = dalloc(&f->tile_ids, ntiles * FRAG_LIST)) != VSR_OK ||
-        (s = dalloc(&f->dmap, n)) != VSR_OK || (s = dalloc(&f->lens_part, 4 * ntiles)) != VSR_OK) {
+        (s = dalloc(&f->dmap, n)) != VSR_OK || (s = dalloc(&f->lens_part, map_backward_partials(ntiles))) != VSR_OK) {
         frags_release_pixels(f);
         return s;
+    }
+    if (cudaMemsetAsync(f->lens_part, 0, sizeof(float), st) != cudaSuccess) {
+        frags_release_pixels(f);
+        return VSR_ERR_CUDA;
     }
     f->npix = n;
     f->ntiles = ntiles;
@@ -126,7 +130,7 @@ vsr_status vsr_raster_shaded(vsr_map m, vsr_scene sc, const float* colors_dev, v
     // the first frame of a shape also sizes the stored bins (see raster_frame)
     if ((s = scene_walk_begin(m, sc, st)) != VSR_OK) return s;
     const int W = m->p.W, H = m->p.H;
-    if ((s = frags_ensure_pixels(f, W, H, (size_t)m->tx * m->ty)) != VSR_OK) return s;
+    if ((s = frags_ensure_pixels(f, W, H, (size_t)m->tx * m->ty, st)) != VSR_OK) return s;
     FragArgs a = frag_args(m, sc, colors_dev, f);
     a.out_id = id_dev;
     a.out_depth = depth_dev;

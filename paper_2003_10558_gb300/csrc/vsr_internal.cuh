@@ -471,7 +471,9 @@ vsr_status launch_frag_backward(const FragArgs& a, const uint32_t* id, const flo
                                 const float* ddepth, float4* grad, float4* dmap, cudaStream_t st);
 vsr_status launch_setup_backward(const float* tris, int T, const float cam[12], const float4* rec, const float4* grad,
                                  float* dtris, float* dcolors, cudaStream_t st);
-size_t map_backward_partials(int W, int H);
+// size of launch_map_backward's workspace in floats, the first of which is a
+// counter, zero between launches
+size_t map_backward_partials(size_t ntiles);
 vsr_status launch_map_backward(int W, int H, int aov, float k, float l, float s, float omega_deg,
                                const float4* dmap, float* partials, double* dlens, cudaStream_t st);
 
