@@ -193,6 +193,8 @@ __device__ __forceinline__ void frag_walk(const FragArgs& v, const Cone& tc, Fra
 
 __global__ void __launch_bounds__(RT, 6) frag_count_kernel(FragArgs v)
 {
+    grid_wait();
+    grid_go();
     __shared__ FragShared s;
     __shared__ uint32_t s_sum[RT / 32], s_base;
     const unsigned FULL = 0xffffffffu;
@@ -265,6 +267,8 @@ constexpr uint32_t FRAG_SORT = 8;
 
 __global__ void __launch_bounds__(RT, 5) frag_fill_kernel(FragArgs v)
 {
+    grid_wait();
+    grid_go();
     __shared__ union {
         FragShared walk;
         struct {
@@ -445,6 +449,8 @@ __device__ __forceinline__ float dot3f(float ax, float ay, float az, const float
 
 __global__ void __launch_bounds__(TILE_PIX) frag_backward_kernel(BackView v)
 {
+    grid_wait();
+    grid_go();
     const int i = blockIdx.x * TILE + (threadIdx.x % TILE);
     const int j = blockIdx.y * TILE + (threadIdx.x / TILE);
     if (i >= v.W || j >= v.H) return;
@@ -586,15 +592,24 @@ struct CamF {
 
 __global__ void __launch_bounds__(128) setup_backward_kernel(const float* __restrict__ tris, int T, CamF cam,
                                                               const float4* __restrict__ rec,
-                                                              const float4* __restrict__ grad,
+                                                              float4* __restrict__ grad,
                                                               float* __restrict__ dtris, float* __restrict__ dcolors)
 {
+    grid_wait();
+    grid_go();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= T) return;
     const size_t TT = (size_t)T;
     const float4 cp2 = rec[rec_at(TT, t, RF_CAP2)];
     float* out = dtris ? dtris + (size_t)t * 9 : nullptr;
-    const float4 gpl = grad[GF_PL * TT + t];
+    // the record's gradient, cleared for the next backward
+    float4 gr[GF_COUNT];
+#pragma unroll
+    for (int q = 0; q < GF_COUNT; ++q) {
+        gr[q] = grad[q * TT + t];
+        grad[q * TT + t] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
+    const float4 gpl = gr[GF_PL];
     if (dcolors) dcolors[t] = cp2.w != 0.0f ? gpl.w : 0.0f;
     if (!out) return;
     if (cp2.w == 0.0f) {  // culled at set-up: no fragments, no gradient
@@ -622,13 +637,13 @@ __global__ void __launch_bounds__(128) setup_backward_kernel(const float* __rest
         const int P = e, Q = e == 2 ? 0 : e + 1;
         const F3 x = cross(V[P], V[Q]);
         const float len = sqrtf(dot(x, x));
-        const F3 dn = xyz(grad[(GF_N1 + e) * TT + t]);
+        const F3 dn = xyz(gr[GF_N1 + e]);
         const F3 dx = sigma * unit_back((1.0f / len) * x, len, dn);
         dV[P] = dV[P] + cross(V[Q], dx);
         dV[Q] = dV[Q] + cross(dx, V[P]);
     }
     // miter
-    const float4 gcap = grad[GF_CAP * TT + t];
+    const float4 gcap = gr[GF_CAP];
     if (gcap.x != 0.0f || gcap.y != 0.0f || gcap.z != 0.0f || gcap.w != 0.0f) {
         F3 U[3];
         float Ul[3];
@@ -678,7 +693,7 @@ __global__ void __launch_bounds__(128) setup_backward_kernel(const float* __rest
         for (int q = 0; q < 3; ++q) dV[q] = dV[q] + unit_back(U[q], Ul[q], dU[q]);
     }
     // plane: shade uses N-hat, depth r = d'/(G.N-hat) with d' = A'.N-hat
-    const float dd = grad[GF_D * TT + t].x;
+    const float dd = gr[GF_D].x;
     const F3 e1 = V[0] - V[1], e2 = V[2] - V[1];
     const F3 N = cross(e1, e2);
     const float nl = sqrtf(dot(N, N));
@@ -703,15 +718,13 @@ __global__ void __launch_bounds__(128) setup_backward_kernel(const float* __rest
 
 vsr_status launch_frag_count(const FragArgs& a, cudaStream_t st)
 {
-    frag_count_kernel<<<a.tiles_x * ((a.H + TILE - 1) / TILE), RT, 0, st>>>(a);
-    VSR_CUDA_TRY(cudaGetLastError());
+    VSR_CUDA_TRY(launch_next(frag_count_kernel, a.tiles_x * ((a.H + TILE - 1) / TILE), RT, st, a));
     return VSR_OK;
 }
 
 vsr_status launch_frag_fill(const FragArgs& a, cudaStream_t st)
 {
-    frag_fill_kernel<<<a.tiles_x * ((a.H + TILE - 1) / TILE), RT, 0, st>>>(a);
-    VSR_CUDA_TRY(cudaGetLastError());
+    VSR_CUDA_TRY(launch_next(frag_fill_kernel, a.tiles_x * ((a.H + TILE - 1) / TILE), RT, st, a));
     return VSR_OK;
 }
 
@@ -720,19 +733,17 @@ vsr_status launch_frag_backward(const FragArgs& a, const uint32_t* id, const flo
 {
     BackView v{a.map, a.W, a.H, a.rec, a.T, a.colors, a.span, a.frags, id, dimage, dcov, ddepth, grad, dmap};
     dim3 grid((a.W + TILE - 1) / TILE, (a.H + TILE - 1) / TILE);
-    frag_backward_kernel<<<grid, TILE_PIX, 0, st>>>(v);
-    VSR_CUDA_TRY(cudaGetLastError());
+    VSR_CUDA_TRY(launch_next(frag_backward_kernel, grid, TILE_PIX, st, v));
     return VSR_OK;
 }
 
-vsr_status launch_setup_backward(const float* tris, int T, const float cam[12], const float4* rec, const float4* grad,
+vsr_status launch_setup_backward(const float* tris, int T, const float cam[12], const float4* rec, float4* grad,
                                  float* dtris, float* dcolors, cudaStream_t st)
 {
     if (T == 0) return VSR_OK;
     CamF c;
     for (int q = 0; q < 3; ++q) c.O[q] = cam[q];
     for (int q = 0; q < 9; ++q) c.M[q] = cam[3 + q];
-    setup_backward_kernel<<<(T + 127) / 128, 128, 0, st>>>(tris, T, c, rec, grad, dtris, dcolors);
-    VSR_CUDA_TRY(cudaGetLastError());
+    VSR_CUDA_TRY(launch_next(setup_backward_kernel, (T + 127) / 128, 128, st, tris, T, c, rec, grad, dtris, dcolors));
     return VSR_OK;
 }

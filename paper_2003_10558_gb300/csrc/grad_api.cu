@@ -20,6 +20,7 @@ struct vsr_frags_s {
     float* lens_part = nullptr;
     float4* grad = nullptr;       // GF_COUNT x grad_T
     int64_t grad_T = 0;
+    bool grad_clean = false;      // grad is all zero
     // the forward the lists belong to
     uint64_t map_gen = 0, scene_gen = 0;
     int W = 0, H = 0;
@@ -183,8 +184,12 @@ vsr_status vsr_raster_backward(vsr_map m, vsr_scene sc, const float* tris_dev, c
         f->grad_T = 0;
         if ((s = dalloc(&f->grad, (size_t)GF_COUNT * (size_t)T)) != VSR_OK) return s;
         f->grad_T = T;
+        f->grad_clean = false;
     }
-    if (T > 0) VSR_CUDA_TRY(cudaMemsetAsync(f->grad, 0, sizeof(float4) * GF_COUNT * (size_t)T, st));
+    // the set-up adjoint leaves the record gradients cleared
+    if (f->grad_T > 0 && !f->grad_clean)
+        VSR_CUDA_TRY(cudaMemsetAsync(f->grad, 0, sizeof(float4) * GF_COUNT * (size_t)f->grad_T, st));
+    f->grad_clean = false;
     FragArgs a = frag_args(m, sc, colors_dev, f);
     if ((s = launch_frag_backward(a, id_dev, dimage_dev, dcov_dev, ddepth_dev, f->grad, f->dmap, st)) != VSR_OK)
         return s;
@@ -192,6 +197,7 @@ vsr_status vsr_raster_backward(vsr_map m, vsr_scene sc, const float* tris_dev, c
         if ((s = launch_setup_backward(tris_dev, (int)T, sc->cam, sc->rec, f->grad, dtris_dev, dcolors_dev, st)) !=
             VSR_OK)
             return s;
+        f->grad_clean = true;
     }
     if (dlens_dev) {
         if ((s = launch_map_backward(m->p.W, m->p.H, m->p.aov, m->p.k, m->p.l, m->p.s, m->p.omega_deg, f->dmap,

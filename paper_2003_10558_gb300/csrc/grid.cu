@@ -21,6 +21,8 @@ constexpr int ROW_THREADS = 128;
 constexpr int ROW_CELLS = (2 * grid_nlat(0) + ROW_THREADS - 1) / ROW_THREADS;  // cells per thread
 __global__ void __launch_bounds__(ROW_THREADS) grid_rows_kernel(TriGrid g)
 {
+    grid_wait();
+    grid_go();
     __shared__ uint32_t s_sum[ROW_THREADS / 32], s_base;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int l = 0, row = blockIdx.x;
@@ -73,6 +75,8 @@ __global__ void __launch_bounds__(ROW_THREADS) grid_rows_kernel(TriGrid g)
 // triangles crowd a few cells does not queue on their counters.
 __global__ void __launch_bounds__(256) grid_file_kernel(const float4* __restrict__ rec, int T, TriGrid g)
 {
+    grid_wait();
+    grid_go();
     const unsigned FULL = 0xffffffffu;
     const int t = blockIdx.x * 256 + threadIdx.x, lane = threadIdx.x & 31;
     if (t == 0) {
@@ -107,6 +111,8 @@ __global__ void __launch_bounds__(WALK_THREADS) bin_walk_kernel(const float4* __
                                                                uint32_t* __restrict__ ids, uint32_t cap, int* status,
                                                                uint32_t* total_host)
 {
+    grid_wait();
+    grid_go();
     __shared__ WalkShared ws;
     __shared__ uint32_t s_ids[WALK_BLOCK];
     __shared__ uint32_t s_n, s_start;
@@ -226,10 +232,8 @@ vsr_status launch_grid_file(const float4* rec, int T, const TriGrid& g, cudaStre
 {
     if (T <= 0) return VSR_OK;
     if ((int64_t)T > g.T || !g.counts) return VSR_ERR_INVALID_ARG;
-    grid_rows_kernel<<<GRID_ROWS + 1, ROW_THREADS, 0, st>>>(g);
-    VSR_CUDA_TRY(cudaGetLastError());
-    grid_file_kernel<<<(T + 255) / 256, 256, 0, st>>>(rec, T, g);
-    VSR_CUDA_TRY(cudaGetLastError());
+    VSR_CUDA_TRY(launch_next(grid_rows_kernel, GRID_ROWS + 1, ROW_THREADS, st, g));
+    VSR_CUDA_TRY(launch_next(grid_file_kernel, (T + 255) / 256, 256, st, rec, T, g));
     return VSR_OK;
 }
 
@@ -238,8 +242,7 @@ vsr_status launch_bin_walk(const float4* rec, int T, const WalkIndex& wi, const 
                            int* status, uint32_t* total_host, cudaStream_t st)
 {
     if (T < 0 || ntiles <= 0 || (!wi.direct && !wi.start)) return VSR_ERR_INVALID_ARG;
-    bin_walk_kernel<<<ntiles, WALK_THREADS, 0, st>>>(rec, T, wi, geom, tiles, ntiles, ctr, starts, ends, ids, cap,
-                                                     status, total_host);
-    VSR_CUDA_TRY(cudaGetLastError());
+    VSR_CUDA_TRY(launch_next(bin_walk_kernel, ntiles, WALK_THREADS, st, rec, T, wi, geom, tiles, ntiles, ctr, starts, ends,
+                             ids, cap, status, total_host));
     return VSR_OK;
 }

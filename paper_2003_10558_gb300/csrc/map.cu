@@ -300,7 +300,9 @@ __global__ void __launch_bounds__(map_threads(P), map_ctas(P)) map_kernel(int W,
                                                                          float4* __restrict__ deriv, int tiles_x,
                                                                          int tiles_y, bool mx, bool my)
 {
+    grid_go();
     // map values of the tile and its halo: direction xyz, w = F's return value
+    // (they depend on the arguments alone: evaluated before the wait)
     __shared__ float4 sv[HW * HW];
     const int tx = blockIdx.x, ty = blockIdx.y;
     const int i0 = tx * TILE - 1, j0 = ty * TILE - 1;
@@ -310,6 +312,7 @@ __global__ void __launch_bounds__(map_threads(P), map_ctas(P)) map_kernel(int W,
         const int ok = fn(i0 + qi, j0 + qj, W, H, v);
         sv[q] = make_float4(v.x, v.y, v.z, (float)ok);
     }
+    grid_wait();  // whoever reads the old map is done
     __syncthreads();
     constexpr int NT = TILE_PIX / P;
     if (threadIdx.x >= NT) return;  // halo-only threads: done
@@ -488,13 +491,12 @@ vsr_status launch_map(int W, int H, int aov, float k, float l, float s, float om
     const int tx = (W + TILE - 1) / TILE, ty = (H + TILE - 1) / TILE;
     const bool mx = W % TILE == 0, my = H % TILE == 0;
     if (mx || my)
-        map_kernel<UniversalFn, VSR_MAP_PPT, true>
-            <<<dim3(mx ? (tx + 1) / 2 : tx, my ? (ty + 1) / 2 : ty), map_threads(VSR_MAP_PPT), 0, st>>>(
-                W, H, UniversalFn{p}, map, tiles, geom, nullptr, tx, ty, mx, my);
+        VSR_CUDA_TRY(launch_next(map_kernel<UniversalFn, VSR_MAP_PPT, true>,
+                                 dim3(mx ? (tx + 1) / 2 : tx, my ? (ty + 1) / 2 : ty), map_threads(VSR_MAP_PPT), st, W,
+                                 H, UniversalFn{p}, map, tiles, geom, (float4*)nullptr, tx, ty, mx, my));
     else
-        map_kernel<UniversalFn, VSR_MAP_PPT, false><<<dim3(tx, ty), map_threads(VSR_MAP_PPT), 0, st>>>(
-            W, H, UniversalFn{p}, map, tiles, geom, nullptr, tx, ty, false, false);
-    VSR_CUDA_TRY(cudaGetLastError());
+        VSR_CUDA_TRY(launch_next(map_kernel<UniversalFn, VSR_MAP_PPT, false>, dim3(tx, ty), map_threads(VSR_MAP_PPT),
+                                 st, W, H, UniversalFn{p}, map, tiles, geom, (float4*)nullptr, tx, ty, false, false));
     return VSR_OK;
 }
 
@@ -517,9 +519,8 @@ vsr_status launch_map_spec(const vsr_map_spec& sp, float4* map, Cone* tiles, flo
         f.a[3] = sp.param[2];
     }
     dim3 grid((sp.W + TILE - 1) / TILE, (sp.H + TILE - 1) / TILE);
-    map_kernel<SpecFn, VSR_MAP_PPT, false><<<grid, map_threads(VSR_MAP_PPT), 0, st>>>(
-        sp.W, sp.H, f, map, tiles, geom, deriv, (int)grid.x, (int)grid.y, false, false);
-    VSR_CUDA_TRY(cudaGetLastError());
+    VSR_CUDA_TRY(launch_next(map_kernel<SpecFn, VSR_MAP_PPT, false>, grid, map_threads(VSR_MAP_PPT), st, sp.W, sp.H, f,
+                             map, tiles, geom, deriv, (int)grid.x, (int)grid.y, false, false));
     return VSR_OK;
 }
 
@@ -635,6 +636,7 @@ __global__ void __launch_bounds__(MAP_THREADS) map_backward_kernel(int W, int H,
     __shared__ float3 sd[4][HW * HW];
     __shared__ unsigned char sok[HW * HW];
     __shared__ float red[4][4][MAP_THREADS / 32];
+    grid_go();
     const int tx = blockIdx.x, ty = blockIdx.y;
     const int i0 = tx * TILE - 1, j0 = ty * TILE - 1;
     if (threadIdx.x < HW * HW) {
@@ -646,6 +648,7 @@ __global__ void __launch_bounds__(MAP_THREADS) map_backward_kernel(int W, int H,
 #pragma unroll
         for (int k = 0; k < 4; ++k) sd[k][q] = ok ? dv[k] : make_float3(0.0f, 0.0f, 0.0f);
     }
+    grid_wait();  // (the tangents depend on the arguments alone)
     __syncthreads();
     const int ux = mx && tiles_x - 1 - tx != tx ? tiles_x - 1 - tx : -1;
     const int uy = my && tiles_y - 1 - ty != ty ? tiles_y - 1 - ty : -1;
@@ -736,6 +739,8 @@ __global__ void __launch_bounds__(LENS_THREADS) lens_reduce_kernel(const float4*
                                                                    double* __restrict__ sums, uint32_t* done,
                                                                    double* __restrict__ dlens)
 {
+    grid_wait();
+    grid_go();
     __shared__ double red[4][LENS_THREADS / 32];
     __shared__ bool s_last;
     double a[4] = {0.0, 0.0, 0.0, 0.0};
@@ -787,11 +792,9 @@ vsr_status launch_map_backward(int W, int H, int aov, float k, float l, float s,
     const int tx = (W + TILE - 1) / TILE, ty = (H + TILE - 1) / TILE;
     const bool mx = W % TILE == 0, my = H % TILE == 0;
     float* tile_sums = partials + LENS_HEAD;
-    map_backward_kernel<<<dim3(mx ? (tx + 1) / 2 : tx, my ? (ty + 1) / 2 : ty), MAP_THREADS, 0, st>>>(
-        W, H, tp, dmap, tile_sums, tx, ty, mx, my);
-    VSR_CUDA_TRY(cudaGetLastError());
-    lens_reduce_kernel<<<LENS_CTAS, LENS_THREADS, 0, st>>>((const float4*)tile_sums, tx * ty, (double*)(partials + 4),
-                                                           (uint32_t*)partials, dlens);
-    VSR_CUDA_TRY(cudaGetLastError());
+    VSR_CUDA_TRY(launch_next(map_backward_kernel, dim3(mx ? (tx + 1) / 2 : tx, my ? (ty + 1) / 2 : ty), MAP_THREADS, st, W,
+                             H, tp, dmap, tile_sums, tx, ty, mx, my));
+    VSR_CUDA_TRY(launch_next(lens_reduce_kernel, LENS_CTAS, LENS_THREADS, st, (const float4*)tile_sums, tx * ty,
+                             (double*)(partials + 4), (uint32_t*)partials, dlens));
     return VSR_OK;
 }

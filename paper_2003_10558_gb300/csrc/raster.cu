@@ -327,6 +327,8 @@ __global__ void __launch_bounds__(RT, VSR_RASTER_CTAS_PER_SM) raster_items_kerne
                                                               const uint32_t* __restrict__ n_extra, int split_max,
                                                               SplitAcc split, int* __restrict__ status)
 {
+    grid_wait();
+    grid_go();
     __shared__ Stage st;
     uint32_t u, k = 0;
     if (blockIdx.x < n_tiles) {
@@ -454,6 +456,8 @@ __global__ void items_kernel(const uint32_t* __restrict__ offsets, const uint32_
                              int32_t* __restrict__ split_slot, uint32_t* __restrict__ counters /* n_split, n_extra */,
                              uint32_t split_cap, uint2* __restrict__ extra, uint32_t extra_cap)
 {
+    grid_wait();
+    grid_go();
     const uint32_t u = blockIdx.x * blockDim.x + threadIdx.x;
     if (u >= n_tiles) return;
     const uint32_t c = (ends ? ends[u] : offsets[u + 1]) - offsets[u];
@@ -506,10 +510,9 @@ vsr_status launch_raster_assign(const uint32_t* offsets, uint32_t n_tiles, uint3
 {
     if (n_tiles == 0) return VSR_OK;
     VSR_CUDA_TRY(cudaMemsetAsync(w.counters, 0, 2 * sizeof(uint32_t), st));
-    items_kernel<<<(n_tiles + 255) / 256, 256, 0, st>>>(offsets, ends, n_tiles, raster_split_items(split_max),
-                                                        w.nsplit_of, w.split_slot, w.counters, w.split_cap, w.extra,
-                                                        raster_extra_cap(cap, w, split_max));
-    VSR_CUDA_TRY(cudaGetLastError());
+    VSR_CUDA_TRY(launch_next(items_kernel, (n_tiles + 255) / 256, 256, st, offsets, ends, n_tiles,
+                             raster_split_items(split_max), w.nsplit_of, w.split_slot, w.counters, w.split_cap, w.extra,
+                             raster_extra_cap(cap, w, split_max)));
     return VSR_OK;
 }
 
@@ -535,9 +538,8 @@ vsr_status launch_raster_items(const RasterView& view, const uint32_t* offsets, 
     const uint32_t extra_cap = raster_extra_cap(cap, w, split_max);
     split_max = raster_split_items(split_max);
     auto kern = host_out ? raster_items_kernel<true> : raster_items_kernel<false>;
-    kern<<<n_tiles + extra_cap, RT, 0, st>>>(view, n_tiles, w.nsplit_of, w.split_slot, w.extra, w.counters + 1,
-                                             split_max, SplitAcc{w.acc, w.key, w.done}, status);
-    VSR_CUDA_TRY(cudaGetLastError());
+    VSR_CUDA_TRY(launch_next(kern, n_tiles + extra_cap, RT, st, view, n_tiles, w.nsplit_of, w.split_slot, w.extra,
+                             w.counters + 1, split_max, SplitAcc{w.acc, w.key, w.done}, status));
     return VSR_OK;
 }
 

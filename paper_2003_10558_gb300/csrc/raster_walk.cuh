@@ -77,6 +77,8 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
                                                                      uint32_t* __restrict__ tile_pairs,
                                                                      int* __restrict__ status)
 {
+    grid_wait();
+    grid_go();
     __shared__ Stage st;
     __shared__ WalkShared ws;
     __shared__ typename Step::Cones wc;
@@ -255,9 +257,8 @@ inline vsr_status launch_walk(const RasterView& view, const typename Step::In& i
     const int split = few ? 2 : (int)WALK_SPLIT_BLOCKS;
     const int helpers = view.T > split * block ? wave : 0;
     auto kern = host_out ? raster_walk_kernel<Step, true> : raster_walk_kernel<Step, false>;
-    kern<<<ntiles + helpers, RT, 0, st>>>(view, in, wi, geom, ntiles, (uint32_t)block, (uint32_t)split, few ? 40 : 0,
-                                          sl, tile_pairs, status);
-    VSR_CUDA_TRY(cudaGetLastError());
+    VSR_CUDA_TRY(launch_next(kern, ntiles + helpers, RT, st, view, in, wi, geom, ntiles, (uint32_t)block,
+                             (uint32_t)split, few ? 40 : 0, sl, tile_pairs, status));
     return VSR_OK;
 }
 

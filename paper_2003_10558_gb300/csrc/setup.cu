@@ -114,6 +114,8 @@ __global__ void __launch_bounds__(128, CAM == CAM_ROTATED ? 2 : 3) setup_pair_ke
                                                                                    float4* __restrict__ rec,
                                                                                    TriGrid grid)
 {
+    grid_wait();
+    grid_go();
     const int t0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     const unsigned am = __ballot_sync(0xffffffffu, t0 < T);  // the lanes that go on
     if (t0 >= T) return;
@@ -261,8 +263,8 @@ vsr_status launch_setup(const float* tris, int T, const float cam[12], float4* r
     for (int q = 0; q < 9; ++q) c.M[q] = cam[3 + q];
     const int pairs = (T + 1) / 2;
     auto kern = identity(c) ? setup_pair_kernel<CAM_IDENT> : setup_pair_kernel<CAM_ROTATED>;
-    kern<<<(pairs + 127) / 128, 128, 0, st>>>(tris, T, c, nullptr, rec, grid ? *grid : TriGrid{});
-    VSR_CUDA_TRY(cudaGetLastError());
+    VSR_CUDA_TRY(launch_next(kern, (pairs + 127) / 128, 128, st, tris, T, c, (const float*)nullptr, rec,
+                             grid ? *grid : TriGrid{}));
     return VSR_OK;
 }
 
@@ -271,8 +273,7 @@ vsr_status launch_setup_view(const float* tris, int T, const float* cam_dev, flo
 {
     if (T == 0) return VSR_OK;
     const int pairs = (T + 1) / 2;
-    setup_pair_kernel<CAM_DEVICE><<<(pairs + 127) / 128, 128, 0, st>>>(tris, T, Cam{}, cam_dev, rec,
-                                                                      grid ? *grid : TriGrid{});
-    VSR_CUDA_TRY(cudaGetLastError());
+    VSR_CUDA_TRY(launch_next(setup_pair_kernel<CAM_DEVICE>, (pairs + 127) / 128, 128, st, tris, T, Cam{}, cam_dev, rec,
+                             grid ? *grid : TriGrid{}));
     return VSR_OK;
 }

@@ -136,6 +136,30 @@ __device__ __forceinline__ bool cap_hits_cone(float3 S, float cos_rho, float sin
         if (_e != cudaSuccess) return VSR_ERR_CUDA;                                                                     \
     } while (0)
 
+// Launches one after another on a stream hand over without draining the GPU
+// in between (programmatic dependent launch): a kernel launched with
+// launch_next may have its CTAs placed while its predecessor's last ones still
+// run, and does nothing before grid_wait has seen the predecessor's end and
+// memory; grid_go in the predecessor allows it.  grid_wait comes first in
+// every such kernel, so nothing but the launch itself overlaps, whatever the
+// predecessor is.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <class... P, class... A>
+inline cudaError_t launch_next(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Kernel launchers (defined in the .cu files, called by the host library).
 // The map kernels write the map, the tile cones and their geometry.
 vsr_status launch_map(int W, int H, int aov, float k, float l, float s, float omega_deg, float4* map, Cone* tiles,
@@ -469,7 +493,8 @@ vsr_status launch_frag_count(const FragArgs& a, cudaStream_t st);
 vsr_status launch_frag_fill(const FragArgs& a, cudaStream_t st);
 vsr_status launch_frag_backward(const FragArgs& a, const uint32_t* id, const float* dimage, const float* dcov,
                                 const float* ddepth, float4* grad, float4* dmap, cudaStream_t st);
-vsr_status launch_setup_backward(const float* tris, int T, const float cam[12], const float4* rec, const float4* grad,
+// (clears the record gradients it reads)
+vsr_status launch_setup_backward(const float* tris, int T, const float cam[12], const float4* rec, float4* grad,
                                  float* dtris, float* dcolors, cudaStream_t st);
 // size of launch_map_backward's workspace in floats, the first of which is a
 // counter, zero between launches
