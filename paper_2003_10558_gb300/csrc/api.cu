@@ -221,12 +221,12 @@ vsr_status ensure_ws(vsr_scene sc, int ntiles, cudaStream_t st)
     cudaFree(sc->offsets);
     sc->offsets = sc->ends = sc->tile_pairs = sc->bin_ctr = nullptr;
     sc->ws_tiles = 0;
-    vsr_status s = dalloc(&sc->offsets, 3 * n + 3);
+    vsr_status s = dalloc(&sc->offsets, 3 * n + 1 + BIN_CTR_WORDS);
     if (s != VSR_OK) return s;
     sc->ends = sc->offsets + n + 1;
     sc->tile_pairs = sc->ends + n;
     sc->bin_ctr = sc->tile_pairs + n;
-    VSR_CUDA_TRY(cudaMemsetAsync(sc->bin_ctr, 0, 2 * sizeof(uint32_t), st));
+    VSR_CUDA_TRY(cudaMemsetAsync(sc->bin_ctr, 0, BIN_CTR_WORDS * sizeof(uint32_t), st));
     sc->ws_tiles = ntiles;
     sc->sized_shape = 0;
     // (the bins' places went with the old arrays)
@@ -584,12 +584,12 @@ static vsr_status bin_scene(vsr_map m, vsr_scene sc, int pstep, cudaStream_t st)
     // binning sizes the bins, which reads this total
     const bool record = resize || !sc->total_pending;
     const WalkIndex wi = walk_index(sc->grid, sc->T, pstep);
-    auto walk = [&](int* status, uint32_t* total_host) {
+    auto walk = [&](bool sizing, uint32_t* total_host) {
         return launch_bin_walk(sc->rec, T, wi, m->idx.geom, m->tiles, ntiles, sc->bin_ctr, sc->offsets, sc->ends,
-                               sc->ids, sc->cap, status, total_host, st);
+                               sc->ids, sc->cap, sizing, scene_status(sc), total_host, st);
     };
     // (a sizing pass reports no overflow: its bins are grown and binned again)
-    if ((s = walk(resize ? nullptr : scene_status(sc), record ? sc->h_total_dev : nullptr)) != VSR_OK) return s;
+    if ((s = walk(resize, record ? sc->h_total_dev : nullptr)) != VSR_OK) return s;
     if (record) {
         VSR_CUDA_TRY(cudaEventRecord(sc->total_event, st));
         sc->total_pending = true;
@@ -604,7 +604,7 @@ static vsr_status bin_scene(vsr_map m, vsr_scene sc, int pstep, cudaStream_t st)
             uint64_t want = (uint64_t)total + total / 4 + 4096;
             if (want > 0xffffffffull) want = 0xffffffffull;
             if ((s = bins_realloc(sc, (uint32_t)want)) != VSR_OK) return s;
-            if ((s = walk(scene_status(sc), nullptr)) != VSR_OK) return s;
+            if ((s = walk(false, nullptr)) != VSR_OK) return s;
         }
         sc->sized_shape = bin_shape_of(m, sc);
         sc->sized_pstep = pstep != 0;
@@ -1034,7 +1034,7 @@ struct BatchView {
     TriGrid grid;
     WalkWork walk;  // split slots of the view's own raster launch
     // stored bins and work items of the pooled raster launches
-    uint32_t* ctr = nullptr;      // 2, zero between binnings
+    uint32_t* ctr = nullptr;      // BIN_CTR_WORDS, zero between binnings
     uint32_t* offsets = nullptr;  // tiles + 1
     uint32_t* ends = nullptr;     // tiles
     uint32_t* ids = nullptr;
@@ -1110,10 +1110,10 @@ vsr_status batch_view_alloc(BatchView& v, int64_t T, int tiles, bool pooled, cud
         raster_work_free(&v.work);
         v.offsets = v.ends = v.ctr = nullptr;
         v.tiles = 0;
-        if ((s = dalloc(&v.offsets, 2 * (size_t)tiles + 3)) != VSR_OK) return s;
+        if ((s = dalloc(&v.offsets, 2 * (size_t)tiles + 1 + BIN_CTR_WORDS)) != VSR_OK) return s;
         v.ends = v.offsets + tiles + 1;
         v.ctr = v.ends + tiles;
-        VSR_CUDA_TRY(cudaMemsetAsync(v.ctr, 0, 2 * sizeof(uint32_t), st));
+        VSR_CUDA_TRY(cudaMemsetAsync(v.ctr, 0, BIN_CTR_WORDS * sizeof(uint32_t), st));
         if ((s = raster_work_alloc(&v.work, (uint32_t)tiles, st)) != VSR_OK) return s;
         v.tiles = tiles;
     }
@@ -1135,14 +1135,14 @@ vsr_status batch_view_raster(vsr_batch b, int v, vsr_map m, int64_t T, uint32_t*
     return launch_raster_walk(rv, walk_index(bv.grid, T), m->idx.geom, bv.walk, nullptr, status_word(), st);
 }
 
-// the stored bins of view v, for a pooled launch (or, without a status, to
-// size them); the total to its pinned word
-vsr_status batch_view_bin(vsr_batch b, int v, vsr_map m, int64_t T, int* status, cudaStream_t st)
+// the stored bins of view v, for a pooled launch (or to size
+// them); the total to its pinned word
+vsr_status batch_view_bin(vsr_batch b, int v, vsr_map m, int64_t T, bool sizing, cudaStream_t st)
 {
     BatchView& bv = b->views[v];
     const int tiles = m->tx * m->ty;
     vsr_status s = launch_bin_walk(bv.rec, (int)T, walk_index(bv.grid, T), m->idx.geom, m->tiles, tiles, bv.ctr,
-                                   bv.offsets, bv.ends, bv.ids, bv.cap, status, nullptr, st);
+                                   bv.offsets, bv.ends, bv.ids, bv.cap, sizing, status_word(), nullptr, st);
     if (s != VSR_OK) return s;
     VSR_CUDA_TRY(cudaMemcpyAsync(b->h_total + v, bv.offsets + tiles, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
     return VSR_OK;
@@ -1339,7 +1339,7 @@ vsr_status vsr_batch_render(vsr_batch b, int nviews, const vsr_map* maps, const 
     // one synchronisation
     for (int v = 0; v < nviews; ++v) {
         if ((s = batch_view_setup(b, v, tris_dev, T, st)) != VSR_OK) return s;
-        if (try_pool && (s = batch_view_bin(b, v, maps[v], T, nullptr, st)) != VSR_OK) return s;
+        if (try_pool && (s = batch_view_bin(b, v, maps[v], T, true, st)) != VSR_OK) return s;
         if ((s = batch_view_raster(b, v, maps[v], T, out_ptr(id_dev, v), out_ptr(depth_dev, v), out_ptr(cov_dev, v),
                                    st)) != VSR_OK)
             return s;
@@ -1401,7 +1401,7 @@ vsr_status vsr_batch_render(vsr_batch b, int nviews, const vsr_map* maps, const 
                                         out_ptr(cov_dev, v), vs);
             if (cst == VSR_OK && pooled) {
                 const BatchView& bv = b->views[v];
-                cst = batch_view_bin(b, v, maps[v], T, status_word(), vs);
+                cst = batch_view_bin(b, v, maps[v], T, false, vs);
                 if (cst == VSR_OK)
                     cst = launch_raster_assign(bv.offsets, (uint32_t)(maps[v]->tx * maps[v]->ty), bv.cap, bv.work,
                                                split, vs, bv.ends);

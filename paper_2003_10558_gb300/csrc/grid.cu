@@ -102,9 +102,57 @@ __global__ void __launch_bounds__(256) grid_file_kernel(const float4* __restrict
 // shared memory, the tile's range of the bins taken with one atomic.  More:
 // a pass that counts and a pass that writes.  The last CTA to finish stores
 // the total and clears the counters.
+//
+// The walk is a chain of loads, so a tile of many candidates (one at a rim
+// whose cone spans a good part of the sphere) would outlast all the others:
+// by itself a tile that tests 300k triangles took 2.1 ms, the rest of its view
+// 30 us; shared, the binning of that view takes 105 us, and a burst of 32
+// requests with two such views 3.7 ms instead of 4.3.  Tiles of more than `split` blocks are published in a BinShare,
+// and the CTAs past the tiles (helpers) take blocks from them: first one claim
+// per block that counts its hits, then, once every block is counted and the
+// range taken, one per block that writes them.  A CTA waits for the counting
+// only after it has claimed a block to write; every block to count was claimed
+// before that, by a CTA that is running and does not wait.
+constexpr int BIN_FEW = 12;  // CTAs of this kernel resident on an SM, about
+struct BinShare {
+    uint32_t tile, blocks;  // blocks: 0 until published
+    uint32_t claim;         // blocks claimed, for counting and then for writing
+    uint32_t done, n;       // blocks counted, hits found in them
+    uint32_t cursor;        // next place in the bins
+    uint32_t ready, pad;    // the range is taken
+};
+static_assert(sizeof(BinShare) == BIN_SHARE_WORDS * sizeof(uint32_t), "BIN_CTR_WORDS");
+
+struct BinBlock {
+    uint32_t n, claim, start;
+    int entry, ok;
+};
+
+// The hits of candidates [i0, i1), at most WALK_BLOCK, into s_ids (all
+// threads; the caller has cleared bb.n and waits for the CTA on both sides).
+__device__ __forceinline__ void bin_block(const Walk& w, const WalkIndex& wi, const float4* __restrict__ rec, int T,
+                                          const WalkShared& ws, uint32_t i0, uint32_t i1, uint32_t* s_ids,
+                                          BinBlock& bb)
+{
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    for (uint32_t i = i0; i < i1; i += WALK_THREADS) {
+        const uint32_t idx = i + threadIdx.x;
+        uint32_t t;
+        const bool hit = w.test(wi, rec, T, ws, idx, idx < i1, t);
+        const unsigned m = __ballot_sync(FULL, hit);
+        if (!m) continue;
+        uint32_t base = 0;
+        if (lane == 0) base = atomicAdd(&bb.n, (uint32_t)__popc(m));
+        base = __shfl_sync(FULL, base, 0);
+        if (hit) s_ids[base + (uint32_t)__popc(m & ((1u << lane) - 1u))] = t;
+    }
+}
+
 __global__ void __launch_bounds__(WALK_THREADS) bin_walk_kernel(const float4* __restrict__ rec, int T, WalkIndex wi,
                                                                const float4* __restrict__ geom,
                                                                const Cone* __restrict__ tiles, int ntiles,
+                                                               uint32_t split, int looks, bool sizing,
                                                                uint32_t* __restrict__ ctr,
                                                                uint32_t* __restrict__ starts,
                                                                uint32_t* __restrict__ ends,
@@ -115,69 +163,174 @@ __global__ void __launch_bounds__(WALK_THREADS) bin_walk_kernel(const float4* __
     grid_go();
     __shared__ WalkShared ws;
     __shared__ uint32_t s_ids[WALK_BLOCK];
-    __shared__ uint32_t s_n, s_start;
-    const unsigned FULL = 0xffffffffu;
-    const int tile = blockIdx.x, lane = threadIdx.x & 31;
-    const uint32_t lt = (1u << lane) - 1u;
-    const Cone c = tiles[tile];
-    if (threadIdx.x < 32) walk_ranges(wi, T, geom[tile], c.c0.y, ws);
-    if (threadIdx.x == 0) s_n = 0u;
-    __syncthreads();
-    const uint32_t E = ws.total;
-    const bool one_pass = E <= WALK_BLOCK;
-    Walk w;
-    w.init(wi, c, ws);
-    for (uint32_t i0 = 0; i0 < E; i0 += WALK_THREADS) {
-        const uint32_t idx = i0 + threadIdx.x;
-        uint32_t t;
-        const bool hit = w.test(wi, rec, T, ws, idx, idx < E, t);
-        const unsigned m = __ballot_sync(FULL, hit);
-        if (!m) continue;
-        uint32_t base = 0;
-        if (lane == 0) base = atomicAdd(&s_n, (uint32_t)__popc(m));
-        base = __shfl_sync(FULL, base, 0);
-        if (hit && one_pass) s_ids[base + (uint32_t)__popc(m & lt)] = t;
-    }
-    __syncthreads();
-    const uint32_t n = s_n;
-    if (threadIdx.x == 0) {
+    __shared__ BinBlock bb;
+    const bool helper = blockIdx.x >= (uint32_t)ntiles;
+    BinShare* shares = (BinShare*)(ctr + BIN_CTR_SHARES);
+    volatile uint32_t* published = ctr + 2;
+    // takes the range of a tile with n hits
+    auto take_range = [&](int tile, uint32_t n) {
         const uint32_t start = n ? atomicAdd(&ctr[0], n) : 0u;
-        if ((uint64_t)start + n > cap) raise_status(status, VSR_ERR_BIN_OVERFLOW);
+        if (!sizing && (uint64_t)start + n > cap) raise_status(status, VSR_ERR_BIN_OVERFLOW);
         starts[tile] = start;
         ends[tile] = start + n;
-        s_start = start;
-    }
-    __syncthreads();
-    const uint32_t start = s_start;
-    if (one_pass) {
-        for (uint32_t j = threadIdx.x; j < n; j += WALK_THREADS)
-            if (start + j < cap) ids[start + j] = s_ids[j];
-    } else {
-        if (threadIdx.x == 0) s_n = 0u;
-        __syncthreads();
-        for (uint32_t i0 = 0; i0 < E; i0 += WALK_THREADS) {
-            const uint32_t idx = i0 + threadIdx.x;
-            uint32_t t;
-            const bool hit = w.test(wi, rec, T, ws, idx, idx < E, t);
-            const unsigned m = __ballot_sync(FULL, hit);
-            if (!m) continue;
-            uint32_t base = 0;
-            if (lane == 0) base = atomicAdd(&s_n, (uint32_t)__popc(m));
-            base = start + __shfl_sync(FULL, base, 0) + (uint32_t)__popc(m & lt);
-            if (hit && base < cap) ids[base] = t;
+        return start;
+    };
+    for (;;) {
+        int tile = (int)blockIdx.x;
+        if (helper) {
+            // a published tile with blocks left, the first from a start of
+            // this CTA's own
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                for (; !*published && looks > 0; --looks) __nanosleep(250);
+                bb.claim = min(*published, (uint32_t)BIN_SHARES);
+                bb.entry = BIN_SHARES;
+            }
+            __syncthreads();
+            const int ne = (int)bb.claim, from = ne ? (int)((blockIdx.x * 37u) % (uint32_t)ne) : 0;
+            int mine = BIN_SHARES;
+            for (int i = threadIdx.x; i < ne && mine == BIN_SHARES; i += WALK_THREADS) {
+                volatile BinShare* e = &shares[(from + i) % ne];
+                if (e->claim < 2u * e->blocks) mine = i;
+            }
+            if (mine < BIN_SHARES) atomicMin(&bb.entry, mine);
+            __syncthreads();
+            const int found = bb.entry;
+            if (found == BIN_SHARES) break;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                bb.entry = (from + found) % ne;
+                __threadfence();
+                bb.claim = *(volatile uint32_t*)&shares[bb.entry].tile;
+            }
+            __syncthreads();
+            tile = (int)bb.claim;
         }
+        const Cone c = tiles[tile];
+        if (threadIdx.x < 32) walk_ranges(wi, T, geom[tile], c.c0.y, ws);
+        if (threadIdx.x == 0) {
+            bb.n = 0u;
+            const uint32_t nb = (ws.total + WALK_BLOCK - 1) / WALK_BLOCK;
+            if (!helper) {
+                bb.entry = -1;
+                if (nb > split) {
+                    const uint32_t i = atomicAdd(&ctr[2], 1u);
+                    if (i < (uint32_t)BIN_SHARES) {
+                        shares[i].tile = (uint32_t)tile;
+                        __threadfence();
+                        atomicExch(&shares[i].blocks, nb);
+                        bb.entry = (int)i;
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        const uint32_t E = ws.total;
+        Walk w;
+        w.init(wi, c, ws);
+        if (bb.entry >= 0) {
+            BinShare* e = &shares[bb.entry];
+            const uint32_t nb = (E + WALK_BLOCK - 1) / WALK_BLOCK;
+            for (;;) {
+                __syncthreads();
+                if (threadIdx.x == 0) {
+                    bb.claim = atomicAdd(&e->claim, 1u);
+                    bb.n = 0u;
+                }
+                __syncthreads();
+                const uint32_t b = bb.claim;
+                if (b >= 2u * nb) break;
+                const uint32_t i0 = (b < nb ? b : b - nb) * WALK_BLOCK, i1 = min(E, i0 + WALK_BLOCK);
+                bin_block(w, wi, rec, T, ws, i0, i1, s_ids, bb);
+                __syncthreads();
+                const uint32_t n = bb.n;
+                if (b < nb) {
+                    if (threadIdx.x == 0) {
+                        atomicAdd(&e->n, n);
+                        __threadfence();
+                        if (atomicAdd(&e->done, 1u) == nb - 1u) {
+                            __threadfence();
+                            atomicExch(&e->cursor, take_range(tile, atomicAdd(&e->n, 0u)));
+                            __threadfence();
+                            atomicExch(&e->ready, 1u);
+                        }
+                    }
+                    continue;
+                }
+                if (threadIdx.x == 0) {
+                    // microseconds; a second of looks, then an error instead
+                    uint32_t look = 0;
+                    while (!*(volatile uint32_t*)&e->ready && look < 5000000u) {
+                        __nanosleep(200);
+                        ++look;
+                    }
+                    __threadfence();
+                    bb.ok = *(volatile uint32_t*)&e->ready != 0u;
+                    if (bb.ok)
+                        bb.start = atomicAdd(&e->cursor, n);
+                    else
+                        raise_status(status, VSR_ERR_TIMEOUT);
+                }
+                __syncthreads();
+                if (!bb.ok) break;
+                const uint32_t start = bb.start;
+                for (uint32_t j = threadIdx.x; j < n; j += WALK_THREADS)
+                    if (start + j < cap) ids[start + j] = s_ids[j];
+            }
+        } else if (E <= WALK_BLOCK) {
+            bin_block(w, wi, rec, T, ws, 0u, E, s_ids, bb);
+            __syncthreads();
+            const uint32_t n = bb.n;
+            if (threadIdx.x == 0) bb.start = take_range(tile, n);
+            __syncthreads();
+            const uint32_t start = bb.start;
+            for (uint32_t j = threadIdx.x; j < n; j += WALK_THREADS)
+                if (start + j < cap) ids[start + j] = s_ids[j];
+        } else {
+            // block by block: count, take the range, write
+            uint32_t total = 0, start = 0;
+            for (int pass = 0; pass < 2; ++pass) {
+                for (uint32_t i0 = 0; i0 < E; i0 += WALK_BLOCK) {
+                    bin_block(w, wi, rec, T, ws, i0, min(E, i0 + WALK_BLOCK), s_ids, bb);
+                    __syncthreads();
+                    const uint32_t n = bb.n;
+                    if (pass)
+                        for (uint32_t j = threadIdx.x; j < n; j += WALK_THREADS)
+                            if (start + j < cap) ids[start + j] = s_ids[j];
+                    start += pass ? n : 0u;
+                    total += pass ? 0u : n;
+                    __syncthreads();
+                    if (threadIdx.x == 0) bb.n = 0u;
+                    __syncthreads();
+                }
+                if (!pass) {
+                    if (threadIdx.x == 0) bb.start = take_range(tile, total);
+                    __syncthreads();
+                    start = bb.start;
+                }
+            }
+        }
+        if (!helper) break;
     }
+    __syncthreads();  // this CTA's last look at the shares
     if (threadIdx.x == 0) {
         __threadfence();
-        if (atomicAdd(&ctr[1], 1u) == gridDim.x - 1) {
-            __threadfence();
-            const uint32_t total = atomicExch(&ctr[0], 0u);
-            ctr[1] = 0u;
-            starts[ntiles] = total;
-            if (total_host) {  // straight into the host's pinned word (read after an event)
-                *(volatile uint32_t*)total_host = total;
-                __threadfence_system();
-            }
+        bb.ok = atomicAdd(&ctr[1], 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!bb.ok) return;
+    __threadfence();
+    const uint32_t used = min(*published, (uint32_t)BIN_SHARES) * BIN_SHARE_WORDS;
+    for (uint32_t i = threadIdx.x; i < used; i += WALK_THREADS) ctr[BIN_CTR_SHARES + i] = 0u;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const uint32_t total = atomicExch(&ctr[0], 0u);
+        ctr[1] = 0u;
+        ctr[2] = 0u;
+        starts[ntiles] = total;
+        if (total_host) {  // straight into the host's pinned word (read after an event)
+            *(volatile uint32_t*)total_host = total;
+            __threadfence_system();
         }
     }
 }
@@ -239,10 +392,17 @@ vsr_status launch_grid_file(const float4* rec, int T, const TriGrid& g, cudaStre
 
 vsr_status launch_bin_walk(const float4* rec, int T, const WalkIndex& wi, const float4* geom, const Cone* tiles,
                            int ntiles, uint32_t* ctr, uint32_t* starts, uint32_t* ends, uint32_t* ids, uint32_t cap,
-                           int* status, uint32_t* total_host, cudaStream_t st)
+                           bool sizing, int* status, uint32_t* total_host, cudaStream_t st)
 {
     if (T < 0 || ntiles <= 0 || (!wi.direct && !wi.start)) return VSR_ERR_INVALID_ARG;
-    VSR_CUDA_TRY(launch_next(bin_walk_kernel, ntiles, WALK_THREADS, st, rec, T, wi, geom, tiles, ntiles, ctr, starts, ends,
-                             ids, cap, status, total_host));
+    const int sms = sm_count();
+    if (sms < 0) return VSR_ERR_CUDA;
+    // helpers, four CTAs per SM, only where a tile can have enough candidates;
+    // with few tiles they start together with them and look for a while
+    const bool few = ntiles < BIN_FEW * sms;
+    const uint32_t split = few ? 2u : 4u;
+    const int helpers = (uint32_t)T > split * WALK_BLOCK ? 4 * sms : 0;
+    VSR_CUDA_TRY(launch_next(bin_walk_kernel, ntiles + helpers, WALK_THREADS, st, rec, T, wi, geom, tiles, ntiles, split,
+                             few ? 40 : 0, sizing, ctr, starts, ends, ids, cap, status, total_host));
     return VSR_OK;
 }

@@ -51,7 +51,7 @@ struct vsr_scene_s {
     // bins: tile u's at ids[offsets[u] .. ends[u]) (offsets[ntiles]: the total)
     uint32_t* offsets = nullptr;  // ntiles + 1
     uint32_t* ends = nullptr;     // ntiles
-    uint32_t* bin_ctr = nullptr;  // 2, zero between binnings
+    uint32_t* bin_ctr = nullptr;  // BIN_CTR_WORDS, zero between binnings
     uint32_t* ids = nullptr;
     uint32_t cap = 0;
     TriGrid grid = {};  // the set-up's triangles by cap cell (T > GRID_DIRECT)

@@ -109,12 +109,12 @@ size_t work_estimate(int64_t T, int W, int H)
     const size_t tiles = (size_t)((W + TILE - 1) / TILE) * ((H + TILE - 1) / TILE);
     const size_t split = tiles < SPLIT_SLOTS ? tiles : SPLIT_SLOTS;
     return (size_t)T * (REC_F * sizeof(float4) + 4 * sizeof(uint32_t)) + (grid_used(T) ? grid_bytes(T) : 0) +
-           tiles * 5 * sizeof(uint32_t) + split * TILE_PIX * 2 * sizeof(uint64_t) + EXTRA_ITEMS * sizeof(uint2);
+           (tiles * 5 + BIN_CTR_WORDS) * sizeof(uint32_t) + split * TILE_PIX * 2 * sizeof(uint64_t) + EXTRA_ITEMS * sizeof(uint2);
 }
 
 size_t scene_bytes(const vsr_scene_s* s)
 {
-    size_t b = (size_t)s->T_alloc * REC_F * sizeof(float4) + (size_t)s->ws_tiles * 3 * sizeof(uint32_t) +
+    size_t b = (size_t)s->T_alloc * REC_F * sizeof(float4) + (s->ws_tiles ? (size_t)s->ws_tiles * 3 + BIN_CTR_WORDS : 0) * sizeof(uint32_t) +
                (size_t)s->cap * sizeof(uint32_t);
     if (s->grid.counts) b += grid_bytes(s->grid.T);
     if (s->walk.mem) b += WALK_WORK_BYTES;

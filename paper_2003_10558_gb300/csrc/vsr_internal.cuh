@@ -314,13 +314,16 @@ inline WalkIndex walk_index(const TriGrid& g, int64_t T, int pstep = 0)
 }
 // binning by the walk: every tile's bin, in one launch.  starts / ends: ntiles
 // + 1 / ntiles words, tile u's ids at [starts[u], ends[u]) in no order of
-// tiles, starts[ntiles] the total; ctr: two words, zero between binnings.
+// tiles, starts[ntiles] the total; ctr: BIN_CTR_WORDS words, zero between
+// binnings (pairs, CTAs done, tiles shared between CTAs, and those tiles' words).
 // With more pairs than cap the bins are cut at cap and VSR_ERR_BIN_OVERFLOW is
-// raised; total_host (optional): the device address of a pinned host word that
+// raised, unless the launch only sizes the bins; total_host (optional): the device address of a pinned host word that
 // also receives the total.
+constexpr int BIN_SHARES = 1024, BIN_SHARE_WORDS = 8, BIN_CTR_SHARES = 8;
+constexpr int BIN_CTR_WORDS = BIN_CTR_SHARES + BIN_SHARES * BIN_SHARE_WORDS;
 vsr_status launch_bin_walk(const float4* rec, int T, const WalkIndex& wi, const float4* geom, const Cone* tiles,
                            int ntiles, uint32_t* ctr, uint32_t* starts, uint32_t* ends, uint32_t* ids, uint32_t cap,
-                           int* status, uint32_t* total_host, cudaStream_t st);
+                           bool sizing, int* status, uint32_t* total_host, cudaStream_t st);
 // One view as the raster kernel sees it: its map, tile cones, set-up
 // records, bin offsets (indexed by the view's own tile number), bin ids and
 // outputs.

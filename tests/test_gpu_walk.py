@@ -74,6 +74,8 @@ CASES = [
     (96, 80, 0.0, 1.0, 1.0, 8.0, lambda: _crowd(12000, 0.004, 11), "pole"),   # one cell
     (800, 608, 0.0, 1.0, 1.0, 60.0, lambda: np.concatenate([  # shared tiles among many: helpers after the tiles
         _crowd(6000, 0.02, 12), scenes.random_triangles(6000, 1.0, 40.0, 0.02, 13)]), "front"),
+    # more tiles of many candidates than can be shared at a time
+    (800, 608, 0.1, 0.9, 0.9, 170.0, lambda: scenes.random_triangles(6000, 1.0, 30.0, 0.9, 15), None),
 ]
 
 
