@@ -291,10 +291,10 @@ __global__ void __launch_bounds__(RT, 5) frag_fill_kernel(FragArgs v)
         inimg[p] = tp.px < v.W && tp.py + 4 * p < v.H;
         if (inimg[p]) span[p] = v.span[(size_t)(tp.py + 4 * p) * v.W + tp.px];
     }
-    // (room beyond the buffer is never given out once the host has sized it)
+    // (beyond the buffer: only before the host has sized it)
     const bool fits = (uint64_t)span[0].x + span[0].y <= v.fcap && (uint64_t)span[1].x + span[1].y <= v.fcap;
     if (!fits) {
-        raise_status(v.status, VSR_ERR_FRAG_OVERFLOW);
+        if (!v.early) raise_status(v.status, VSR_ERR_FRAG_OVERFLOW);
         span[0].y = span[1].y = 0u;
     }
     uint32_t cnt[PPT] = {0u, 0u};

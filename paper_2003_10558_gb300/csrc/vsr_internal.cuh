@@ -486,6 +486,7 @@ struct FragArgs {
     uint4* bits;          // per pixel: a bit per triangle of the tile's list that is a fragment
     float4* frags;        // fragment records (r, t, m^f, shade)
     uint32_t fcap;
+    bool early;           // the room is not known to be enough: what does not fit is left out, not an error
     float* image;
     float* cov;
     uint32_t* out_id;

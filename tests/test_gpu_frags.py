@@ -54,3 +54,18 @@ def test_lists(vsr, W, H, T, jitter):
                             cam=np.asarray(cam, dtype=np.float64))
     for a, b in ((g["dtris"], og["dtris"]), (g["dcolors"], og["dcolors"])):
         assert np.linalg.norm(a.cpu().numpy() - b) <= 1e-3 * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("n", [1, 2, 5])
+def test_lists_grow(vsr, n):
+    """Frames of ever more fragments into lists filled before their number is
+    known: the same as into lists of their own, and no error."""
+    m = vsr.Map(61, 45, 0.3, 0.8, 0.9, 200.0)
+    frags = vsr.Frags()
+    for q in range(3):
+        sc = vsr.Scene(torch.from_numpy(scenes.random_triangles(20 * (4 * n) ** q, 1.0, 10.0, 0.2, seed=q)).cuda(),
+                       scenes.camera())
+        out, ref = (vsr.raster_shaded(m, sc, f) for f in (frags, vsr.Frags()))
+        for key in ref:
+            assert torch.equal(out[key].view(torch.int32), ref[key].view(torch.int32)), key
+    assert vsr.last_device_status() == 0
