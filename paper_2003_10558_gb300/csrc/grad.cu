@@ -33,6 +33,8 @@
 // per-triangle record gradients accumulate with float4 atomics; the
 // per-pixel (dG, d delta) go to the map adjoint (map.cu), and the set-up
 // adjoint below takes the record gradients to the world vertices.
+#include <type_traits>
+
 #include "tile.cuh"
 #include "walk.cuh"
 
@@ -88,7 +90,7 @@ __device__ __forceinline__ bool frag_start(const FragArgs& v, const TilePos& tp,
 // and classification.
 struct FragEval {
     float gm[PPT], r[PPT], D[PPT];
-    bool f[PPT], in[PPT];
+    bool f[PPT];
 };
 // false (for the whole warp): no fragment
 __device__ __forceinline__ bool frag_eval(const Stage& st, int j, const FragPix& q, FragEval& o)
@@ -106,12 +108,10 @@ __device__ __forceinline__ bool frag_eval(const Stage& st, int j, const FragPix&
     const float2 Dp = plane_distance2(q.dgx, q.dgy, q.dgz, st.s5[j]);
     o.D[0] = Dp.x;
     o.D[1] = Dp.y;
-    const unsigned ties = __float_as_uint(st.s0[j].w);
 #pragma unroll
     for (int p = 0; p < PPT; ++p) {
         o.r[p] = __fdividef(b.w, o.D[p]);
         o.f[p] = (p ? f1 : f0) && __float_as_uint(o.r[p]) - 1u < DEPTH_LIM;  // 0 < r < inf
-        o.in[p] = o.f[p] && centre_inside(p ? g1.y : g1.x, p ? g2.y : g2.x, p ? g3.y : g3.x, g3m[p], ties);
     }
     return true;
 }
@@ -131,12 +131,12 @@ struct FragShared {
 };
 
 // The tile's triangles, walked block by block and staged chunk by chunk; each
-// survivor of the warp's cull goes to each(j, group, k): staged slot j = 32
-// group + k.  Called by every thread of the CTA after walk_ranges, frag_start
+// survivor of the warp's cull goes to each(j, k): staged slot j = 32 g + k;
+// group(g) follows each 32 slots.  Called by every thread of the CTA after walk_ranges, frag_start
 // and a barrier; staged(t, j) runs in the thread that stages triangle t.
-template <class Stage1, class Each>
+template <class Stage1, class Each, class Group>
 __device__ __forceinline__ void frag_walk(const FragArgs& v, const Cone& tc, FragShared& s, bool active, Stage1 staged,
-                                          Each each)
+                                          Each each, Group group)
 {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -172,26 +172,76 @@ __device__ __forceinline__ void frag_walk(const FragArgs& v, const Cone& tc, Fra
             }
             __syncthreads();
             if (!active) continue;
-#pragma unroll
-            for (int g = 0; g < STAGE_CHUNK / 32; ++g) {
+            for (int g = 0; 32 * g < nc; ++g) {
                 const int jj = 32 * g + lane;
-                if (32 * g >= nc) break;
                 bool keep = false;
                 if (jj < nc && __float_as_uint(s.st.s6[jj].w) != STAGE_EMPTY)
                     keep = cone_may_hit(s.st.s0[jj], s.st.s1[jj], s.st.s2[jj], s.st.s3[jj], s.st.s4[jj],
                                         s.wc.c[warp][0], s.wc.c[warp][1], false);
-                unsigned mask = __ballot_sync(FULL, keep);
+                unsigned mask = __ballot_sync(0xffffffffu, keep);
                 while (mask) {
                     const int k = 31 - __clz(mask);
                     mask ^= 1u << k;
-                    each(32 * g + k, g, k);
+                    each(32 * g + k, k);
                 }
+                group(g);
             }
         }
     }
 }
 
-__global__ void __launch_bounds__(RT, 6) frag_count_kernel(FragArgs v)
+// One staged triangle in the count: as the coverage kernel's evaluation
+// (eval_slot of raster.cu), with a count and a bit in place of the coverage.
+struct FragCount {
+    uint32_t cnt[PPT], bits[PPT];  // fragments; those of the current group of 32 slots
+    unsigned long long key[PPT];   // ((bits(r) - 1) << 32) | t of the nearest centre-inside fragment, or KEY_NONE
+};
+__device__ __forceinline__ void frag_count(const Stage& st, int j, int k, const FragPix& q, FragCount& n)
+{
+    const float4 b = st.s1[j], e = st.s6[j];
+    const float2 g4 = miter_distance2(q.dgx, q.dgy, q.dgz, e, b, q.eg);
+    const float2 g1 = plane_distance2(q.dgx, q.dgy, q.dgz, st.s2[j]);
+    const float2 g2 = plane_distance2(q.dgx, q.dgy, q.dgz, st.s3[j]);
+    const float2 g3 = plane_distance2(q.dgx, q.dgy, q.dgz, st.s4[j]);
+    const float g3m[PPT] = {fminf(fminf(g1.x, g2.x), g3.x), fminf(fminf(g1.y, g2.y), g3.y)};
+    const bool f[PPT] = {fminf(g3m[0], g4.x) > q.lim[0], fminf(g3m[1], g4.y) > q.lim[1]};
+    if (!__any_sync(0xffffffffu, f[0] || f[1])) return;
+    const float2 Dp = plane_distance2(q.dgx, q.dgy, q.dgz, st.s5[j]);
+    const float D[PPT] = {Dp.x, Dp.y};
+    auto post = [&](auto rare_t) {
+        constexpr bool RARE = decltype(rare_t)::value;
+        uint32_t rq[PPT];
+        bool inn[PPT];
+#pragma unroll
+        for (int p = 0; p < PPT; ++p) {
+            const float r = RARE ? __fdividef(b.w, D[p]) : __fmul_rn(b.w, rcp_fast(D[p]));
+            rq[p] = __float_as_uint(r) - 1u;
+            const bool frag = f[p] && rq[p] < DEPTH_LIM;
+            n.cnt[p] += frag;
+            n.bits[p] |= (frag ? 1u : 0u) << k;
+            inn[p] = f[p] && g3m[p] > 0.0f;
+            if (RARE && f[p] && g3m[p] == 0.0f) {
+                const float dx = p ? q.dgx.y : q.dgx.x, dy = p ? q.dgy.y : q.dgy.x, dz = p ? q.dgz.y : q.dgz.x;
+                inn[p] = centre_inside(plane_distance(dx, dy, dz, st.s2[j]), plane_distance(dx, dy, dz, st.s3[j]),
+                                       plane_distance(dx, dy, dz, st.s4[j]), g3m[p], __float_as_uint(st.s0[j].w));
+            }
+        }
+        if (__any_sync(0xffffffffu, inn[0] || inn[1])) {
+#pragma unroll
+            for (int p = 0; p < PPT; ++p) {
+                const unsigned long long kk = ((unsigned long long)rq[p] << 32) | __float_as_uint(e.w);
+                n.key[p] = inn[p] && kk < n.key[p] ? kk : n.key[p];
+            }
+        }
+    };
+    const float tiny = fminf(fminf(fabsf(g3m[0]), fabsf(g3m[1])), fminf(fabsf(D[0]), fabsf(D[1])));
+    if (__any_sync(0xffffffffu, tiny < 1.17549435e-38f))
+        post(std::true_type{});
+    else
+        post(std::false_type{});
+}
+
+__global__ void __launch_bounds__(RT, 8) frag_count_kernel(FragArgs v)
 {
     grid_wait();
     grid_go();
@@ -205,26 +255,21 @@ __global__ void __launch_bounds__(RT, 6) frag_count_kernel(FragArgs v)
     if (threadIdx.x == 0) s.n = 0u;
     FragPix q;
     const bool active = frag_start(v, tp, tc.c0, q, s.wc);
-    uint32_t cnt[PPT] = {0u, 0u}, bits[PPT][4] = {};
-    unsigned long long key[PPT] = {~0ull, ~0ull};
+    FragCount c{{0u, 0u}, {0u, 0u}, {KEY_NONE, KEY_NONE}};
     __syncthreads();
     frag_walk(
-        v, tc, s, active, [](uint32_t, int) {},
-        [&](int j, int g, int k) {
-            FragEval o;
-            if (!frag_eval(s.st, j, q, o)) return;
-            const uint32_t t = __float_as_uint(s.st.s6[j].w);
+        v, tc, s, active, [](uint32_t, int) {}, [&](int j, int k) { frag_count(s.st, j, k, q, c); },
+        [&](int g) {  // (one chunk, if the tile keeps a list)
+            if (s.ws.total <= (uint32_t)WALK_BLOCK && s.n <= (uint32_t)FRAG_LIST) {
 #pragma unroll
-            for (int p = 0; p < PPT; ++p) {
-                cnt[p] += o.f[p];
-                // (g is a constant of the unrolled loop: bits stay in registers)
-                bits[p][g] |= (o.f[p] ? 1u : 0u) << k;
-                const unsigned long long kk = ((unsigned long long)__float_as_uint(o.r[p]) << 32) | t;
-                if (o.in[p] && kk < key[p]) key[p] = kk;
+                for (int p = 0; p < PPT; ++p)
+                    if (tp.px < v.W && tp.py + 4 * p < v.H)
+                        v.bits[((size_t)g * v.H + tp.py + 4 * p) * v.W + tp.px] = c.bits[p];
             }
+            c.bits[0] = c.bits[1] = 0u;
         });
     // the tile's range of the lists, its pixels in thread order
-    const uint32_t mine = cnt[0] + cnt[1];
+    const uint32_t mine = c.cnt[0] + c.cnt[1];
     uint32_t incl = mine;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -251,13 +296,12 @@ __global__ void __launch_bounds__(RT, 6) frag_count_kernel(FragArgs v)
     for (int p = 0; p < PPT; ++p) {
         if (tp.px < v.W && tp.py + 4 * p < v.H) {
             const size_t o = (size_t)(tp.py + 4 * p) * v.W + tp.px;
-            v.span[o] = make_uint2(off, cnt[p]);
-            if (list) v.bits[o] = make_uint4(bits[p][0], bits[p][1], bits[p][2], bits[p][3]);
-            const bool hit = key[p] != ~0ull;
-            if (v.out_id) v.out_id[o] = hit ? (uint32_t)(key[p] & 0xffffffffull) : 0xffffffffu;
-            if (v.out_depth) v.out_depth[o] = hit ? __uint_as_float((uint32_t)(key[p] >> 32)) : INFINITY;
+            v.span[o] = make_uint2(off, c.cnt[p]);
+            const bool hit = c.key[p] != KEY_NONE;
+            if (v.out_id) v.out_id[o] = hit ? (uint32_t)(c.key[p] & 0xffffffffull) : 0xffffffffu;
+            if (v.out_depth) v.out_depth[o] = hit ? __uint_as_float((uint32_t)(c.key[p] >> 32) + 1u) : INFINITY;
         }
-        off += cnt[p];
+        off += c.cnt[p];
     }
 }
 
@@ -265,7 +309,7 @@ __global__ void __launch_bounds__(RT, 6) frag_count_kernel(FragArgs v)
 // it is stored
 constexpr uint32_t FRAG_SORT = 8;
 
-__global__ void __launch_bounds__(RT, 5) frag_fill_kernel(FragArgs v)
+__global__ void __launch_bounds__(RT, 6) frag_fill_kernel(FragArgs v)
 {
     grid_wait();
     grid_go();
@@ -315,8 +359,13 @@ __global__ void __launch_bounds__(RT, 5) frag_fill_kernel(FragArgs v)
         uint4 bits[PPT];
 #pragma unroll
         for (int p = 0; p < PPT; ++p) {
-            bits[p] = make_uint4(0u, 0u, 0u, 0u);
-            if (inimg[p] && span[p].y) bits[p] = v.bits[(size_t)(tp.py + 4 * p) * v.W + tp.px];
+            const uint32_t* __restrict__ at = v.bits + (size_t)(tp.py + 4 * p) * v.W + tp.px;
+            const size_t pic = (size_t)v.H * v.W;
+            const bool some = inimg[p] && span[p].y;
+            bits[p].x = some ? at[0] : 0u;
+            bits[p].y = some && n > 32u ? at[pic] : 0u;
+            bits[p].z = some && n > 64u ? at[2 * pic] : 0u;
+            bits[p].w = some && n > 96u ? at[3 * pic] : 0u;
             sorted[p] = span[p].y <= FRAG_SORT;
         }
         __syncthreads();
@@ -384,14 +433,15 @@ __global__ void __launch_bounds__(RT, 5) frag_fill_kernel(FragArgs v)
         frag_walk(
             v, tc, s.walk, active,
             [&](uint32_t t, int j) { scol[j] = v.colors && t < (uint32_t)v.T ? v.colors[t] : 1.0f; },
-            [&](int j, int, int) {
+            [&](int j, int) {
                 FragEval o;
                 if (!frag_eval(s.walk.st, j, q, o)) return;
                 const uint32_t t = __float_as_uint(s.walk.st.s6[j].w);
 #pragma unroll
                 for (int p = 0; p < PPT; ++p)
                     if (o.f[p]) put(o, p, t, scol[j]);
-            });
+            },
+            [](int) {});
     }
 #pragma unroll
     for (int p = 0; p < PPT; ++p) {

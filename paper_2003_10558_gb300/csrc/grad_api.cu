@@ -8,7 +8,7 @@
 struct vsr_frags_s {
     size_t npix = 0, ntiles = 0;  // per-pixel and per-tile buffers sized for these
     uint2* span = nullptr;        // npix
-    uint4* bits = nullptr;        // npix
+    uint32_t* bits = nullptr;     // npix x FRAG_LIST / 32
     uint32_t* tile_n = nullptr;   // ntiles
     uint32_t* tile_ids = nullptr; // ntiles x FRAG_LIST
     uint32_t* cursor = nullptr;
@@ -53,7 +53,7 @@ vsr_status frags_ensure_pixels(vsr_frags f, int W, int H, size_t ntiles, cudaStr
     if (!f->cursor && (s = dalloc(&f->cursor, 1)) != VSR_OK) return s;
     if (n <= f->npix && ntiles <= f->ntiles) return VSR_OK;
     frags_release_pixels(f);
-    if ((s = dalloc(&f->span, n)) != VSR_OK || (s = dalloc(&f->bits, n)) != VSR_OK ||
+    if ((s = dalloc(&f->span, n)) != VSR_OK || (s = dalloc(&f->bits, n * (FRAG_LIST / 32))) != VSR_OK ||
         (s = dalloc(&f->tile_n, ntiles)) != VSR_OK || (s = dalloc(&f->tile_ids, ntiles * FRAG_LIST)) != VSR_OK ||
         (s = dalloc(&f->dmap, n)) != VSR_OK || (s = dalloc(&f->lens_part, map_backward_partials(ntiles))) != VSR_OK) {
         frags_release_pixels(f);

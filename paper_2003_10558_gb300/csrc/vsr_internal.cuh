@@ -483,7 +483,7 @@ struct FragArgs {
     uint32_t* tile_n;     // per tile: its triangles, or ~0 (more than FRAG_LIST)
     uint32_t* tile_ids;   // per tile: FRAG_LIST of them
     uint2* span;          // per pixel: (first fragment, fragments)
-    uint4* bits;          // per pixel: a bit per triangle of the tile's list that is a fragment
+    uint32_t* bits;       // FRAG_LIST / 32 pictures: a bit per triangle of the tile's list that is a fragment
     float4* frags;        // fragment records (r, t, m^f, shade)
     uint32_t fcap;
     bool early;           // the room is not known to be enough: what does not fit is left out, not an error
