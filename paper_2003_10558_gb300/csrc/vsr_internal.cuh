@@ -288,8 +288,7 @@ struct TriGrid {
     uint32_t* start = nullptr;   // GRID_WORDS: first entry of each cell, each row closed by its end
     uint32_t* hdr = nullptr;     // GRID_HDR
     uint32_t* where = nullptr;   // T: cell word, or ~0 without a cap
-    float4* ent = nullptr;       // T entries: (S-hat xyz, cos rho)
-    float2* ent2 = nullptr;      // (sin rho, triangle bits)
+    float4* ent = nullptr;       // 2 per entry: (S-hat xyz, cos rho), (sin rho, triangle bits, 0, 0)
     int64_t T = 0;               // capacity
     bool dirty = false;          // host side: a failed set-up may have left counters behind
 };
@@ -303,14 +302,13 @@ struct WalkIndex {
     const uint32_t* start;
     const uint32_t* hdr;
     const float4* ent;
-    const float2* ent2;
     int direct;
     int pstep;  // caps of the per-fragment pixel step
 };
 inline bool grid_used(int64_t T) { return T > GRID_DIRECT; }
 inline WalkIndex walk_index(const TriGrid& g, int64_t T, int pstep = 0)
 {
-    return WalkIndex{g.start, g.hdr, g.ent, g.ent2, grid_used(T) ? 0 : 1, pstep};
+    return WalkIndex{g.start, g.hdr, g.ent, grid_used(T) ? 0 : 1, pstep};
 }
 // binning by the walk: every tile's bin, in one launch.  starts / ends: ntiles
 // + 1 / ntiles words, tile u's ids at [starts[u], ends[u]) in no order of

@@ -245,10 +245,10 @@ struct Walk {
                 const uint4 r = ws.rng[o];
                 const uint32_t k = idx - r.x;
                 const uint32_t e = k < r.z ? r.y + k : r.w + k;
-                q = wi.ent[e];
-                const float2 s = wi.ent2[e];
-                sr = s.x;
-                t = __float_as_uint(s.y);
+                const F8 c = ld_f8(wi.ent + 2 * (size_t)e);
+                q = c.a;
+                sr = c.b.x;
+                t = __float_as_uint(c.b.y);
             }
         }
         float cb, sb;
