@@ -138,7 +138,6 @@ template <class Stage1, class Each, class Group>
 __device__ __forceinline__ void frag_walk(const FragArgs& v, const Cone& tc, FragShared& s, bool active, Stage1 staged,
                                           Each each, Group group)
 {
-    const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (uint32_t e0 = 0; e0 < s.ws.total; e0 += WALK_BLOCK) {
         if (e0) {
@@ -146,20 +145,9 @@ __device__ __forceinline__ void frag_walk(const FragArgs& v, const Cone& tc, Fra
             if (threadIdx.x == 0) s.n = 0u;
             __syncthreads();
         }
-        const uint32_t e1 = min(s.ws.total, e0 + (uint32_t)WALK_BLOCK);
         Walk w;
         w.init(v.wi, tc, s.ws);
-        for (uint32_t i0 = e0; i0 < e1; i0 += WALK_THREADS) {
-            const uint32_t idx = i0 + threadIdx.x;
-            uint32_t t;
-            const bool hit = w.test(v.wi, v.rec, v.T, s.ws, idx, idx < e1, t);
-            const unsigned m = __ballot_sync(FULL, hit);
-            if (!m) continue;
-            uint32_t base = 0;
-            if (lane == 0) base = atomicAdd(&s.n, (uint32_t)__popc(m));
-            base = __shfl_sync(FULL, base, 0);
-            if (hit) s.ids[base + (uint32_t)__popc(m & ((1u << lane) - 1u))] = t;
-        }
+        walk_hits(w, v.wi, v.rec, v.T, s.ws, e0, min(s.ws.total, e0 + (uint32_t)WALK_BLOCK), s.ids, &s.n);
         __syncthreads();
         const uint32_t n = s.n;
         for (uint32_t base = 0; base < n; base += STAGE_CHUNK) {

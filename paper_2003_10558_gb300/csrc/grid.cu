@@ -130,27 +130,6 @@ struct BinBlock {
     int entry, ok;
 };
 
-// The hits of candidates [i0, i1), at most WALK_BLOCK, into s_ids (all
-// threads; the caller has cleared bb.n and waits for the CTA on both sides).
-__device__ __forceinline__ void bin_block(const Walk& w, const WalkIndex& wi, const float4* __restrict__ rec, int T,
-                                          const WalkShared& ws, uint32_t i0, uint32_t i1, uint32_t* s_ids,
-                                          BinBlock& bb)
-{
-    const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    for (uint32_t i = i0; i < i1; i += WALK_THREADS) {
-        const uint32_t idx = i + threadIdx.x;
-        uint32_t t;
-        const bool hit = w.test(wi, rec, T, ws, idx, idx < i1, t);
-        const unsigned m = __ballot_sync(FULL, hit);
-        if (!m) continue;
-        uint32_t base = 0;
-        if (lane == 0) base = atomicAdd(&bb.n, (uint32_t)__popc(m));
-        base = __shfl_sync(FULL, base, 0);
-        if (hit) s_ids[base + (uint32_t)__popc(m & ((1u << lane) - 1u))] = t;
-    }
-}
-
 __global__ void __launch_bounds__(WALK_THREADS) bin_walk_kernel(const float4* __restrict__ rec, int T, WalkIndex wi,
                                                                const float4* __restrict__ geom,
                                                                const Cone* __restrict__ tiles, int ntiles,
@@ -243,7 +222,7 @@ __global__ void __launch_bounds__(WALK_THREADS) bin_walk_kernel(const float4* __
                 const uint32_t b = bb.claim;
                 if (b >= 2u * nb) break;
                 const uint32_t i0 = (b < nb ? b : b - nb) * WALK_BLOCK, i1 = min(E, i0 + WALK_BLOCK);
-                bin_block(w, wi, rec, T, ws, i0, i1, s_ids, bb);
+                walk_hits(w, wi, rec, T, ws, i0, i1, s_ids, &bb.n);
                 __syncthreads();
                 const uint32_t n = bb.n;
                 if (b < nb) {
@@ -280,7 +259,7 @@ __global__ void __launch_bounds__(WALK_THREADS) bin_walk_kernel(const float4* __
                     if (start + j < cap) ids[start + j] = s_ids[j];
             }
         } else if (E <= WALK_BLOCK) {
-            bin_block(w, wi, rec, T, ws, 0u, E, s_ids, bb);
+            walk_hits(w, wi, rec, T, ws, 0u, E, s_ids, &bb.n);
             __syncthreads();
             const uint32_t n = bb.n;
             if (threadIdx.x == 0) bb.start = take_range(tile, n);
@@ -293,7 +272,7 @@ __global__ void __launch_bounds__(WALK_THREADS) bin_walk_kernel(const float4* __
             uint32_t total = 0, start = 0;
             for (int pass = 0; pass < 2; ++pass) {
                 for (uint32_t i0 = 0; i0 < E; i0 += WALK_BLOCK) {
-                    bin_block(w, wi, rec, T, ws, i0, min(E, i0 + WALK_BLOCK), s_ids, bb);
+                    walk_hits(w, wi, rec, T, ws, i0, min(E, i0 + WALK_BLOCK), s_ids, &bb.n);
                     __syncthreads();
                     const uint32_t n = bb.n;
                     if (pass)

@@ -85,7 +85,6 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
     __shared__ WalkTile wt;
     __shared__ uint32_t s_ids[WALK_BLOCK];
     static_assert(RT == WALK_THREADS, "the walk's CTA");
-    const unsigned FULL = 0xffffffffu;
     const bool helper = blockIdx.x >= (uint32_t)ntiles;
     for (;;) {
         typename Step::Pix q;
@@ -164,19 +163,8 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
             {
                 Walk w;
                 w.init(wi, wt.cone, ws);
-                const uint32_t e0 = wt.next * block, e1 = min(ws.total, e0 + block);
-                const int lane = threadIdx.x & 31;
-                for (uint32_t i0 = e0; i0 < e1; i0 += RT) {
-                    const uint32_t idx = i0 + threadIdx.x;
-                    uint32_t t;
-                    const bool hit = w.test(wi, view.rec, view.T, ws, idx, idx < e1, t);
-                    const unsigned m = __ballot_sync(FULL, hit);
-                    if (!m) continue;
-                    uint32_t base = 0;
-                    if (lane == 0) base = atomicAdd(&wt.n, (uint32_t)__popc(m));
-                    base = __shfl_sync(FULL, base, 0);
-                    if (hit) s_ids[base + (uint32_t)__popc(m & ((1u << lane) - 1u))] = t;
-                }
+                const uint32_t e0 = wt.next * block;
+                walk_hits(w, wi, view.rec, view.T, ws, e0, min(ws.total, e0 + block), s_ids, &wt.n);
             }
             __syncthreads();
             for (uint32_t base = 0; base < wt.n; base += CHUNK) {

@@ -211,24 +211,27 @@ struct Walk {
         ex0 = ws.rng[lane].x;
     }
 
-    // candidate idx < total (one per thread, consecutive within a warp;
-    // `in`: whether this thread's exists -- all lanes call): the triangle and
-    // whether its cap may reach the tile's cone
-    __device__ __forceinline__ bool test(const WalkIndex& wi, const float4* __restrict__ rec, int T,
-                                         const WalkShared& ws, uint32_t idx, bool in, uint32_t& t) const
-    {
+    // A candidate as read: its cap (centre, cos and sin of its radius) and triangle.
+    struct Cand {
         float4 q;
         float sr;
-        bool ok = in;
+        uint32_t t;
+        bool ok;
+    };
+
+    // candidate idx < total (one per thread, consecutive within a warp;
+    // `in`: whether this thread's exists -- all lanes call)
+    __device__ __forceinline__ Cand read(const WalkIndex& wi, const float4* __restrict__ rec, int T,
+                                         const WalkShared& ws, uint32_t idx, bool in) const
+    {
+        Cand c{make_float4(0.0f, 0.0f, 0.0f, 0.0f), 0.0f, 0u, in};
         if (wi.direct) {
-            q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            sr = 0.0f;
-            t = idx;
+            c.t = idx;
             if (in) {
                 const F8 cap = ld_f8(rec + rec_at((size_t)T, idx, RF_CAP));
-                q = cap.a;
-                sr = cap.b.x;
-                ok = cap.b.w != 0.0f;
+                c.q = cap.a;
+                c.sr = cap.b.x;
+                c.ok = cap.b.w != 0.0f;
             }
         } else {
             // the range of the warp's first candidate by a vote per group of
@@ -237,20 +240,25 @@ struct Walk {
             const uint32_t lane = threadIdx.x & 31, first = idx - lane;
             int o = __popc(__ballot_sync(FULL, ex0 <= first)) - 1;
             for (int g = 1; g < ws.groups; ++g) o += __popc(__ballot_sync(FULL, ws.rng[32 * g + lane].x <= first));
-            q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            sr = 0.0f;
-            t = 0;
             if (in) {
                 while (ws.rng[o + 1].x <= idx) ++o;
                 const uint4 r = ws.rng[o];
                 const uint32_t k = idx - r.x;
                 const uint32_t e = k < r.z ? r.y + k : r.w + k;
-                const F8 c = ld_f8(wi.ent + 2 * (size_t)e);
-                q = c.a;
-                sr = c.b.x;
-                t = __float_as_uint(c.b.y);
+                const F8 ent = ld_f8(wi.ent + 2 * (size_t)e);
+                c.q = ent.a;
+                c.sr = ent.b.x;
+                c.t = __float_as_uint(ent.b.y);
             }
         }
+        return c;
+    }
+
+    // whether the cap may reach the tile's cone
+    __device__ __forceinline__ bool reaches(const WalkIndex& wi, const Cand& c) const
+    {
+        const float4& q = c.q;
+        const float sr = c.sr;
         float cb, sb;
         if (wi.pstep) {
             cb = fmaf(q.w, ce, -sr * se);
@@ -264,6 +272,35 @@ struct Walk {
         // angle(S, axis) <= alpha + beta (always when alpha + beta >= pi); the
         // margin covers the FP32 rounding of the products
         const float cg = fmaf(q.x, ax, fmaf(q.y, ay, q.z * az));
-        return ok && (cb + ca <= 2e-6f || cg >= fmaf(ca, cb, -sa * sb) - 2e-6f);
+        return c.ok && (cb + ca <= 2e-6f || cg >= fmaf(ca, cb, -sa * sb) - 2e-6f);
     }
 };
+
+// The hits of candidates [i0, i1), at most WALK_BLOCK, appended to ids (*n of
+// them so far, both in shared memory).  Called by every thread of the CTA; the
+// caller synchronizes on both sides.  A thread reads two candidates before it
+// tests either (1M triangles from inside: 427.5 -> 421.5 us a frame; the pixel
+// step at 1280 x 720: 119.5 -> 115.9 us).  Prefetching the hits' records as
+// they are found changed nothing (421.3, 116.4 us).
+__device__ __forceinline__ void walk_hits(const Walk& w, const WalkIndex& wi, const float4* __restrict__ rec, int T,
+                                          const WalkShared& ws, uint32_t i0, uint32_t i1, uint32_t* ids, uint32_t* n)
+{
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const uint32_t lt = (1u << lane) - 1u;
+    for (uint32_t i = i0; i < i1; i += 2 * WALK_THREADS) {
+        const uint32_t ia = i + threadIdx.x, ib = ia + WALK_THREADS;
+        const bool two = i + WALK_THREADS < i1;
+        const Walk::Cand a = w.read(wi, rec, T, ws, ia, ia < i1);
+        Walk::Cand b{};
+        if (two) b = w.read(wi, rec, T, ws, ib, ib < i1);
+        const bool ha = w.reaches(wi, a), hb = two && w.reaches(wi, b);
+        const unsigned ma = __ballot_sync(FULL, ha), mb = __ballot_sync(FULL, hb);
+        if (!(ma | mb)) continue;
+        uint32_t at = 0;
+        if (lane == 0) at = atomicAdd(n, (uint32_t)(__popc(ma) + __popc(mb)));
+        at = __shfl_sync(FULL, at, 0);
+        if (ha) ids[at + (uint32_t)__popc(ma & lt)] = a.t;
+        if (hb) ids[at + (uint32_t)(__popc(ma) + __popc(mb & lt))] = b.t;
+    }
+}
