@@ -165,7 +165,7 @@ vsr_status ensure_tile_index(vsr_map m, cudaStream_t st)
 // Set-up of T triangles with the camera in host (cam) or device (cam_dev)
 // memory: records, and the triangle grid where it is used.
 vsr_status setup_records(const float* tris_dev, int64_t T, const float* cam, const float* cam_dev, float4* rec,
-                         TriGrid& grid, cudaStream_t st)
+                         TriGrid& grid, cudaStream_t st, bool on_host = false)
 {
     const TriGrid* g = grid_used(T) ? &grid : nullptr;
     vsr_status s;
@@ -178,12 +178,13 @@ vsr_status setup_records(const float* tris_dev, int64_t T, const float* cam, con
             VSR_CUDA_TRY(cudaMemsetAsync(grid.counts, 0, sizeof(uint32_t) * ((size_t)GRID_WORDS + GRID_HDR), st));
     }
     s = cam_dev ? launch_setup_view(tris_dev, (int)T, cam_dev, rec, g, st)
-                : launch_setup(tris_dev, (int)T, cam, rec, g, st);
+                : launch_setup(tris_dev, (int)T, cam, rec, g, st, on_host);
     if (s == VSR_OK && g && (s = launch_grid_file(rec, (int)T, grid, st)) == VSR_OK) grid.dirty = false;
     return s;
 }
 
-vsr_status scene_setup(vsr_scene sc, const float* tris_dev, int64_t T, const float cam[12], cudaStream_t st)
+vsr_status scene_setup(vsr_scene sc, const float* tris_dev, int64_t T, const float cam[12], cudaStream_t st,
+                       bool on_host = false)
 {
     if (T > sc->T_alloc) {
         cudaFree(sc->rec);
@@ -196,7 +197,7 @@ vsr_status scene_setup(vsr_scene sc, const float* tris_dev, int64_t T, const flo
     sc->T = T;
     for (int q = 0; q < 12; ++q) sc->cam[q] = cam[q];
     // the records are laid out for exactly T triangles
-    vsr_status s = setup_records(tris_dev, T, cam, nullptr, sc->rec, sc->grid, st);
+    vsr_status s = setup_records(tris_dev, T, cam, nullptr, sc->rec, sc->grid, st, on_host);
     sc->gen = g_gen.fetch_add(1);
     return s == VSR_OK ? scene_used(sc, st) : s;
 }
@@ -806,6 +807,7 @@ vsr_status host_frame_front(vsr_map m, vsr_scene sc, const float* tris_host, int
         VSR_CUDA_TRY(cudaEventRecord(sc->use_event, st));
     }
     VSR_CUDA_TRY(cudaStreamWaitEvent(sc->side, sc->use_event, 0));
+    const bool on_host = tris_src != nullptr;
     if (T > 0 && !tris_src) {
         if (T > sc->tris_alloc) {
             cudaFree(sc->tris_dev);
@@ -837,7 +839,7 @@ vsr_status host_frame_front(vsr_map m, vsr_scene sc, const float* tris_host, int
         if (f->stage_cov) f->cov_d = (float*)((char*)sc->out_dev + 8 * f->npix);
     }
     f->in_place = (id_host && !f->stage_id) || (depth_host && !f->stage_depth) || (cov_host && !f->stage_cov);
-    if ((s = scene_setup(sc, tris_src, T, cam, sc->side)) != VSR_OK) return s;
+    if ((s = scene_setup(sc, tris_src, T, cam, sc->side, on_host)) != VSR_OK) return s;
     VSR_CUDA_TRY(cudaEventRecord(sc->setup_event, sc->side));
     VSR_CUDA_TRY(cudaStreamWaitEvent(st, sc->setup_event, 0));
     return VSR_OK;

@@ -107,15 +107,35 @@ __device__ __forceinline__ uint32_t grid_cell(float x, float y, float z, float c
 // rotated camera, whose transform wants the registers: 220k triangles, identity
 // 33.2 -> 30.3 us at 3; 1M triangles, rotated 141.6 us at 2, 144.2 us at 3.
 enum { CAM_IDENT, CAM_ROTATED, CAM_DEVICE };
-template <int CAM>
-__global__ void __launch_bounds__(128, CAM == CAM_ROTATED ? 2 : 3) setup_pair_kernel(const float* __restrict__ tris,
-                                                                                   int T, Cam cam,
-                                                                                   const float* __restrict__ cams_dev,
-                                                                                   float4* __restrict__ rec,
-                                                                                   TriGrid grid)
+constexpr int SETUP_THREADS = 128;
+// STAGED: the vertices come through shared memory in whole lines instead of 18
+// strided loads per thread.  For vertices in host memory (each of those loads
+// goes over the link: 220k triangles 78.2 us, staged 50.3) and a camera read
+// from the device (12 views of 1M triangles: 5.63 -> 5.57 ms); not for the
+// identity camera and vertices on the device, whose registers it takes (220k
+// triangles 30.0 us, staged 31.3).
+template <int CAM, bool STAGED>
+__global__ void __launch_bounds__(SETUP_THREADS, CAM == CAM_ROTATED ? 2 : 3)
+    setup_pair_kernel(const float* __restrict__ tris, int T, Cam cam, const float* __restrict__ cams_dev,
+                      float4* __restrict__ rec, TriGrid grid)
 {
     grid_wait();
     grid_go();
+    __shared__ __align__(16) float s_in[STAGED ? 2 * SETUP_THREADS * 9 : 4];
+    if (STAGED) {
+        // the CTA's vertices in whole lines, 16 bytes a lane where the buffer allows
+        const size_t first = (size_t)blockIdx.x * (2 * SETUP_THREADS);
+        const int words = 9 * (int)min((size_t)(2 * SETUP_THREADS), (size_t)T - first);
+        const float* __restrict__ src = tris + 9 * first;
+        const int quads = ((uintptr_t)src & 15u) == 0 ? words / 4 : 0;
+#pragma unroll
+        for (int q = 0; q < (2 * SETUP_THREADS * 9 / 4 + SETUP_THREADS - 1) / SETUP_THREADS; ++q) {
+            const int i = q * SETUP_THREADS + threadIdx.x;
+            if (i < quads) ((float4*)s_in)[i] = ((const float4*)src)[i];
+        }
+        for (int i = 4 * quads + threadIdx.x; i < words; i += SETUP_THREADS) s_in[i] = src[i];
+        __syncthreads();
+    }
     const int t0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     const unsigned am = __ballot_sync(0xffffffffu, t0 < T);  // the lanes that go on
     if (t0 >= T) return;
@@ -131,8 +151,8 @@ __global__ void __launch_bounds__(128, CAM == CAM_ROTATED ? 2 : 3) setup_pair_ke
     float w0[9], w1[9];
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
-        w0[q] = tris[(size_t)t0 * 9 + q];
-        w1[q] = tris[(size_t)t1 * 9 + q];
+        w0[q] = STAGED ? s_in[18 * threadIdx.x + q] : tris[(size_t)t0 * 9 + q];
+        w1[q] = STAGED ? s_in[18 * threadIdx.x + (has1 ? 9 : 0) + q] : tris[(size_t)t1 * 9 + q];
     }
     // an identity rotation (the common camera) needs only the exact
     // differences A - O: the pair products by 1 and sums with 0 of the
@@ -255,15 +275,17 @@ __global__ void __launch_bounds__(128, CAM == CAM_ROTATED ? 2 : 3) setup_pair_ke
 }  // namespace
 
 vsr_status launch_setup(const float* tris, int T, const float cam[12], float4* rec, const TriGrid* grid,
-                        cudaStream_t st)
+                        cudaStream_t st, bool on_host)
 {
     if (T == 0) return VSR_OK;
     Cam c;
     for (int q = 0; q < 3; ++q) c.O[q] = cam[q];
     for (int q = 0; q < 9; ++q) c.M[q] = cam[3 + q];
     const int pairs = (T + 1) / 2;
-    auto kern = identity(c) ? setup_pair_kernel<CAM_IDENT> : setup_pair_kernel<CAM_ROTATED>;
-    VSR_CUDA_TRY(launch_next(kern, (pairs + 127) / 128, 128, st, tris, T, c, (const float*)nullptr, rec,
+    auto kern = !identity(c) ? (on_host ? setup_pair_kernel<CAM_ROTATED, true> : setup_pair_kernel<CAM_ROTATED, false>)
+                : on_host    ? setup_pair_kernel<CAM_IDENT, true>
+                             : setup_pair_kernel<CAM_IDENT, false>;
+    VSR_CUDA_TRY(launch_next(kern, (pairs + SETUP_THREADS - 1) / SETUP_THREADS, SETUP_THREADS, st, tris, T, c, (const float*)nullptr, rec,
                              grid ? *grid : TriGrid{}));
     return VSR_OK;
 }
@@ -273,7 +295,7 @@ vsr_status launch_setup_view(const float* tris, int T, const float* cam_dev, flo
 {
     if (T == 0) return VSR_OK;
     const int pairs = (T + 1) / 2;
-    VSR_CUDA_TRY(launch_next(setup_pair_kernel<CAM_DEVICE>, (pairs + 127) / 128, 128, st, tris, T, Cam{}, cam_dev, rec,
+    VSR_CUDA_TRY(launch_next(setup_pair_kernel<CAM_DEVICE, true>, (pairs + SETUP_THREADS - 1) / SETUP_THREADS, SETUP_THREADS, st, tris, T, Cam{}, cam_dev, rec,
                              grid ? *grid : TriGrid{}));
     return VSR_OK;
 }

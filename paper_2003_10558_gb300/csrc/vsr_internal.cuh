@@ -170,9 +170,10 @@ vsr_status launch_map_cones(const float4* map, int W, int H, Cone* tiles, float4
 vsr_status launch_map_spec(const vsr_map_spec& spec, float4* map, Cone* tiles, float4* geom, float4* deriv,
                            cudaStream_t st);
 struct TriGrid;
-// grid: count the triangles' cells for launch_grid_file (NULL: no grid)
+// grid: count the triangles' cells for launch_grid_file (NULL: no grid);
+// on_host: tris is the device address of host memory
 vsr_status launch_setup(const float* tris, int T, const float cam[12], float4* rec, const TriGrid* grid,
-                        cudaStream_t st);
+                        cudaStream_t st, bool on_host);
 
 // Device memory of a tile index (sized for IDX_CELLS_MAX cells, ntiles tiles).
 // The cones of the small tiles are stored sorted by home cell, so the cells
