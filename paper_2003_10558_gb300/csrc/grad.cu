@@ -8,16 +8,17 @@
 //     m^fc = min(m^f, 1 - m^b);  I += m^fc shade;  m^b += m^fc
 // Unlike coverage, the image depends on the order, so every fragment is
 // kept, as the float4 (r, t, m^f, shade), sorted per pixel.  Two launches:
-//  * frag_count_kernel walks the triangle grid (walk.cuh), evaluates every
-//    pixel x triangle pair, counts each pixel's fragments, takes the tile's
-//    range of the lists with one atomic (so no scan over the pixels runs) and
-//    keeps what the second launch needs: the tile's triangles and, per pixel,
-//    a bit for each that is a fragment.  Ids and depths are final here.
-//  * frag_fill_kernel, after the host has read the total, evaluates only the
-//    triangles with a fragment in the warp's block, sorts each pixel's
-//    fragments on their way in (shared memory), writes and merges them.
-// A tile with more than FRAG_LIST triangles keeps no list: the fill walks and
-// evaluates it again.
+//  * the count (FragCountStep, a walking raster) evaluates every pixel x
+//    triangle pair, counts each pixel's fragments, takes the tile's range of
+//    the lists with one atomic (so no scan over the pixels runs) and keeps
+//    what the second launch needs: the tile's triangles and, per pixel, a bit
+//    for each that is a fragment.  Ids and depths are final here.
+//  * frag_fill_kernel evaluates only the triangles with a fragment in the
+//    warp's block, sorts each pixel's fragments on their way in (shared
+//    memory), writes and merges them.
+// A tile with more than FRAG_LIST triangles or of several blocks of candidates
+// keeps no list: where there are such tiles, a third launch (FragFillStep,
+// again a walking raster) walks and evaluates them once more.
 //
 // Backward (vsr_raster_backward).  Per pixel, with upstream gradients dI,
 // dcov, ddepth: the merge takes m^fc = m^f until the first fragment f* with
@@ -35,8 +36,7 @@
 // adjoint below takes the record gradients to the world vertices.
 #include <type_traits>
 
-#include "tile.cuh"
-#include "walk.cuh"
+#include "raster_walk.cuh"
 
 namespace {
 
@@ -53,22 +53,18 @@ struct FragPix {
     float delta[PPT], lim[PPT];  // as PixPair of raster.cu
 };
 
-__device__ __forceinline__ bool frag_start(const FragArgs& v, const TilePos& tp, const float4& axis, FragPix& q,
-                                           WarpCones& wc)
+__device__ __forceinline__ bool frag_start(const float4 (&g)[PPT], const float4& axis, FragPix& q, WarpCones& wc)
 {
     float gx[PPT], gy[PPT], gz[PPT], h[PPT];
     bool pv[PPT];
 #pragma unroll
     for (int p = 0; p < PPT; ++p) {
-        const int y = tp.py + 4 * p;
-        float4 g = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (tp.px < v.W && y < v.H) g = v.map[(size_t)y * v.W + tp.px];
-        pv[p] = g.w > 0.0f;
-        gx[p] = g.x;
-        gy[p] = g.y;
-        gz[p] = g.z;
-        h[p] = pv[p] ? 0.5f / g.w : 0.0f;
-        q.delta[p] = g.w;
+        pv[p] = g[p].w > 0.0f;
+        gx[p] = g[p].x;
+        gy[p] = g[p].y;
+        gz[p] = g[p].z;
+        h[p] = pv[p] ? 0.5f / g[p].w : 0.0f;
+        q.delta[p] = g[p].w;
         q.lim[p] = pv[p] ? -h[p] : INFINITY;
     }
     q.dgx = make_float2(pv[0] ? gx[0] - axis.x : 0.0f, pv[1] ? gx[1] - axis.x : 0.0f);
@@ -122,69 +118,38 @@ __device__ __forceinline__ float4 frag_record(const FragEval& o, const FragPix& 
                        colour * fabsf(o.D[p]));
 }
 
-struct FragShared {
-    Stage st;
-    WalkShared ws;
-    WarpCones wc;
-    uint32_t ids[WALK_BLOCK];
-    uint32_t n;
-};
-
-// The tile's triangles, walked block by block and staged chunk by chunk; each
-// survivor of the warp's cull goes to each(j, k): staged slot j = 32 g + k;
-// group(g) follows each 32 slots.  Called by every thread of the CTA after walk_ranges, frag_start
-// and a barrier; staged(t, j) runs in the thread that stages triangle t.
-template <class Stage1, class Each, class Group>
-__device__ __forceinline__ void frag_walk(const FragArgs& v, const Cone& tc, FragShared& s, bool active, Stage1 staged,
-                                          Each each, Group group)
+// Sorts a pixel's m fragments where they are stored (insertion, by (r, t))
+// and merges them.  (Other CTAs may have written them: the first read of each
+// goes past the L1.)
+__device__ __forceinline__ void frag_merge(const FragArgs& v, size_t pixel, float4* F, uint32_t m)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (uint32_t e0 = 0; e0 < s.ws.total; e0 += WALK_BLOCK) {
-        if (e0) {
-            __syncthreads();
-            if (threadIdx.x == 0) s.n = 0u;
-            __syncthreads();
+    for (uint32_t u = 0; u < m; ++u) {
+        const float4 x = __ldcg(F + u);
+        uint32_t w = u;
+        while (w > 0 && frag_less(x, F[w - 1])) {
+            F[w] = F[w - 1];
+            --w;
         }
-        Walk w;
-        w.init(v.wi, tc, s.ws);
-        walk_hits(w, v.wi, v.rec, v.T, s.ws, e0, min(s.ws.total, e0 + (uint32_t)WALK_BLOCK), s.ids, &s.n);
-        __syncthreads();
-        const uint32_t n = s.n;
-        for (uint32_t base = 0; base < n; base += STAGE_CHUNK) {
-            const int nc = (int)min((uint32_t)STAGE_CHUNK, n - base);
-            if (base) __syncthreads();
-            if ((int)threadIdx.x < nc) {
-                const uint32_t t = s.ids[base + threadIdx.x];
-                stage_checked(v.rec, v.T, t, tc.c0, s.st, threadIdx.x, v.status);
-                staged(t, (int)threadIdx.x);
-            }
-            __syncthreads();
-            if (!active) continue;
-            for (int g = 0; 32 * g < nc; ++g) {
-                const int jj = 32 * g + lane;
-                bool keep = false;
-                if (jj < nc && __float_as_uint(s.st.s6[jj].w) != STAGE_EMPTY)
-                    keep = cone_may_hit(s.st.s0[jj], s.st.s1[jj], s.st.s2[jj], s.st.s3[jj], s.st.s4[jj],
-                                        s.wc.c[warp][0], s.wc.c[warp][1], false);
-                unsigned mask = __ballot_sync(0xffffffffu, keep);
-                while (mask) {
-                    const int k = 31 - __clz(mask);
-                    mask ^= 1u << k;
-                    each(32 * g + k, k);
-                }
-                group(g);
-            }
-        }
+        F[w] = x;
     }
+    float mb = 0.0f, img = 0.0f;
+    for (uint32_t u = 0; u < m && mb < 1.0f; ++u) {
+        const float4 x = F[u];
+        const float mfc = fminf(x.z, 1.0f - mb);
+        img = fmaf(mfc, x.w, img);
+        mb += mfc;
+    }
+    if (v.image) v.image[pixel] = img;
+    if (v.cov) v.cov[pixel] = mb;
 }
 
 // One staged triangle in the count: as the coverage kernel's evaluation
 // (eval_slot of raster.cu), with a count and a bit in place of the coverage.
-struct FragCount {
-    uint32_t cnt[PPT], bits[PPT];  // fragments; those of the current group of 32 slots
+struct FragCount : FragPix {
+    uint32_t acc[PPT], bits[PPT];  // fragments; those of the current group of 32 slots
     unsigned long long key[PPT];   // ((bits(r) - 1) << 32) | t of the nearest centre-inside fragment, or KEY_NONE
 };
-__device__ __forceinline__ void frag_count(const Stage& st, int j, int k, const FragPix& q, FragCount& n)
+__device__ __forceinline__ void frag_count(const Stage& st, int j, FragCount& q)
 {
     const float4 b = st.s1[j], e = st.s6[j];
     const float2 g4 = miter_distance2(q.dgx, q.dgy, q.dgz, e, b, q.eg);
@@ -205,8 +170,8 @@ __device__ __forceinline__ void frag_count(const Stage& st, int j, int k, const 
             const float r = RARE ? __fdividef(b.w, D[p]) : __fmul_rn(b.w, rcp_fast(D[p]));
             rq[p] = __float_as_uint(r) - 1u;
             const bool frag = f[p] && rq[p] < DEPTH_LIM;
-            n.cnt[p] += frag;
-            n.bits[p] |= (frag ? 1u : 0u) << k;
+            q.acc[p] += frag;
+            q.bits[p] |= (frag ? 1u : 0u) << (j & 31);
             inn[p] = f[p] && g3m[p] > 0.0f;
             if (RARE && f[p] && g3m[p] == 0.0f) {
                 const float dx = p ? q.dgx.y : q.dgx.x, dy = p ? q.dgy.y : q.dgy.x, dz = p ? q.dgz.y : q.dgz.x;
@@ -218,7 +183,7 @@ __device__ __forceinline__ void frag_count(const Stage& st, int j, int k, const 
 #pragma unroll
             for (int p = 0; p < PPT; ++p) {
                 const unsigned long long kk = ((unsigned long long)rq[p] << 32) | __float_as_uint(e.w);
-                n.key[p] = inn[p] && kk < n.key[p] ? kk : n.key[p];
+                q.key[p] = inn[p] && kk < q.key[p] ? kk : q.key[p];
             }
         }
     };
@@ -229,69 +194,183 @@ __device__ __forceinline__ void frag_count(const Stage& st, int j, int k, const 
         post(std::false_type{});
 }
 
-__global__ void __launch_bounds__(RT, 8) frag_count_kernel(FragArgs v)
-{
-    grid_wait();
-    grid_go();
-    __shared__ FragShared s;
-    __shared__ uint32_t s_sum[RT / 32], s_base;
-    const unsigned FULL = 0xffffffffu;
-    const int tile = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const TilePos tp(tile, v.tiles_x);
-    const Cone tc = v.tiles[tile];
-    if (threadIdx.x < 32) walk_ranges(v.wi, v.T, v.geom[tile], tc.c0.y, s.ws);
-    if (threadIdx.x == 0) s.n = 0u;
-    FragPix q;
-    const bool active = frag_start(v, tp, tc.c0, q, s.wc);
-    FragCount c{{0u, 0u}, {0u, 0u}, {KEY_NONE, KEY_NONE}};
-    __syncthreads();
-    frag_walk(
-        v, tc, s, active, [](uint32_t, int) {}, [&](int j, int k) { frag_count(s.st, j, k, q, c); },
-        [&](int g) {  // (one chunk, if the tile keeps a list)
-            if (s.ws.total <= (uint32_t)WALK_BLOCK && s.n <= (uint32_t)FRAG_LIST) {
-#pragma unroll
-                for (int p = 0; p < PPT; ++p)
-                    if (tp.px < v.W && tp.py + 4 * p < v.H)
-                        v.bits[((size_t)g * v.H + tp.py + 4 * p) * v.W + tp.px] = c.bits[p];
-            }
-            c.bits[0] = c.bits[1] = 0u;
-        });
-    // the tile's range of the lists, its pixels in thread order
-    const uint32_t mine = c.cnt[0] + c.cnt[1];
-    uint32_t incl = mine;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(FULL, incl, o);
-        if (lane >= o) incl += y;
+// The count as a step of the walking raster, so tiles of many candidates are
+// shared between CTAs here too (see raster_walk_kernel).  A frame with its
+// backward: 145 -> 138 us at 1024 x 1024 with 10k triangles, where no tile is
+// shared; 3.8 -> 1.4 ms at 128 x 128 with 300k triangles, where all are.
+struct FragStep {
+    using Cones = WarpCones;
+    using In = FragArgs;
+    static constexpr int FEW_BLOCK = WALK_BLOCK;  // a tile of one block can keep its list
+    static constexpr bool SATURATES = false, HOST_OUT = false;
+    __device__ __forceinline__ static bool cull(const Stage& st, int j, const Cones& wc, int warp)
+    {
+        return cone_may_hit(st.s0[j], st.s1[j], st.s2[j], st.s3[j], st.s4[j], wc.c[warp][0], wc.c[warp][1], false);
     }
-    if (lane == 31) s_sum[warp] = incl;
-    __syncthreads();
-    uint32_t before = 0, total = 0;
-#pragma unroll
-    for (int w = 0; w < RT / 32; ++w) {
-        if (w < warp) before += s_sum[w];
-        total += s_sum[w];
+};
+
+struct FragCountStep : FragStep {
+    static constexpr bool SKIPS = false;
+    static constexpr int CTAS = 8;  // 64 registers; 7: 40.2 us, 6: 44.0 us against 39.4 us
+    using Pix = FragCount;
+    using Ctx = WalkCtx<FragArgs>;
+    struct Raw {
+        float4 g[PPT];
+    };
+    __device__ __forceinline__ static void load(const RasterView& view, const In&, const TilePos& tp, Raw& r)
+    {
+        load_pixels(view, tp, r.g);
     }
-    const bool list = s.ws.total <= (uint32_t)WALK_BLOCK && s.n <= (uint32_t)FRAG_LIST;
-    if (threadIdx.x == 0) {
-        s_base = total ? atomicAdd(v.cursor, total) : 0u;
-        v.tile_n[tile] = list ? s.n : 0xffffffffu;
+    __device__ __forceinline__ static bool start(const Raw& r, const float4& axis, Pix& q, Cones& wc)
+    {
+        q.acc[0] = q.acc[1] = q.bits[0] = q.bits[1] = 0u;
+        q.key[0] = q.key[1] = KEY_NONE;
+        return frag_start(r.g, axis, q, wc);
     }
-    if (list && threadIdx.x < s.n) v.tile_ids[(size_t)tile * FRAG_LIST + threadIdx.x] = s.ids[threadIdx.x];
-    __syncthreads();
-    uint32_t off = s_base + before + incl - mine;
+    __device__ __forceinline__ static bool skip(const In&, int) { return false; }
+    __device__ __forceinline__ static void clamp(Pix&) {}
+    __device__ __forceinline__ static void eval(const Ctx&, const Stage& st, int j, Pix& q) { frag_count(st, j, q); }
+    __device__ __forceinline__ static uint32_t final_acc(const Pix& q, int p) { return q.acc[p]; }
+    // does the tile keep a list?  (known with its only block's hits)
+    __device__ __forceinline__ static bool list(const Ctx& cx)
+    {
+        return cx.wt.nblk <= 1u && cx.wt.slot < 0 && cx.wt.n <= (uint32_t)FRAG_LIST;
+    }
+    __device__ __forceinline__ static void group(const Ctx& cx, int g, Pix& q)
+    {
+        if (list(cx)) {
+            const FragArgs& v = cx.in;
+            const TilePos tp(cx.wt.tile, v.tiles_x);
 #pragma unroll
-    for (int p = 0; p < PPT; ++p) {
-        if (tp.px < v.W && tp.py + 4 * p < v.H) {
-            const size_t o = (size_t)(tp.py + 4 * p) * v.W + tp.px;
-            v.span[o] = make_uint2(off, c.cnt[p]);
-            const bool hit = c.key[p] != KEY_NONE;
-            if (v.out_id) v.out_id[o] = hit ? (uint32_t)(c.key[p] & 0xffffffffull) : 0xffffffffu;
-            if (v.out_depth) v.out_depth[o] = hit ? __uint_as_float((uint32_t)(c.key[p] >> 32) + 1u) : INFINITY;
+            for (int p = 0; p < PPT; ++p)
+                if (tp.px < v.W && tp.py + 4 * p < v.H)
+                    v.bits[((size_t)g * v.H + tp.py + 4 * p) * v.W + tp.px] = q.bits[p];
         }
-        off += c.cnt[p];
+        q.bits[0] = q.bits[1] = 0u;
     }
-}
+    // the tile's range of the lists, its pixels in thread order
+    template <bool ROWS>
+    __device__ __forceinline__ static void finish(const Ctx& cx, const TilePos& tp, const Pix& q, int*)
+    {
+        __shared__ uint32_t s_sum[RT / 32], s_base;
+        const FragArgs& v = cx.in;
+        const int tile = cx.wt.tile, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        const uint32_t mine = q.acc[0] + q.acc[1];
+        uint32_t incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) s_sum[warp] = incl;
+        __syncthreads();
+        uint32_t before = 0, total = 0;
+#pragma unroll
+        for (int w = 0; w < RT / 32; ++w) {
+            if (w < warp) before += s_sum[w];
+            total += s_sum[w];
+        }
+        const bool keep = list(cx);
+        const uint32_t n = cx.wt.n;
+        if (threadIdx.x == 0) {
+            s_base = total ? atomicAdd(v.cursor, total) : 0u;
+            v.tile_n[tile] = keep ? n : 0xffffffffu;
+            if (!keep) atomicAdd(v.cursor + 1, 1u);
+        }
+        if (keep && threadIdx.x < n) v.tile_ids[(size_t)tile * FRAG_LIST + threadIdx.x] = cx.ids[threadIdx.x];
+        __syncthreads();
+        uint32_t off = s_base + before + incl - mine;
+#pragma unroll
+        for (int p = 0; p < PPT; ++p) {
+            if (tp.px < v.W && tp.py + 4 * p < v.H) {
+                const size_t o = (size_t)(tp.py + 4 * p) * v.W + tp.px;
+                v.span[o] = make_uint2(off, q.acc[p]);
+                const bool hit = q.key[p] != KEY_NONE;
+                if (v.out_id) v.out_id[o] = hit ? (uint32_t)(q.key[p] & 0xffffffffull) : 0xffffffffu;
+                if (v.out_depth) v.out_depth[o] = hit ? __uint_as_float((uint32_t)(q.key[p] >> 32) + 1u) : INFINITY;
+            }
+            off += q.acc[p];
+        }
+    }
+};
+
+// The fill of the tiles without a list: walked and evaluated again, fragments
+// appended to their pixels' lists in any order (a shared tile's parts take
+// their places from the slot's accumulators) and sorted by the part that
+// finishes the tile.
+struct FragAppend : FragPix {
+    uint32_t at[PPT], room[PPT];  // the pixel's list
+    uint32_t acc[PPT];            // fragments appended (a shared tile: counted in its slot)
+    unsigned long long key[PPT];  // unused
+};
+struct FragFillStep : FragStep {
+    static constexpr bool SKIPS = true;
+    static constexpr int CTAS = 5;
+    using Pix = FragAppend;
+    using Ctx = WalkCtx<FragArgs>;
+    struct Raw {
+        float4 g[PPT];
+        uint32_t at[PPT], room[PPT];
+    };
+    __device__ __forceinline__ static void load(const RasterView& view, const In& v, const TilePos& tp, Raw& r)
+    {
+        load_pixels(view, tp, r.g);
+#pragma unroll
+        for (int p = 0; p < PPT; ++p) {
+            uint2 s = make_uint2(0u, 0u);
+            if (tp.px < v.W && tp.py + 4 * p < v.H) s = v.span[(size_t)(tp.py + 4 * p) * v.W + tp.px];
+            r.at[p] = s.x;
+            r.room[p] = (uint64_t)s.x + s.y <= v.fcap ? s.y : 0u;  // (finish reports a list cut short)
+        }
+    }
+    __device__ __forceinline__ static bool start(const Raw& r, const float4& axis, Pix& q, Cones& wc)
+    {
+#pragma unroll
+        for (int p = 0; p < PPT; ++p) {
+            q.at[p] = r.at[p];
+            q.room[p] = r.room[p];
+            q.acc[p] = 0u;
+            q.key[p] = KEY_NONE;
+        }
+        return frag_start(r.g, axis, q, wc);
+    }
+    __device__ __forceinline__ static bool skip(const In& v, int tile) { return v.tile_n[tile] <= (uint32_t)FRAG_LIST; }
+    __device__ __forceinline__ static void clamp(Pix&) {}
+    __device__ __forceinline__ static void group(const Ctx&, int, Pix&) {}
+    __device__ __forceinline__ static uint32_t final_acc(const Pix& q, int p) { return q.acc[p]; }
+    __device__ __forceinline__ static void eval(const Ctx& cx, const Stage& st, int j, Pix& q)
+    {
+        FragEval o;
+        if (!frag_eval(st, j, q, o)) return;
+        const FragArgs& v = cx.in;
+        const uint32_t t = __float_as_uint(st.s6[j].w);
+        const float colour = v.colors ? v.colors[t] : 1.0f;
+        const int slot = cx.wt.slot;
+        const TilePos tp(0, 1);
+#pragma unroll
+        for (int p = 0; p < PPT; ++p) {
+            if (!o.f[p]) continue;
+            const uint32_t u = slot < 0 ? q.acc[p]++
+                                        : (uint32_t)atomicAdd(&cx.slots.split.acc[(size_t)slot * TILE_PIX + tp.lx +
+                                                                                  TILE * (tp.ly + 4 * p)],
+                                                              1ull);
+            if (u < q.room[p]) v.frags[(size_t)q.at[p] + u] = frag_record(o, q, p, t, colour);
+        }
+    }
+    template <bool ROWS>
+    __device__ __forceinline__ static void finish(const Ctx& cx, const TilePos& tp, const Pix& q, int* status)
+    {
+        const FragArgs& v = cx.in;
+#pragma unroll 1
+        for (int p = 0; p < PPT; ++p) {
+            if (tp.px >= v.W || tp.py + 4 * p >= v.H) continue;
+            const uint32_t n = p ? q.acc[1] : q.acc[0], room = p ? q.room[1] : q.room[0];
+            // spans of another frame, or no room (see FragArgs::early)
+            if (n != room && !(v.early && room == 0u)) raise_status(status, VSR_ERR_FRAG_OVERFLOW);
+            frag_merge(v, (size_t)(tp.py + 4 * p) * v.W + tp.px, v.frags + (p ? q.at[1] : q.at[0]), min(n, room));
+        }
+    }
+};
 
 // fragments of a pixel sorted in shared memory; a longer list is sorted where
 // it is stored
@@ -301,160 +380,111 @@ __global__ void __launch_bounds__(RT, 6) frag_fill_kernel(FragArgs v)
 {
     grid_wait();
     grid_go();
-    __shared__ union {
-        FragShared walk;
-        struct {
-            Stage st;
-            float4 rec[FRAG_SORT][RT];
-        } list;
-    } s;
+    __shared__ Stage st;
+    __shared__ float4 rec[FRAG_SORT][RT];
     __shared__ float scol[STAGE_CHUNK];
+    __shared__ WarpCones wc;
     const unsigned FULL = 0xffffffffu;
     const int tile = blockIdx.x;
     const TilePos tp(tile, v.tiles_x);
-    const Cone tc = v.tiles[tile];
-    if (tile == 0 && threadIdx.x == 0) *v.cursor = 0u;  // for the next frame
+    if (tile == 0 && threadIdx.x < 2) v.cursor[threadIdx.x] = 0u;  // for the next frame
     const uint32_t n = v.tile_n[tile];
-    FragPix q;
+    if (n > (uint32_t)FRAG_LIST) return;
+    const Cone tc = v.tiles[tile];
+    if (threadIdx.x < n) {
+        const uint32_t t = v.tile_ids[(size_t)tile * FRAG_LIST + threadIdx.x];
+        stage_checked(v.rec, v.T, t, tc.c0, st, threadIdx.x, v.status);
+        scol[threadIdx.x] = v.colors && t < (uint32_t)v.T ? v.colors[t] : 1.0f;
+    }
+    float4 gp[PPT];
     uint2 span[PPT] = {};
     bool inimg[PPT];
 #pragma unroll
     for (int p = 0; p < PPT; ++p) {
         inimg[p] = tp.px < v.W && tp.py + 4 * p < v.H;
-        if (inimg[p]) span[p] = v.span[(size_t)(tp.py + 4 * p) * v.W + tp.px];
+        gp[p] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (inimg[p]) {
+            gp[p] = v.map[(size_t)(tp.py + 4 * p) * v.W + tp.px];
+            span[p] = v.span[(size_t)(tp.py + 4 * p) * v.W + tp.px];
+        }
     }
+    FragPix q;
+    frag_start(gp, tc.c0, q, wc);
     // (beyond the buffer: only before the host has sized it)
     const bool fits = (uint64_t)span[0].x + span[0].y <= v.fcap && (uint64_t)span[1].x + span[1].y <= v.fcap;
     if (!fits) {
         if (!v.early) raise_status(v.status, VSR_ERR_FRAG_OVERFLOW);
         span[0].y = span[1].y = 0u;
     }
-    uint32_t cnt[PPT] = {0u, 0u};
-    bool sorted[PPT] = {false, false};
-    auto put = [&](const FragEval& o, int p, uint32_t t, float colour) {
-        // append (lists that are not sorted on their way in)
-        if (cnt[p] < span[p].y) v.frags[(size_t)span[p].x + cnt[p]] = frag_record(o, q, p, t, colour);
-        ++cnt[p];
-    };
-    if (n <= (uint32_t)FRAG_LIST) {
-        __shared__ WarpCones wc;
-        if (threadIdx.x < n) {
-            const uint32_t t = v.tile_ids[(size_t)tile * FRAG_LIST + threadIdx.x];
-            stage_checked(v.rec, v.T, t, tc.c0, s.list.st, threadIdx.x, v.status);
-            scol[threadIdx.x] = v.colors && t < (uint32_t)v.T ? v.colors[t] : 1.0f;
-        }
-        frag_start(v, tp, tc.c0, q, wc);
-        uint4 bits[PPT];
-#pragma unroll
-        for (int p = 0; p < PPT; ++p) {
-            const uint32_t* __restrict__ at = v.bits + (size_t)(tp.py + 4 * p) * v.W + tp.px;
-            const size_t pic = (size_t)v.H * v.W;
-            const bool some = inimg[p] && span[p].y;
-            bits[p].x = some ? at[0] : 0u;
-            bits[p].y = some && n > 32u ? at[pic] : 0u;
-            bits[p].z = some && n > 64u ? at[2 * pic] : 0u;
-            bits[p].w = some && n > 96u ? at[3 * pic] : 0u;
-            sorted[p] = span[p].y <= FRAG_SORT;
-        }
-        __syncthreads();
-        // (one pixel's list at a time in shared memory: the first pixels of
-        // the lanes, then the second)
-#pragma unroll
-        for (int p = 0; p < PPT; ++p) {
-#pragma unroll
-            for (int g = 0; g < 4; ++g) {
-                const uint32_t b = g == 0 ? bits[p].x : (g == 1 ? bits[p].y : (g == 2 ? bits[p].z : bits[p].w));
-                unsigned any = __reduce_or_sync(FULL, b);
-                while (any) {
-                    const int k = 31 - __clz(any);
-                    any ^= 1u << k;
-                    const int j = 32 * g + k;
-                    if (!(b >> k & 1u)) continue;
-                    // this pixel's distances in scalar form (bit for bit the packed ones)
-                    const float dx = p ? q.dgx.y : q.dgx.x, dy = p ? q.dgy.y : q.dgy.x, dz = p ? q.dgz.y : q.dgz.x;
-                    const float4 c = s.list.st.s1[j], e = s.list.st.s6[j];
-                    const float g4 = miter_distance(dx, dy, dz, e, c, p ? q.eg.y : q.eg.x);
-                    const float g3m = fminf(fminf(plane_distance(dx, dy, dz, s.list.st.s2[j]),
-                                                  plane_distance(dx, dy, dz, s.list.st.s3[j])),
-                                            plane_distance(dx, dy, dz, s.list.st.s4[j]));
-                    const float D = plane_distance(dx, dy, dz, s.list.st.s5[j]);
-                    const float4 x = make_float4(__fdividef(c.w, D), e.w,
-                                                 __saturatef(fmaf(fminf(g3m, g4), q.delta[p], 0.5f)),
-                                                 scol[j] * fabsf(D));
-                    if (cnt[p] >= span[p].y) {
-                        ++cnt[p];  // spans of another frame: reported below
-                    } else if (sorted[p]) {
-                        uint32_t u = cnt[p];
-                        while (u > 0 && frag_less(x, s.list.rec[u - 1][threadIdx.x])) {
-                            s.list.rec[u][threadIdx.x] = s.list.rec[u - 1][threadIdx.x];
-                            --u;
-                        }
-                        s.list.rec[u][threadIdx.x] = x;
-                        ++cnt[p];
-                    } else {
-                        v.frags[(size_t)span[p].x + cnt[p]] = x;
-                        ++cnt[p];
-                    }
-                }
-            }
-            if (!sorted[p] || !inimg[p]) continue;
-            // the pixel's merge, and its list
-            float mb = 0.0f, img = 0.0f;
-            for (uint32_t u = 0; u < min(cnt[p], span[p].y); ++u) {
-                const float4 x = s.list.rec[u][threadIdx.x];
-                v.frags[(size_t)span[p].x + u] = x;
-                if (mb < 1.0f) {
-                    const float mfc = fminf(x.z, 1.0f - mb);
-                    img = fmaf(mfc, x.w, img);
-                    mb += mfc;
-                }
-            }
-            const size_t o = (size_t)(tp.py + 4 * p) * v.W + tp.px;
-            if (v.image) v.image[o] = img;
-            if (v.cov) v.cov[o] = mb;
-        }
-    } else {
-        if (threadIdx.x < 32) walk_ranges(v.wi, v.T, v.geom[tile], tc.c0.y, s.walk.ws);
-        if (threadIdx.x == 0) s.walk.n = 0u;
-        const bool active = frag_start(v, tp, tc.c0, q, s.walk.wc);
-        __syncthreads();
-        frag_walk(
-            v, tc, s.walk, active,
-            [&](uint32_t t, int j) { scol[j] = v.colors && t < (uint32_t)v.T ? v.colors[t] : 1.0f; },
-            [&](int j, int) {
-                FragEval o;
-                if (!frag_eval(s.walk.st, j, q, o)) return;
-                const uint32_t t = __float_as_uint(s.walk.st.s6[j].w);
-#pragma unroll
-                for (int p = 0; p < PPT; ++p)
-                    if (o.f[p]) put(o, p, t, scol[j]);
-            },
-            [](int) {});
-    }
+    uint4 bits[PPT];
 #pragma unroll
     for (int p = 0; p < PPT; ++p) {
-        if (!inimg[p]) continue;
-        if (fits && cnt[p] != span[p].y) raise_status(v.status, VSR_ERR_FRAG_OVERFLOW);  // spans of another frame
-        if (sorted[p]) continue;
-        const size_t o = (size_t)(tp.py + 4 * p) * v.W + tp.px;
-        const uint32_t m = min(cnt[p], span[p].y);
-        float4* F = v.frags + span[p].x;
-        // insertion sort by (r, t)
-        for (uint32_t u = 1; u < m; ++u) {
-            const float4 x = F[u];
-            uint32_t w = u;
-            while (w > 0 && frag_less(x, F[w - 1])) {
-                F[w] = F[w - 1];
-                --w;
+        const uint32_t* __restrict__ at = v.bits + (size_t)(tp.py + 4 * p) * v.W + tp.px;
+        const size_t pic = (size_t)v.H * v.W;
+        const bool some = inimg[p] && span[p].y;
+        bits[p].x = some ? at[0] : 0u;
+        bits[p].y = some && n > 32u ? at[pic] : 0u;
+        bits[p].z = some && n > 64u ? at[2 * pic] : 0u;
+        bits[p].w = some && n > 96u ? at[3 * pic] : 0u;
+    }
+    __syncthreads();
+    // (one pixel's list at a time in shared memory: the first pixels of
+    // the lanes, then the second)
+#pragma unroll
+    for (int p = 0; p < PPT; ++p) {
+        const bool sorted = span[p].y <= FRAG_SORT;
+        uint32_t cnt = 0u;
+#pragma unroll
+        for (int g = 0; g < FRAG_LIST / 32; ++g) {
+            const uint32_t b = g == 0 ? bits[p].x : (g == 1 ? bits[p].y : (g == 2 ? bits[p].z : bits[p].w));
+            unsigned any = __reduce_or_sync(FULL, b);
+            while (any) {
+                const int k = 31 - __clz(any);
+                any ^= 1u << k;
+                const int j = 32 * g + k;
+                if (!(b >> k & 1u)) continue;
+                // this pixel's distances in scalar form (bit for bit the packed ones)
+                const float dx = p ? q.dgx.y : q.dgx.x, dy = p ? q.dgy.y : q.dgy.x, dz = p ? q.dgz.y : q.dgz.x;
+                const float4 c = st.s1[j], e = st.s6[j];
+                const float g4 = miter_distance(dx, dy, dz, e, c, p ? q.eg.y : q.eg.x);
+                const float g3m = fminf(fminf(plane_distance(dx, dy, dz, st.s2[j]), plane_distance(dx, dy, dz, st.s3[j])),
+                                        plane_distance(dx, dy, dz, st.s4[j]));
+                const float D = plane_distance(dx, dy, dz, st.s5[j]);
+                const float4 x = make_float4(__fdividef(c.w, D), e.w, __saturatef(fmaf(fminf(g3m, g4), q.delta[p], 0.5f)),
+                                             scol[j] * fabsf(D));
+                if (cnt < span[p].y) {  // (else spans of another frame: reported below)
+                    uint32_t u = cnt;
+                    if (sorted) {
+                        while (u > 0 && frag_less(x, rec[u - 1][threadIdx.x])) {
+                            rec[u][threadIdx.x] = rec[u - 1][threadIdx.x];
+                            --u;
+                        }
+                        rec[u][threadIdx.x] = x;
+                    } else {
+                        v.frags[(size_t)span[p].x + u] = x;
+                    }
+                }
+                ++cnt;
             }
-            F[w] = x;
         }
+        if (!inimg[p]) continue;
+        if (fits && cnt != span[p].y) raise_status(v.status, VSR_ERR_FRAG_OVERFLOW);  // spans of another frame
+        const size_t o = (size_t)(tp.py + 4 * p) * v.W + tp.px;
+        const uint32_t m = min(cnt, span[p].y);
+        if (!sorted) {
+            frag_merge(v, o, v.frags + span[p].x, m);
+            continue;
+        }
+        // the pixel's merge, and its list
         float mb = 0.0f, img = 0.0f;
-        for (uint32_t u = 0; u < m && mb < 1.0f; ++u) {
-            const float4 x = F[u];
-            const float mfc = fminf(x.z, 1.0f - mb);
-            img = fmaf(mfc, x.w, img);
-            mb += mfc;
+        for (uint32_t u = 0; u < m; ++u) {
+            const float4 x = rec[u][threadIdx.x];
+            v.frags[(size_t)span[p].x + u] = x;
+            if (mb < 1.0f) {
+                const float mfc = fminf(x.z, 1.0f - mb);
+                img = fmaf(mfc, x.w, img);
+                mb += mfc;
+            }
         }
         if (v.image) v.image[o] = img;
         if (v.cov) v.cov[o] = mb;
@@ -754,16 +784,27 @@ __global__ void __launch_bounds__(128) setup_backward_kernel(const float* __rest
 
 }  // namespace
 
-vsr_status launch_frag_count(const FragArgs& a, cudaStream_t st)
+namespace {
+RasterView frag_view(const FragArgs& a)
 {
-    VSR_CUDA_TRY(launch_next(frag_count_kernel, a.tiles_x * ((a.H + TILE - 1) / TILE), RT, st, a));
-    return VSR_OK;
+    return RasterView{a.map, a.W, a.H, a.tiles, a.tiles_x, a.rec, a.T, nullptr, nullptr, 0u, nullptr, nullptr, nullptr};
+}
+}  // namespace
+
+vsr_status launch_frag_count(const FragArgs& a, const WalkWork& work, cudaStream_t st)
+{
+    return launch_walk<FragCountStep>(frag_view(a), a, a.wi, a.geom, work, nullptr, a.status, st, false);
 }
 
 vsr_status launch_frag_fill(const FragArgs& a, cudaStream_t st)
 {
     VSR_CUDA_TRY(launch_next(frag_fill_kernel, a.tiles_x * ((a.H + TILE - 1) / TILE), RT, st, a));
     return VSR_OK;
+}
+
+vsr_status launch_frag_fill_walk(const FragArgs& a, const WalkWork& work, cudaStream_t st)
+{
+    return launch_walk<FragFillStep>(frag_view(a), a, a.wi, a.geom, work, nullptr, a.status, st, false);
 }
 
 vsr_status launch_frag_backward(const FragArgs& a, const uint32_t* id, const float* dimage, const float* dcov,

@@ -15,7 +15,8 @@ struct vsr_frags_s {
     bool dirty = true;            // the cursor is not known to be zero
     float4* frags = nullptr;
     uint32_t fcap = 0;
-    uint32_t* h_total = nullptr;  // pinned
+    bool unlisted = false;        // the last frame had tiles without a list
+    uint32_t* h_total = nullptr;  // pinned: fragments, tiles without a list
     cudaEvent_t counted = nullptr;  // the total is in h_total
     float4* dmap = nullptr;       // npix
     float* lens_part = nullptr;
@@ -50,7 +51,7 @@ vsr_status frags_ensure_pixels(vsr_frags f, int W, int H, size_t ntiles, cudaStr
 {
     const size_t n = (size_t)W * H;
     vsr_status s;
-    if (!f->cursor && (s = dalloc(&f->cursor, 1)) != VSR_OK) return s;
+    if (!f->cursor && (s = dalloc(&f->cursor, 2)) != VSR_OK) return s;
     if (n <= f->npix && ntiles <= f->ntiles) return VSR_OK;
     frags_release_pixels(f);
     if ((s = dalloc(&f->span, n)) != VSR_OK || (s = dalloc(&f->bits, n * (FRAG_LIST / 32))) != VSR_OK ||
@@ -102,7 +103,7 @@ vsr_status vsr_frags_create(vsr_frags* out)
     *out = nullptr;
     vsr_frags f = new (std::nothrow) vsr_frags_s;
     if (!f) return VSR_ERR_OOM;
-    if (cudaMallocHost((void**)&f->h_total, sizeof(uint32_t)) != cudaSuccess ||
+    if (cudaMallocHost((void**)&f->h_total, 2 * sizeof(uint32_t)) != cudaSuccess ||
         cudaEventCreateWithFlags(&f->counted, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
         if (f->h_total) cudaFreeHost(f->h_total);
@@ -139,10 +140,10 @@ vsr_status vsr_raster_shaded(vsr_map m, vsr_scene sc, const float* colors_dev, v
     FragArgs a = frag_args(m, sc, colors_dev, f);
     a.out_id = id_dev;
     a.out_depth = depth_dev;
-    if (f->dirty) VSR_CUDA_TRY(cudaMemsetAsync(f->cursor, 0, sizeof(uint32_t), st));
+    if (f->dirty) VSR_CUDA_TRY(cudaMemsetAsync(f->cursor, 0, 2 * sizeof(uint32_t), st));
     f->dirty = true;  // until the fill, which clears it, is queued
-    if ((s = launch_frag_count(a, st)) != VSR_OK) return s;
-    VSR_CUDA_TRY(cudaMemcpyAsync(f->h_total, f->cursor, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+    if ((s = launch_frag_count(a, sc->walk, st)) != VSR_OK) return s;
+    VSR_CUDA_TRY(cudaMemcpyAsync(f->h_total, f->cursor, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
     VSR_CUDA_TRY(cudaEventRecord(f->counted, st));
     a.image = image_dev;
     a.cov = cov_dev;
@@ -151,14 +152,15 @@ vsr_status vsr_raster_shaded(vsr_map m, vsr_scene sc, const float* colors_dev, v
     // device does not stand still for the host's round trip (1024^2 pixels, 10k
     // triangles, a frame with its backward: 158.7 us before, 153.0 with it).
     // If it was not, once more with more.
-    const bool early = f->fcap > 0;
+    const bool early = f->fcap > 0, early_walk = early && f->unlisted;
     if (early) {
         a.early = true;
         if ((s = launch_frag_fill(a, st)) != VSR_OK) return s;
+        if (early_walk && (s = launch_frag_fill_walk(a, sc->walk, st)) != VSR_OK) return s;
         a.early = false;
     }
     VSR_CUDA_TRY(cudaEventSynchronize(f->counted));
-    const uint32_t total = *f->h_total;
+    const uint32_t total = f->h_total[0], unlisted = f->h_total[1];
     if (total > f->fcap) {
         cudaFree(f->frags);
         f->frags = nullptr;
@@ -168,11 +170,14 @@ vsr_status vsr_raster_shaded(vsr_map m, vsr_scene sc, const float* colors_dev, v
         if ((s = dalloc(&f->frags, (size_t)want)) != VSR_OK) return s;
         f->fcap = (uint32_t)want;
     }
-    if (!early || a.fcap != f->fcap) {
+    const bool again = !early || a.fcap != f->fcap;
+    if (again) {
         a.frags = f->frags;
         a.fcap = f->fcap;
         if ((s = launch_frag_fill(a, st)) != VSR_OK) return s;
     }
+    f->unlisted = unlisted > 0;
+    if (f->unlisted && (again || !early_walk) && (s = launch_frag_fill_walk(a, sc->walk, st)) != VSR_OK) return s;
     f->dirty = false;
     f->map_gen = m->gen;
     f->scene_gen = sc->gen;

@@ -48,6 +48,8 @@ __device__ __forceinline__ float2 width2(const PstepPix& q, const float4& n)
 __device__ __forceinline__ float ramp(float g, float w) { return __fmaf_rn(g, rcp_fast(fmaxf(w, 1e-30f)), 0.5f); }
 
 struct PstepStep {
+    static constexpr int FEW_BLOCK = WALK_BLOCK / 4;
+    static constexpr bool SATURATES = true, HOST_OUT = false, SKIPS = false;
     static constexpr int CTAS = 6;  // 80 registers; 5: 135.3 us, 4: 142.7 us against 130.4 us
     using Pix = PstepPix;
     using Cones = PstepCones;
@@ -134,7 +136,7 @@ struct PstepStep {
                fmaf(c0.x, n3.x, fmaf(c0.y, n3.y, c0.z * n3.z)) > lim;
     }
     // staged slot j at the lane's two pixels; all 32 lanes together
-    __device__ __forceinline__ static void eval(const Stage& st, int j, Pix& q)
+    __device__ __forceinline__ static void eval(const WalkCtx<In>&, const Stage& st, int j, Pix& q)
     {
         const float4 a = st.s0[j], b = st.s1[j], e = st.s6[j];
         const float4 n1 = st.s2[j], n2 = st.s3[j], n3 = st.s4[j];
@@ -185,6 +187,18 @@ struct PstepStep {
             post(std::false_type{});
     }
     __device__ __forceinline__ static uint32_t final_acc(const Pix& q, int p) { return min(q.acc[p], COV_ONE); }
+    __device__ __forceinline__ static void group(const WalkCtx<In>&, int, Pix&) {}
+    __device__ __forceinline__ static bool skip(const In&, int) { return false; }
+    __device__ __forceinline__ static void clamp(Pix& q)
+    {
+#pragma unroll
+        for (int p = 0; p < PPT; ++p) q.acc[p] = min(q.acc[p], COV_ONE);
+    }
+    template <bool ROWS>
+    __device__ __forceinline__ static void finish(const WalkCtx<In>& cx, const TilePos& tp, const Pix& q, int*)
+    {
+        write_tile<ROWS>(cx.view, tp, q);
+    }
 };
 
 }  // namespace

@@ -198,7 +198,8 @@ __device__ __forceinline__ void eval_chunk(const Stage& st, int n, const WarpCon
 
 // The global step for the walking raster.
 struct GlobalStep {
-    static constexpr int CTAS = VSR_RASTER_CTAS_PER_SM;
+    static constexpr int CTAS = VSR_RASTER_CTAS_PER_SM, FEW_BLOCK = WALK_BLOCK / 4;
+    static constexpr bool SATURATES = true, HOST_OUT = true, SKIPS = false;
     using Pix = PixPair;
     using Cones = WarpCones;
     struct In {};
@@ -217,12 +218,24 @@ struct GlobalStep {
     {
         return cone_may_hit(st.s0[j], st.s1[j], st.s2[j], st.s3[j], st.s4[j], wc.c[warp][0], wc.c[warp][1], false);
     }
-    __device__ __forceinline__ static void eval(const Stage& st, int j, Pix& q)
+    __device__ __forceinline__ static void eval(const WalkCtx<In>&, const Stage& st, int j, Pix& q)
     {
         uint32_t unused = 0;
         eval_slot<false>(st, j, q, unused);
     }
     __device__ __forceinline__ static uint32_t final_acc(const Pix& q, int p) { return ::final_acc(q, p); }
+    __device__ __forceinline__ static void group(const WalkCtx<In>&, int, Pix&) {}
+    __device__ __forceinline__ static bool skip(const In&, int) { return false; }
+    __device__ __forceinline__ static void clamp(Pix& q)
+    {
+#pragma unroll
+        for (int p = 0; p < PPT; ++p) q.acc[p] = min(q.acc[p], COV_ONE);
+    }
+    template <bool ROWS>
+    __device__ __forceinline__ static void finish(const WalkCtx<In>& cx, const TilePos& tp, const Pix& q, int*)
+    {
+        write_tile<ROWS>(cx.view, tp, q);
+    }
 };
 
 template <bool STATS, bool ROWS = false>
@@ -546,9 +559,9 @@ vsr_status launch_raster_items(const RasterView& view, const uint32_t* offsets, 
 vsr_status walk_work_alloc(WalkWork* w, cudaStream_t st)
 {
     if (w->mem) return VSR_OK;
-    // accumulators | keys | claims | done | nblk | hits | hint, active
+    // accumulators | keys | claims | done | nblk | hits | hint, active, begun, ended
     const size_t pix = sizeof(unsigned long long) * TILE_PIX * (size_t)WALK_SLOTS;
-    const size_t rest = sizeof(unsigned long long) * WALK_SLOTS + 3 * sizeof(uint32_t) * WALK_SLOTS + 2 * sizeof(uint32_t);
+    const size_t rest = sizeof(unsigned long long) * WALK_SLOTS + 3 * sizeof(uint32_t) * WALK_SLOTS + 4 * sizeof(uint32_t);
     char* m = nullptr;
     if (cudaMalloc((void**)&m, 2 * pix + rest) != cudaSuccess) {
         cudaGetLastError();

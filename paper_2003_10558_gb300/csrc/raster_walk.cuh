@@ -25,8 +25,10 @@ namespace {
 // so one made on a slot that has changed hands is still a claim of the slot's
 // present tile; a claim past the tile's last block is no block.  While a part
 // holds unmerged blocks its slot cannot be freed.  Nobody waits for another,
-// but that helpers which start together with the tiles (fewer tiles than
-// resident CTAs) look again for about 10 us before they give up.
+// but that helpers which may start before the tiles have been published
+// (`early`: fewer tiles than resident CTAs, or tiles that are skipped) look
+// until every tile has got that far, 100 us at most: 480 x 480 pixels, 5000
+// triangles 31 us a frame against 51 with 10 us of looks each.
 struct WalkSlots {
     SplitAcc split;             // WALK_SLOTS accumulators
     unsigned long long* claim;  // WALK_SLOTS: (tile << 32) | blocks claimed
@@ -34,6 +36,8 @@ struct WalkSlots {
     uint32_t* hits;             // WALK_SLOTS: hits of the parts merged so far
     uint32_t* hint;             // where the next owner looks first
     uint32_t* active;           // published tiles
+    uint32_t* begun;            // tiles published or known not to be (zero between launches)
+    uint32_t* ended;            // CTAs that have ended (zero between launches)
 };
 
 // What a CTA knows of its tile, in shared memory: uniform, and needed only
@@ -46,12 +50,22 @@ struct WalkTile {
     uint32_t n;            // hits of the current block
 };
 
+// What a step's evaluation may want besides the staged triangle and the pixels.
+template <class In>
+struct WalkCtx {
+    const RasterView& view;
+    const In& in;
+    const WalkSlots& slots;
+    const WalkTile& wt;
+    const uint32_t* ids;  // the current block's hits
+};
+
 // The n staged triangles of a chunk at the warp's pixels: a lane-parallel cull
 // of 32 triangles at a time against the warp's cone, then the survivors one by
 // one.
 template <class Step>
-__device__ __forceinline__ void walk_eval(const Stage& st, int n, const typename Step::Cones& wc,
-                                          typename Step::Pix& q)
+__device__ __forceinline__ void walk_eval(const WalkCtx<typename Step::In>& cx, const Stage& st, int n,
+                                          const typename Step::Cones& wc, typename Step::Pix& q)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int gbase = 0; gbase < n; gbase += 32) {
@@ -62,17 +76,19 @@ __device__ __forceinline__ void walk_eval(const Stage& st, int n, const typename
         while (mask) {
             const int k = 31 - __clz(mask);  // any order: from the top, one instruction less than from the bottom
             mask ^= 1u << k;
-            Step::eval(st, gbase + k, q);
+            Step::eval(cx, st, gbase + k, q);
         }
+        Step::group(cx, gbase / 32, q);
     }
 }
 
-// Step: how pixels are loaded, culled against and evaluated (the global step
-// of raster.cu, the per-fragment step of pstep.cu).
+// Step: how pixels are loaded, culled against, evaluated and written (the
+// global step of raster.cu, the per-fragment step of pstep.cu, the fragment
+// lists of grad.cu).
 template <class Step, bool ROWS>
 __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView view, typename Step::In in, WalkIndex wi,
                                                                      const float4* __restrict__ geom, int ntiles,
-                                                                     uint32_t block, uint32_t split_blocks, int looks,
+                                                                     uint32_t block, uint32_t split_blocks, bool early,
                                                                      WalkSlots slots,
                                                                      uint32_t* __restrict__ tile_pairs,
                                                                      int* __restrict__ status)
@@ -86,7 +102,18 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
     __shared__ uint32_t s_ids[WALK_BLOCK];
     static_assert(RT == WALK_THREADS, "the walk's CTA");
     const bool helper = blockIdx.x >= (uint32_t)ntiles;
-    for (;;) {
+    int looks = early ? 400 : 0;
+    // a tile is past its publication
+    auto begun = [&] {
+        if (early) {
+            __threadfence();
+            atomicAdd(slots.begun, 1u);
+        }
+    };
+    const bool skip = !helper && Step::skip(in, (int)blockIdx.x);
+    if (skip && threadIdx.x == 0) begun();
+    const WalkCtx<typename Step::In> cx{view, in, slots, wt, s_ids};
+    while (!skip) {
         typename Step::Pix q;
         bool warp_active;
         {
@@ -97,14 +124,15 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
                 // a start of this CTA's own
                 __syncthreads();
                 if (threadIdx.x == 0) {
-                    while (!*(volatile uint32_t*)slots.active && looks > 0) {
-                        --looks;
+                    for (; looks > 0 && !*(volatile uint32_t*)slots.active &&
+                           *(volatile uint32_t*)slots.begun < (uint32_t)ntiles;
+                         --looks)
                         __nanosleep(250);
-                    }
+                    __threadfence();
                     wt.slot = *(volatile uint32_t*)slots.active ? WALK_SLOTS : -1;
                 }
                 __syncthreads();
-                if (wt.slot < 0) return;
+                if (wt.slot < 0) break;
                 const int from = (int)((blockIdx.x * 37u) % WALK_SLOTS);
                 int mine = WALK_SLOTS;
                 for (int i = threadIdx.x; i < WALK_SLOTS && mine == WALK_SLOTS; i += RT) {
@@ -117,7 +145,7 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
                 if (mine < WALK_SLOTS) atomicMin(&wt.slot, mine);
                 __syncthreads();
                 slot = wt.slot;
-                if (slot == WALK_SLOTS) return;
+                if (slot == WALK_SLOTS) break;
                 slot = (from + slot) % WALK_SLOTS;
                 if (threadIdx.x == 0) {
                     const unsigned long long c = atomicAdd(&slots.claim[slot], 1ull);
@@ -127,7 +155,7 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
                 __syncthreads();
                 tile = wt.tile;
                 first = wt.next;
-                if (tile >= ntiles) return;
+                if (tile >= ntiles) break;
             }
             const float4 axis = view.tiles[tile].c0;
             typename Step::Raw g;
@@ -154,6 +182,7 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
                 wt.nblk = nblk;
                 wt.next = first;
                 wt.units = wt.hits = wt.n = 0u;
+                if (!helper) begun();
             }
             warp_active = Step::start(g, axis, q, wc);
             __syncthreads();
@@ -169,13 +198,12 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
             __syncthreads();
             for (uint32_t base = 0; base < wt.n; base += CHUNK) {
                 const int nc = (int)min((uint32_t)CHUNK, wt.n - base);
-#pragma unroll
-                for (int p = 0; p < PPT; ++p) q.acc[p] = min(q.acc[p], COV_ONE);
+                Step::clamp(q);
                 if (base) __syncthreads();
                 if ((int)threadIdx.x < nc)
                     stage_checked(view.rec, view.T, s_ids[base + threadIdx.x], wt.cone.c0, st, threadIdx.x, status);
                 __syncthreads();
-                if (warp_active) walk_eval<Step>(st, nc, wc, q);
+                if (warp_active) walk_eval<Step>(cx, st, nc, wc, q);
             }
             // the only block of a tile that is not shared (almost every tile):
             // no one waits for the others' evaluation
@@ -197,7 +225,7 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
         bool last = true;
         if (slot >= 0) {
             if (threadIdx.x == 0 && hits) atomicAdd(&slots.hits[slot], hits);
-            last = merge_slot(slots.split, slot, tp, q, wt.units, wt.nblk);
+            last = merge_slot<Step::SATURATES>(slots.split, slot, tp, q, wt.units, wt.nblk);
             if (last) {
                 __threadfence();
                 __syncthreads();
@@ -211,9 +239,16 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
         }
         if (last) {
             if (tile_pairs && threadIdx.x == 0) tile_pairs[tile] = hits;
-            write_tile<ROWS>(view, tp, q);
+            Step::template finish<ROWS>(cx, tp, q, status);
         }
-        if (!helper) return;
+        if (!helper) break;
+    }
+    if (early && threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(slots.ended, 1u) == gridDim.x - 1) {
+            atomicExch(slots.begun, 0u);
+            atomicExch(slots.ended, 0u);
+        }
     }
 }
 
@@ -237,16 +272,19 @@ inline vsr_status launch_walk(const RasterView& view, const typename Step::In& i
     sl.hits = sl.nblk + WALK_SLOTS;
     sl.hint = sl.hits + WALK_SLOTS;
     sl.active = sl.hint + 1;
+    sl.begun = sl.hint + 2;
+    sl.ended = sl.hint + 3;
     // helpers only where a tile can have enough candidates; few tiles: smaller
     // blocks, handed out from the second on
     const int wave = sms * Step::CTAS;
     const bool few = ntiles < wave;
-    const int block = few ? WALK_BLOCK / 4 : WALK_BLOCK;
+    const int block = few ? Step::FEW_BLOCK : WALK_BLOCK;
     const int split = few ? 2 : (int)WALK_SPLIT_BLOCKS;
     const int helpers = view.T > split * block ? wave : 0;
-    auto kern = host_out ? raster_walk_kernel<Step, true> : raster_walk_kernel<Step, false>;
+    auto kern = raster_walk_kernel<Step, false>;
+    if constexpr (Step::HOST_OUT) kern = host_out ? raster_walk_kernel<Step, true> : kern;
     VSR_CUDA_TRY(launch_next(kern, ntiles + helpers, RT, st, view, in, wi, geom, ntiles, (uint32_t)block,
-                             (uint32_t)split, few ? 40 : 0, sl, tile_pairs, status));
+                             (uint32_t)split, helpers && (few || Step::SKIPS), sl, tile_pairs, status));
     return VSR_OK;
 }
 

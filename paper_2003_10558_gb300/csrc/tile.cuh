@@ -158,8 +158,8 @@ __device__ __forceinline__ void stage_checked(const float4* __restrict__ rec, in
 // Merge the lane's pixels into accumulator slot `slot` of a tile processed in
 // several parts; the part that brings the count of `done` units to `target`
 // gets the tile's result in q, clears the slot and returns true.  Called by
-// every thread of the CTA.
-template <class Pix>
+// every thread of the CTA.  SATURATES: the sum is a coverage, at most COV_ONE.
+template <bool SATURATES = true, class Pix>
 __device__ __forceinline__ bool merge_slot(const SplitAcc& split, int slot, const TilePos& tp, Pix& q,
                                            uint32_t units, uint32_t target)
 {
@@ -180,7 +180,8 @@ __device__ __forceinline__ bool merge_slot(const SplitAcc& split, int slot, cons
     __threadfence();
 #pragma unroll
     for (int p = 0; p < PPT; ++p) {
-        q.acc[p] = (uint32_t)min(atomicExch(&sacc[lp0 + TILE * 4 * p], 0ull), (unsigned long long)COV_ONE);
+        const unsigned long long sum = atomicExch(&sacc[lp0 + TILE * 4 * p], 0ull);
+        q.acc[p] = (uint32_t)(SATURATES ? min(sum, (unsigned long long)COV_ONE) : sum);
         q.key[p] = min(atomicExch(&skey[lp0 + TILE * 4 * p], ~0ull), KEY_NONE);
     }
     if (threadIdx.x == 0) split.done[slot] = 0u;

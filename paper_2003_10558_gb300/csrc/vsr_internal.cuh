@@ -435,7 +435,7 @@ struct WalkWork {
 // (cleared on st; a launch leaves the slots as it found them)
 vsr_status walk_work_alloc(WalkWork* w, cudaStream_t st);
 void walk_work_free(WalkWork* w);
-constexpr size_t WALK_WORK_BYTES = (size_t)WALK_SLOTS * (16 * TILE_PIX + 20) + 8;
+constexpr size_t WALK_WORK_BYTES = (size_t)WALK_SLOTS * (16 * TILE_PIX + 20) + 16;
 // view: no bins needed; tile_pairs (optional): the triangles found per tile;
 // host_out: as launch_raster_items
 vsr_status launch_raster_walk(const RasterView& view, const WalkIndex& wi, const float4* geom, const WalkWork& work,
@@ -478,8 +478,8 @@ struct FragArgs {
     int T;
     WalkIndex wi;
     const float* colors;  // per triangle, NULL = 1
-    uint32_t* cursor;     // fragments given out (zero before the count, cleared by the fill)
-    uint32_t* tile_n;     // per tile: its triangles, or ~0 (more than FRAG_LIST)
+    uint32_t* cursor;     // fragments given out, tiles without a list (zero before the count, cleared by the fill)
+    uint32_t* tile_n;     // per tile: its triangles, or ~0: no list (see grad.cu)
     uint32_t* tile_ids;   // per tile: FRAG_LIST of them
     uint2* span;          // per pixel: (first fragment, fragments)
     uint32_t* bits;       // FRAG_LIST / 32 pictures: a bit per triangle of the tile's list that is a fragment
@@ -492,8 +492,9 @@ struct FragArgs {
     float* out_depth;
     int* status;
 };
-vsr_status launch_frag_count(const FragArgs& a, cudaStream_t st);
-vsr_status launch_frag_fill(const FragArgs& a, cudaStream_t st);
+vsr_status launch_frag_count(const FragArgs& a, const WalkWork& work, cudaStream_t st);
+vsr_status launch_frag_fill(const FragArgs& a, cudaStream_t st);  // tiles with a list; clears the cursor
+vsr_status launch_frag_fill_walk(const FragArgs& a, const WalkWork& work, cudaStream_t st);  // the others
 vsr_status launch_frag_backward(const FragArgs& a, const uint32_t* id, const float* dimage, const float* dcov,
                                 const float* ddepth, float4* grad, float4* dmap, cudaStream_t st);
 // (clears the record gradients it reads)
