@@ -674,7 +674,9 @@ vsr_status scene_walk_begin(vsr_map m, vsr_scene sc, cudaStream_t st)
 }
 
 // One frame of (m, s) without statistics.  The walking raster needs no bins
-// (1920x1080, 220k triangles: see the figures at raster_walk_kernel), but the
+// (1920x1080, 220k triangles: 124 us instead of 38 us of binning, 3 us of work
+// items and 103 us of raster; 4096x2176, 1M: 544 us instead of 148 + 3 + 450),
+// but the
 // first frame of a shape goes through stored ones, as does every frame of a
 // scene that renders again on a bin overflow (async_sizing): the bins are
 // then allocated and sized, with the one synchronisation of a new shape, and
@@ -685,6 +687,8 @@ static vsr_status raster_frame(vsr_map m, vsr_scene sc, uint32_t* id_dev, float*
     if (!m || !sc) return VSR_ERR_INVALID_ARG;
     vsr_status s;
     if (sc->async_sizing || !bins_sized(m, sc, 0)) {
+        // (and the next frame, which walks, allocates nothing either)
+        if (!sc->async_sizing && (s = walk_work_alloc(&sc->walk, st)) != VSR_OK) return s;
         if ((s = bin_scene(m, sc, 0, st)) != VSR_OK) return s;
         return raster_tiles(m, sc, id_dev, depth_dev, cov_dev, nullptr, st, host_out);
     }

@@ -10,10 +10,12 @@ namespace {
 // Binning and raster in one launch: every tile's CTA walks its candidates
 // (walk.cuh) WALK_BLOCK at a time, lists the hits in shared memory and
 // rasterizes them, so the bins are never stored and no pass over the tiles
-// runs before.  Against the tile pass, the heavy-tile pass, the work-item pass
-// and the raster over stored bins (four launches), the walk's latency is
-// hidden by the other CTAs' evaluation (see the measured figures at
-// vsr_raster).
+// runs before; the walk's latency is hidden by the other CTAs' evaluation.
+// 1920x1080, 220k triangles: 123.5 us, against 45 us for a tile-major binning
+// in three launches, 3 us for the work items and 103 us for this evaluation
+// over stored bins.  Bound by instruction issue (63 % of the cycles, 8 CTAs of
+// 64 registers per SM): about half of the 94 M warp instructions are the
+// evaluation, the rest staging, culls, the walk and the prologue.
 //
 // A tile with many candidates is processed by several CTAs that merge in an
 // accumulator slot (merge_slot): the tile's own CTA takes a free slot and
@@ -274,11 +276,16 @@ inline vsr_status launch_walk(const RasterView& view, const typename Step::In& i
     sl.active = sl.hint + 1;
     sl.begun = sl.hint + 2;
     sl.ended = sl.hint + 3;
-    // helpers only where a tile can have enough candidates; few tiles: smaller
-    // blocks, handed out from the second on
+    // Helpers only where a tile can have enough candidates.  A tile is shared
+    // from its fourth block of 1024 on (1M triangles at 1920x1080, a 340 degree
+    // lens: 912 us; from the second 1417, from the ninth 1149).  Few tiles:
+    // smaller blocks, shared from the third on (200k triangles at 256x256:
+    // 142 us; in blocks of 512 159 us, of 1024 193 us), but one block without
+    // a grid (900 triangles at 256x256: 19 us, shared in blocks of 256 41 us).
     const int wave = sms * Step::CTAS;
     const bool few = ntiles < wave;
-    const int block = few ? Step::FEW_BLOCK : WALK_BLOCK;
+    static_assert(GRID_DIRECT <= WALK_BLOCK, "one block");
+    const int block = few && !wi.direct ? Step::FEW_BLOCK : WALK_BLOCK;
     const int split = few ? 2 : (int)WALK_SPLIT_BLOCKS;
     const int helpers = view.T > split * block ? wave : 0;
     auto kern = raster_walk_kernel<Step, false>;

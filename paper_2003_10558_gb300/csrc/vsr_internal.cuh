@@ -281,9 +281,13 @@ constexpr int GRID_H_CURSOR = 4;  // entries given to rows, while filing
 constexpr int GRID_H_MAX = 8;     // [8 .. 11] the filed triangles' largest sin(cap radius) per level, 0: level empty
 constexpr int GRID_H_N = 12;      // entries
 constexpr int GRID_HDR = 16;
-// scenes of up to this many triangles have no grid: every tile tests them
-// all, two steps of a CTA (the two filing launches cost more, ~5 us)
-constexpr int GRID_DIRECT = 256;
+// Scenes of up to this many triangles have no grid: every tile tests them all,
+// at most five steps of a CTA, against two filing launches and the search for
+// its ranges.  us a frame, without and with a grid: 400 triangles 17.8 / 24.8
+// at 256x256, 55.5 / 66.3 at 1920x1080; 600 triangles 18.6 / 29.4, 59.8 / 67.5,
+// and 201 / 216 at 4096x2176, but 768 triangles 258 / 254 there with a wide
+// lens, and 1024 triangles 242 / 228.
+constexpr int GRID_DIRECT = 640;
 struct TriGrid {
     uint32_t* counts = nullptr;  // GRID_WORDS: triangles counted per cell, then left to place; zero between set-ups
     uint32_t* start = nullptr;   // GRID_WORDS: first entry of each cell, each row closed by its end

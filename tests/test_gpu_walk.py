@@ -49,7 +49,7 @@ def _crowd(n, spread, seed):
 
 def _mixed(n, seed):
     """Caps of every level and of the list, and some culled triangles."""
-    parts = [scenes.random_triangles(max(1, n // 4), 1.0, 30.0, j, seed + q)
+    parts = [scenes.random_triangles(-(-n // 4), 1.0, 30.0, j, seed + q)
              for q, j in enumerate((0.004, 0.03, 0.12, 0.9))]
     t = np.concatenate(parts)[:n] if n < 4 else np.concatenate(parts)
     t = t[:n]
@@ -63,8 +63,9 @@ CASES = [
     # W, H, k, l, s, omega, triangles, rotation
     (64, 48, 0.2, 0.9, 0.9, 120.0, lambda: np.zeros((0, 3, 3), np.float32), None),
     (33, 17, 0.2, 0.9, 0.9, 120.0, lambda: _mixed(1, 1), None),
-    (160, 96, 0.3, 0.8, 0.9, 200.0, lambda: _mixed(256, 2), 3),   # the last direct count
-    (160, 96, 0.3, 0.8, 0.9, 200.0, lambda: _mixed(257, 2), 3),   # the first with a grid
+    (160, 96, 0.3, 0.8, 0.9, 200.0, lambda: _mixed(257, 2), 3),
+    (160, 96, 0.3, 0.8, 0.9, 200.0, lambda: _mixed(640, 2), 3),   # the last direct count
+    (160, 96, 0.3, 0.8, 0.9, 200.0, lambda: _mixed(641, 2), 3),   # the first with a grid
     (251, 143, -0.4, 0.7, 0.8, 300.0, lambda: _mixed(6000, 4), 5),
     (40, 24, -0.2, 1.0, 1.0, 360.0, lambda: _mixed(5000, 6), 7),  # tiles of a radian and more
     (16, 16, 0.0, 1.0, 1.0, 360.0, lambda: _mixed(3000, 8), None),  # one tile, the whole sphere
@@ -115,4 +116,26 @@ def test_tiles_after_an_unstored_frame(vsr):
         b = vsr.raster(m, sc, binned=True)
         for key in a:
             assert torch.equal(a[key].view(torch.int32), b[key].view(torch.int32)), key
+    assert vsr.last_device_status() == 0
+
+
+@pytest.mark.parametrize("T", [200, 5000])
+def test_second_frame_under_capture(vsr, T):
+    """The second frame of a shape is the first that walks: nothing is left
+    for it to allocate, so it can be captured."""
+    sc = vsr.Scene(torch.from_numpy(scenes.random_triangles(T, 1.0, 30.0, 0.05, 16)).cuda(), scenes.camera())
+    m = vsr.Map(200, 120, 0.2, 0.9, 0.9, 150.0)
+    first = vsr.raster(m, sc)
+    out = {key: torch.empty_like(t) for key, t in first.items()}
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        vsr.raster(m, sc, out=out)
+    for _ in range(3):
+        for t in out.values():
+            t.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        for key in first:
+            assert torch.equal(out[key].view(torch.int32), first[key].view(torch.int32)), key
     assert vsr.last_device_status() == 0
