@@ -41,10 +41,9 @@ WORKLOAD = "single-view 1920x1080, k=0.32 l=0.62 s=0.86 Omega=270, icosphere L5 
 UNIT = "tests/s"
 OPS_PER_TEST = 20  # FP32 ops of one algorithmic test: 4 three-term dots (12 FMA), 3 min, ramp FMA, 4 compares
 LANES_PER_SM = 128  # FP32 lanes per Blackwell SM
-# kernels of libvsr.so per step: map (the map stream), set-up, triangle
-# filing, tile bins, work items, raster (the memsets between them are not
-# kernels of the library)
-LAUNCHES_PER_STEP = 6
+# kernels of libvsr.so per step: map (the map stream), set-up, the triangle
+# grid's rows and entries, raster (which finds each tile's triangles itself)
+LAUNCHES_PER_STEP = 5
 
 
 def parse():
@@ -84,9 +83,9 @@ def workload():
     return lens, tris, cam
 
 
-RASTER_SOURCES = ("paper_2003_10558_gb300/csrc/raster.cu", "paper_2003_10558_gb300/csrc/stage.cuh",
-                  "paper_2003_10558_gb300/csrc/df.cuh", "paper_2003_10558_gb300/csrc/vsr_internal.cuh")
-RASTER_PROFILE = "raster_items_kernel_1080p_single_view.md"
+RASTER_SOURCES = tuple("paper_2003_10558_gb300/csrc/" + f for f in (
+    "raster.cu", "raster_walk.cuh", "walk.cuh", "tile.cuh", "stage.cuh", "df.cuh", "df2.cuh", "vsr_internal.cuh"))
+RASTER_PROFILE = "raster_walk_kernel_1080p_single_view.md"
 
 
 def raster_traffic():
@@ -284,12 +283,9 @@ def run_vsr(args, rank, world, local):
         stream.wait_event(ev_map)
         if evs:
             evs[0].record(stream)
-        V.bin(m, sc)  # a3
+        V.raster(m, sc, out=out)  # a3 + a4 + a5
         if evs:
             evs[1].record(stream)
-        V.raster(m, sc, out=out, binned=True)  # a4 + a5
-        if evs:
-            evs[2].record(stream)
 
     # algorithmic units of one step (counted once, untimed)
     V.bin(m, sc)
@@ -311,7 +307,7 @@ def run_vsr(args, rank, world, local):
         return torch.cuda.Event(enable_timing=True)
 
     ev0 = [evt() for _ in range(K)]
-    stage = [[evt() for _ in range(3)] for _ in range(K)]
+    stage = [[evt() for _ in range(2)] for _ in range(K)]
     with ClockSampler(local) as clk:
         clk.load(lambda: (flush.fill_(1.0), step()))
         torch.cuda.synchronize()
@@ -323,11 +319,10 @@ def run_vsr(args, rank, world, local):
         if world > 1:
             dist.barrier()
     assert V.last_device_status() == 0
-    step_ms = [a.elapsed_time(st_[2]) for a, st_ in zip(ev0, stage)]
-    rast_ms = [st_[1].elapsed_time(st_[2]) for st_ in stage]
+    step_ms = [a.elapsed_time(st_[1]) for a, st_ in zip(ev0, stage)]
+    rast_ms = [st_[0].elapsed_time(st_[1]) for st_ in stage]  # binning included
     stage_ms = {"map||setup": statistics.mean(a.elapsed_time(s[0]) for a, s in zip(ev0, stage)),
-                "bin": statistics.mean(s[0].elapsed_time(s[1]) for s in stage),
-                "raster": statistics.mean(rast_ms)}
+                "bin+raster": statistics.mean(rast_ms)}
     # the two overlapped stages alone (untimed diagnostics)
     for name, fn in (("map", lambda: m.update(W, H, lens["k"], lens["l"], lens["s"], lens["omega"])),
                      ("setup", lambda: sc.update(tris, cam))):
@@ -346,14 +341,13 @@ def run_vsr(args, rank, world, local):
         flush.fill_(float(k))
         c0[k].record(stream)
         sc.update(tris, cam)
-        V.bin(m, sc)
-        V.raster(m, sc, out=out, binned=True)
+        V.raster(m, sc, out=out)
         c1[k].record(stream)
     torch.cuda.synchronize()
     assert V.last_device_status() == 0
     cached_ms = statistics.mean(a.elapsed_time(b) for a, b in zip(c0, c1))
-    # the per-fragment pixel step on the same frame (binning for its wider
-    # caps + raster), a quality variant: mean of K calls
+    # the per-fragment pixel step on the same frame (with its wider caps), a
+    # quality variant: mean of K calls
     pm = V.Map.from_spec(V.MAP_UNIVERSAL, W, H, (lens["k"], lens["l"], lens["s"], lens["omega"]), derivatives=True)
     ps_sc = V.Scene(tris, cam)
     V.raster_pstep(pm, ps_sc, out=out)
@@ -380,8 +374,7 @@ def run_vsr(args, rank, world, local):
         a.record(stream)
         dm.update(W, H, lens["k"], lens["l"], lens["s"], lens["omega"], aov=V.AOV_DIAGONAL)
         dsc.update(tris, cam)
-        V.bin(dm, dsc)
-        V.raster(dm, dsc, out=out, binned=True)
+        V.raster(dm, dsc, out=out)
         b.record(stream)
         diag_ms.append((a, b))
     torch.cuda.synchronize()
@@ -408,8 +401,8 @@ def run_vsr(args, rank, world, local):
         dense_ms = a.elapsed_time(b) / KD
         dense = {"kernel": "raster_dense_kernel", "ms": dense_ms, "launches": KD,
                  "pair_tests_per_frame": W * H * T,
-                 "binned_bin_plus_raster_ms": stage_ms["bin"] + stage_ms["raster"],
-                 "speedup_binned_vs_dense": dense_ms / (stage_ms["bin"] + stage_ms["raster"]),
+                 "binned_bin_plus_raster_ms": stage_ms["bin+raster"],
+                 "speedup_binned_vs_dense": dense_ms / stage_ms["bin+raster"],
                  "outputs_identical": bool(same)}
         del ref, dout
     # replicas: tests summed over ranks, time of the slowest rank
@@ -557,7 +550,7 @@ def run_vsr(args, rank, world, local):
                                       "step": "map, set-up, binning, raster in sequence on one stream"}},
         "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_ops / 1e12, "unit": "Tops/s (FP32)",
                      "frac": achieved / peak_ops, "traffic": traffic,
-                     "kernel": "raster_items_kernel", "peak_source": f"{props.multi_processor_count} SMs x "
+                     "kernel": "raster_walk_kernel", "peak_source": f"{props.multi_processor_count} SMs x "
                      f"{LANES_PER_SM} FP32 lanes x {sm_mhz:.0f} MHz ({pk_kind} sm_max_mhz)"},
         "clocks": clk.summary(),
         "gpu_launches": LAUNCHES_PER_STEP * K,

@@ -230,8 +230,9 @@ vsr_status vsr_raster(vsr_map m, vsr_scene s, uint32_t* id_dev, float* depth_dev
  * (S-hat . d G)/sin(rho) for the miter, from the map's differences:
  *   fragment iff every g > -w/2 (bpxstep), m^f = min clamp(g/w + 1/2, 0, 1).
  * The map must be made with VSR_MAP_DERIVATIVES (else VSR_ERR_INVALID_ARG).
- * Bins the scene for the wider caps of this step (bins that vsr_raster_tiles
- * may reuse).  Outputs as vsr_raster. */
+ * The first call for a tile count and T bins the scene for the wider caps of
+ * this step (bins that vsr_raster_tiles may reuse); later ones find each
+ * tile's triangles as they rasterize it.  Outputs as vsr_raster. */
 vsr_status vsr_raster_pstep(vsr_map m, vsr_scene s, uint32_t* id_dev, float* depth_dev, float* cov_dev,
                             void* stream);
 
@@ -487,9 +488,9 @@ typedef struct vsr_frags_s* vsr_frags;
 vsr_status vsr_frags_create(vsr_frags* out);
 void vsr_frags_free(vsr_frags f);
 
-/* vsr_raster_shaded: bins (as vsr_raster), counts the fragments of every
- * pixel, sizes the lists (one synchronisation of `stream` per call: the
- * fragment total is read back), fills, sorts and merges them.
+/* vsr_raster_shaded: finds each tile's triangles (as vsr_raster), counts the
+ * fragments of every pixel, sizes the lists (the call waits for the count and
+ * reads the fragment total back), fills, sorts and merges them.
  * colors_dev: device [T] colour c_t per triangle (NULL: all 1).
  * Outputs (caller-owned device [H][W], any may be NULL): image_dev (I),
  * cov_dev (final m^b of the merge: the coverage of vsr_raster within

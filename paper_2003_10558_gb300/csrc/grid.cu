@@ -377,7 +377,10 @@ vsr_status launch_bin_walk(const float4* rec, int T, const WalkIndex& wi, const 
     const int sms = sm_count();
     if (sms < 0) return VSR_ERR_CUDA;
     // helpers, four CTAs per SM, only where a tile can have enough candidates;
-    // with few tiles they start together with them and look for a while
+    // with few tiles they start together with them and look for a while (the
+    // others would finish the tiles' own blocks later than these start).  A
+    // tile of 4 blocks by itself takes 58 us, about what the rest of a view
+    // does; with few tiles there is nothing to hide 4 behind, so 2.
     const bool few = ntiles < BIN_FEW * sms;
     const uint32_t split = few ? 2u : 4u;
     const int helpers = (uint32_t)T > split * WALK_BLOCK ? 4 * sms : 0;
