@@ -376,6 +376,12 @@ struct FragFillStep : FragStep {
 // it is stored
 constexpr uint32_t FRAG_SORT = 8;
 
+// The fill of the tiles with a list: the evaluations that are fragments, no
+// walk and no cull.  Bound by issue with lanes idle (each triangle's step runs
+// for the pixels that have it) and by the sort; 1024 x 1024, 10k triangles:
+// 28.7 us, 59.7 when every pair was evaluated again and sorted where it was
+// stored, 33.8 while one kernel held the walk of the other tiles too (92
+// registers instead of 72).
 __global__ void __launch_bounds__(RT, 6) frag_fill_kernel(FragArgs v)
 {
     grid_wait();
