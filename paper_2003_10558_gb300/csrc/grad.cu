@@ -797,9 +797,9 @@ RasterView frag_view(const FragArgs& a)
 }
 }  // namespace
 
-vsr_status launch_frag_count(const FragArgs& a, const WalkWork& work, cudaStream_t st)
+vsr_status launch_frag_count(const FragArgs& a, const WalkWork& work, uint32_t* tile_pairs, cudaStream_t st)
 {
-    return launch_walk<FragCountStep>(frag_view(a), a, a.wi, a.geom, work, nullptr, a.status, st, false);
+    return launch_walk<FragCountStep>(frag_view(a), a, a.wi, a.geom, work, tile_pairs, a.status, st, false);
 }
 
 vsr_status launch_frag_fill(const FragArgs& a, cudaStream_t st)

@@ -142,7 +142,7 @@ vsr_status vsr_raster_shaded(vsr_map m, vsr_scene sc, const float* colors_dev, v
     a.out_depth = depth_dev;
     if (f->dirty) VSR_CUDA_TRY(cudaMemsetAsync(f->cursor, 0, 2 * sizeof(uint32_t), st));
     f->dirty = true;  // until the fill, which clears it, is queued
-    if ((s = launch_frag_count(a, sc->walk, st)) != VSR_OK) return s;
+    if ((s = launch_frag_count(a, sc->walk, sc->tile_pairs, st)) != VSR_OK) return s;
     VSR_CUDA_TRY(cudaMemcpyAsync(f->h_total, f->cursor, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
     VSR_CUDA_TRY(cudaEventRecord(f->counted, st));
     a.image = image_dev;

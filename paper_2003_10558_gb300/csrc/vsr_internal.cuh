@@ -496,7 +496,8 @@ struct FragArgs {
     float* out_depth;
     int* status;
 };
-vsr_status launch_frag_count(const FragArgs& a, const WalkWork& work, cudaStream_t st);
+// tile_pairs: the triangles found per tile, as launch_raster_walk
+vsr_status launch_frag_count(const FragArgs& a, const WalkWork& work, uint32_t* tile_pairs, cudaStream_t st);
 vsr_status launch_frag_fill(const FragArgs& a, cudaStream_t st);  // tiles with a list; clears the cursor
 vsr_status launch_frag_fill_walk(const FragArgs& a, const WalkWork& work, cudaStream_t st);  // the others
 vsr_status launch_frag_backward(const FragArgs& a, const uint32_t* id, const float* dimage, const float* dcov,

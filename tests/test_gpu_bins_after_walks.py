@@ -1,0 +1,59 @@
+"""Stored bins and pair counts after frames that stored none."""
+import numpy as np
+import pytest
+
+from paper_2003_10558_gb300 import scenes
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def vsr():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2003_10558_gb300 import build, vsr as V
+    build.build()
+    V.load()
+    return V
+
+
+def _half(n, seed):
+    """n triangles of which all but a few lie around the world's +z axis."""
+    t = scenes.random_triangles(n, 2.0, 20.0, 0.05, seed).astype(np.float64)
+    c = t.mean(axis=1, keepdims=True)
+    rng = np.random.default_rng(seed)
+    d = np.stack([rng.normal(0, 0.2, n), rng.normal(0, 0.2, n), np.ones(n)], 1)
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    moved = (t - c + np.linalg.norm(c, axis=2, keepdims=True) * d[:, None, :]).astype(np.float32)
+    moved[:50] = scenes.random_triangles(50, 2.0, 20.0, 0.05, seed + 1)
+    return moved
+
+
+def _turned(a):
+    """A camera that looks at angle a from +z."""
+    c, s = np.cos(a), np.sin(a)
+    return scenes.camera((0.0, 0.0, 0.0), np.array([[c, 0.0, s], [0.0, 1.0, 0.0], [-s, 0.0, c]]))
+
+
+def test_pairs_of_a_shaded_frame(vsr):
+    """The pair count of a shaded forward is that of its own view."""
+    tris = torch.from_numpy(_half(5000, 6)).cuda()
+    m = vsr.Map(200, 120, 0.2, 0.9, 0.9, 90.0)
+    sc, frags = vsr.Scene(tris, _turned(0.3)), vsr.Frags()
+    for q in range(3):
+        vsr.raster_shaded(m, sc, frags)
+        shaded = sc.bin_pairs()
+        vsr.bin(m, sc)
+        assert sc.bin_pairs() == shaded, q
+        m.update(200, 120, 0.3, 0.8, 0.9, 60.0 + 40.0 * q)
+        sc.update(tris, _turned(0.8 - 0.4 * q))
+    # 24 x 16 pixels of 20,000 triangles: every tile's candidates are shared
+    # between several CTAs
+    tris = torch.from_numpy(_half(20_000, 7)).cuda()
+    m, sc = vsr.Map(24, 16, 0.2, 0.9, 0.9, 90.0), vsr.Scene(tris, _turned(0.0))
+    vsr.raster_shaded(m, sc, frags)
+    shaded = sc.bin_pairs()
+    vsr.bin(m, sc)
+    assert sc.bin_pairs() == shaded
+    assert vsr.last_device_status() == 0
