@@ -242,13 +242,16 @@ vsr_status vsr_raster_pstep(vsr_map m, vsr_scene s, uint32_t* id_dev, float* dep
  * (made first, if the last vsr_raster of (m, s) stored none) and returns
  * VSR_ERR_INVALID_ARG if there is neither a binning nor a vsr_raster of this
  * map and set-up.
- * Bins are sized with one synchronisation of `stream` the first time and
- * whenever the map's tile count or the scene's T changes; otherwise no call
- * synchronises: the bins grow ahead of need from the pair count of an earlier
- * binning, and a binning that still outgrows them (e.g. after the camera
- * moved) raises VSR_ERR_BIN_OVERFLOW in the device status
+ * Bins are sized with one synchronisation of `stream` the first time,
+ * whenever the map's tile count or the scene's T changes, and where frames
+ * that stored no bins (vsr_raster and others) came since the last binning;
+ * otherwise no call synchronises: the bins grow ahead of need from the pair
+ * count of an earlier binning, and a binning that still outgrows them (e.g.
+ * after the camera moved) raises VSR_ERR_BIN_OVERFLOW in the device status
  * (vsr_last_device_status) with that frame's outputs incomplete, the next
- * call growing the bins. */
+ * call growing the bins.  A binning inside a stream capture keeps the bins
+ * as they are: vsr_bin of the densest view to come, before the capture,
+ * makes the room. */
 vsr_status vsr_bin(vsr_map m, vsr_scene s, void* stream);
 
 /* Diagnostics of one rasterization (all optional, NULL to skip). */

@@ -564,14 +564,18 @@ static vsr_status bin_scene(vsr_map m, vsr_scene sc, int pstep, cudaStream_t st)
     if (s != VSR_OK) return s;
     const int T = (int)sc->T;
     sc->last_ntiles = ntiles;
-    // Bin capacity.  Sized synchronously the first time and whenever the
-    // number of tiles or triangles changes (the first time only, for a scene
-    // with async_sizing); otherwise the pair total of the previous binning
-    // (copied to pinned memory, read only once its event has completed, never
-    // waited for) grows the capacity ahead of need, and the binning kernels
-    // report any overflow in the status word.
-    const bool resize = !bins_sized(m, sc, pstep);
-    if (!resize && sc->total_pending && cudaEventQuery(sc->total_event) == cudaSuccess) {
+    // Bin capacity.  Sized synchronously the first time, whenever the number
+    // of tiles or triangles changes, and where frames have walked since the
+    // last binning, whose totals the host has not seen (the first time only,
+    // for a scene with async_sizing); otherwise the pair total of the previous
+    // binning (copied to pinned memory, read only once its event has
+    // completed, never waited for) grows the capacity ahead of need, and the
+    // binning kernels report any overflow in the status word.  A capture can
+    // neither wait nor query: it takes the bins as they are.
+    bool captures;
+    if ((s = stream_captures(st, &captures)) != VSR_OK) return s;
+    const bool resize = !bins_sized(m, sc, pstep) || (sc->walked_last && !sc->async_sizing && !captures);
+    if (!resize && !captures && sc->total_pending && cudaEventQuery(sc->total_event) == cudaSuccess) {
         sc->total_pending = false;
         const uint64_t last = *sc->h_total;
         if (last + last / 8 > sc->cap) {
@@ -583,7 +587,7 @@ static vsr_status bin_scene(vsr_map m, vsr_scene sc, int pstep, cudaStream_t st)
     // the pair total also goes to the pinned host word (its device address)
     // unless an earlier total has not been read yet -- and always when this
     // binning sizes the bins, which reads this total
-    const bool record = resize || !sc->total_pending;
+    const bool record = resize || (!sc->total_pending && !captures);
     const WalkIndex wi = walk_index(sc->grid, sc->T, pstep);
     auto walk = [&](bool sizing, uint32_t* total_host) {
         return launch_bin_walk(sc->rec, T, wi, m->idx.geom, m->tiles, ntiles, sc->bin_ctr, sc->offsets, sc->ends,
@@ -599,7 +603,6 @@ static vsr_status bin_scene(vsr_map m, vsr_scene sc, int pstep, cudaStream_t st)
     }
     if (resize) {
         VSR_CUDA_TRY(cudaEventSynchronize(sc->total_event));
-        sc->total_pending = false;
         const uint32_t total = *sc->h_total;
         if (total > sc->cap || sc->cap == 0) {
             uint64_t want = (uint64_t)total + total / 4 + 4096;
@@ -607,8 +610,12 @@ static vsr_status bin_scene(vsr_map m, vsr_scene sc, int pstep, cudaStream_t st)
             if ((s = bins_realloc(sc, (uint32_t)want)) != VSR_OK) return s;
             if ((s = walk(false, nullptr)) != VSR_OK) return s;
         }
-        sc->sized_shape = bin_shape_of(m, sc);
-        sc->sized_pstep = pstep != 0;
+        // (a total near the capacity stays to be read by the next binning)
+        sc->total_pending = (uint64_t)total + total / 8 > sc->cap;
+        // (the capacity never shrinks: bins sized for the wider caps stay so)
+        const uint64_t shape = bin_shape_of(m, sc);
+        sc->sized_pstep = pstep != 0 || (sc->sized_pstep && sc->sized_shape == shape);
+        sc->sized_shape = shape;
     }
     sc->binned_map = m->gen;
     sc->binned_scene = sc->gen;
@@ -679,8 +686,8 @@ vsr_status scene_walk_begin(vsr_map m, vsr_scene sc, cudaStream_t st)
 // but the
 // first frame of a shape goes through stored ones, as does every frame of a
 // scene that renders again on a bin overflow (async_sizing): the bins are
-// then allocated and sized, with the one synchronisation of a new shape, and
-// a vsr_raster_tiles that follows later needs neither, also under capture.
+// then allocated and sized, with the one synchronisation of a new shape, so
+// that a vsr_raster_tiles that follows can be captured.
 static vsr_status raster_frame(vsr_map m, vsr_scene sc, uint32_t* id_dev, float* depth_dev, float* cov_dev,
                                cudaStream_t st, bool host_out)
 {

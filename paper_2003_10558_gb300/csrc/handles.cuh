@@ -84,8 +84,8 @@ struct vsr_scene_s {
     // bins sized without waiting for the device when the map's shape changes
     // (the capacity of earlier binnings is kept and only grows): an owner
     // that renders a request again after a bin overflow (the server) needs
-    // no synchronisation per new shape; everyone else gets exact bins on
-    // every call
+    // no synchronisation per new shape; everyone else's bins are sized for
+    // each new shape and after frames that stored none (bin_scene)
     bool async_sizing = false;
     // vsr_render_host runs the set-up on a stream of the scene's own, beside
     // work the caller queued before the call that does not touch the scene
@@ -112,18 +112,27 @@ inline int* scene_status(const vsr_scene_s* s) { return s->status ? s->status : 
 // that they are sized (see raster_frame in api.cu).
 vsr_status scene_walk_begin(vsr_map m, vsr_scene sc, cudaStream_t st);
 
+// Whether work queued on st now is captured, to run when its graph is launched.
+inline vsr_status stream_captures(cudaStream_t st, bool* captures)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+        cudaGetLastError();
+        return VSR_ERR_CUDA;
+    }
+    *captures = cs != cudaStreamCaptureStatusNone;
+    return VSR_OK;
+}
+
 // Note a use of the scene's buffers queued on st (see use_event).
 inline vsr_status scene_used(vsr_scene_s* s, cudaStream_t st)
 {
     if (!s->use_event) return VSR_OK;
     // uses inside a stream capture run when their graph is launched: the
     // caller orders those launches
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
-        cudaGetLastError();
-        return VSR_ERR_CUDA;
-    }
-    if (cs == cudaStreamCaptureStatusNone && cudaEventRecord(s->use_event, st) != cudaSuccess) {
+    bool captures;
+    if (stream_captures(st, &captures) != VSR_OK) return VSR_ERR_CUDA;
+    if (!captures && cudaEventRecord(s->use_event, st) != cudaSuccess) {
         cudaGetLastError();
         return VSR_ERR_CUDA;
     }

@@ -1,4 +1,6 @@
-"""Stored bins and pair counts after frames that stored none."""
+"""Stored bins and pair counts after frames that stored none: a view that goes
+from almost no triangles to most of the scene over frames that bin as they
+rasterize, then every call that reads stored bins."""
 import numpy as np
 import pytest
 
@@ -6,6 +8,8 @@ from paper_2003_10558_gb300 import scenes
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
+
+KEYS = ("id", "depth", "cov")
 
 
 @pytest.fixture(scope="module")
@@ -34,6 +38,38 @@ def _turned(a):
     """A camera that looks at angle a from +z."""
     c, s = np.cos(a), np.sin(a)
     return scenes.camera((0.0, 0.0, 0.0), np.array([[c, 0.0, s], [0.0, 1.0, 0.0], [-s, 0.0, c]]))
+
+
+def _equal(a, b):
+    for key in KEYS:
+        assert torch.equal(a[key].view(torch.int32), b[key].view(torch.int32)), key
+
+
+READERS = {
+    "tiles": lambda vsr, m, sc: vsr.raster(m, sc, binned=True),
+    "statistics": lambda vsr, m, sc: vsr.raster(m, sc, stats=True),
+    "bin": lambda vsr, m, sc: (vsr.bin(m, sc), vsr.raster(m, sc, binned=True))[1],
+}
+
+
+@pytest.mark.parametrize("T", [600, 20_000])
+@pytest.mark.parametrize("reader", sorted(READERS))
+def test_bins_hold_a_denser_view(vsr, reader, T):
+    tris = torch.from_numpy(_half(T, 5)).cuda()
+    m = vsr.Map(320, 240, 0.2, 0.9, 0.9, 60.0)
+    sc = vsr.Scene(tris, _turned(np.pi))
+    vsr.raster(m, sc)  # sized for a view of almost nothing
+    sparse = sc.bin_pairs()
+    for a in np.linspace(np.pi, 0.0, 9)[1:]:
+        sc.update(tris, _turned(a))
+        out = vsr.raster(m, sc)
+    pairs = sc.bin_pairs()
+    assert pairs > 2 * sparse + 8192 or T < 1000
+    ref = vsr.raster_dense(m, sc)
+    _equal(out, ref)
+    _equal(READERS[reader](vsr, m, sc), ref)
+    assert sc.bin_pairs() == pairs
+    assert vsr.last_device_status() == 0
 
 
 def test_pairs_of_a_shaded_frame(vsr):
