@@ -22,7 +22,7 @@ struct vsr_frags_s {
     float* lens_part = nullptr;
     float4* grad = nullptr;       // GF_COUNT x grad_T
     int64_t grad_T = 0;
-    bool grad_clean = false;      // grad is all zero
+    bool grad_clean = false;      // grad is all zero, after the work queued so far and between replays of captured work
     // the forward the lists belong to
     uint64_t map_gen = 0, scene_gen = 0;
     int W = 0, H = 0;
@@ -209,10 +209,16 @@ vsr_status vsr_raster_backward(vsr_map m, vsr_scene sc, const float* tris_dev, c
         f->grad_T = T;
         f->grad_clean = false;
     }
-    // the set-up adjoint leaves the record gradients cleared
-    if (f->grad_T > 0 && !f->grad_clean)
+    // Every backward leaves the record gradients cleared, the set-up adjoint
+    // by itself.  A captured one does so at each replay and changes nothing
+    // before, so the flag stays what it was: a clear that the buffer still
+    // needs is captured with it, and the next eager call has its own.
+    bool captures;
+    if ((s = stream_captures(st, &captures)) != VSR_OK) return s;
+    const bool clean = f->grad_clean;
+    if (f->grad_T > 0 && !clean)
         VSR_CUDA_TRY(cudaMemsetAsync(f->grad, 0, sizeof(float4) * GF_COUNT * (size_t)f->grad_T, st));
-    f->grad_clean = false;
+    f->grad_clean = false;  // until all of it is queued
     FragArgs a = frag_args(m, sc, colors_dev, f);
     if ((s = launch_frag_backward(a, id_dev, dimage_dev, dcov_dev, ddepth_dev, f->grad, f->dmap, st)) != VSR_OK)
         return s;
@@ -220,8 +226,10 @@ vsr_status vsr_raster_backward(vsr_map m, vsr_scene sc, const float* tris_dev, c
         if ((s = launch_setup_backward(tris_dev, (int)T, sc->cam, sc->rec, f->grad, dtris_dev, dcolors_dev, st)) !=
             VSR_OK)
             return s;
-        f->grad_clean = true;
+    } else if (T > 0) {
+        VSR_CUDA_TRY(cudaMemsetAsync(f->grad, 0, sizeof(float4) * GF_COUNT * (size_t)T, st));
     }
+    f->grad_clean = !captures || clean;
     if (dlens_dev) {
         if ((s = launch_map_backward(m->p.W, m->p.H, m->p.aov, m->p.k, m->p.l, m->p.s, m->p.omega_deg, f->dmap,
                                      f->lens_part, dlens_dev, st)) != VSR_OK)
