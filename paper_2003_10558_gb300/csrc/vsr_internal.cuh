@@ -397,6 +397,11 @@ struct RasterWork {
 };
 // SMs of the current device (looked up once per device), or -1.
 int sm_count();
+// Clears (bytes of value `byte`) workspace that the library has just allocated
+// or found dirty: on st, before the launches that follow there; where st
+// captures, at once, since eager work may use it before the graph's first
+// launch, and replays find it as any launch leaves it.
+vsr_status clear_workspace(void* p, int byte, size_t n, cudaStream_t st);
 
 // A view's raster work for the pooled launch: the view, its item assignment
 // (from launch_raster_assign) and its split accumulators.
@@ -436,7 +441,7 @@ constexpr uint32_t WALK_SPLIT_BLOCKS = 3;  // blocks of candidates up to which a
 struct WalkWork {
     char* mem = nullptr;
 };
-// (cleared on st; a launch leaves the slots as it found them)
+// (cleared with clear_workspace; a launch leaves the slots as it found them)
 vsr_status walk_work_alloc(WalkWork* w, cudaStream_t st);
 void walk_work_free(WalkWork* w);
 constexpr size_t WALK_WORK_BYTES = (size_t)WALK_SLOTS * (16 * TILE_PIX + 20) + 16;
@@ -446,9 +451,8 @@ vsr_status launch_raster_walk(const RasterView& view, const WalkIndex& wi, const
                               uint32_t* tile_pairs, int* status, cudaStream_t st, bool host_out = false);
 // the dense reference: every pixel against every triangle, no bins
 vsr_status launch_raster_dense(const RasterView& view, int* status, cudaStream_t st);
-// allocate / free a RasterWork for up to n_tiles tiles (accumulators
-// initialised on st, before the launches that follow there: a clear on another
-// stream would race with them)
+// allocate / free a RasterWork for up to n_tiles tiles (accumulators cleared
+// with clear_workspace: a clear on another stream would race with the launches)
 vsr_status raster_work_alloc(RasterWork* w, uint32_t n_tiles, cudaStream_t st);
 void raster_work_free(RasterWork* w);
 int raster_threads_per_cta();
