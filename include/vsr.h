@@ -320,8 +320,9 @@ vsr_status vsr_scene_bin_pairs(vsr_scene s, void* stream, int64_t* pairs);
  * into the map and returns id/depth/cov (W*H each, host; any may be NULL),
  * then synchronises `stream`.  Same outputs as vsr_raster.  A bin overflow
  * of a frame through stored bins would be rendered again with grown bins
- * before the call returns, and one that persists returned by the call
- * (VSR_ERR_BIN_OVERFLOW) instead of being raised in the per-device status.
+ * before the call returns; one that persists (VSR_ERR_BIN_OVERFLOW), and any
+ * other error that the frame's kernels raise, is returned by the call instead
+ * of being raised in the per-device status.
  * Buffers in pinned host memory mapped into the device's address space
  * (cudaHostAlloc, cudaMallocHost, torch pin_memory) are read and written in
  * place by the kernels over the host link, so the transfers overlap the
@@ -352,7 +353,8 @@ vsr_status vsr_render_host(vsr_map m, vsr_scene s, const float* tris_host, int64
  * vsr_render_host_wait returns VSR_OK (outputs complete),
  * VSR_ERR_BIN_OVERFLOW (the frame outgrew the scene's bins: its outputs are
  * incomplete; the next render of the scene grows them -- render it again),
- * or VSR_ERR_CUDA; VSR_OK also when no frame of `s` is queued. */
+ * another error that its kernels raised, or VSR_ERR_CUDA; VSR_OK also when no
+ * frame of `s` is queued. */
 vsr_status vsr_render_host_async(vsr_map m, vsr_scene s, const float* tris_host, int64_t T, const float cam[12],
                                  uint32_t* id_host, float* depth_host, float* cov_host, void* stream);
 vsr_status vsr_render_host_wait(vsr_scene s);
@@ -427,8 +429,9 @@ void vsr_batch_free(vsr_batch b);
  * requests run, and fails with VSR_ERR_BUDGET if it cannot fit alone.  A
  * request whose bins outgrew their capacity is rendered again with grown
  * bins (counted in `reruns`; the server's workspaces report to status words
- * of their own, so vsr_last_device_status does not see them).  Completion is polled on the host; no device
- * code waits.  Timestamps are seconds of one steady clock (vsr_serve_now). */
+ * of their own, so vsr_last_device_status does not see them); any other error
+ * that its kernels raise is its result's status.  Completion is polled on the
+ * host.  Timestamps are seconds of one steady clock (vsr_serve_now). */
 typedef struct vsr_server_s* vsr_server;
 typedef struct {
     int64_t budget_bytes; /* device memory for maps and workspaces */

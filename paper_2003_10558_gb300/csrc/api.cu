@@ -547,7 +547,7 @@ void vsr_scene_free(vsr_scene sc)
     if (sc->side) cudaStreamDestroy(sc->side);
     if (sc->use_event) cudaEventDestroy(sc->use_event);
     if (sc->setup_event) cudaEventDestroy(sc->setup_event);
-    cudaFree(sc->host_status);
+    sc->host_status.release();
     delete sc;
 }
 
@@ -821,17 +821,14 @@ vsr_status host_frame_front(vsr_map m, vsr_scene sc, const float* tris_host, int
             cudaEventCreateWithFlags(&sc->use_event, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&sc->setup_event, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&sc->host_done, cudaEventDisableTiming) != cudaSuccess ||
-            cudaMalloc((void**)&sc->host_status, sizeof(int)) != cudaSuccess ||
-            cudaMemset(sc->host_status, 0, sizeof(int)) != cudaSuccess) {
+            sc->host_status.alloc(1) != VSR_OK) {
             cudaGetLastError();
             if (sc->side) cudaStreamDestroy(sc->side);
             if (sc->use_event) cudaEventDestroy(sc->use_event);
             if (sc->setup_event) cudaEventDestroy(sc->setup_event);
             if (sc->host_done) cudaEventDestroy(sc->host_done);
-            cudaFree(sc->host_status);
             sc->side = nullptr;
             sc->use_event = sc->setup_event = sc->host_done = nullptr;
-            sc->host_status = nullptr;
             return VSR_ERR_CUDA;
         }
         // uses queued before the tracking began are unknown: this once, the
@@ -883,7 +880,7 @@ vsr_status host_frame_back(vsr_map m, vsr_scene sc, const HostFrame& f, uint32_t
                            float* cov_host, cudaStream_t st)
 {
     int* const saved_status = sc->status;
-    sc->status = sc->host_status;
+    sc->status = sc->host_status.dev;
     vsr_status s = raster_frame(m, sc, f.id_d, f.depth_d, f.cov_d, st, f.in_place);
     sc->status = saved_status;
     if (s == VSR_OK && f.stage_id && cudaMemcpyAsync(id_host, f.id_d, 4 * f.npix, cudaMemcpyDeviceToHost, st))
@@ -897,11 +894,15 @@ vsr_status host_frame_back(vsr_map m, vsr_scene sc, const HostFrame& f, uint32_t
     return s;
 }
 
-// After the frame completed: did it outgrow its bins (the pair total, stored
-// into pinned memory by the scan, above the capacity)?
-bool host_frame_outgrew(vsr_scene sc, uint64_t map_gen)
+// The result of a frame that has completed: VSR_ERR_BIN_OVERFLOW if it
+// outgrew its bins (the pair total, stored into pinned memory by the binning,
+// above the capacity), else what its kernels raised.
+vsr_status host_frame_result(vsr_scene sc, uint64_t map_gen)
 {
-    return sc->total_pending && sc->total_map == map_gen && sc->total_scene == sc->gen && *sc->h_total > sc->cap;
+    const vsr_status raised = sc->host_status.take();
+    const bool outgrew =
+        sc->total_pending && sc->total_map == map_gen && sc->total_scene == sc->gen && *sc->h_total > sc->cap;
+    return outgrew ? VSR_ERR_BIN_OVERFLOW : raised;
 }
 
 }  // namespace
@@ -921,12 +922,14 @@ vsr_status vsr_render_host(vsr_map m, vsr_scene sc, const float* tris_host, int6
     // is rendered again: the next binning grows the bins from its total.
     for (int attempt = 0;; ++attempt) {
         s = host_frame_back(m, sc, f, id_host, depth_host, cov_host, st);
-        if (s == VSR_OK && cudaStreamSynchronize(st) != cudaSuccess) s = VSR_ERR_CUDA;
-        if (s != VSR_OK || !host_frame_outgrew(sc, m->gen)) break;
-        if (attempt == 2) return VSR_ERR_BIN_OVERFLOW;
+        if (s == VSR_OK && cudaStreamSynchronize(st) != cudaSuccess) {
+            cudaGetLastError();
+            s = VSR_ERR_CUDA;
+        }
+        if (s != VSR_OK) return s;
+        s = host_frame_result(sc, m->gen);
+        if (s != VSR_ERR_BIN_OVERFLOW || attempt == 2) return s;
     }
-    if (s != VSR_OK) cudaGetLastError();
-    return s;
 }
 
 vsr_status vsr_render_host_async(vsr_map m, vsr_scene sc, const float* tris_host, int64_t T, const float cam[12],
@@ -954,7 +957,7 @@ vsr_status vsr_render_host_wait(vsr_scene sc)
         cudaGetLastError();
         return VSR_ERR_CUDA;
     }
-    return host_frame_outgrew(sc, sc->host_map_gen) ? VSR_ERR_BIN_OVERFLOW : VSR_OK;
+    return host_frame_result(sc, sc->host_map_gen);
 }
 
 }  // extern "C"

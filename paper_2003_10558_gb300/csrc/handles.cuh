@@ -40,7 +40,41 @@ struct vsr_map_s {
     uint64_t gen = 0;
 };
 
+// Status words in host memory that kernels raise errors in (mapped into the
+// device's address space): zero between frames, read and cleared by the host
+// once a frame's launches have completed.
+struct HostStatus {
+    int* host = nullptr;
+    int* dev = nullptr;
+    vsr_status alloc(int n)
+    {
+        if (cudaHostAlloc((void**)&host, sizeof(int) * (size_t)n, cudaHostAllocMapped) != cudaSuccess ||
+            cudaHostGetDevicePointer((void**)&dev, host, 0) != cudaSuccess) {
+            cudaGetLastError();
+            release();
+            return VSR_ERR_OOM;
+        }
+        for (int i = 0; i < n; ++i) host[i] = 0;
+        return VSR_OK;
+    }
+    vsr_status take(int i = 0)
+    {
+        const int v = *(volatile int*)&host[i];
+        *(volatile int*)&host[i] = 0;
+        return (vsr_status)v;
+    }
+    void release()
+    {
+        if (host) cudaFreeHost(host);
+        host = dev = nullptr;
+    }
+};
+
 struct vsr_scene_s {
+    // the status word of vsr_render_host's frames: an overflow it raised
+    // renders the frame again, any other error is the call's result (first in
+    // the handle, where the tests reach it to raise one)
+    HostStatus host_status;
     int64_t T = 0;
     float cam[12] = {};  // camera of the current set-up
     int64_t T_alloc = 0;
@@ -95,9 +129,6 @@ struct vsr_scene_s {
     cudaStream_t side = nullptr;
     cudaEvent_t use_event = nullptr;
     cudaEvent_t setup_event = nullptr;
-    // its device status word: a frame that outgrew its bins is rendered
-    // again, so the overflow it raised goes here, not to the per-device word
-    int* host_status = nullptr;
     // vsr_render_host_async: the frame's completion, whether one is queued
     // and not yet waited for, and the map generation it was binned against
     cudaEvent_t host_done = nullptr;

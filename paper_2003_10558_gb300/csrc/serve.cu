@@ -16,8 +16,10 @@
 // the device when a request's map shape differs from the previous one's
 // (the capacity only grows), so admitting a request never blocks the worker;
 // a request whose bins outgrew their capacity (known from the pair count
-// once it has finished) is rendered again with grown bins; the slots' workspaces report to status words of their own, so such
-// handled overflows do not reach vsr_last_device_status.  Every request's
+// once it has finished) is rendered again with grown bins; the slots'
+// workspaces report to status words of their own, so such handled overflows do
+// not reach vsr_last_device_status, and what else their kernels raise becomes
+// the request's status.  Every request's
 // output equals that of rendering it alone: the arithmetic is per request and
 // order-free.
 #include <math.h>
@@ -79,7 +81,6 @@ struct Request {
 struct Slot {
     cudaStream_t stream = nullptr;
     cudaEvent_t done = nullptr;
-    int* status = nullptr;  // device status word of this slot's workspaces
     bool busy = false;
     Request req;
     std::list<MapEntry>::iterator map;
@@ -127,6 +128,9 @@ size_t scene_bytes(const vsr_scene_s* s)
 }  // namespace
 
 struct vsr_server_s {
+    // a word per slot for the errors of its workspaces' kernels (first in the
+    // handle, where the tests reach it to raise one)
+    HostStatus status;
     vsr_serve_cfg cfg;
     std::mutex mu;
     std::condition_variable cv;
@@ -300,6 +304,7 @@ struct vsr_server_s {
                     continue;
                 }
                 vsr_scene_s* w = sl.work;
+                const vsr_status raised = status.take((int)(&sl - slots.data()));
                 const bool overflow = *w->h_total > w->cap;
                 if (overflow && sl.req.reruns < 3) {
                     // the bins overflowed: vsr_bin grows them from this count; render again
@@ -308,8 +313,9 @@ struct vsr_server_s {
                     if (launch(sl) == VSR_OK) continue;
                 }
                 sl.map->refs--;
-                // outputs of bins that still overflow are incomplete: say so
-                finish(sl.req, overflow ? VSR_ERR_BIN_OVERFLOW : VSR_OK, sl.t_start, sl.hit);
+                // outputs of bins that still overflow, or of kernels that
+                // raised another error, are incomplete: say so
+                finish(sl.req, overflow ? VSR_ERR_BIN_OVERFLOW : raised, sl.t_start, sl.hit);
                 sl.busy = false;
                 progressed = true;
             }
@@ -339,7 +345,7 @@ struct vsr_server_s {
                         finish(q, VSR_ERR_OOM, now_s(), hit);
                         continue;
                     }
-                    w->status = sl.status;  // overflows are handled here, not reported globally
+                    w->status = status.dev + si;  // its errors are this server's, not the device's
                     w->async_sizing = true;  // a bin overflow renders the request again (below)
                 }
                 sl.req = q;
@@ -386,12 +392,15 @@ vsr_status vsr_serve_create(const vsr_serve_cfg* cfg, vsr_server* out)
         delete s;
         return VSR_ERR_CUDA;
     }
+    if (s->status.alloc(cfg->slots) != VSR_OK) {
+        delete s;
+        return VSR_ERR_OOM;
+    }
     s->slots.resize(cfg->slots);
     s->work.resize(cfg->slots);
     for (Slot& sl : s->slots) {
         if (cudaStreamCreateWithFlags(&sl.stream, cudaStreamNonBlocking) != cudaSuccess ||
-            cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming) != cudaSuccess ||
-            cudaMalloc((void**)&sl.status, sizeof(int)) != cudaSuccess || cudaMemset(sl.status, 0, sizeof(int)) != cudaSuccess) {
+            cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming) != cudaSuccess) {
             cudaGetLastError();
             vsr_serve_destroy(s);
             return VSR_ERR_CUDA;
@@ -509,7 +518,7 @@ vsr_status vsr_serve_destroy(vsr_server s)
     }
     for (auto& per_slot : s->work)
         for (vsr_scene w : per_slot) vsr_scene_free(w);
-    for (Slot& sl : s->slots) cudaFree(sl.status);
+    s->status.release();
     for (MapEntry& e : s->cache) {
         vsr_map_free(e.map);
         if (e.ready) cudaEventDestroy(e.ready);
