@@ -698,7 +698,7 @@ def _autograd_function():
         @staticmethod
         def forward(ctx, tris, colors, lens, renderer):
             ctx.set_materialize_grads(False)  # an unused output costs no zeros
-            lv = lens.detach().cpu().double().tolist()
+            lv = [float(x) for x in lens.detach().cpu().double()]  # (a vector or a column)
             eff = renderer.set_lens(*lv)
             tris_c = tris.detach().contiguous()
             col_c = colors.detach().contiguous()
