@@ -425,7 +425,7 @@ __global__ void __launch_bounds__(RT, 6) frag_fill_kernel(FragArgs v)
     uint4 bits[PPT];
 #pragma unroll
     for (int p = 0; p < PPT; ++p) {
-        const uint32_t* __restrict__ at = v.bits + (size_t)(tp.py + 4 * p) * v.W + tp.px;
+        const uint32_t* at = v.bits + (size_t)(tp.py + 4 * p) * v.W + tp.px;
         const size_t pic = (size_t)v.H * v.W;
         const bool some = inimg[p] && span[p].y;
         bits[p].x = some ? at[0] : 0u;
@@ -541,7 +541,7 @@ __global__ void __launch_bounds__(TILE_PIX) frag_backward_kernel(BackView v)
     const float dD = v.ddepth ? v.ddepth[o] : 0.0f;
     const uint2 span = v.span[o];
     const uint32_t n = span.y;
-    const float4* __restrict__ F = v.frags + span.x;
+    const float4* F = v.frags + span.x;
 
     // the saturating fragment, replaying the forward merge's arithmetic
     uint32_t fstar = n;
@@ -664,8 +664,8 @@ struct CamF {
     float M[9];
 };
 
-__global__ void __launch_bounds__(128) setup_backward_kernel(const float* __restrict__ tris, int T, CamF cam,
-                                                              const float4* __restrict__ rec,
+__global__ void __launch_bounds__(128) setup_backward_kernel(const float* tris, int T, CamF cam,
+                                                              const float4* rec,
                                                               float4* __restrict__ grad,
                                                               float* __restrict__ dtris, float* __restrict__ dcolors)
 {

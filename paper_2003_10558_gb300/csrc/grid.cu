@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(ROW_THREADS) grid_rows_kernel(TriGrid g)
 // scattered writes: an entry is one 32-byte sector, written and later read
 // whole (1M triangles: 20.5 us; as 16 + 8 bytes in two arrays 27.8).  Finding
 // the lanes that share costs 0.7 us of it.
-__global__ void __launch_bounds__(256) grid_file_kernel(const float4* __restrict__ rec, int T, TriGrid g)
+__global__ void __launch_bounds__(256) grid_file_kernel(const float4* rec, int T, TriGrid g)
 {
     grid_wait();
     grid_go();
@@ -130,9 +130,9 @@ struct BinBlock {
     int entry, ok;
 };
 
-__global__ void __launch_bounds__(WALK_THREADS) bin_walk_kernel(const float4* __restrict__ rec, int T, WalkIndex wi,
-                                                               const float4* __restrict__ geom,
-                                                               const Cone* __restrict__ tiles, int ntiles,
+__global__ void __launch_bounds__(WALK_THREADS) bin_walk_kernel(const float4* rec, int T, WalkIndex wi,
+                                                               const float4* geom,
+                                                               const Cone* tiles, int ntiles,
                                                                uint32_t split, int looks, bool sizing,
                                                                uint32_t* __restrict__ ctr,
                                                                uint32_t* __restrict__ starts,

@@ -628,7 +628,7 @@ __device__ __forceinline__ bool map_tangent(int i, int j, int W, int H, const Ta
 // bit for bit that of a kernel that evaluates the tile itself.  Bound by the
 // tangents' instructions: at 1024 x 1024, a quarter of the evaluations.
 __global__ void __launch_bounds__(MAP_THREADS) map_backward_kernel(int W, int H, TanP tp,
-                                                                    const float4* __restrict__ dmap,
+                                                                    const float4* dmap,
                                                                     float* __restrict__ partials, int tiles_x,
                                                                     int tiles_y, bool mx, bool my)
 {
@@ -735,7 +735,7 @@ __device__ __forceinline__ double warp_sum_d(double x)
     for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
     return x;
 }
-__global__ void __launch_bounds__(LENS_THREADS) lens_reduce_kernel(const float4* __restrict__ partials, int nblocks,
+__global__ void __launch_bounds__(LENS_THREADS) lens_reduce_kernel(const float4* partials, int nblocks,
                                                                    double* __restrict__ sums, uint32_t* done,
                                                                    double* __restrict__ dlens)
 {

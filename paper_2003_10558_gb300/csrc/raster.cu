@@ -244,7 +244,7 @@ __device__ __forceinline__ void raster_tile(const RasterView& view, int tile, St
                                             int* __restrict__ status, int range_lo = 0, int range_hi = -1,
                                             int split_slot = -1, int nsplit = 1, SplitAcc split = SplitAcc{})
 {
-    const uint32_t* __restrict__ ids = view.ids;
+    const uint32_t* ids = view.ids;
     const uint32_t cap = view.cap;
     const TilePos tp(tile, view.tiles_x);
     const Cone tc = view.tiles[tile];
@@ -334,10 +334,10 @@ __global__ void __launch_bounds__(RT, 7) raster_kernel(RasterView view, unsigned
 // return at once.
 template <bool ROWS>
 __global__ void __launch_bounds__(RT, VSR_RASTER_CTAS_PER_SM) raster_items_kernel(RasterView view, uint32_t n_tiles,
-                                                              const uint32_t* __restrict__ nsplit_of,
-                                                              const int32_t* __restrict__ split_slot,
-                                                              const uint2* __restrict__ extra,
-                                                              const uint32_t* __restrict__ n_extra, int split_max,
+                                                              const uint32_t* nsplit_of,
+                                                              const int32_t* split_slot,
+                                                              const uint2* extra,
+                                                              const uint32_t* n_extra, int split_max,
                                                               SplitAcc split, int* __restrict__ status)
 {
     grid_wait();
@@ -464,7 +464,7 @@ __global__ void __launch_bounds__(RT) raster_dense_kernel(RasterView view, int* 
 
 // Work items per tile: ceil(bin / split_max) when a split slot and room in
 // the extra list are free, else 1 (the tile runs in one CTA).
-__global__ void items_kernel(const uint32_t* __restrict__ offsets, const uint32_t* __restrict__ ends,
+__global__ void items_kernel(const uint32_t* offsets, const uint32_t* ends,
                              uint32_t n_tiles, int split_max, uint32_t* __restrict__ nsplit_of,
                              int32_t* __restrict__ split_slot, uint32_t* __restrict__ counters /* n_split, n_extra */,
                              uint32_t split_cap, uint2* __restrict__ extra, uint32_t extra_cap)

@@ -89,7 +89,7 @@ __device__ __forceinline__ void walk_eval(const WalkCtx<typename Step::In>& cx, 
 // lists of grad.cu).
 template <class Step, bool ROWS>
 __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView view, typename Step::In in, WalkIndex wi,
-                                                                     const float4* __restrict__ geom, int ntiles,
+                                                                     const float4* geom, int ntiles,
                                                                      uint32_t block, uint32_t split_blocks, bool early,
                                                                      WalkSlots slots,
                                                                      uint32_t* __restrict__ tile_pairs,

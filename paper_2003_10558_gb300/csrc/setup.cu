@@ -116,7 +116,7 @@ constexpr int SETUP_THREADS = 128;
 // triangles 30.0 us, staged 31.3).
 template <int CAM, bool STAGED>
 __global__ void __launch_bounds__(SETUP_THREADS, CAM == CAM_ROTATED ? 2 : 3)
-    setup_pair_kernel(const float* __restrict__ tris, int T, Cam cam, const float* __restrict__ cams_dev,
+    setup_pair_kernel(const float* tris, int T, Cam cam, const float* cams_dev,
                       float4* __restrict__ rec, TriGrid grid)
 {
     grid_wait();
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(SETUP_THREADS, CAM == CAM_ROTATED ? 2 : 3)
         // the CTA's vertices in whole lines, 16 bytes a lane where the buffer allows
         const size_t first = (size_t)blockIdx.x * (2 * SETUP_THREADS);
         const int words = 9 * (int)min((size_t)(2 * SETUP_THREADS), (size_t)T - first);
-        const float* __restrict__ src = tris + 9 * first;
+        const float* src = tris + 9 * first;
         const int quads = ((uintptr_t)src & 15u) == 0 ? words / 4 : 0;
 #pragma unroll
         for (int q = 0; q < (2 * SETUP_THREADS * 9 / 4 + SETUP_THREADS - 1) / SETUP_THREADS; ++q) {

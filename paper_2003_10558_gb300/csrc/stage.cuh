@@ -28,7 +28,7 @@ struct __align__(16) Stage {
 constexpr uint32_t STAGE_EMPTY = 0xffffffffu;  // s6.w of a slot that holds no triangle
 
 // Stage triangle t (a valid record index) into slot j for the tile axis a.
-__device__ __forceinline__ void stage_triangle(const float4* __restrict__ rec, size_t TT, uint32_t t, float ax,
+__device__ __forceinline__ void stage_triangle(const float4* rec, size_t TT, uint32_t t, float ax,
                                                float ay, float az, Stage& st, int j)
 {
     const F8 n12 = ld_f8(rec + rec_at(TT, t, RF_N1)), n3p = ld_f8(rec + rec_at(TT, t, RF_N3));

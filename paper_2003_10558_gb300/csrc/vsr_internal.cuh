@@ -40,16 +40,22 @@ __host__ __device__ __forceinline__ size_t rec_at(size_t TT, size_t t, int f)
 }
 
 // Two consecutive fields (32 bytes, 32-byte aligned: an even field) in one
-// 256-bit access of sm_100+.
+// 256-bit access of sm_100+.  A plain load that stays where it stands: what it
+// reads is written by a kernel that may end while this one's CTAs are already
+// resident (grid_wait), so it is not read-only for this kernel's lifetime, as
+// ld.global.nc wants it.  For the same reason a kernel that waits takes no
+// `const T* __restrict__`, which lets the compiler choose that load.
 struct __align__(16) F8 {
     float4 a, b;
 };
 __device__ __forceinline__ F8 ld_f8(const float4* p)
 {
     F8 v;
-    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=f"(v.a.x), "=f"(v.a.y), "=f"(v.a.z), "=f"(v.a.w), "=f"(v.b.x), "=f"(v.b.y), "=f"(v.b.z), "=f"(v.b.w)
-        : "l"(p));
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v.a.x), "=f"(v.a.y), "=f"(v.a.z), "=f"(v.a.w), "=f"(v.b.x), "=f"(v.b.y), "=f"(v.b.z),
+                   "=f"(v.b.w)
+                 : "l"(p)
+                 : "memory");
     return v;
 }
 __device__ __forceinline__ void st_f8(float4* p, const float4& a, const float4& b)

@@ -126,7 +126,7 @@ __device__ __forceinline__ void walk_ranges(const WalkIndex& wi, int T, const fl
         if (i < R - 1) {
             const int nlat = grid_nlat_of(l);
             const int ncol = grid_ncol(nlat, row);
-            const uint32_t* __restrict__ st = wi.start + grid_base_of(l) + row * (2 * nlat + 1);
+            const uint32_t* st = wi.start + grid_base_of(l) + row * (2 * nlat + 1);
             int c0 = 0, c1 = ncol - 1;
             if (fabsf(g.y) + gl < 0.5f * IDX_PI - 0.1f) {
                 // the cap's longitude half-width over this row: at the
@@ -221,7 +221,7 @@ struct Walk {
 
     // candidate idx < total (one per thread, consecutive within a warp;
     // `in`: whether this thread's exists -- all lanes call)
-    __device__ __forceinline__ Cand read(const WalkIndex& wi, const float4* __restrict__ rec, int T,
+    __device__ __forceinline__ Cand read(const WalkIndex& wi, const float4* rec, int T,
                                          const WalkShared& ws, uint32_t idx, bool in) const
     {
         Cand c{make_float4(0.0f, 0.0f, 0.0f, 0.0f), 0.0f, 0u, in};
@@ -282,7 +282,7 @@ struct Walk {
 // tests either (1M triangles from inside: 427.5 -> 421.5 us a frame; the pixel
 // step at 1280 x 720: 119.5 -> 115.9 us).  Prefetching the hits' records as
 // they are found changed nothing (421.3, 116.4 us).
-__device__ __forceinline__ void walk_hits(const Walk& w, const WalkIndex& wi, const float4* __restrict__ rec, int T,
+__device__ __forceinline__ void walk_hits(const Walk& w, const WalkIndex& wi, const float4* rec, int T,
                                           const WalkShared& ws, uint32_t i0, uint32_t i1, uint32_t* ids, uint32_t* n)
 {
     const unsigned FULL = 0xffffffffu;
