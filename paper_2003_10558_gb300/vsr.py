@@ -178,9 +178,10 @@ def _stream_ptr(stream):
     if stream is not None:
         return stream.cuda_stream
     import torch
-    if not torch.cuda.is_initialized():
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)  # not public: may be gone one day
+    if raw is None:
         return torch.cuda.current_stream().cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return raw(torch.cuda.current_device())
 
 
 def _dptr(t):
