@@ -676,13 +676,19 @@ __global__ void __launch_bounds__(128) setup_backward_kernel(const float* tris, 
     const size_t TT = (size_t)T;
     const float4 cp2 = rec[rec_at(TT, t, RF_CAP2)];
     float* out = dtris ? dtris + (size_t)t * 9 : nullptr;
-    // the record's gradient, cleared for the next backward
+    // The record's gradient, cleared for the next backward where it holds
+    // anything: most fields of most triangles are zero already (hidden, or no
+    // pixel at that edge), and a store between the loads makes them a chain.  A
+    // backward to the vertices of 1M triangles, 640x480: 334 us with a load and
+    // a store per field, 214 with the stores after the loads, 103 like this (140
+    // with a memset per call instead); of 10k, 1024x1024: 25.9, 25.1, 25.0 us.
     float4 gr[GF_COUNT];
 #pragma unroll
-    for (int q = 0; q < GF_COUNT; ++q) {
-        gr[q] = grad[q * TT + t];
-        grad[q * TT + t] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    }
+    for (int q = 0; q < GF_COUNT; ++q) gr[q] = grad[q * TT + t];
+#pragma unroll
+    for (int q = 0; q < GF_COUNT; ++q)
+        if (gr[q].x != 0.0f || gr[q].y != 0.0f || gr[q].z != 0.0f || gr[q].w != 0.0f)
+            grad[q * TT + t] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     const float4 gpl = gr[GF_PL];
     if (dcolors) dcolors[t] = cp2.w != 0.0f ? gpl.w : 0.0f;
     if (!out) return;
