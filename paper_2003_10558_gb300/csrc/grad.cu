@@ -118,13 +118,57 @@ __device__ __forceinline__ float4 frag_record(const FragEval& o, const FragPix& 
                        colour * fabsf(o.D[p]));
 }
 
-// Sorts a pixel's m fragments where they are stored (insertion, by (r, t))
-// and merges them.  (Other CTAs may have written them: the first read of each
-// goes past the L1.)
-__device__ __forceinline__ void frag_merge(const FragArgs& v, size_t pixel, float4* F, uint32_t m)
+// Sorts a pixel's m fragments where they are stored, by (r, t), and merges
+// them: the first CAP by insertion of their depths in shared memory (one column
+// a thread), then each record into its place along the permutation's cycles;
+// what is beyond CAP by insertion among the records.  Insertion of the records
+// alone is a chain of dependent loads and stores that needs the lists in the
+// L1, which holds those of a few CTAs.  A shaded forward of 1024 x 1024 pixels:
+// 5000 triangles, 12 fragments a pixel, 1578 -> 540 us; 50k, 16 a pixel, 2630 ->
+// 1055; 20k, 6 a pixel, 328 -> 222.  (Counting the smaller depths instead of
+// inserting, with one move a turn for all lanes: 1577 us on the first.)
+// OTHERS: other CTAs may have written the records, so the first read of each
+// goes past the L1 (and it is stored again); such tiles are few, and insertion
+// of the records is the faster one.
+template <int CAP>
+struct FragKeys {
+    float r[CAP][RT];
+    unsigned char at[CAP][RT];  // which record
+};
+template <bool OTHERS, int CAP>
+__device__ __forceinline__ void frag_merge(const FragArgs& v, size_t pixel, float4* F, uint32_t m, FragKeys<CAP>& key)
 {
-    for (uint32_t u = 0; u < m; ++u) {
-        const float4 x = __ldcg(F + u);
+    const uint32_t me = threadIdx.x, mk = OTHERS ? 0u : min(m, (uint32_t)CAP);
+    for (uint32_t u = 0; u < mk; ++u) {
+        const float r = F[u].x;
+        uint32_t w = u;
+        while (w > 0) {
+            const float q = key.r[w - 1][me];
+            const unsigned char a = key.at[w - 1][me];
+            if (!(r < q || (r == q && __float_as_uint(F[u].y) < __float_as_uint(F[a].y)))) break;
+            key.r[w][me] = q;
+            key.at[w][me] = a;
+            --w;
+        }
+        key.r[w][me] = r;
+        key.at[w][me] = (unsigned char)u;
+    }
+    for (uint32_t u = 0; u < mk; ++u) {
+        uint32_t from = key.at[u][me];
+        if (from == u) continue;
+        const float4 first = F[u];
+        uint32_t to = u;
+        while (from != u) {
+            F[to] = F[from];
+            key.at[to][me] = (unsigned char)to;
+            to = from;
+            from = key.at[to][me];
+        }
+        F[to] = first;
+        key.at[to][me] = (unsigned char)to;
+    }
+    for (uint32_t u = mk; u < m; ++u) {
+        const float4 x = OTHERS ? __ldcg(F + u) : F[u];
         uint32_t w = u;
         while (w > 0 && frag_less(x, F[w - 1])) {
             F[w] = F[w - 1];
@@ -360,21 +404,41 @@ struct FragFillStep : FragStep {
     template <bool ROWS>
     __device__ __forceinline__ static void finish(const Ctx& cx, const TilePos& tp, const Pix& q, int* status)
     {
+        using Keys = FragKeys<sizeof(Stage) / (5 * RT)>;
+        static_assert(sizeof(Keys) <= sizeof(Stage), "the keys take the triangles' place");
+        Keys& key = *(Keys*)&cx.stage;
         const FragArgs& v = cx.in;
+        const bool shared = cx.wt.slot >= 0;
+        __syncthreads();  // no warp evaluates any more
 #pragma unroll 1
         for (int p = 0; p < PPT; ++p) {
             if (tp.px >= v.W || tp.py + 4 * p >= v.H) continue;
             const uint32_t n = p ? q.acc[1] : q.acc[0], room = p ? q.room[1] : q.room[0];
             // spans of another frame, or no room (see FragArgs::early)
             if (n != room && !(v.early && room == 0u)) raise_status(status, VSR_ERR_FRAG_OVERFLOW);
-            frag_merge(v, (size_t)(tp.py + 4 * p) * v.W + tp.px, v.frags + (p ? q.at[1] : q.at[0]), min(n, room));
+            const size_t o = (size_t)(tp.py + 4 * p) * v.W + tp.px;
+            float4* F = v.frags + (p ? q.at[1] : q.at[0]);
+            if (shared)
+                frag_merge<true>(v, o, F, min(n, room), key);
+            else
+                frag_merge<false>(v, o, F, min(n, room), key);
         }
     }
 };
 
-// fragments of a pixel sorted in shared memory; a longer list is sorted where
-// it is stored
+// fragments of a pixel sorted in shared memory as they are found; a longer list
+// is stored and then sorted (frag_merge, its keys in the same memory)
 constexpr uint32_t FRAG_SORT = 8;
+struct FillBuffers {
+    Stage st;
+    float4 rec[FRAG_SORT][RT];
+};
+using FillKeys = FragKeys<sizeof(FillBuffers) / (RT * 5)>;
+union __align__(16) FillShared {
+    FillBuffers b;
+    FillKeys key;
+    __device__ FillShared() {}
+};
 
 // The fill of the tiles with a list: the evaluations that are fragments, no
 // walk and no cull.  Bound by issue with lanes idle (each triangle's step runs
@@ -386,8 +450,9 @@ __global__ void __launch_bounds__(RT, 6) frag_fill_kernel(FragArgs v)
 {
     grid_wait();
     grid_go();
-    __shared__ Stage st;
-    __shared__ float4 rec[FRAG_SORT][RT];
+    __shared__ FillShared sh;
+    Stage& st = sh.b.st;
+    float4 (&rec)[FRAG_SORT][RT] = sh.b.rec;
     __shared__ float scol[STAGE_CHUNK];
     __shared__ WarpCones wc;
     const unsigned FULL = 0xffffffffu;
@@ -436,6 +501,7 @@ __global__ void __launch_bounds__(RT, 6) frag_fill_kernel(FragArgs v)
     __syncthreads();
     // (one pixel's list at a time in shared memory: the first pixels of
     // the lanes, then the second)
+    unsigned longer = 0u;  // pixels with a longer list
 #pragma unroll
     for (int p = 0; p < PPT; ++p) {
         const bool sorted = span[p].y <= FRAG_SORT;
@@ -478,7 +544,8 @@ __global__ void __launch_bounds__(RT, 6) frag_fill_kernel(FragArgs v)
         const size_t o = (size_t)(tp.py + 4 * p) * v.W + tp.px;
         const uint32_t m = min(cnt, span[p].y);
         if (!sorted) {
-            frag_merge(v, o, v.frags + span[p].x, m);
+            span[p].y = m;  // below, with every warp done with the triangles
+            longer |= 1u << p;
             continue;
         }
         // the pixel's merge, and its list
@@ -495,6 +562,12 @@ __global__ void __launch_bounds__(RT, 6) frag_fill_kernel(FragArgs v)
         if (v.image) v.image[o] = img;
         if (v.cov) v.cov[o] = mb;
     }
+    if (!__syncthreads_or(longer)) return;
+#pragma unroll 1
+    for (int p = 0; p < PPT; ++p)
+        if (longer >> p & 1u)
+            frag_merge<false>(v, (size_t)(tp.py + 4 * p) * v.W + tp.px, v.frags + (p ? span[1].x : span[0].x),
+                              p ? span[1].y : span[0].y, sh.key);
 }
 
 // ---------------------------------------------------------------------------

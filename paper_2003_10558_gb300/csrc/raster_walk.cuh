@@ -60,6 +60,7 @@ struct WalkCtx {
     const WalkSlots& slots;
     const WalkTile& wt;
     const uint32_t* ids;  // the current block's hits
+    Stage& stage;  // a finish may use its memory, after a barrier: other warps may still evaluate
 };
 
 // The n staged triangles of a chunk at the warp's pixels: a lane-parallel cull
@@ -114,7 +115,7 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
     };
     const bool skip = !helper && Step::skip(in, (int)blockIdx.x);
     if (skip && threadIdx.x == 0) begun();
-    const WalkCtx<typename Step::In> cx{view, in, slots, wt, s_ids};
+    const WalkCtx<typename Step::In> cx{view, in, slots, wt, s_ids, st};
     while (!skip) {
         typename Step::Pix q;
         bool warp_active;
