@@ -136,10 +136,15 @@ __device__ __forceinline__ bool cap_hits_cone(float3 S, float cos_rho, float sin
     return cg >= cos_a * cb - sin_a * sb - eps;
 }
 
+// (the failed call's error is taken from the runtime, or a later check of
+// another launch would find it)
 #define VSR_CUDA_TRY(expr)                                                                                              \
     do {                                                                                                                \
         cudaError_t _e = (expr);                                                                                        \
-        if (_e != cudaSuccess) return VSR_ERR_CUDA;                                                                     \
+        if (_e != cudaSuccess) {                                                                                        \
+            cudaGetLastError();                                                                                         \
+            return VSR_ERR_CUDA;                                                                                        \
+        }                                                                                                               \
     } while (0)
 
 // Launches one after another on a stream hand over without draining the GPU
