@@ -20,7 +20,6 @@
 #include <algorithm>
 #include <atomic>
 
-
 #include "vsr_internal.cuh"
 
 namespace {

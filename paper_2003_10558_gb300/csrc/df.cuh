@@ -129,17 +129,3 @@ __device__ __forceinline__ df3 df3_add(df3 a, df3 b) { return {df_add(a.x, b.x),
 __device__ __forceinline__ df3 df3_scale(df3 a, df s) { return {df_mul(a.x, s), df_mul(a.y, s), df_mul(a.z, s)}; }
 __device__ __forceinline__ df3 df3_div(df3 a, df s) { return {df_div(a.x, s), df_div(a.y, s), df_div(a.z, s)}; }
 __device__ __forceinline__ df3 df3_neg(df3 a) { return {df_neg(a.x), df_neg(a.y), df_neg(a.z)}; }
-
-// a . (b_hi + b_lo) for an FP32 vector a and a double-word vector b
-// (Ogita-Rump-Oishi style compensated dot product), rounded to one float.
-__device__ __forceinline__ float dot_f_df(float ax, float ay, float az, df3 b)
-{
-    df p = two_prod(ax, b.x.hi);
-    df q = two_prod(ay, b.y.hi);
-    df r = two_prod(az, b.z.hi);
-    df s = two_sum(p.hi, q.hi);
-    df t = two_sum(s.hi, r.hi);
-    float err = __fadd_rn(__fadd_rn(__fadd_rn(p.lo, q.lo), __fadd_rn(r.lo, s.lo)), t.lo);
-    float lo = __fmaf_rn(ax, b.x.lo, __fmaf_rn(ay, b.y.lo, __fmul_rn(az, b.z.lo)));
-    return __fadd_rn(t.hi, __fadd_rn(err, lo));
-}

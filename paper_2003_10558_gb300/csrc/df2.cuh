@@ -152,8 +152,9 @@ __device__ __forceinline__ df3_2 df3_2_sel(bool cx, bool cy, df3_2 a, df3_2 b)
     return {df2_sel(cx, cy, a.x, b.x), df2_sel(cx, cy, a.y, b.y), df2_sel(cx, cy, a.z, b.z)};
 }
 
-// dot_f_df of the FP32 vector a with two double-word vectors at once (b's
-// components x and y), bit for bit the scalar function's results.
+// a . (b_hi + b_lo) for an FP32 vector a and two double-word vectors at once
+// (b's components x and y): a compensated dot product (Ogita-Rump-Oishi style),
+// rounded to one float.
 __device__ __forceinline__ float2 dot_f_df2(float ax, float ay, float az, df3_2 b)
 {
     const df2 p = two_prod2(f2(ax), b.x.hi);

@@ -33,7 +33,7 @@ struct PstepPix {
 
 struct PstepCones {
     float4 c[RT / 32][2];  // as WarpCones (the widest ramp of any distance for h)
-    float2 e[RT / 32];     // cos, sin of 4h: what the ramp adds to a cap's radius (see pstep_cap)
+    float2 e[RT / 32];     // pstep_ramp of h
 };
 
 // |n . d_i G| + |n . d_j G| of both pixels
@@ -111,9 +111,7 @@ struct PstepStep {
             const int w = threadIdx.x >> 5;
             wc.c[w][0] = c0;
             wc.c[w][1] = c1;
-            float2 e = make_float2(-1.0f, 0.0f);
-            if (4.0f * c1.y < 3.14159265f) sincosf(4.0f * c1.y, &e.y, &e.x);
-            wc.e[w] = e;
+            wc.e[w] = pstep_ramp(c1.y);
         }
         __syncwarp();
         return c1.z > 0.0f;
@@ -124,11 +122,9 @@ struct PstepStep {
         const float2 e = wc.e[warp];
         const float4 a = st.s0[j], b = st.s1[j];
         // the cap widened by the ramp (pstep_cap)
-        const float cr = 1.0f - 0.5f * b.y;
-        float cb = fmaf(cr, e.x, -b.x * e.y), sb = fmaf(b.x, e.x, cr * e.y);
-        if (e.x <= -1.0f || (sb < 0.0f && cb < 0.0f)) cb = -1.0f;  // past the antipode: the whole sphere
-        const bool keep = cap_hits_cone(make_float3(a.x, a.y, a.z), cb, fmaxf(sb, 0.0f), make_float3(c0.x, c0.y, c0.z),
-                                        c0.w, c1.x, 0.0f);
+        const float2 cap = pstep_cap(1.0f - 0.5f * b.y, b.x, e);
+        const bool keep = cap_hits_cone(make_float3(a.x, a.y, a.z), cap.x, fmaxf(cap.y, 0.0f),
+                                        make_float3(c0.x, c0.y, c0.z), c0.w, c1.x, 0.0f);
         const float lim = -(c1.y + c1.x + (1.0f - c0.w) + 1e-6f);
         const float4 n1 = st.s2[j], n2 = st.s3[j], n3 = st.s4[j];
         return keep && fmaf(c0.x, n1.x, fmaf(c0.y, n1.y, c0.z * n1.z)) > lim &&

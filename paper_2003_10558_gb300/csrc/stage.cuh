@@ -61,19 +61,9 @@ __device__ __forceinline__ void stage_triangle(const float4* rec, size_t TT, uin
                            __uint_as_float(t));
 }
 
-// |G|^2 - 1, error-free (TwoProd / TwoSum): the chord form of the miter
-// distance equals (G.S-hat - cos rho)/sin rho for any G only with this term,
-// and FP32 map directions are unit to ~1e-7, not exactly.
-__device__ __forceinline__ float norm2_minus_one(float x, float y, float z)
-{
-    const df px2 = two_prod(x, x), py2 = two_prod(y, y), pz2 = two_prod(z, z);
-    const df s1 = two_sum(px2.hi, py2.hi);
-    const df s2 = two_sum(s1.hi, pz2.hi);
-    const float tail = __fadd_rn(__fadd_rn(__fadd_rn(px2.lo, py2.lo), __fadd_rn(pz2.lo, s1.lo)), s2.lo);
-    return __fadd_rn(__fadd_rn(s2.hi, -1.0f), tail);
-}
-
-// the same of two directions at once, bit for bit
+// |G|^2 - 1 of two directions at once, error-free (TwoProd / TwoSum): the chord
+// form of the miter distance equals (G.S-hat - cos rho)/sin rho for any G only
+// with this term, and FP32 map directions are unit to ~1e-7, not exactly.
 __device__ __forceinline__ float2 norm2_minus_one2(float2 x, float2 y, float2 z)
 {
     const df2 px2 = two_prod2(x, x), py2 = two_prod2(y, y), pz2 = two_prod2(z, z);
@@ -144,20 +134,4 @@ __device__ __forceinline__ bool centre_inside(float g1, float g2, float g3, floa
         in = (g1 > 0.0f || (g1 == 0.0f && (ties & 1u))) && (g2 > 0.0f || (g2 == 0.0f && (ties & 2u))) &&
              (g3 > 0.0f || (g3 == 0.0f && (ties & 4u)));
     return in;
-}
-
-__device__ __forceinline__ float warp_sum(float v)
-{
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-__device__ __forceinline__ float warp_min(float v)
-{
-    for (int o = 16; o; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-__device__ __forceinline__ float warp_max(float v)
-{
-    for (int o = 16; o; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
 }

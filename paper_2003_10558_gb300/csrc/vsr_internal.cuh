@@ -377,17 +377,20 @@ struct BinView {
 // not scaled by sin rho like the global step's, and |S.d G| <= sin(theta)
 // |d G| at angle theta from S, so with h >= the widest ramp half-width
 // (|d_i G| + |d_j G|)/2 every fragment lies within the angle rho + 4h of S.
-// Returns (cos, sin) of that radius.
-__device__ __forceinline__ float2 pstep_cap(float cos_rho, float sin_rho, float h)
+// pstep_ramp: (cos, sin) of 4h, (-1, 0) from pi on; pstep_cap: (cos, sin) of
+// rho + 4h, cos -1 (the whole sphere) past the antipode.
+__device__ __forceinline__ float2 pstep_ramp(float h)
 {
-    const float e = 4.0f * h;
-    if (e >= 3.14159265f) return make_float2(-1.0f, 0.0f);
-    float se, ce;
-    sincosf(e, &se, &ce);
-    const float c = fmaf(cos_rho, ce, -sin_rho * se);
-    const float s = fmaf(sin_rho, ce, cos_rho * se);
-    // past the antipode the cap is the whole sphere
-    return (s < 0.0f && c < 0.0f) ? make_float2(-1.0f, 0.0f) : make_float2(c, fmaxf(s, 0.0f));
+    float2 e = make_float2(-1.0f, 0.0f);
+    if (4.0f * h < IDX_PI) sincosf(4.0f * h, &e.y, &e.x);
+    return e;
+}
+__device__ __forceinline__ float2 pstep_cap(float cos_rho, float sin_rho, float2 ramp)
+{
+    float c = fmaf(cos_rho, ramp.x, -sin_rho * ramp.y);
+    const float s = fmaf(sin_rho, ramp.x, cos_rho * ramp.y);
+    if (ramp.x <= -1.0f || (s < 0.0f && c < 0.0f)) c = -1.0f;
+    return make_float2(c, s);
 }
 
 // Work items of the raster: a tile whose bin is longer than split_max

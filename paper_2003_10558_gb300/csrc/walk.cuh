@@ -188,7 +188,7 @@ __device__ __forceinline__ void walk_ranges(const WalkIndex& wi, int T, const fl
 // The walk as one thread sees it, after the barrier that follows walk_ranges.
 struct Walk {
     float ax, ay, az, ca, sa, h;  // the tile's cone and widest ramp
-    float ce, se;                 // pixel step: cos / sin of 4h
+    float2 ramp;                  // pixel step: pstep_ramp(h)
     uint32_t ex0;                 // first candidate of range `lane`
 
     __device__ __forceinline__ void init(const WalkIndex& wi, const Cone& c, const WalkShared& ws)
@@ -200,14 +200,7 @@ struct Walk {
         ca = c.c0.w;
         sa = c.c1.x;
         h = c.c1.y;
-        ce = 1.0f;
-        se = 0.0f;
-        if (wi.pstep) {
-            if (4.0f * h < IDX_PI)
-                sincosf(4.0f * h, &se, &ce);
-            else
-                ce = -1.0f;
-        }
+        ramp = wi.pstep ? pstep_ramp(h) : make_float2(1.0f, 0.0f);
         ex0 = ws.rng[lane].x;
     }
 
@@ -261,9 +254,9 @@ struct Walk {
         const float sr = c.sr;
         float cb, sb;
         if (wi.pstep) {
-            cb = fmaf(q.w, ce, -sr * se);
-            sb = fmaf(sr, ce, q.w * se);
-            if (ce <= -1.0f || (sb < 0.0f && cb < 0.0f)) cb = -1.0f;  // past the antipode: the whole sphere
+            const float2 c4 = pstep_cap(q.w, sr, ramp);
+            cb = c4.x;
+            sb = c4.y;
         } else {
             cb = fmaf(-h, sr, q.w);
             const float s2 = fmaxf(fmaf(-cb, cb, 1.0f), 1e-30f);
