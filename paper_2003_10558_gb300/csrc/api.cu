@@ -40,23 +40,25 @@ int* status_word()
     return g_status[dev];
 }
 
-vsr_status clear_workspace(void* p, int byte, size_t n, cudaStream_t st)
+vsr_status clear_workspace(std::initializer_list<Fill> fills, cudaStream_t st)
 {
     bool captures;
     const vsr_status s = stream_captures(st, &captures);
     if (s != VSR_OK) return s;
     if (!captures) {
-        VSR_CUDA_TRY(cudaMemsetAsync(p, byte, n, st));
+        for (const Fill& f : fills) VSR_CUDA_TRY(cudaMemsetAsync(f.p, f.byte, f.n, st));
         return VSR_OK;
     }
     // a stream of its own, which the capture's mode must not forbid to wait for
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     VSR_CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
     cudaStream_t own = nullptr;
-    const bool ok = cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking) == cudaSuccess &&
-                    cudaMemsetAsync(p, byte, n, own) == cudaSuccess && cudaStreamSynchronize(own) == cudaSuccess;
+    bool ok = cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking) == cudaSuccess;
+    for (const Fill& f : fills) ok = ok && cudaMemsetAsync(f.p, f.byte, f.n, own) == cudaSuccess;
+    ok = ok && cudaStreamSynchronize(own) == cudaSuccess;
     if (own) cudaStreamDestroy(own);
     cudaThreadExchangeStreamCaptureMode(&mode);
+    if (!ok) cudaGetLastError();
     return ok ? VSR_OK : VSR_ERR_CUDA;
 }
 
@@ -195,7 +197,7 @@ vsr_status setup_records(const float* tris_dev, int64_t T, const float* cam, con
         const bool was_dirty = grid.dirty;
         grid.dirty = true;
         if (was_dirty &&
-            (s = clear_workspace(grid.counts, 0, sizeof(uint32_t) * ((size_t)GRID_WORDS + GRID_HDR), st)) != VSR_OK)
+            (s = clear_workspace({{grid.counts, 0, sizeof(uint32_t) * ((size_t)GRID_WORDS + GRID_HDR)}}, st)) != VSR_OK)
             return s;
     }
     s = cam_dev ? launch_setup_view(tris_dev, (int)T, cam_dev, rec, g, st)
@@ -248,7 +250,7 @@ vsr_status ensure_ws(vsr_scene sc, int ntiles, cudaStream_t st)
     sc->ends = sc->offsets + n + 1;
     sc->tile_pairs = sc->ends + n;
     sc->bin_ctr = sc->tile_pairs + n;
-    if ((s = clear_workspace(sc->bin_ctr, 0, BIN_CTR_WORDS * sizeof(uint32_t), st)) != VSR_OK) return s;
+    if ((s = clear_workspace({{sc->bin_ctr, 0, BIN_CTR_WORDS * sizeof(uint32_t)}}, st)) != VSR_OK) return s;
     sc->ws_tiles = ntiles;
     sc->sized_shape = 0;
     // (the bins' places went with the old arrays)

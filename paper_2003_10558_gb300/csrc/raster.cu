@@ -567,8 +567,7 @@ vsr_status walk_work_alloc(WalkWork* w, cudaStream_t st)
         cudaGetLastError();
         return VSR_ERR_OOM;
     }
-    if (clear_workspace(m, 0, pix, st) != VSR_OK || clear_workspace(m + pix, 0xff, pix, st) != VSR_OK ||
-        clear_workspace(m + 2 * pix, 0, rest, st) != VSR_OK) {
+    if (clear_workspace({{m, 0, pix}, {m + pix, 0xff, pix}, {m + 2 * pix, 0, rest}}, st) != VSR_OK) {
         cudaFree(m);
         return VSR_ERR_CUDA;
     }
@@ -621,8 +620,7 @@ vsr_status raster_work_alloc(RasterWork* w, uint32_t n_tiles, cudaStream_t st)
     w->counters = (uint32_t*)(m + 2 * pix + extra + done + 2 * tiles);
     w->split_cap = (uint32_t)cap;
     w->extra_cap = EXTRA_ITEMS;
-    if (clear_workspace(w->acc, 0, pix, st) != VSR_OK || clear_workspace(w->key, 0xff, pix, st) != VSR_OK ||
-        clear_workspace(w->done, 0, done, st) != VSR_OK) {
+    if (clear_workspace({{w->acc, 0, pix}, {w->key, 0xff, pix}, {w->done, 0, done}}, st) != VSR_OK) {
         raster_work_free(w);
         return VSR_ERR_CUDA;
     }

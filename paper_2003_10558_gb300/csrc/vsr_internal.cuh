@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <initializer_list>
+
 #include "../../include/vsr.h"
 
 // ---------------------------------------------------------------------------
@@ -411,11 +413,16 @@ struct RasterWork {
 };
 // SMs of the current device (looked up once per device), or -1.
 int sm_count();
-// Clears (bytes of value `byte`) workspace that the library has just allocated
-// or found dirty: on st, before the launches that follow there; where st
+// Fills workspace that the library has just allocated or found dirty with its
+// initial bytes: on st, before the launches that follow there; where st
 // captures, at once, since eager work may use it before the graph's first
 // launch, and replays find it as any launch leaves it.
-vsr_status clear_workspace(void* p, int byte, size_t n, cudaStream_t st);
+struct Fill {
+    void* p;
+    int byte;
+    size_t n;
+};
+vsr_status clear_workspace(std::initializer_list<Fill> fills, cudaStream_t st);
 
 // A view's raster work for the pooled launch: the view, its item assignment
 // (from launch_raster_assign) and its split accumulators.
