@@ -219,9 +219,9 @@ int64_t vsr_scene_size(vsr_scene s);
  * bins, as vsr_bin and vsr_raster_tiles, sized with one synchronisation of
  * `stream`; later frames bin and rasterize in one launch that stores none,
  * and do not synchronise.  The outputs are the same.
- * Scratch (the grid, 28 B per triangle; the bins, sized by the first frame;
- * accumulators of shared tiles) is held by the scene handle.  A scene must
- * not be rasterized on two streams at the same time. */
+ * Scratch (the grid, 36 B per triangle and 0.8 MB of cell counters; the bins,
+ * sized by the first frame; accumulators of shared tiles) is held by the scene
+ * handle.  A scene must not be rasterized on two streams at the same time. */
 vsr_status vsr_raster(vsr_map m, vsr_scene s, uint32_t* id_dev, float* depth_dev, float* cov_dev, void* stream);
 
 /* vsr_raster_pstep: vsr_raster with the per-fragment pixel step of Sec.
@@ -392,10 +392,10 @@ vsr_status vsr_render_host_wait(vsr_scene s);
  * bin capacity re-sizes the bins and captures again (as for a new
  * configuration); a frame whose cameras outgrow the bins before that raises
  * VSR_ERR_BIN_OVERFLOW in the device status with its outputs incomplete; the
- * next call grows the bins.  Device memory per view: T x 188 B of set-up
- * records and triangle grid, 4 MB of accumulators, and for pooled launches
- * its bins.  A batch must not render on two
- * streams at once. */
+ * next call grows the bins.  Device memory per view: T x 196 B of set-up
+ * records and triangle grid, 0.8 MB of cell counters, 4 MB of accumulators,
+ * and for pooled launches its bins.  A batch must not render on two streams
+ * at once. */
 typedef struct vsr_batch_s* vsr_batch;
 vsr_status vsr_batch_create(vsr_batch* out);
 vsr_status vsr_batch_render(vsr_batch b, int nviews, const vsr_map* maps, const float* tris_dev, int64_t T,

@@ -706,9 +706,8 @@ vsr_status scene_walk_begin(vsr_map m, vsr_scene sc, cudaStream_t st)
 // One frame of (m, s) without statistics.  The walking raster needs no bins
 // (1920x1080, 220k triangles: 124 us instead of 38 us of binning, 3 us of work
 // items and 103 us of raster; 4096x2176, 1M: 544 us instead of 148 + 3 + 450),
-// but the
-// first frame of a shape goes through stored ones, as does every frame of a
-// scene that renders again on a bin overflow (async_sizing): the bins are
+// but the first frame of a shape goes through stored ones, as does every frame
+// of a scene that renders again on a bin overflow (async_sizing): the bins are
 // then allocated and sized, with the one synchronisation of a new shape, so
 // that a vsr_raster_tiles that follows can be captured.
 static vsr_status raster_frame(vsr_map m, vsr_scene sc, uint32_t* id_dev, float* depth_dev, float* cov_dev,
@@ -921,7 +920,8 @@ vsr_status vsr_render_host(vsr_map m, vsr_scene sc, const float* tris_host, int6
     vsr_status s = host_frame_front(m, sc, tris_host, T, cam, id_host, depth_host, cov_host, st, &f);
     if (s != VSR_OK) return s;
     // The call waits for the frame anyway, so a frame that outgrew its bins
-    // is rendered again: the next binning grows the bins from its total.
+    // (through stored ones: the first of a shape) is rendered again: the next
+    // binning grows the bins from its total.
     for (int attempt = 0;; ++attempt) {
         s = host_frame_back(m, sc, f, id_host, depth_host, cov_host, st);
         if (s == VSR_OK && cudaStreamSynchronize(st) != cudaSuccess) {

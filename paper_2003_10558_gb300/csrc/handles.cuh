@@ -71,7 +71,7 @@ struct HostStatus {
 };
 
 struct vsr_scene_s {
-    // the status word of vsr_render_host's frames: an overflow it raised
+    // the status word of vsr_render_host's frames: an overflow of stored bins
     // renders the frame again, any other error is the call's result (first in
     // the handle, where the tests reach it to raise one)
     HostStatus host_status;

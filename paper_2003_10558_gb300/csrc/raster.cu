@@ -238,6 +238,9 @@ struct GlobalStep {
     }
 };
 
+// One 16x16 tile of one view over its stored bin.  Called by every thread of a
+// CTA of RT threads; `st` is the CTA's staging area (reusable across calls:
+// every use is fenced by the barriers of the chunk loop).
 template <bool STATS, bool ROWS = false>
 __device__ __forceinline__ void raster_tile(const RasterView& view, int tile, Stage& st, bool count_alg,
                                             uint32_t& cnt_alg, uint32_t& cnt_exec, int32_t* __restrict__ n_inside,

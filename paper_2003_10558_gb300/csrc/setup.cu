@@ -55,7 +55,7 @@ __device__ __forceinline__ bool vless(const float* P, const float* Q)
 // each record is bit for bit what the scalar double-word algorithms of
 // df.cuh give for its triangle.  What would branch per triangle is a
 // per-component select: the canonical operand order of each edge, the miter
-// case (every case is formed), the invalid triangles.
+// case (the circumcentre and one midpoint are formed), the invalid triangles.
 __device__ __forceinline__ df3_2 normalize3_2(df3_2 v) { return df3_2_scale(v, df2_rsqrt(df2_dot(v, v))); }
 
 __device__ __forceinline__ df3_2 edge_normal2(const float* P0, const float* Q0, const float* P1, const float* Q1,
@@ -184,8 +184,8 @@ __global__ void __launch_bounds__(SETUP_THREADS, CAM == CAM_ROTATED ? 2 : 3)
     const df3_2 n2 = edge_normal2(w0 + 3, w0 + 6, w1 + 3, w1 + 6, V[1], V[2], flip0, flip1);
     const df3_2 n3 = edge_normal2(w0 + 6, w0 + 0, w1 + 6, w1 + 0, V[2], V[0], flip0, flip1);
 
-    // miter: smallest circle over the unit vertices; every case formed, the
-    // triangle's own selected
+    // miter: smallest circle over the unit vertices; the circumcentre and the
+    // midpoint that the triangle would take are formed, one selected
     const df3_2 U0 = normalize3_2(V[0]), U1 = normalize3_2(V[1]), U2 = normalize3_2(V[2]);
     const df3_2 ea = df3_2_sub(U1, U2), eb = df3_2_sub(U2, U0), ec = df3_2_sub(U0, U1);
     const df2 a2 = df2_dot(ea, ea), b2 = df2_dot(eb, eb), c2 = df2_dot(ec, ec);

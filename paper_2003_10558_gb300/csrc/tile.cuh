@@ -15,9 +15,6 @@ static_assert(RT * PPT == TILE_PIX, "one CTA covers one tile");
 #define VSR_RASTER_CTAS_PER_SM 8
 #endif
 
-// One 16x16 tile of one view.  Called by every thread of a CTA of RT
-// threads; `st` is the CTA's staging area (reusable across calls: every use
-// is fenced by the barriers of the chunk loop).
 // Split tiles: a tile whose bin is longer than split_max triangles (a
 // multiple of CHUNK) is processed as several work items of at most
 // split_max triangles each.  The

@@ -152,10 +152,11 @@ __device__ __forceinline__ bool cap_hits_cone(float3 S, float cos_rho, float sin
 // Launches one after another on a stream hand over without draining the GPU
 // in between (programmatic dependent launch): a kernel launched with
 // launch_next may have its CTAs placed while its predecessor's last ones still
-// run, and does nothing before grid_wait has seen the predecessor's end and
-// memory; grid_go in the predecessor allows it.  grid_wait comes first in
-// every such kernel, so nothing but the launch itself overlaps, whatever the
-// predecessor is.  A frame's five launches: about 10 us less.
+// run; grid_go in the predecessor allows it.  Nothing before grid_wait, which
+// returns with the predecessor's end and memory, touches global memory: most
+// kernels wait first, and the map kernels evaluate what depends on their
+// arguments alone, in registers and shared memory, before they wait.  A
+// frame's five launches: about 10 us less.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <class... P, class... A>
@@ -397,7 +398,7 @@ __device__ __forceinline__ float2 pstep_cap(float cos_rho, float sin_rho, float2
 
 // Work items of the raster: a tile whose bin is longer than split_max
 // triangles is processed by several CTAs whose results merge order-free
-// (see SplitAcc in raster.cu).
+// (see SplitAcc in tile.cuh).
 constexpr uint32_t SPLIT_SLOTS = 4096;    // split tiles per launch (others run unsplit)
 constexpr uint32_t EXTRA_ITEMS = 1u << 16;  // extra items per launch
 constexpr int SPLIT_MAX_DEFAULT = 512;    // triangles per item of a split tile

@@ -40,7 +40,7 @@ __device__ __forceinline__ int grid_base_of(int l)
     return l == 0 ? grid_base(0) : (l == 1 ? grid_base(1) : (l == 2 ? grid_base(2) : grid_base(3)));
 }
 // latitude and longitude of a cap centre for its place in the grid, by the
-// polynomials 4.4.45 (arccos, error 7e-5) and 4.4.49 (arctan, error 1e-5) of
+// polynomials 4.4.45 (arccos, error 7e-5) and 4.4.47 (arctan, error 1e-5) of
 // Abramowitz and Stegun: the walk's margin of 3e-4 rad covers both errors
 __device__ __forceinline__ float grid_lat(float y)
 {
