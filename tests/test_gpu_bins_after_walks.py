@@ -93,3 +93,31 @@ def test_pairs_of_a_shaded_frame(vsr):
     vsr.bin(m, sc)
     assert sc.bin_pairs() == shaded
     assert vsr.last_device_status() == 0
+
+
+def test_captured_binning_after_walked_frames(vsr):
+    """A binning captured after frames that stored none, its replays, and the
+    eager calls around them; the bins made room for this view before."""
+    tris = torch.from_numpy(_half(8000, 8)).cuda()
+    m = vsr.Map(200, 120, 0.2, 0.9, 0.9, 90.0)
+    sc = vsr.Scene(tris, _turned(0.0))
+    vsr.raster(m, sc)
+    for a in (0.1, 0.2):
+        sc.update(tris, _turned(a))
+        vsr.raster(m, sc)
+    ref = vsr.raster_dense(m, sc)
+    out = {key: torch.zeros_like(ref[key]) for key in KEYS}
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        vsr.bin(m, sc)
+        vsr.raster(m, sc, out=out, binned=True)
+    for _ in range(3):
+        vsr.bin(m, sc)
+        _equal(vsr.raster(m, sc, binned=True), ref)
+        g.replay()
+        torch.cuda.synchronize()
+        _equal(out, ref)
+        _equal(vsr.raster_dense(m, sc), ref)
+        _equal(vsr.raster(m, sc), ref)
+    assert vsr.last_device_status() == 0
