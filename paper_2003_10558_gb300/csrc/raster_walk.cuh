@@ -2,6 +2,8 @@
 // the candidates of a tile), for any pixel step.
 #pragma once
 
+#include <algorithm>
+
 #include "tile.cuh"
 #include "walk.cuh"
 
@@ -283,11 +285,12 @@ inline vsr_status launch_walk(const RasterView& view, const typename Step::In& i
     // smaller blocks, shared from the third on (200k triangles at 256x256:
     // 142 us; in blocks of 512 159 us, of 1024 193 us), but one block without
     // a grid (900 triangles at 256x256: 19 us, shared in blocks of 256 41 us).
+    // A step may share later (SHARE_FROM).
     const int wave = sms * Step::CTAS;
     const bool few = ntiles < wave;
     static_assert(GRID_DIRECT <= WALK_BLOCK, "one block");
     const int block = few && !wi.direct ? Step::FEW_BLOCK : WALK_BLOCK;
-    const int split = few ? 2 : (int)WALK_SPLIT_BLOCKS;
+    const int split = std::max(Step::SHARE_FROM, few ? 2 : (int)WALK_SPLIT_BLOCKS);
     const int helpers = view.T > split * block ? wave : 0;
     auto kern = raster_walk_kernel<Step, false>;
     if constexpr (Step::HOST_OUT) kern = host_out ? raster_walk_kernel<Step, true> : kern;
