@@ -220,7 +220,7 @@ int64_t vsr_scene_size(vsr_scene s);
  * `stream`; later frames bin and rasterize in one launch that stores none,
  * and do not synchronise.  The outputs are the same.
  * Scratch (the grid, 36 B per triangle and 0.8 MB of cell counters; the bins,
- * sized by the first frame; accumulators of shared tiles) is held by the scene
+ * sized by the first frame; 5 MB of accumulators of shared tiles) is held by the scene
  * handle.  A scene must not be rasterized on two streams at the same time. */
 vsr_status vsr_raster(vsr_map m, vsr_scene s, uint32_t* id_dev, float* depth_dev, float* cov_dev, void* stream);
 
@@ -393,7 +393,7 @@ vsr_status vsr_render_host_wait(vsr_scene s);
  * configuration); a frame whose cameras outgrow the bins before that raises
  * VSR_ERR_BIN_OVERFLOW in the device status with its outputs incomplete; the
  * next call grows the bins.  Device memory per view: T x 196 B of set-up
- * records and triangle grid, 0.8 MB of cell counters, 4 MB of accumulators,
+ * records and triangle grid, 0.8 MB of cell counters, 5 MB of accumulators,
  * and for pooled launches its bins.  A batch must not render on two streams
  * at once. */
 typedef struct vsr_batch_s* vsr_batch;

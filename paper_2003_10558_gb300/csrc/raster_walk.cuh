@@ -34,14 +34,15 @@ namespace {
 // until every tile has got that far, 100 us at most: 480 x 480 pixels, 5000
 // triangles 31 us a frame against 51 with 10 us of looks each.
 struct WalkSlots {
-    SplitAcc split;             // WALK_SLOTS accumulators
-    unsigned long long* claim;  // WALK_SLOTS: (tile << 32) | blocks claimed
-    uint32_t* nblk;             // WALK_SLOTS: blocks of the slot's tile; 0 free, ~0 being set up
-    uint32_t* hits;             // WALK_SLOTS: hits of the parts merged so far
+    SplitAcc split;             // accumulators
+    unsigned long long* claim;  // per slot: (tile << 32) | blocks claimed
+    uint32_t* nblk;             // per slot: blocks of its tile; 0 free, ~0 being set up
+    uint32_t* hits;             // per slot: hits of the parts merged so far
     uint32_t* hint;             // where the next owner looks first
     uint32_t* active;           // published tiles
     uint32_t* begun;            // tiles published or known not to be (zero between launches)
     uint32_t* ended;            // CTAs that have ended (zero between launches)
+    uint32_t n;                 // slots that this launch uses: as many as it has tiles, WALK_SLOTS at most
 };
 
 // What a CTA knows of its tile, in shared memory: uniform, and needed only
@@ -134,24 +135,27 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
                          --looks)
                         __nanosleep(250);
                     __threadfence();
-                    wt.slot = *(volatile uint32_t*)slots.active ? WALK_SLOTS : -1;
+                    wt.slot = *(volatile uint32_t*)slots.active ? (int)slots.n : -1;
                 }
                 __syncthreads();
                 if (wt.slot < 0) break;
-                const int from = (int)((blockIdx.x * 37u) % WALK_SLOTS);
-                int mine = WALK_SLOTS;
-                for (int i = threadIdx.x; i < WALK_SLOTS && mine == WALK_SLOTS; i += RT) {
-                    const int c = (from + i) % WALK_SLOTS;
+                // (read from shared memory: as an argument it would be held in a
+                // register through the evaluation)
+                const int ns = wt.slot, from = (int)((blockIdx.x * 37u) % (uint32_t)ns);
+                __syncthreads();
+                int mine = ns;
+                for (int i = threadIdx.x; i < ns && mine == ns; i += RT) {
+                    const int c = from + i < ns ? from + i : from + i - ns;
                     const uint32_t nb = *(volatile uint32_t*)&slots.nblk[c];
                     if (nb != 0u && nb != 0xffffffffu &&
                         (uint32_t)*(volatile unsigned long long*)&slots.claim[c] < nb)
                         mine = i;
                 }
-                if (mine < WALK_SLOTS) atomicMin(&wt.slot, mine);
+                if (mine < ns) atomicMin(&wt.slot, mine);
                 __syncthreads();
                 slot = wt.slot;
-                if (slot == WALK_SLOTS) break;
-                slot = (from + slot) % WALK_SLOTS;
+                if (slot == ns) break;
+                slot = from + slot < ns ? from + slot : from + slot - ns;
                 if (threadIdx.x == 0) {
                     const unsigned long long c = atomicAdd(&slots.claim[slot], 1ull);
                     wt.tile = (int)(c >> 32);
@@ -172,7 +176,7 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
                 if (!helper && nblk > split_blocks) {
                     const uint32_t from = atomicAdd(slots.hint, 1u);
                     for (uint32_t i = 0; i < 8u && slot < 0; ++i) {
-                        const uint32_t c = (from + i) % WALK_SLOTS;
+                        const uint32_t c = (from + i) % slots.n;
                         if (atomicCAS(&slots.nblk[c], 0u, 0xffffffffu) == 0u) {
                             atomicExch(&slots.claim[c], (unsigned long long)(uint32_t)tile << 32 | 1ull);
                             __threadfence();
@@ -276,6 +280,7 @@ inline vsr_status launch_walk(const RasterView& view, const typename Step::In& i
     sl.nblk = sl.split.done + WALK_SLOTS;
     sl.hits = sl.nblk + WALK_SLOTS;
     sl.hint = sl.hits + WALK_SLOTS;
+    sl.n = (uint32_t)std::min(ntiles, WALK_SLOTS);
     sl.active = sl.hint + 1;
     sl.begun = sl.hint + 2;
     sl.ended = sl.hint + 3;
