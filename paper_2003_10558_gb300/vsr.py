@@ -178,10 +178,12 @@ def _stream_ptr(stream):
     if stream is not None:
         return stream.cuda_stream
     import torch
-    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)  # not public: may be gone one day
-    if raw is None:
-        return torch.cuda.current_stream().cuda_stream
-    return raw(torch.cuda.current_device())
+    if torch.cuda.is_initialized():
+        try:  # not public: may be gone one day
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        except AttributeError:
+            pass
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _dptr(t):

@@ -16,7 +16,7 @@ def test_given_stream():
 @pytest.mark.parametrize("private", [True, False])
 def test_current_stream(monkeypatch, private):
     monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
-    monkeypatch.setattr(torch.cuda, "current_device", lambda: 2)
+    monkeypatch.setattr(torch._C, "_cuda_getDevice", lambda: 2, raising=False)
     monkeypatch.setattr(torch.cuda, "current_stream", lambda: SimpleNamespace(cuda_stream=40))
     if private:
         monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda d: 38 + d, raising=False)
