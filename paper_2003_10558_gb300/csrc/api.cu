@@ -822,7 +822,7 @@ vsr_status host_frame_front(vsr_map m, vsr_scene sc, const float* tris_host, int
             cudaEventCreateWithFlags(&sc->use_event, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&sc->setup_event, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&sc->host_done, cudaEventDisableTiming) != cudaSuccess ||
-            sc->host_status.alloc(1, sc->side) != VSR_OK) {
+            sc->host_status.alloc(1) != VSR_OK) {
             cudaGetLastError();
             if (sc->side) cudaStreamDestroy(sc->side);
             if (sc->use_event) cudaEventDestroy(sc->use_event);
@@ -880,8 +880,8 @@ vsr_status host_frame_front(vsr_map m, vsr_scene sc, const float* tris_host, int
 vsr_status host_frame_back(vsr_map m, vsr_scene sc, const HostFrame& f, uint32_t* id_host, float* depth_host,
                            float* cov_host, cudaStream_t st)
 {
-    const StatusRef saved_status = sc->status;
-    sc->status = sc->host_status.ref();
+    int* const saved_status = sc->status;
+    sc->status = sc->host_status.dev;
     vsr_status s = raster_frame(m, sc, f.id_d, f.depth_d, f.cov_d, st, f.in_place);
     sc->status = saved_status;
     if (s == VSR_OK && f.stage_id && cudaMemcpyAsync(id_host, f.id_d, 4 * f.npix, cudaMemcpyDeviceToHost, st))
@@ -900,9 +900,7 @@ vsr_status host_frame_back(vsr_map m, vsr_scene sc, const HostFrame& f, uint32_t
 // above the capacity), else what its kernels raised.
 vsr_status host_frame_result(vsr_scene sc, uint64_t map_gen)
 {
-    // (cleared on the scene's own stream, which later frames' launches follow)
-    const vsr_status raised = sc->host_status.take(sc->side);
-    if (raised != VSR_OK && cudaStreamSynchronize(sc->side) != cudaSuccess) return VSR_ERR_CUDA;
+    const vsr_status raised = sc->host_status.take();
     const bool outgrew =
         sc->total_pending && sc->total_map == map_gen && sc->total_scene == sc->gen && *sc->h_total > sc->cap;
     return outgrew ? VSR_ERR_BIN_OVERFLOW : raised;

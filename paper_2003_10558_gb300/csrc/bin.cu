@@ -276,7 +276,7 @@ constexpr int BIN_BIG_CHUNK = 16;
 template <bool FILL, int CB, int TPW>
 __global__ void __launch_bounds__(128, CB == 1 ? 12 : (CB == 2 ? 10 : 1)) bin_kernel(BinView v, int T,
                                                                                    uint32_t* __restrict__ ids,
-                                                                     uint32_t cap, StatusRef status)
+                                                                     uint32_t cap, int* status)
 {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -587,7 +587,7 @@ vsr_status launch_bin_count(const float4* rec, int T, TileIndex idx, uint32_t* c
 }
 
 vsr_status launch_bin_fill(const float4* rec, int T, TileIndex idx, const uint32_t* offsets, uint32_t* counts,
-                           uint32_t* ids, uint32_t cap, StatusRef status, cudaStream_t st)
+                           uint32_t* ids, uint32_t cap, int* status, cudaStream_t st)
 {
     if (T == 0) return VSR_OK;
     const BinView v{idx.hdr, idx.cell_start, idx.sorted, idx.big, rec, counts, offsets, idx.ntiles};

@@ -295,7 +295,7 @@ struct FragCountStep : FragStep {
     }
     // the tile's range of the lists, its pixels in thread order
     template <bool ROWS>
-    __device__ __forceinline__ static void finish(const Ctx& cx, const TilePos& tp, const Pix& q, const StatusRef&)
+    __device__ __forceinline__ static void finish(const Ctx& cx, const TilePos& tp, const Pix& q, int*)
     {
         __shared__ uint32_t s_sum[RT / 32], s_base;
         const FragArgs& v = cx.in;
@@ -409,7 +409,7 @@ struct FragFillStep : FragStep {
         }
     }
     template <bool ROWS>
-    __device__ __forceinline__ static void finish(const Ctx& cx, const TilePos& tp, const Pix& q, StatusRef status)
+    __device__ __forceinline__ static void finish(const Ctx& cx, const TilePos& tp, const Pix& q, int* status)
     {
         using Keys = FragKeys<sizeof(Stage) / (5 * RT)>;
         static_assert(sizeof(Keys) <= sizeof(Stage), "the keys take the triangles' place");

@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(WALK_THREADS) bin_walk_kernel(const float4* re
                                                                uint32_t* __restrict__ ctr,
                                                                uint32_t* __restrict__ starts,
                                                                uint32_t* __restrict__ ends,
-                                                               uint32_t* __restrict__ ids, uint32_t cap, StatusRef status,
+                                                               uint32_t* __restrict__ ids, uint32_t cap, int* status,
                                                                uint32_t* total_host)
 {
     grid_wait();
@@ -371,7 +371,7 @@ vsr_status launch_grid_file(const float4* rec, int T, const TriGrid& g, cudaStre
 
 vsr_status launch_bin_walk(const float4* rec, int T, const WalkIndex& wi, const float4* geom, const Cone* tiles,
                            int ntiles, uint32_t* ctr, uint32_t* starts, uint32_t* ends, uint32_t* ids, uint32_t cap,
-                           bool sizing, StatusRef status, uint32_t* total_host, cudaStream_t st)
+                           bool sizing, int* status, uint32_t* total_host, cudaStream_t st)
 {
     if (T < 0 || ntiles <= 0 || (!wi.direct && !wi.start)) return VSR_ERR_INVALID_ARG;
     const int sms = sm_count();

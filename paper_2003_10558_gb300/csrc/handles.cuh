@@ -40,22 +40,16 @@ struct vsr_map_s {
     uint64_t gen = 0;
 };
 
-// Status words that kernels raise errors in and the host learns of without a
-// copy: device words, each with a word in mapped host memory that receives the
-// first error.  Both are zero between frames; `take` reads and clears once a
-// frame's launches have completed, the device word (only after an error) on st,
-// before the owner's next launches there.
+// Status words in host memory that kernels raise errors in (mapped into the
+// device's address space): zero between frames, read and cleared by the host
+// once a frame's launches have completed.
 struct HostStatus {
     int* host = nullptr;
-    int* host_dev = nullptr;  // its device address
-    int* word = nullptr;
-    vsr_status alloc(int n, cudaStream_t st)
+    int* dev = nullptr;
+    vsr_status alloc(int n)
     {
         if (cudaHostAlloc((void**)&host, sizeof(int) * (size_t)n, cudaHostAllocMapped) != cudaSuccess ||
-            cudaHostGetDevicePointer((void**)&host_dev, host, 0) != cudaSuccess ||
-            cudaMalloc((void**)&word, sizeof(int) * (size_t)n) != cudaSuccess ||
-            cudaMemsetAsync(word, 0, sizeof(int) * (size_t)n, st) != cudaSuccess ||
-            cudaStreamSynchronize(st) != cudaSuccess) {
+            cudaHostGetDevicePointer((void**)&dev, host, 0) != cudaSuccess) {
             cudaGetLastError();
             release();
             return VSR_ERR_OOM;
@@ -63,23 +57,16 @@ struct HostStatus {
         for (int i = 0; i < n; ++i) host[i] = 0;
         return VSR_OK;
     }
-    StatusRef ref(int i = 0) const { return StatusRef(word + i, host_dev + i); }
-    vsr_status take(cudaStream_t st, int i = 0)
+    vsr_status take(int i = 0)
     {
         const int v = *(volatile int*)&host[i];
-        if (v == 0) return VSR_OK;
         *(volatile int*)&host[i] = 0;
-        if (cudaMemsetAsync(word + i, 0, sizeof(int), st) != cudaSuccess) {
-            cudaGetLastError();
-            return VSR_ERR_CUDA;
-        }
         return (vsr_status)v;
     }
     void release()
     {
         if (host) cudaFreeHost(host);
-        cudaFree(word);
-        host = host_dev = word = nullptr;
+        host = dev = nullptr;
     }
 };
 
@@ -125,9 +112,9 @@ struct vsr_scene_s {
     int64_t tris_alloc = 0;
     void* out_dev = nullptr;  // id | depth | cov staging, 12 B per pixel
     size_t out_alloc = 0;
-    // status word of this scene's kernels: NULL = the per-device word of
-    // vsr_last_device_status; the server gives its workspaces their own
-    StatusRef status;
+    // device status word of this scene's kernels: NULL = the per-device word
+    // of vsr_last_device_status; the server gives its workspaces their own
+    int* status = nullptr;
     // bins sized without waiting for the device when the map's shape changes
     // (the capacity of earlier binnings is kept and only grows): an owner
     // that renders a request again after a bin overflow (the server) needs
@@ -149,7 +136,7 @@ struct vsr_scene_s {
     uint64_t host_map_gen = 0;
 };
 
-inline StatusRef scene_status(const vsr_scene_s* s) { return s->status.word ? s->status : StatusRef(status_word()); }
+inline int* scene_status(const vsr_scene_s* s) { return s->status ? s->status : status_word(); }
 
 // A launch that walks the scene's grid follows on st: its workspace and
 // bookkeeping; the first frame of a shape goes through stored bins first, so

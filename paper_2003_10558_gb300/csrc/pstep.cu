@@ -192,7 +192,7 @@ struct PstepStep {
         for (int p = 0; p < PPT; ++p) q.acc[p] = min(q.acc[p], COV_ONE);
     }
     template <bool ROWS>
-    __device__ __forceinline__ static void finish(const WalkCtx<In>& cx, const TilePos& tp, const Pix& q, const StatusRef&)
+    __device__ __forceinline__ static void finish(const WalkCtx<In>& cx, const TilePos& tp, const Pix& q, int*)
     {
         write_tile<ROWS>(cx.view, tp, q);
     }
@@ -201,7 +201,7 @@ struct PstepStep {
 }  // namespace
 
 vsr_status launch_raster_pstep(const RasterView& view, const float4* deriv, const WalkIndex& wi, const float4* geom,
-                               const WalkWork& work, uint32_t* tile_pairs, StatusRef status, cudaStream_t st)
+                               const WalkWork& work, uint32_t* tile_pairs, int* status, cudaStream_t st)
 {
     return launch_walk<PstepStep>(view, PstepStep::In{deriv}, wi, geom, work, tile_pairs, status, st, false);
 }

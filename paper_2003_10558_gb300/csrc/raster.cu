@@ -233,7 +233,7 @@ struct GlobalStep {
         for (int p = 0; p < PPT; ++p) q.acc[p] = min(q.acc[p], COV_ONE);
     }
     template <bool ROWS>
-    __device__ __forceinline__ static void finish(const WalkCtx<In>& cx, const TilePos& tp, const Pix& q, const StatusRef&)
+    __device__ __forceinline__ static void finish(const WalkCtx<In>& cx, const TilePos& tp, const Pix& q, int*)
     {
         write_tile<ROWS>(cx.view, tp, q);
     }
@@ -245,7 +245,7 @@ struct GlobalStep {
 template <bool STATS, bool ROWS = false>
 __device__ __forceinline__ void raster_tile(const RasterView& view, int tile, Stage& st, bool count_alg,
                                             uint32_t& cnt_alg, uint32_t& cnt_exec, int32_t* __restrict__ n_inside,
-                                            StatusRef status, int range_lo = 0, int range_hi = -1,
+                                            int* __restrict__ status, int range_lo = 0, int range_hi = -1,
                                             int split_slot = -1, int nsplit = 1, SplitAcc split = SplitAcc{})
 {
     const uint32_t* ids = view.ids;
@@ -301,7 +301,7 @@ __device__ __forceinline__ void raster_tile(const RasterView& view, int tile, St
 template <bool STATS>
 __global__ void __launch_bounds__(RT, 7) raster_kernel(RasterView view, unsigned long long* __restrict__ n_alg,
                                                         unsigned long long* __restrict__ n_exec,
-                                                        int32_t* __restrict__ n_inside, StatusRef status)
+                                                        int32_t* __restrict__ n_inside, int* __restrict__ status)
 {
     __shared__ Stage st;
     __shared__ unsigned long long red[2][RT / 32];
@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(RT, VSR_RASTER_CTAS_PER_SM) raster_items_kerne
                                                               const int32_t* split_slot,
                                                               const uint2* extra,
                                                               const uint32_t* n_extra, int split_max,
-                                                              SplitAcc split, StatusRef status)
+                                                              SplitAcc split, int* __restrict__ status)
 {
     grid_wait();
     grid_go();
@@ -376,7 +376,7 @@ __global__ void __launch_bounds__(RT, VSR_RASTER_CTAS_PER_SM) raster_items_kerne
 __global__ void __launch_bounds__(RT, VSR_RASTER_CTAS_PER_SM) raster_pool_kernel(const PoolView* __restrict__ views,
                                                                                  const uint32_t* __restrict__ item_start,
                                                                                  int nviews, uint32_t* __restrict__ queue,
-                                                                                 int split_max, StatusRef status)
+                                                                                 int split_max, int* __restrict__ status)
 {
     __shared__ Stage st;
     __shared__ uint32_t s_item;
@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(RT, VSR_RASTER_CTAS_PER_SM) raster_pool_kernel
 // else the coverage kernel's own evaluation follows.  The outputs equal the
 // binned path's bit for bit (the same arithmetic per pair, and the merge is
 // order-free); its cost is that of W x H x T pair tests.
-__global__ void __launch_bounds__(RT) raster_dense_kernel(RasterView view, StatusRef status)
+__global__ void __launch_bounds__(RT) raster_dense_kernel(RasterView view, int* __restrict__ status)
 {
     __shared__ Stage st;
     const int T = view.T;
@@ -501,7 +501,7 @@ __global__ void items_kernel(const uint32_t* offsets, const uint32_t* ends,
 vsr_status launch_raster(const float4* map, int W, int H, const Cone* tiles, const float4* rec, int T,
                          const uint32_t* offsets, const uint32_t* ids, uint32_t cap, uint32_t* id, float* depth,
                          float* cov, unsigned long long* n_alg, unsigned long long* n_exec, int32_t* n_inside,
-                         StatusRef status, cudaStream_t st, const uint32_t* ends)
+                         int* status, cudaStream_t st, const uint32_t* ends)
 {
     const int tx = (W + TILE - 1) / TILE, ty = (H + TILE - 1) / TILE;
     const RasterView v{map, W, H, tiles, tx, rec, T, offsets, ids, cap, id, depth, cov, ends};
@@ -534,7 +534,7 @@ vsr_status launch_raster_assign(const uint32_t* offsets, uint32_t n_tiles, uint3
 }
 
 vsr_status launch_raster_pool(const PoolView* views_dev, const uint32_t* item_start_dev, int nviews,
-                              uint32_t* queue, int split_max, StatusRef status, cudaStream_t st)
+                              uint32_t* queue, int split_max, int* status, cudaStream_t st)
 {
     if (nviews == 0) return VSR_OK;
     const int sms = sm_count();
@@ -547,7 +547,7 @@ vsr_status launch_raster_pool(const PoolView* views_dev, const uint32_t* item_st
 }
 
 vsr_status launch_raster_items(const RasterView& view, const uint32_t* offsets, uint32_t n_tiles, uint32_t cap,
-                               RasterWork w, int split_max, StatusRef status, cudaStream_t st, bool host_out)
+                               RasterWork w, int split_max, int* status, cudaStream_t st, bool host_out)
 {
     if (n_tiles == 0) return VSR_OK;
     vsr_status s = launch_raster_assign(offsets, n_tiles, cap, w, split_max, st, view.ends);
@@ -586,12 +586,12 @@ void walk_work_free(WalkWork* w)
 }
 
 vsr_status launch_raster_walk(const RasterView& view, const WalkIndex& wi, const float4* geom, const WalkWork& work,
-                              uint32_t* tile_pairs, StatusRef status, cudaStream_t st, bool host_out)
+                              uint32_t* tile_pairs, int* status, cudaStream_t st, bool host_out)
 {
     return launch_walk<GlobalStep>(view, GlobalStep::In{}, wi, geom, work, tile_pairs, status, st, host_out);
 }
 
-vsr_status launch_raster_dense(const RasterView& view, StatusRef status, cudaStream_t st)
+vsr_status launch_raster_dense(const RasterView& view, int* status, cudaStream_t st)
 {
     const int n_tiles = view.tiles_x * ((view.H + TILE - 1) / TILE);
     if (n_tiles == 0) return VSR_OK;

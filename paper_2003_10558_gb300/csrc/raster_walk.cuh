@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
                                                                      uint32_t block, uint32_t split_blocks, bool early,
                                                                      WalkSlots slots,
                                                                      uint32_t* __restrict__ tile_pairs,
-                                                                     StatusRef status)
+                                                                     int* __restrict__ status)
 {
     grid_wait();
     grid_go();
@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
 // grid and arguments of a walking raster over `work`'s slots
 template <class Step>
 inline vsr_status launch_walk(const RasterView& view, const typename Step::In& in, const WalkIndex& wi,
-                              const float4* geom, const WalkWork& work, uint32_t* tile_pairs, StatusRef status,
+                              const float4* geom, const WalkWork& work, uint32_t* tile_pairs, int* status,
                               cudaStream_t st, bool host_out)
 {
     const int ntiles = view.tiles_x * ((view.H + TILE - 1) / TILE);

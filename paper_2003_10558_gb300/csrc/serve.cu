@@ -304,7 +304,7 @@ struct vsr_server_s {
                     continue;
                 }
                 vsr_scene_s* w = sl.work;
-                const vsr_status raised = status.take(sl.stream, (int)(&sl - slots.data()));
+                const vsr_status raised = status.take((int)(&sl - slots.data()));
                 const bool overflow = *w->h_total > w->cap;
                 if (overflow && sl.req.reruns < 3) {
                     // the bins overflowed: vsr_bin grows them from this count; render again
@@ -345,7 +345,7 @@ struct vsr_server_s {
                         finish(q, VSR_ERR_OOM, now_s(), hit);
                         continue;
                     }
-                    w->status = status.ref(si);  // its errors are this server's, not the device's
+                    w->status = status.dev + si;  // its errors are this server's, not the device's
                     w->async_sizing = true;  // a bin overflow renders the request again (below)
                 }
                 sl.req = q;
@@ -392,6 +392,10 @@ vsr_status vsr_serve_create(const vsr_serve_cfg* cfg, vsr_server* out)
         delete s;
         return VSR_ERR_CUDA;
     }
+    if (s->status.alloc(cfg->slots) != VSR_OK) {
+        delete s;
+        return VSR_ERR_OOM;
+    }
     s->slots.resize(cfg->slots);
     s->work.resize(cfg->slots);
     for (Slot& sl : s->slots) {
@@ -401,10 +405,6 @@ vsr_status vsr_serve_create(const vsr_serve_cfg* cfg, vsr_server* out)
             vsr_serve_destroy(s);
             return VSR_ERR_CUDA;
         }
-    }
-    if (s->status.alloc(cfg->slots, s->slots[0].stream) != VSR_OK) {
-        vsr_serve_destroy(s);
-        return VSR_ERR_OOM;
     }
     s->worker = std::thread([s] { s->loop(); });
     *out = s;

@@ -142,7 +142,7 @@ struct WarpCones {
 // Stage triangle t into slot j (an index beyond the records -- never left by a
 // completed binning or grid -- empties the slot and raises the status).
 __device__ __forceinline__ void stage_checked(const float4* rec, int T, uint32_t t, const float4& axis,
-                                              Stage& st, int j, StatusRef status)
+                                              Stage& st, int j, int* status)
 {
     if (t >= (uint32_t)T) {
         raise_status(status, VSR_ERR_BIN_OVERFLOW);

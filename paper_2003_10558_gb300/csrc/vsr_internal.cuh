@@ -114,19 +114,11 @@ struct TileIndexHdr {
     unsigned hist[IDX_HIST];    // third-of-an-octave histogram of half-angles
 };
 
-// Device-side status word (vsr_status values; 0 = OK), one int per device, host
-// path or server slot, passed to the kernels that can fail.  `host` (optional):
-// the device address of a word in host memory to which the first to raise an
-// error copies it: an overflow is raised by thousands of tiles, whose atomics
-// do not cross the host link.
-struct StatusRef {
-    int* word;
-    int* host;
-    __host__ __device__ StatusRef(int* w = nullptr, int* h = nullptr) : word(w), host(h) {}
-};
-__device__ __forceinline__ void raise_status(const StatusRef& status, int code)
+// Device-side status word (vsr_status values; 0 = OK), one int per device
+// owned by the host library and passed to the kernels that can fail.
+__device__ __forceinline__ void raise_status(int* status, int code)
 {
-    if (status.word && atomicCAS(status.word, 0, code) == 0 && status.host) *(volatile int*)status.host = code;
+    if (status) atomicCAS(status, 0, code);
 }
 
 // Conservative test: may a cap (centre S, cos/sin of radius, enlarged by the
@@ -263,7 +255,7 @@ __device__ __forceinline__ Cone index_entry(const Cone& c, int i)
 vsr_status launch_bin_count(const float4* rec, int T, TileIndex idx, uint32_t* counts, cudaStream_t st);
 vsr_status launch_scan(const uint32_t* counts, int n, uint32_t* offsets, cudaStream_t st);
 vsr_status launch_bin_fill(const float4* rec, int T, TileIndex idx, const uint32_t* offsets, uint32_t* counts,
-                           uint32_t* ids, uint32_t cap, StatusRef status, cudaStream_t st);
+                           uint32_t* ids, uint32_t cap, int* status, cudaStream_t st);
 
 // ---------------------------------------------------------------------------
 // Triangle grid: the triangles of a set-up by the place of their caps on the
@@ -348,7 +340,7 @@ constexpr int BIN_SHARES = 1024, BIN_SHARE_WORDS = 8, BIN_CTR_SHARES = 8;
 constexpr int BIN_CTR_WORDS = BIN_CTR_SHARES + BIN_SHARES * BIN_SHARE_WORDS;
 vsr_status launch_bin_walk(const float4* rec, int T, const WalkIndex& wi, const float4* geom, const Cone* tiles,
                            int ntiles, uint32_t* ctr, uint32_t* starts, uint32_t* ends, uint32_t* ids, uint32_t cap,
-                           bool sizing, StatusRef status, uint32_t* total_host, cudaStream_t st);
+                           bool sizing, int* status, uint32_t* total_host, cudaStream_t st);
 // One view as the raster kernel sees it: its map, tile cones, set-up
 // records, bin offsets (indexed by the view's own tile number), bin ids and
 // outputs.
@@ -458,12 +450,12 @@ vsr_status launch_raster_assign(const uint32_t* offsets, uint32_t n_tiles, uint3
 // items item_start[v] .. item_start[v + 1] - 1 (its tiles, then its extra
 // items); queue: a device counter (zeroed here)
 vsr_status launch_raster_pool(const PoolView* views_dev, const uint32_t* item_start_dev, int nviews,
-                              uint32_t* queue, int split_max, StatusRef status, cudaStream_t st);
+                              uint32_t* queue, int split_max, int* status, cudaStream_t st);
 // items + raster over all tiles of a view; offsets: its bin offsets
 // (n_tiles + 1 entries, or the bins' starts with view.ends); cap: the bins' capacity (bounds the extra items);
 // host_out: the outputs are pinned host memory (written in whole tile rows)
 vsr_status launch_raster_items(const RasterView& view, const uint32_t* offsets, uint32_t n_tiles, uint32_t cap,
-                               RasterWork w, int split_max, StatusRef status, cudaStream_t st, bool host_out = false);
+                               RasterWork w, int split_max, int* status, cudaStream_t st, bool host_out = false);
 // binning and raster in one launch over the grid (raster_walk_kernel): the
 // slots in which the parts of a tile with many candidates merge
 // (at least the tiles of one wave of CTAs, so that where every tile of a small
@@ -481,9 +473,9 @@ constexpr size_t WALK_WORK_BYTES = (size_t)WALK_SLOTS * (16 * TILE_PIX + 20) + 1
 // view: no bins needed; tile_pairs (optional): the triangles found per tile;
 // host_out: as launch_raster_items
 vsr_status launch_raster_walk(const RasterView& view, const WalkIndex& wi, const float4* geom, const WalkWork& work,
-                              uint32_t* tile_pairs, StatusRef status, cudaStream_t st, bool host_out = false);
+                              uint32_t* tile_pairs, int* status, cudaStream_t st, bool host_out = false);
 // the dense reference: every pixel against every triangle, no bins
-vsr_status launch_raster_dense(const RasterView& view, StatusRef status, cudaStream_t st);
+vsr_status launch_raster_dense(const RasterView& view, int* status, cudaStream_t st);
 // allocate / free a RasterWork for up to n_tiles tiles (accumulators cleared
 // with clear_workspace: a clear on another stream would race with the launches)
 vsr_status raster_work_alloc(RasterWork* w, uint32_t n_tiles, cudaStream_t st);
@@ -495,7 +487,7 @@ vsr_status launch_setup_view(const float* tris, int T, const float* cam_dev, flo
 vsr_status launch_raster(const float4* map, int W, int H, const Cone* tiles, const float4* rec, int T,
                          const uint32_t* offsets, const uint32_t* ids, uint32_t cap, uint32_t* id, float* depth,
                          float* cov, unsigned long long* n_alg, unsigned long long* n_exec, int32_t* n_inside,
-                         StatusRef status, cudaStream_t st, const uint32_t* ends = nullptr);
+                         int* status, cudaStream_t st, const uint32_t* ends = nullptr);
 
 // ---------------------------------------------------------------------------
 // Differentiable path (grad.cu, map.cu).
@@ -531,7 +523,7 @@ struct FragArgs {
     float* cov;
     uint32_t* out_id;
     float* out_depth;
-    StatusRef status;
+    int* status;
 };
 // tile_pairs: the triangles found per tile, as launch_raster_walk
 vsr_status launch_frag_count(const FragArgs& a, const WalkWork& work, uint32_t* tile_pairs, cudaStream_t st);
@@ -552,4 +544,4 @@ vsr_status launch_map_backward(int W, int H, int aov, float k, float l, float s,
 // launch_raster_walk with a pstep index; deriv: 2 float4 per pixel from
 // launch_map_spec
 vsr_status launch_raster_pstep(const RasterView& view, const float4* deriv, const WalkIndex& wi, const float4* geom,
-                               const WalkWork& work, uint32_t* tile_pairs, StatusRef status, cudaStream_t st);
+                               const WalkWork& work, uint32_t* tile_pairs, int* status, cudaStream_t st);

@@ -1,7 +1,7 @@
 """Errors that the kernels of the host path and of the server raise reach the
 caller: the frame that raised one reports it, the next one is clean again.  The
-error is raised from the host, in the host memory that the kernels copy theirs
-to (the first member of either handle), between frames."""
+error is raised from the host, in the status word that the kernels would raise
+it in (the first member of either handle, mapped host memory), between frames."""
 import ctypes
 
 import numpy as np
