@@ -91,7 +91,10 @@ __device__ __forceinline__ void walk_eval(const WalkCtx<typename Step::In>& cx, 
 // Step: how pixels are loaded, culled against, evaluated and written (the
 // global step of raster.cu, the per-fragment step of pstep.cu, the fragment
 // lists of grad.cu).
-template <class Step, bool ROWS>
+// SHARE: the launch has helpers (no tile of one without them has enough
+// candidates to be shared, and a small frame waits for every line of code that
+// its kernel has to fetch).
+template <class Step, bool ROWS, bool SHARE>
 __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView view, typename Step::In in, WalkIndex wi,
                                                                      const float4* geom, int ntiles,
                                                                      uint32_t block, uint32_t split_blocks, bool early,
@@ -107,11 +110,11 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
     __shared__ WalkTile wt;
     __shared__ uint32_t s_ids[WALK_BLOCK];
     static_assert(RT == WALK_THREADS, "the walk's CTA");
-    const bool helper = blockIdx.x >= (uint32_t)ntiles;
+    const bool helper = SHARE && blockIdx.x >= (uint32_t)ntiles;
     int looks = early ? 400 : 0;
     // a tile is past its publication
     auto begun = [&] {
-        if (early) {
+        if (SHARE && early) {
             __threadfence();
             atomicAdd(slots.begun, 1u);
         }
@@ -173,7 +176,7 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
             if (threadIdx.x < 32) walk_ranges(wi, view.T, geom[tile], axis.y, ws);
             if (threadIdx.x == 0) {
                 const uint32_t nblk = (ws.total + block - 1) / block;
-                if (!helper && nblk > split_blocks) {
+                if (SHARE && !helper && nblk > split_blocks) {
                     const uint32_t from = atomicAdd(slots.hint, 1u);
                     for (uint32_t i = 0; i < 8u && slot < 0; ++i) {
                         const uint32_t c = (from + i) % slots.n;
@@ -216,13 +219,13 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
             }
             // the only block of a tile that is not shared (almost every tile):
             // no one waits for the others' evaluation
-            if (wt.nblk == 1u && wt.slot < 0) break;
+            if (wt.nblk == 1u && (!SHARE || wt.slot < 0)) break;
             __syncthreads();
             if (threadIdx.x == 0) {
                 wt.hits += wt.n;
                 wt.n = 0u;
                 ++wt.units;
-                wt.next = wt.slot >= 0 ? (uint32_t)atomicAdd(&slots.claim[wt.slot], 1ull) : wt.next + 1u;
+                wt.next = SHARE && wt.slot >= 0 ? (uint32_t)atomicAdd(&slots.claim[wt.slot], 1ull) : wt.next + 1u;
             }
             __syncthreads();
         }
@@ -232,7 +235,7 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
         const TilePos tp(tile, view.tiles_x);
         uint32_t hits = wt.hits + wt.n;
         bool last = true;
-        if (slot >= 0) {
+        if (SHARE && slot >= 0) {
             if (threadIdx.x == 0 && hits) atomicAdd(&slots.hits[slot], hits);
             last = merge_slot<Step::SATURATES>(slots.split, slot, tp, q, wt.units, wt.nblk);
             if (last) {
@@ -252,7 +255,7 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
         }
         if (!helper) break;
     }
-    if (early && threadIdx.x == 0) {
+    if (SHARE && early && threadIdx.x == 0) {
         __threadfence();
         if (atomicAdd(slots.ended, 1u) == gridDim.x - 1) {
             atomicExch(slots.begun, 0u);
@@ -297,8 +300,10 @@ inline vsr_status launch_walk(const RasterView& view, const typename Step::In& i
     const int block = few && !wi.direct ? Step::FEW_BLOCK : WALK_BLOCK;
     const int split = std::max(Step::SHARE_FROM, few ? 2 : (int)WALK_SPLIT_BLOCKS);
     const int helpers = view.T > split * block ? wave : 0;
-    auto kern = raster_walk_kernel<Step, false>;
-    if constexpr (Step::HOST_OUT) kern = host_out ? raster_walk_kernel<Step, true> : kern;
+    auto kern = helpers ? raster_walk_kernel<Step, false, true> : raster_walk_kernel<Step, false, false>;
+    if constexpr (Step::HOST_OUT) {
+        if (host_out) kern = helpers ? raster_walk_kernel<Step, true, true> : raster_walk_kernel<Step, true, false>;
+    }
     VSR_CUDA_TRY(launch_next(kern, ntiles + helpers, RT, st, view, in, wi, geom, ntiles, (uint32_t)block,
                              (uint32_t)split, helpers && (few || Step::SKIPS), sl, tile_pairs, status));
     return VSR_OK;
