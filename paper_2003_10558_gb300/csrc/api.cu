@@ -594,10 +594,11 @@ static vsr_status bin_scene(vsr_map m, vsr_scene sc, int pstep, cudaStream_t st)
     // binning (copied to pinned memory, read only once its event has
     // completed, never waited for) grows the capacity ahead of need, and the
     // binning kernels report any overflow in the status word.  A capture can
-    // neither wait nor query: it takes the bins as they are.
+    // neither wait nor query: it takes the bins as they are, and the next
+    // eager binning sizes them.
     bool captures;
     if ((s = stream_captures(st, &captures)) != VSR_OK) return s;
-    const bool resize = !bins_sized(m, sc, pstep) || (sc->walked_last && !sc->async_sizing && !captures);
+    const bool resize = !bins_sized(m, sc, pstep) || (sc->size_due && !sc->async_sizing && !captures);
     if (!resize && !captures && sc->total_pending && cudaEventQuery(sc->total_event) == cudaSuccess) {
         sc->total_pending = false;
         const uint64_t last = *sc->h_total;
@@ -639,6 +640,7 @@ static vsr_status bin_scene(vsr_map m, vsr_scene sc, int pstep, cudaStream_t st)
         const uint64_t shape = bin_shape_of(m, sc);
         sc->sized_pstep = pstep != 0 || (sc->sized_pstep && sc->sized_shape == shape);
         sc->sized_shape = shape;
+        sc->size_due = false;
     }
     sc->binned_map = m->gen;
     sc->binned_scene = sc->gen;
@@ -692,6 +694,7 @@ vsr_status walk_begin(vsr_map m, vsr_scene sc, cudaStream_t st)
     sc->walked_map = m->gen;
     sc->walked_scene = sc->gen;
     sc->walked_last = true;
+    sc->size_due = true;
     return VSR_OK;
 }
 }  // namespace

@@ -96,6 +96,7 @@ struct vsr_scene_s {
     uint32_t* tile_pairs = nullptr;
     uint64_t walked_map = 0, walked_scene = 0;
     bool walked_last = false;
+    bool size_due = false;              // frames have walked since the bins were sized
     uint64_t sized_shape = 0;           // (tiles, T) the bins were last sized for,
     bool sized_pstep = false;           // with the wider caps of the pixel step
     uint32_t* h_total = nullptr;        // pinned: pair total of a recent binning

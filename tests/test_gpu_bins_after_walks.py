@@ -121,3 +121,26 @@ def test_captured_binning_after_walked_frames(vsr):
         _equal(vsr.raster_dense(m, sc), ref)
         _equal(vsr.raster(m, sc), ref)
     assert vsr.last_device_status() == 0
+
+
+def test_eager_bins_after_a_capture_that_sized_none(vsr):
+    """A capture between the walked frames and an eager binning sizes nothing:
+    the eager one still holds the denser view."""
+    tris = torch.from_numpy(_half(20_000, 9)).cuda()
+    m = vsr.Map(320, 240, 0.2, 0.9, 0.9, 60.0)
+    sc = vsr.Scene(tris, _turned(np.pi))
+    out = vsr.raster(m, sc)  # sized for a view of almost nothing
+    vsr.raster(m, sc, out=out, binned=True)  # what a captured binned raster allocates
+    sparse = sc.bin_pairs()
+    for a in np.linspace(np.pi, 0.0, 5)[1:]:
+        sc.update(tris, _turned(a))
+        vsr.raster(m, sc, out=out)
+    assert sc.bin_pairs() > 2 * sparse + 8192
+    ref = vsr.raster_dense(m, sc)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):  # (never launched: its bins are too small for this view)
+        vsr.bin(m, sc)
+    vsr.bin(m, sc)
+    _equal(vsr.raster(m, sc, binned=True), ref)
+    assert vsr.last_device_status() == 0
