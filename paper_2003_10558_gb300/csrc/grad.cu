@@ -255,7 +255,7 @@ struct FragStep {
 
 struct FragCountStep : FragStep {
     static constexpr bool SKIPS = false;
-    static constexpr int SHARE_FROM = 0;
+    static constexpr int FEW_FROM = 2, SHARE_FROM = 3;
     static constexpr int CTAS = 8;  // 64 registers; 7: 40.2 us, 6: 44.0 us against 39.4 us
     using Pix = FragCount;
     using Ctx = WalkCtx<FragArgs>;
@@ -355,7 +355,7 @@ struct FragFillStep : FragStep {
     // third, seventh, eleventh block: 5000 triangles of 0.3 rad at 64x64 484,
     // 334, 335 us; 50k of 0.1 rad at 256x256 486, 417, 412; 100k small ones at
     // 128x128 652, 578, 575; 300k 1243, 1233, 1514.
-    static constexpr int SHARE_FROM = 6;
+    static constexpr int FEW_FROM = 6, SHARE_FROM = 6;
     static constexpr int CTAS = 5;
     using Pix = FragAppend;
     using Ctx = WalkCtx<FragArgs>;

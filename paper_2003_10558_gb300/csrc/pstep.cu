@@ -50,7 +50,7 @@ __device__ __forceinline__ float ramp(float g, float w) { return __fmaf_rn(g, rc
 struct PstepStep {
     static constexpr int FEW_BLOCK = WALK_BLOCK / 4;
     static constexpr bool SATURATES = true, HOST_OUT = false, SKIPS = false;
-    static constexpr int SHARE_FROM = 0;
+    static constexpr int FEW_FROM = 2, SHARE_FROM = 1;
     static constexpr int CTAS = 6;  // 80 registers; 5: 135.3 us, 4: 142.7 us against 130.4 us
     using Pix = PstepPix;
     using Cones = PstepCones;

@@ -200,7 +200,7 @@ __device__ __forceinline__ void eval_chunk(const Stage& st, int n, const WarpCon
 struct GlobalStep {
     static constexpr int CTAS = VSR_RASTER_CTAS_PER_SM, FEW_BLOCK = WALK_BLOCK / 4;
     static constexpr bool SATURATES = true, HOST_OUT = true, SKIPS = false;
-    static constexpr int SHARE_FROM = 0;
+    static constexpr int FEW_FROM = 2, SHARE_FROM = 1;
     using Pix = PixPair;
     using Cones = WarpCones;
     struct In {};

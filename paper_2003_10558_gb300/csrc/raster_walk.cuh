@@ -38,7 +38,7 @@ struct WalkSlots {
     unsigned long long* claim;  // per slot: (tile << 32) | blocks claimed
     uint32_t* nblk;             // per slot: blocks of its tile; 0 free, ~0 being set up
     uint32_t* hits;             // per slot: hits of the parts merged so far
-    uint32_t* hint;             // where the next owner looks first
+    uint32_t* hint;             // owners so far: where the next one looks first, times WALK_SLOT_STEP
     uint32_t* active;           // published tiles
     uint32_t* begun;            // tiles published or known not to be (zero between launches)
     uint32_t* ended;            // CTAs that have ended (zero between launches)
@@ -50,6 +50,7 @@ struct WalkSlots {
 struct WalkTile {
     Cone cone;
     uint32_t nblk, next;  // blocks of the tile, this CTA's next one
+    uint32_t block;       // candidates of a block
     uint32_t units, hits;  // blocks done and hits found by this CTA
     int tile, slot;        // slot: -1 unless the tile is shared
     uint32_t n;            // hits of the current block
@@ -91,14 +92,16 @@ __device__ __forceinline__ void walk_eval(const WalkCtx<typename Step::In>& cx, 
 // Step: how pixels are loaded, culled against, evaluated and written (the
 // global step of raster.cu, the per-fragment step of pstep.cu, the fragment
 // lists of grad.cu).
+// block: candidates of a block where one CTA has the tile; share_from: tiles of
+// more candidates are shared, in blocks of share_block.
 // SHARE: the launch has helpers (no tile of one without them has enough
 // candidates to be shared, and a small frame waits for every line of code that
 // its kernel has to fetch).
 template <class Step, bool ROWS, bool SHARE>
 __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView view, typename Step::In in, WalkIndex wi,
                                                                      const float4* geom, int ntiles,
-                                                                     uint32_t block, uint32_t split_blocks, bool early,
-                                                                     WalkSlots slots,
+                                                                     uint32_t block, uint32_t share_from,
+                                                                     uint32_t share_block, bool early, WalkSlots slots,
                                                                      uint32_t* __restrict__ tile_pairs,
                                                                      int* __restrict__ status)
 {
@@ -175,15 +178,16 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
             if (threadIdx.x == RT - 1) wt.cone = view.tiles[tile];
             if (threadIdx.x < 32) walk_ranges(wi, view.T, geom[tile], axis.y, ws);
             if (threadIdx.x == 0) {
-                const uint32_t nblk = (ws.total + block - 1) / block;
-                if (SHARE && !helper && nblk > split_blocks) {
-                    const uint32_t from = atomicAdd(slots.hint, 1u);
+                const bool crowded = SHARE && ws.total > share_from;
+                const uint32_t parts = (ws.total + share_block - 1) / share_block;
+                if (crowded && !helper) {
+                    const uint32_t from = atomicAdd(slots.hint, 1u) * WALK_SLOT_STEP;
                     for (uint32_t i = 0; i < 8u && slot < 0; ++i) {
                         const uint32_t c = (from + i) % slots.n;
                         if (atomicCAS(&slots.nblk[c], 0u, 0xffffffffu) == 0u) {
                             atomicExch(&slots.claim[c], (unsigned long long)(uint32_t)tile << 32 | 1ull);
                             __threadfence();
-                            atomicExch(&slots.nblk[c], nblk);
+                            atomicExch(&slots.nblk[c], parts);
                             atomicAdd(slots.active, 1u);
                             slot = (int)c;
                         }
@@ -191,7 +195,9 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
                 }
                 wt.tile = tile;
                 wt.slot = slot;
-                wt.nblk = nblk;
+                const bool shared = SHARE && (helper || slot >= 0);
+                wt.block = shared ? share_block : block;
+                wt.nblk = shared ? parts : (ws.total + block - 1) / block;
                 wt.next = first;
                 wt.units = wt.hits = wt.n = 0u;
                 if (!helper) begun();
@@ -204,8 +210,8 @@ __global__ void __launch_bounds__(RT, Step::CTAS) raster_walk_kernel(RasterView 
             {
                 Walk w;
                 w.init(wi, wt.cone, ws);
-                const uint32_t e0 = wt.next * block;
-                walk_hits(w, wi, view.rec, view.T, ws, e0, min(ws.total, e0 + block), s_ids, &wt.n);
+                const uint32_t e0 = wt.next * wt.block;
+                walk_hits(w, wi, view.rec, view.T, ws, e0, min(ws.total, e0 + wt.block), s_ids, &wt.n);
             }
             __syncthreads();
             for (uint32_t base = 0; base < wt.n; base += CHUNK) {
@@ -287,25 +293,34 @@ inline vsr_status launch_walk(const RasterView& view, const typename Step::In& i
     sl.active = sl.hint + 1;
     sl.begun = sl.hint + 2;
     sl.ended = sl.hint + 3;
-    // Helpers only where a tile can have enough candidates.  A tile is shared
-    // from its fourth block of 1024 on (1M triangles at 1920x1080, a 340 degree
-    // lens: 912 us; from the second 1417, from the ninth 1149).  Few tiles:
-    // smaller blocks, shared from the third on (200k triangles at 256x256:
-    // 142 us; in blocks of 512 159 us, of 1024 193 us), but one block without
-    // a grid (900 triangles at 256x256: 19 us, shared in blocks of 256 41 us).
-    // A step may share later (SHARE_FROM).
+    // Helpers only where a tile can have enough candidates.  Pictures of fewer
+    // tiles than CTAs are resident: small blocks, a tile shared from its third
+    // on (200k triangles at 256x256: 142 us; in blocks of 512 159 us, of 1024
+    // 193 us), but one block without a grid (900 triangles at 256x256: 19 us,
+    // shared in blocks of 256 41 us).  Larger pictures: large blocks, but a tile
+    // of more than one is shared, in small ones, so that an object in few tiles
+    // is not left to few CTAs.  1920x1080, a raster shared so, shared from the
+    // fourth large block on, and over bins stored before it: 200k triangles in
+    // 0.06 rad 240, 302, 297 us; 100k in 0.02 rad 151, 251, 222; in an even
+    // cloud under a 340 degree lens 300k 205, 361, 246, 1M 419, 452, 454; of
+    // 200k small ones 121.5 both, 140 stored.  Where an even cloud already gives
+    // its tiles that many (over 128 triangles a tile), from the third large block
+    // on: 1M at 1024x1024 from inside 231 us from the second, 226 from the third
+    // or the fourth.  A step may share later (FEW_FROM, SHARE_FROM).
     const int wave = sms * Step::CTAS;
     const bool few = ntiles < wave;
-    static_assert(GRID_DIRECT <= WALK_BLOCK, "one block");
+    static_assert(GRID_DIRECT <= WALK_BLOCK && Step::FEW_BLOCK <= WALK_BLOCK, "one block, and its hits");
     const int block = few && !wi.direct ? Step::FEW_BLOCK : WALK_BLOCK;
-    const int split = std::max(Step::SHARE_FROM, few ? 2 : (int)WALK_SPLIT_BLOCKS);
-    const int helpers = view.T > split * block ? wave : 0;
+    const int share = few ? Step::FEW_FROM : std::max(Step::SHARE_FROM, view.T / 128 > ntiles ? 2 : 1);
+    const int share_from = share * block;
+    const int helpers = view.T > share_from ? wave : 0;
     auto kern = helpers ? raster_walk_kernel<Step, false, true> : raster_walk_kernel<Step, false, false>;
     if constexpr (Step::HOST_OUT) {
         if (host_out) kern = helpers ? raster_walk_kernel<Step, true, true> : raster_walk_kernel<Step, true, false>;
     }
     VSR_CUDA_TRY(launch_next(kern, ntiles + helpers, RT, st, view, in, wi, geom, ntiles, (uint32_t)block,
-                             (uint32_t)split, helpers && (few || Step::SKIPS), sl, tile_pairs, status));
+                             (uint32_t)share_from, (uint32_t)Step::FEW_BLOCK, helpers && (few || Step::SKIPS), sl,
+                             tile_pairs, status));
     return VSR_OK;
 }
 
