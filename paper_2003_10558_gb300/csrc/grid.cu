@@ -151,7 +151,9 @@ __global__ void __launch_bounds__(WALK_THREADS) bin_walk_kernel(const float4* re
     // takes the range of a tile with n hits
     auto take_range = [&](int tile, uint32_t n) {
         const uint32_t start = n ? atomicAdd(&ctr[0], n) : 0u;
-        if (!sizing && (uint64_t)start + n > cap) raise_status(status, VSR_ERR_BIN_OVERFLOW);
+        // (raised once, by the tile that lies across the bins' end: the word may
+        // be host memory, and thousands can lie beyond)
+        if (!sizing && start <= cap && (uint64_t)start + n > cap) raise_status(status, VSR_ERR_BIN_OVERFLOW);
         starts[tile] = start;
         ends[tile] = start + n;
         return start;

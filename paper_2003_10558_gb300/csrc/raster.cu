@@ -263,7 +263,7 @@ __device__ __forceinline__ void raster_tile(const RasterView& view, int tile, St
         b0 = view.offsets[tile];
         b1 = view.ends ? view.ends[tile] : view.offsets[tile + 1];
         if (b1 > cap) {
-            if (threadIdx.x == 0) raise_status(status, VSR_ERR_BIN_OVERFLOW);
+            if (threadIdx.x == 0 && b0 <= cap) raise_status(status, VSR_ERR_BIN_OVERFLOW);  // (as the binning, once)
             b1 = cap;
             b0 = min(b0, cap);
         }
